@@ -29,6 +29,7 @@
 #include "metric.cuh"
 #include "pivot_dense.cuh"
 #include "tile_l1.cuh"
+#include "tile_l2f.cuh"
 #include "tile_str.cuh"
 #include "tile_tc.cuh"
 #include "scan.cuh"
@@ -38,6 +39,11 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kWarpsPerBlock = kT / 32;
+constexpr int64_t kF32TileEntries = 4;           // FP32 tiles: least last-level entries per node
+constexpr int64_t kF32TilePairs = 6 << 20;       // and least (entry, row) pairs (f32_tiles_pay)
+constexpr int64_t kF32DenseQueries = 64;         // dense pivot matrices in FP32: one full tile of queries
+constexpr int64_t kF32TileBudget = (int64_t)1 << 30;   // and least memory budget: the regrouped records take about
+                                                       // 60 bytes per entry beside the budgeted tables
 constexpr int kKeepCap = 2048;   // exact-key candidates staged in shared memory per query
 
 inline unsigned nblocks(int64_t work, int per) {
@@ -2369,6 +2375,7 @@ struct Runner {
     StageClock clk;
     bool use_tc = false;   // BF16 tensor-core tiles at the last level (L2)
     bool use_l1 = false;   // FP32 CUDA-core tiles at the last level (L1)
+    bool use_f32 = false;  // GTS_PREC_FP32: FP32 CUDA-core tiles where the last level's nodes hold enough queries
     bool use_qg = false;   // 3-gram filtering tiles at the last level (edit distance)
     bool use_scan = false; // low-dim vectors: node-major table scan + CUDA-core verification
     Tuning tu;             // launch parameters (a copy of the index's)
@@ -2427,7 +2434,7 @@ struct Runner {
     // reaches the level if its frontier holds at least a quarter of the
     // batch's (query, node) pairs and the matrix fits an eighth of the budget.
     const float *dense_for(int l, int64_t E) {
-        if (!(use_tc || use_l1 || use_scan) || d.dim == 0) return nullptr;
+        if (!(use_tc || use_l1 || use_scan || (use_f32 && qb.nq >= kF32DenseQueries)) || d.dim == 0) return nullptr;
         if ((int)dense_state.size() < h) {
             dense_state.assign(h, 0);
             dense.resize(h);
@@ -2553,7 +2560,7 @@ struct Runner {
 
     void process(Level &L, int64_t e0, int64_t e1, int l) {
         if (e1 <= e0) return;
-        if ((use_tc || use_l1 || use_scan) && l == h - 1) {
+        if (l == h - 1 && (use_tc || use_l1 || use_scan || (use_f32 && f32_tiles_pay(e1 - e0)))) {
             last_level_tc(L, e0, e1, l);
             return;
         }
@@ -2960,8 +2967,12 @@ struct Runner {
             scan_leaf(L, e0, e1, mask, ncount);
             return;
         }
-        if (use_l1) {
+        if (use_l1 || (use_f32 && d.metric == GTS_L1)) {
             l1_leaf(L, e0, e1, mask, ncount);
+            return;
+        }
+        if (use_f32) {
+            l2f_leaf(L, e0, e1, mask, ncount);
             return;
         }
         TcQuery tq = tc_query_base();
@@ -3088,6 +3099,58 @@ struct Runner {
         verify_and_collect(q2, r2, C);
     }
 
+    // GTS_PREC_FP32: whether the last level's E entries run as FP32 tiles or
+    // candidate by candidate.  The tiles cost the regrouping (80 to 200 us of
+    // launches and host round trips) and then 4 ps per pair at 128
+    // dimensions, the plain path about 140 ps.  kNN batches, plain / tiles in
+    // us: 3 * 10^5 x 128, 32 queries (5 M pairs) 1501 / 1518, 100 (15 M) 2424 /
+    // 1813, 1000 15877 / 5444; 3 * 10^5 x 17, 32: 1102 / 1161, 100: 1419 /
+    // 1280; L1, 2 * 10^4 x 64, 100 (1 M): 895 / 1082, 3 * 10^5, 100: 2053 / 1743.
+    bool f32_tiles_pay(int64_t E) const {
+        const int64_t nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
+        return E >= kF32TileEntries * nn && E * ((ix->tree.n + nn - 1) / nn) >= kF32TilePairs;
+    }
+
+    // Last level on the FP32 L2 tiles: regroup the entries by node, run the
+    // tiles (leaf mask, visibility and the FP32 distance bound), then verify
+    // the kept pairs as the plain path does.
+    void l2f_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask, DBuf<int32_t> *ncount) {
+        TcQuery tq;
+        tq.E = e1 - e0;
+        tq.nq = qb.nq;
+        tq.eq = L.q.get() + e0;
+        tq.enode = L.node.get() + e0;
+        tq.path = L.path.get() + e0 * h;
+        tq.emask = mask.get();
+        tq.Q = d.Q;
+        tq.qseq = d.qseq;
+        tq.thr = thr.get();
+        tq.epsc = d.epsc;
+        tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
+        TcRegroup rg;
+        clk.begin(GTS_STAGE_OTHER, 6);
+        tc_regroup(ix->tree, tq, rg, st, ncount ? ncount->get() : nullptr);
+        clk.end();
+        st_tiles += rg.n_items;
+        st_tile_entries += rg.n_entries;
+        st_tile_pairs += rg.n_pairs;
+        L2fQuery lq;
+        lq.Q = d.Q;
+        lq.absf = d.absf;
+        lq.any_deleted = tq.any_deleted;
+        const int64_t per_q = ix->f32_pairs_hint[knn ? 1 : 0].load();
+        const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+        DBuf<int32_t> oq, orow;
+        int nl = 0;
+        clk.begin(GTS_STAGE_TILE);
+        const int64_t C = l2f_run(ix->tree, lq, qb.nq, rg, oq, orow, hint, &nl, st);
+        clk.end();
+        if (rg.n_items > 0 && qb.nq > 0)
+            ix->f32_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+        ++st_groups;
+        if (C > 0) verify_and_collect(oq, orow, C, /*query_major=*/false);
+    }
+
     // Last level on the L1 tiles: regroup the entries by node, run the tiles
     // (leaf mask, visibility and FP32 distance with its error band), then
     // decide the kept pairs (range) or merge them into the answer (kNN).  kNN
@@ -3145,6 +3208,10 @@ struct Runner {
             if (qb.nq > 0) ix->l1_pairs_hint[slot].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
             ++st_groups;
             if (C == 0) continue;
+            if (!knn && use_f32) {   // GTS_PREC_FP32 reports the plain path's FP32 distances
+                verify_and_collect(oq, orow, C, /*query_major=*/false);
+                continue;
+            }
             st_cands += C;
             DBuf<uint8_t> keep(C, st);
             if (knn) {   // the merge wants query-major order
@@ -3427,6 +3494,11 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
                          t.n > 0 && t.n < ((int64_t)1 << 31);
     if (precision == GTS_PREC_BF16 && low_dim) R.use_scan = true;
     if (precision == GTS_PREC_BF16 && !low_dim && l1_tiles_supported(t, qb.Q)) R.use_l1 = true;
+    // GTS_PREC_FP32: node-major FP32 tiles for batches (the diagnostic count
+    // needs the plain scan, whose candidates are the counted pairs)
+    if (precision == GTS_PREC_FP32 && !low_dim && budget >= kF32TileBudget && !qb.count_table_pass &&
+        (l2f_tiles_supported(t) || l1_tiles_supported(t, qb.Q)))
+        R.use_f32 = true;
     if (precision == GTS_PREC_BF16 && t.dim == 0 && t.n > 0 && t.n < ((int64_t)1 << 31) && R.tu.str_qgram > 0)
         R.use_qg = true;
     if (precision == GTS_PREC_BF16 && !low_dim && tc_supported(t)) {
