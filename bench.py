@@ -69,7 +69,7 @@ SCAN_TRAFFIC = 328.7e6
 # of the bit-parallel edit-distance kernels: sm__inst_executed_pipe_alu.sum x 32
 # over the cells of every launch of one batch pair of the dna workload at 0.2
 # scale (profiles/dp_str_dna_200k_r8.md).  None once the kernels change.
-INT_OPS_PER_CELL = {"pivot_dist": 0.600, "verify": 0.619}
+INT_OPS_PER_CELL = {"pivot_dist": None, "verify": None}
 
 
 def workload(scale: float = 1.0):

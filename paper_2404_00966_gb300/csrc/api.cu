@@ -285,7 +285,7 @@ void cache_append(gts_index *ix, const DevObjects &o, int64_t *ids_out) {
     } else {
         if (c.h_Soff.empty()) c.h_Soff.push_back(0);
         const int64_t add = o.h_off[m];
-        grow(c.S, c.s_bytes, c.s_bytes + add + 1, st);
+        grow(c.S, c.s_bytes, c.s_bytes + add + kTextPad, st);
         if (add) GTS_CUDA(cudaMemcpyAsync(c.S.get() + c.s_bytes, o.v.S, add, cudaMemcpyDeviceToDevice, st));
         for (int64_t i = 1; i <= m; ++i) c.h_Soff.push_back(c.s_bytes + o.h_off[i]);
         c.s_bytes += add;

@@ -136,13 +136,13 @@ __global__ void k_map_vec(const float *__restrict__ X, int dim, const int32_t *_
 // Mapping for strings: a block takes a run of table positions; for every node
 // in the run it loads the node pivot's match masks into shared memory and each
 // thread computes one object's distance to the pivot (pattern = pivot).
-template <int W>
+template <int B>
 __global__ void k_map_str(const uint8_t *__restrict__ S, const int64_t *__restrict__ Soff,
                           const int32_t *__restrict__ perm, const int32_t *__restrict__ pos_node,
                           const int32_t *__restrict__ piv_obj, const int32_t *__restrict__ lpos,
                           const int32_t *__restrict__ lsize, int64_t n, int chunk, float *__restrict__ Tl,
                           int32_t *__restrict__ node_of) {
-    __shared__ uint64_t Peq[256 * W];
+    __shared__ __align__(16) uint32_t Peq[256 * B];
     const int64_t p0 = (int64_t)blockIdx.x * chunk;
     const int64_t p1 = p0 + chunk < n ? p0 + chunk : n;
     int64_t s = p0;
@@ -152,11 +152,11 @@ __global__ void k_map_str(const uint8_t *__restrict__ S, const int64_t *__restri
         if (e > p1) e = p1;
         const int32_t pv = piv_obj[node];
         const int m = (int)(Soff[pv + 1] - Soff[pv]);
-        if (m > 0) build_peq<W>(Peq, S + Soff[pv], m);
+        if (m > 0) build_peq<B>(Peq, S + Soff[pv], m);
         for (int64_t p = s + threadIdx.x; p < e; p += blockDim.x) {
             const int32_t o = perm[p];
             const int len = (int)(Soff[o + 1] - Soff[o]);
-            const int d = m > 0 ? myers_edit<W>(Peq, m, S + Soff[o], len) : len;
+            const int d = m > 0 ? edit_bits<B, TextBytes>(Peq, m, S + Soff[o], len) : len;
             Tl[o] = (float)d;
             node_of[o] = node;
         }
@@ -257,12 +257,12 @@ __global__ void k_piv_rows(int32_t *__restrict__ piv, int64_t cnt, const int32_t
         if (piv[i] >= 0) piv[i] = inv[piv[i]];
 }
 
-template <int W>
+template <int B>
 void launch_map_str(const Objects &o, const int32_t *perm, const int32_t *pos_node, const int32_t *piv,
                     const int32_t *lpos, const int32_t *lsize, int64_t n, float *Tl, int32_t *node_of,
                     cudaStream_t st) {
     const int chunk = 256;
-    k_map_str<W><<<blocks_for(n, chunk), 128, 0, st>>>(o.S, o.Soff, perm, pos_node, piv, lpos, lsize, n, chunk, Tl,
+    k_map_str<B><<<blocks_for(n, chunk), 128, 0, st>>>(o.S, o.Soff, perm, pos_node, piv, lpos, lsize, n, chunk, Tl,
                                                        node_of);
 }
 
@@ -329,7 +329,6 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
     cub::DeviceRadixSort::SortPairs(nullptr, sort_tmp_bytes, keys.get(), keys2.get(), perm.get(), perm2.get(), n, 0,
                                     64, st);
     DBuf<uint8_t> sort_tmp(sort_tmp_bytes, st);
-    int W = 1;   // 64-bit words per pivot pattern (strings)
     for (int l = 0; l < h; ++l) {
         const int64_t nn = t.lvl_off[l + 1] - t.lvl_off[l];
         int32_t *lpos = t.npos.get() + t.lvl_off[l];
@@ -346,12 +345,16 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
                 k_map_vec<false><<<blocks_for(n), kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), pos_node.get(), lpiv,
                                                                      n, Tl, node_of.get());
         } else {
-            W = (t.max_len + 63) / 64;
-            if (W <= 1) launch_map_str<1>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st);
-            else if (W <= 2) launch_map_str<2>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st);
-            else if (W <= 4) launch_map_str<4>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st);
-            else if (W <= 8) launch_map_str<8>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st);
-            else launch_map_str<16>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st);
+            const int W = (t.max_len + 31) / 32;   // 32-bit words of the longest pattern
+#define GTS_MAP_STR(BB) \
+    launch_map_str<BB>(objs, perm.get(), pos_node.get(), lpiv, lpos, lsize, n, Tl, node_of.get(), st)
+            if (W <= 1) GTS_MAP_STR(1);
+            else if (W <= 2) GTS_MAP_STR(2);
+            else if (W <= 4) GTS_MAP_STR(4);
+            else if (W <= 8) GTS_MAP_STR(8);
+            else if (W <= 16) GTS_MAP_STR(16);
+            else GTS_MAP_STR(32);
+#undef GTS_MAP_STR
         }
         check_launch("mapping");
         k_keys<<<blocks_for(n), kThreads, 0, st>>>(node_of.get(), Tl, n, keys.get(), perm2.get());
@@ -392,7 +395,7 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
         int64_t total = 0;
         GTS_CUDA(cudaMemcpyAsync(&total, t.Soff.get() + n, 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        t.S.alloc(total > 0 ? total : 1, st);
+        t.S.alloc(total + kTextPad, st);
         k_gather_str<<<blocks_for(n * 32), kThreads, 0, st>>>(objs.S, objs.Soff, perm.get(), n, t.Soff.get(),
                                                             t.S.get());
     }

@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "gts_impl.cuh"
+#include "metric.cuh"
 
 namespace gts {
 
@@ -86,12 +87,13 @@ struct Reader {
         raw(v.data(), (size_t)bytes);
         return v;
     }
-    // an array into a new device buffer of at least `min_count` elements
+    // an array into a new device buffer of at least `min_count` elements,
+    // with `spare` more after the array
     template <class T>
-    int64_t dev(DBuf<T> &b, int64_t min_count, cudaStream_t st) {
+    int64_t dev(DBuf<T> &b, int64_t min_count, cudaStream_t st, int64_t spare = 0) {
         std::vector<T> h = host<T>();
         const int64_t count = (int64_t)h.size();
-        b.alloc((size_t)std::max<int64_t>(std::max<int64_t>(count, min_count), 1), st);
+        b.alloc((size_t)std::max<int64_t>(std::max<int64_t>(count + spare, min_count), 1), st);
         if (count) GTS_CUDA(cudaMemcpyAsync(b.get(), h.data(), count * sizeof(T), cudaMemcpyHostToDevice, st));
         GTS_CUDA(cudaStreamSynchronize(st));
         return count;
@@ -264,7 +266,7 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
             expect((int64_t)soff.size(), n + 1, "string offsets");
             t.Soff.alloc(n + 1, st);
             GTS_CUDA(cudaMemcpyAsync(t.Soff.get(), soff.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
-            expect(r.dev(t.S, 1, st), soff[n], "strings");
+            expect(r.dev(t.S, 1, st, kTextPad), soff[n], "strings");
         }
         expect(r.dev(t.row_id, 1, st), n, "ids");
         expect(r.dev(t.table, 1, st), (int64_t)h * n, "table");
@@ -287,7 +289,7 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
             GTS_REQUIRE((int64_t)c.h_Soff.size() == (c.count > 0 ? c.count + 1 : (int64_t)c.h_Soff.size()),
                         GTS_EINVAL, "index file is corrupt (cache offsets)");
             c.s_bytes = c.h_Soff.empty() ? 0 : c.h_Soff.back();
-            expect(r.dev(c.S, 1, st), c.s_bytes, "cache strings");
+            expect(r.dev(c.S, 1, st, kTextPad), c.s_bytes, "cache strings");
             c.Soff.alloc(c.h_Soff.size() + 1, st);
             if (!c.h_Soff.empty())
                 GTS_CUDA(cudaMemcpyAsync(c.Soff.get(), c.h_Soff.data(), c.h_Soff.size() * 8, cudaMemcpyHostToDevice,
