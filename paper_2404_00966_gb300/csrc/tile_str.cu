@@ -24,8 +24,9 @@ namespace gts {
 namespace {
 
 constexpr int kRowsS = 128;     // rows of one node block (the regrouping's block size)
-constexpr int kThreadsS = 256;  // thread = (row tid % 128, query half tid / 128)
+constexpr int kThreadsS = 256;  // warp w: rows [64 (w % 2), + 64), two per lane; queries of group w / 2
 constexpr int kWords = 16;      // 64 one-byte buckets as 16 words
+constexpr int kGroups = 4;      // query groups of a chunk
 
 struct StrArgs {
     int F;
@@ -44,19 +45,24 @@ struct StrArgs {
     unsigned long long *out_count;
 };
 
-// NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 2 per thread
+// NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 4 per thread.
+// The ALU pipe bounds it: 16 four-byte sums of absolute differences per pair
+// (19 T a second on the device, 60 of 64 lanes per SM and cycle: 2 * 10^10
+// pairs cannot take less than 16.8 ms).  A lane therefore holds two rows, so
+// that a query's 64 bytes -- four 16-byte broadcast loads -- serve 64 rows of
+// its warp, and the leaf and visibility tests run on the few pairs that pass:
+// 33.1 ms for 1.9 * 10^10 pairs (one row a lane and 4-byte loads: 53.0 ms).
 template <int NQS>
 __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
-    constexpr int kNQS = NQS;
-    constexpr int kQPTS = NQS / 2;
-    __shared__ __align__(16) uint32_t sQ[kNQS][kWords + 1];
-    __shared__ uint64_t sMask[kNQS];
-    __shared__ int64_t sSeq[kNQS];
-    __shared__ float sLim[kNQS];
-    __shared__ int32_t sQid[kNQS];
+    constexpr int kPer = NQS / kGroups;
+    __shared__ uint4 sQ[NQS][kWords / 4];
+    __shared__ uint64_t sMask[NQS];
+    __shared__ int64_t sSeq[NQS];
+    __shared__ uint32_t sLim[NQS];
+    __shared__ int32_t sQid[NQS];
     __shared__ int s_item;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int r = tid % kRowsS, half = tid / kRowsS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int group = warp >> 1;
     for (;;) {
         if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
         __syncthreads();
@@ -68,54 +74,76 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
         const int rb = it.w * kRowsS;
         const int32_t pos = a.npos[g], size = a.nsize[g];
         const int nrow = min(kRowsS, size - rb);
-        const int64_t row = (int64_t)pos + rb + r;
-        const bool valid = r < nrow;
-        // this thread's row: bucket counts, leaf bit, delete mark
         const int32_t avg = size / a.F;
-        int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
-        if (jl > a.F - 1) jl = a.F - 1;
-        const uint64_t rowbit = valid ? (1ull << jl) : 0ull;
-        const int64_t rdel = (valid && a.any_deleted) ? a.row_del[row] : kNever;
-        uint32_t rw[kWords];
-        if (valid) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + row * 64);
+        // this lane's two rows: bucket counts, leaf bits, delete marks
+        uint32_t rw[2][kWords];
+        uint64_t rowbit[2];
+        int64_t rdel[2];
+        const int r0 = (warp & 1) * 64 + lane;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = r0 + 32 * h;
+            const bool valid = r < nrow;
+            const int64_t row = (int64_t)pos + rb + r;
+            int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
+            if (jl > a.F - 1) jl = a.F - 1;
+            rowbit[h] = valid ? (1ull << jl) : 0ull;
+            rdel[h] = (valid && a.any_deleted) ? a.row_del[row] : kNever;
+            const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + (valid ? row : (int64_t)pos) * 64);
 #pragma unroll
             for (int v = 0; v < kWords / 4; ++v) {
                 const uint4 x = src[v];
-                rw[4 * v] = x.x;
-                rw[4 * v + 1] = x.y;
-                rw[4 * v + 2] = x.z;
-                rw[4 * v + 3] = x.w;
+                rw[h][4 * v] = x.x;
+                rw[h][4 * v + 1] = x.y;
+                rw[h][4 * v + 2] = x.z;
+                rw[h][4 * v + 3] = x.w;
             }
-        } else {
-#pragma unroll
-            for (int w = 0; w < kWords; ++w) rw[w] = 0;
         }
-        for (int c0 = 0; c0 < total; c0 += kNQS) {
-            const int cnt = min(kNQS, total - c0);
+        // the leaves of the warp's rows: a query that kept none of them is passed over
+        const uint64_t both = rowbit[0] | rowbit[1];
+        const uint64_t wmask = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)both) |
+                               ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(both >> 32)) << 32);
+        for (int c0 = 0; c0 < total; c0 += NQS) {
+            const int cnt = min(NQS, total - c0);
             __syncthreads();   // the previous chunk's shared data is no longer read
             for (int j = tid; j < cnt; j += kThreadsS) {
                 const TileRec rc = a.grec[first + c0 + j];
                 sMask[j] = rc.mask;
                 sSeq[j] = rc.seq;
-                sLim[j] = 6.f * rc.thr;   // keep iff L1 <= 6 t
+                // keep iff L1 <= 6 t (whole numbers; an unbounded t keeps all)
+                sLim[j] = rc.thr < 1e8f ? (uint32_t)(6.f * rc.thr) : 0xffffffffu;
                 sQid[j] = rc.q;
             }
-            for (int t = tid; t < cnt * kWords; t += kThreadsS) {
-                const int j = t / kWords, w = t - j * kWords;
-                sQ[j][w] = reinterpret_cast<const uint32_t *>(a.qgq + (int64_t)a.grec[first + c0 + j].q * 64)[w];
+            for (int t = tid; t < cnt * (kWords / 4); t += kThreadsS) {
+                const int j = t / (kWords / 4), w = t - j * (kWords / 4);
+                sQ[j][w] = reinterpret_cast<const uint4 *>(a.qgq + (int64_t)a.grec[first + c0 + j].q * 64)[w];
             }
             __syncthreads();
-            uint32_t pass = 0;
-#pragma unroll 1
-            for (int jj = 0; jj < kQPTS; ++jj) {
-                const int j = half * kQPTS + jj;
-                if (j >= cnt) break;
-                if (!(sMask[j] & rowbit) || rdel <= sSeq[j]) continue;
-                uint32_t l1 = 0;
+            uint32_t pass = 0;   // bit jj: row r0, bit 16 + jj: row r0 + 32
+            const int j0 = group * kPer, j1 = min(j0 + kPer, cnt);
+#pragma unroll 2
+            for (int j = j0; j < j1; ++j) {
+                if (!(sMask[j] & wmask)) continue;   // warp-uniform
+                uint32_t l0 = 0, l1 = 0;
 #pragma unroll
-                for (int w = 0; w < kWords; ++w) l1 = __vsadu4(rw[w], sQ[j][w]) + l1;
-                if ((float)l1 <= sLim[j]) pass |= 1u << jj;
+                for (int v = 0; v < kWords / 4; ++v) {
+                    const uint4 x = sQ[j][v];
+                    l0 = __vsadu4(rw[0][4 * v], x.x) + l0;
+                    l1 = __vsadu4(rw[1][4 * v], x.x) + l1;
+                    l0 = __vsadu4(rw[0][4 * v + 1], x.y) + l0;
+                    l1 = __vsadu4(rw[1][4 * v + 1], x.y) + l1;
+                    l0 = __vsadu4(rw[0][4 * v + 2], x.z) + l0;
+                    l1 = __vsadu4(rw[1][4 * v + 2], x.z) + l1;
+                    l0 = __vsadu4(rw[0][4 * v + 3], x.w) + l0;
+                    l1 = __vsadu4(rw[1][4 * v + 3], x.w) + l1;
+                }
+                const uint32_t lim = sLim[j];
+                if (l0 <= lim) pass |= 1u << (j - j0);
+                if (l1 <= lim) pass |= 65536u << (j - j0);
+            }
+            for (uint32_t left = pass; left; left &= left - 1) {   // leaf and visibility of the passing pairs
+                const int b = __ffs(left) - 1, h = b >> 4, j = j0 + (b & 15);
+                if (!(sMask[j] & (h ? rowbit[1] : rowbit[0])) || (h ? rdel[1] : rdel[0]) <= sSeq[j]) pass &= ~(1u << b);
             }
             const int np = __popc(pass);
             int incl = np;
@@ -131,11 +159,11 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
                 base = __shfl_sync(0xffffffffu, base, 31);
                 unsigned long long o = base + (unsigned long long)(incl - np);
                 while (pass) {
-                    const int jj = __ffs(pass) - 1;
+                    const int b = __ffs(pass) - 1;
                     pass &= pass - 1;
                     if ((int64_t)o < a.cap) {
-                        a.out_q[o] = sQid[half * kQPTS + jj];
-                        a.out_row[o] = (int32_t)row;
+                        a.out_q[o] = sQid[j0 + (b & 15)];
+                        a.out_row[o] = pos + rb + r0 + 32 * (b >> 4);
                     }
                     ++o;
                 }
