@@ -1225,6 +1225,28 @@ __global__ void k_qgram_hist(const uint8_t *__restrict__ S, const int64_t *__res
     }
 }
 
+// How selective the 3-gram bound is: of ns pairs spread over the entries [e0,
+// e0 + E) of a level (an entry's query, a row of its node), how many pass.
+__global__ void k_qgram_sample(Dev d, const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
+                               int64_t lvl_base, int64_t e0, int64_t E, const float *__restrict__ thr_q, int ns,
+                               unsigned long long *__restrict__ passed) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool pass = false;
+    if (i < ns) {
+        const int64_t e = e0 + (int64_t)i * E / ns;
+        const int32_t q = eq[e];
+        const int64_t g = lvl_base + enode[e];
+        const int64_t row = d.npos[g] + (uint32_t)(i * 2654435761u) % (uint32_t)d.nsize[g];
+        const uint32_t *qw = reinterpret_cast<const uint32_t *>(d.qgq + (int64_t)q * kQgBuckets);
+        const uint32_t *rw = reinterpret_cast<const uint32_t *>(d.qg + row * kQgBuckets);
+        uint32_t l1 = 0;
+        for (int w = 0; w < kQgBuckets / 4; ++w) l1 = __vsadu4(qw[w], rw[w]) + l1;
+        pass = (float)l1 <= 6.f * thr_q[q];
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, pass);
+    if ((threadIdx.x & 31) == 0 && b) atomicAdd(passed, (unsigned long long)__popc(b));
+}
+
 // Verification of (query, row) pairs under edit distance; consecutive pairs
 // mostly share their query, whose match masks a block builds once per run.  A
 // pair is kept if its distance is at most the run's threshold t, so queries of
@@ -2605,6 +2627,10 @@ struct Runner {
                                                                    nullptr, nullptr, nullptr, cmask.get());
             clk.end();
             check_launch("expand count");
+            if (use_qg && !knn && l == h - 2 && filter_beats_last_pivots(L, e0, e1, cnt)) {
+                str_leaf_children(L, e0, e1, cmask);
+                return;
+            }
             DBuf<int64_t> off;
             scan_i32(cnt, E, off);
             const int64_t total = d2h_i64(off.get() + E, st);
@@ -3078,31 +3104,86 @@ struct Runner {
         verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
     }
 
-    // Last level for strings on the 3-gram tiles: regroup the entries by
-    // node, keep the pairs the 3-gram count bound does not exclude, then run
-    // the exact bit-parallel DP on those (query-major for its match masks).
-    void str_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
-        TcQuery tq;
+    // Range queries on the 3-gram tiles: whether to leave the last pivot level
+    // out and filter every row of the children that survived the level above.
+    // Per (query, last-level node) entry the pivot costs 0.6 ps per word-step
+    // of its DP and 150 ps for the entry (its expansion, leaf mask and
+    // regrouped record); filtering all R rows of the node costs 1 ps a row
+    // and 90 ps for each pair the bound lets through (sorting and verifying
+    // it).  The pass rate is measured on a sample.  (10^6 reads of 108, r = 8:
+    // R = 125, pass rate below 10^-3, and the pivots exclude 5 % of the
+    // entries: 100.5 -> 39.3 ms without them.  Dictionary words at r = 2: a
+    // third passes, so the pivots stay.)
+    bool filter_beats_last_pivots(Level &L, int64_t e0, int64_t e1, DBuf<int32_t> &cnt) {
+        if (qb.count_table_pass || h < 2) return false;
+        const Tree &t = ix->tree;
+        const double nn = (double)(t.lvl_off[h] - t.lvl_off[h - 1]);
+        const double rows = (double)t.n / nn;
+        const double pivot_ps = 0.6 * W * ((double)t.S.bytes() / (double)t.n) + 150.0;
+        if (rows > pivot_ps) return false;
+        constexpr int kSample = 8192;
+        DBuf<unsigned long long> c(2, st);
+        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 16, st));
+        clk.begin(GTS_STAGE_OTHER, 2);
+        k_qgram_sample<<<kSample / kT, kT, 0, st>>>(d, L.q.get(), L.node.get(), t.lvl_off[h - 2], e0, e1 - e0,
+                                                    thr.get(), kSample, c.get());
+        k_sum_i32<<<cap(nblocks(e1 - e0, kT)), kT, 0, st>>>(cnt.get(), e1 - e0, c.get() + 1);
+        clk.end();
+        check_launch("3-gram sample");
+        unsigned long long hc[2];
+        GTS_CUDA(cudaMemcpyAsync(hc, c.get(), 16, cudaMemcpyDeviceToHost, st));
+        GTS_CUDA(cudaStreamSynchronize(st));
+        const double f = (double)hc[0] / kSample;
+        if (rows * (1.0 + 90.0 * f) > pivot_ps) return false;
+        st_frontier += (int64_t)hc[1];
+        return true;
+    }
+
+    // The rows of every child of [e0, e1)'s nodes (level h - 2) that its
+    // query's mask kept, through the 3-gram tiles.
+    void str_leaf_children(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &cmask) {
+        TcQuery tq = str_query_base(L, e0, e1, cmask);
+        TcRegroup rg;
+        clk.begin(GTS_STAGE_OTHER, 6);
+        tc_regroup_children(ix->tree, tq, rg, st);
+        clk.end();
+        str_tiles(rg, tq.any_deleted, true);
+    }
+
+    TcQuery str_query_base(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+        TcQuery tq;   // (no path distances: the 3-gram tiles do not read them)
         tq.E = e1 - e0;
         tq.nq = qb.nq;
         tq.eq = L.q.get() + e0;
         tq.enode = L.node.get() + e0;
-        tq.path = L.path.get() + e0 * h;
         tq.emask = mask.get();
         tq.qseq = d.qseq;
         tq.thr = thr.get();
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
+        return tq;
+    }
+
+    // Last level for strings on the 3-gram tiles: regroup the entries by
+    // node, keep the pairs the 3-gram count bound does not exclude, then run
+    // the exact bit-parallel DP on those (query-major for its match masks).
+    void str_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+        TcQuery tq = str_query_base(L, e0, e1, mask);
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
         tc_regroup(ix->tree, tq, rg, st, nullptr, false);
         clk.end();
+        str_tiles(rg, tq.any_deleted, false);
+    }
+
+    void str_tiles(TcRegroup &rg, int any_deleted, bool children) {
         st_tiles += rg.n_items;
         st_tile_entries += rg.n_entries;
         st_tile_pairs += rg.n_pairs;
         StrQuery sq;
         sq.qg = d.qg;
         sq.qgq = d.qgq;
-        sq.any_deleted = tq.any_deleted;
+        sq.any_deleted = any_deleted;
+        sq.children = children;
         sq.queries = tu.str_qgram == 32 ? 32 : 64;
         const int64_t per_q = ix->tc_pairs_hint[knn ? 1 : 0].load();
         const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);

@@ -34,6 +34,7 @@ struct StrArgs {
     int64_t lvl_last;
     const int64_t *row_del;
     int any_deleted;
+    int children;               // the masks' bits are the parent's children, not the node's leaves
     const uint8_t *qg;          // rows' bucket counts [n, 64]
     const uint8_t *qgq;         // queries' bucket counts [nq, 64]
     const TileRec *grec;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
             const int64_t row = (int64_t)pos + rb + r;
             int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
             if (jl > a.F - 1) jl = a.F - 1;
+            if (a.children) jl = it.x % a.F;
             rowbit[h] = valid ? (1ull << jl) : 0ull;
             rdel[h] = (valid && a.any_deleted) ? a.row_del[row] : kNever;
             const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + (valid ? row : (int64_t)pos) * 64);
@@ -204,6 +206,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<i
         a.lvl_last = t.lvl_off[t.h - 1];
         a.row_del = t.row_del.get();
         a.any_deleted = sq.any_deleted;
+        a.children = sq.children ? 1 : 0;
         a.qg = sq.qg;
         a.qgq = sq.qgq;
         a.grec = rg.grec.get();

@@ -750,7 +750,8 @@ __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__
         r.mask = m;
         grec[o] = r;
         gq[o] = q;
-        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
+        if (path)
+            for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
     }
 }
 
@@ -816,7 +817,8 @@ __device__ __forceinline__ void write_rec(int64_t e, int64_t o, const int32_t *e
     r.mask = emask[e];
     grec[o] = r;
     gq[o] = q;
-    for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
+    if (path)
+        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
 }
 
 __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
@@ -858,6 +860,32 @@ __global__ void k_fill_items(const int32_t *__restrict__ ncount, const int32_t *
         const int32_t blocks = (nsize[i] + kRows - 1) / kRows;
         const int flag = c >= win_min ? kWindowItem : 0;
         for (int32_t b = 0; b < blocks; ++b) items[ioff[i] + b] = make_int4((int)i, (int)noff[i], c, b | flag);
+    }
+}
+
+// The same for items over the children (level `cnode` sizes) of the counted
+// nodes: thread per child.
+__global__ void k_child_items(const int32_t *__restrict__ ncount, const int32_t *__restrict__ csize, int64_t nc, int F,
+                              int64_t *__restrict__ nitems, unsigned long long *__restrict__ pairs) {
+    unsigned long long p = 0;
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t k = ncount[c / F];
+        nitems[c] = k > 0 ? (int64_t)((csize[c] + kRows - 1) / kRows) : 0;
+        p += (unsigned long long)k * (unsigned long long)csize[c];
+    }
+    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+    if ((threadIdx.x & 31) == 0 && p) atomicAdd(pairs, p);
+    if (blockIdx.x == 0 && threadIdx.x == 0) nitems[nc] = 0;
+}
+
+__global__ void k_fill_child_items(const int32_t *__restrict__ ncount, const int32_t *__restrict__ csize,
+                                   const int64_t *__restrict__ noff, const int64_t *__restrict__ ioff, int64_t nc,
+                                   int F, int4 *__restrict__ items) {
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t k = ncount[c / F];
+        if (k == 0) continue;
+        const int32_t blocks = (csize[c] + kRows - 1) / kRows;
+        for (int32_t b = 0; b < blocks; ++b) items[ioff[c] + b] = make_int4((int)c, (int)noff[c / F], k, b);
     }
 }
 
@@ -939,19 +967,20 @@ bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E) {
     return words * 8 <= ((int64_t)1 << 30) && words <= 4 * E;
 }
 
-int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st, const int32_t *counts,
-                   bool window_ok) {
+// the entries' records by node of their level (nn nodes; counts, if given, are
+// the nodes' entries with a set mask): rg.grec / gq / gpath and rg.noff;
+// returns the nodes' counts (in `own` unless given)
+static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup &rg, int64_t nn, bool use_bits,
+                                    const int32_t *counts, DBuf<int32_t> &own, cudaStream_t st) {
     const int64_t E = tq.E;
-    const int64_t nn = t.lvl_off[t.h] - t.lvl_off[t.h - 1];
-    // the bitmap form when its two (node x query-word) arrays stay small
     const int64_t nw = (tq.nq + 31) / 32;
-    const bool use_bits = regroup_uses_bits(t, tq.nq, E);
     DBuf<uint32_t> &bits = rg.bits;
     DBuf<int32_t> &wpre = rg.wpre;
     bits.alloc(use_bits ? nn * nw : 0, st);
     wpre.alloc(use_bits ? nn * nw : 0, st);
     rg.nw = use_bits ? nw : 0;
-    DBuf<int32_t> own((counts && !use_bits) ? 0 : nn, st), cursor(use_bits ? 0 : nn, st);
+    own.alloc((counts && !use_bits) ? 0 : nn, st);
+    DBuf<int32_t> cursor(use_bits ? 0 : nn, st);
     if (use_bits) {
         GTS_CUDA(cudaMemsetAsync(bits.get(), 0, nn * nw * 4, st));
         k_bits_set<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, E, nw, bits.get());
@@ -964,7 +993,7 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
         }
     }
     const int32_t *ncnt = (counts && !use_bits) ? counts : own.get();
-    DBuf<int64_t> c64(nn + 1, st), nitems(nn + 1, st), ioff(nn + 1, st);
+    DBuf<int64_t> c64(nn + 1, st);
     DBuf<int64_t> &noff = rg.noff;
     noff.alloc(nn + 1, st);
     k_i32_to_i64_tc<<<nblk(nn), 256, 0, st>>>(ncnt, nn, c64.get());
@@ -976,7 +1005,7 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
     const int hp = (t.h + 3) & ~3;
     rg.grec.alloc(ne, st);
     rg.gq.alloc(ne, st);
-    rg.gpath.alloc(ne * hp, st);
+    rg.gpath.alloc(tq.path ? ne * hp : 1, st);
     if (use_bits)
         k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, t.h, hp, E, tq.thr, tq.qn2,
                                                      tq.cE1, tq.cE2, tq.qseq, noff.get(), bits.get(), wpre.get(), nw, rg.grec.get(),
@@ -985,6 +1014,20 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
         k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, t.h, hp, E, tq.thr, tq.qn2,
                                                 tq.cE1, tq.cE2, tq.qseq, noff.get(), cursor.get(), rg.grec.get(), rg.gq.get(),
                                                 rg.gpath.get());
+    rg.n_entries = total_entries;
+    rg.n_chunks = (total_entries + 127) / 128;
+    return ncnt;
+}
+
+int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st, const int32_t *counts,
+                   bool window_ok) {
+    const int64_t nn = t.lvl_off[t.h] - t.lvl_off[t.h - 1];
+    // the bitmap form when its two (node x query-word) arrays stay small
+    const bool use_bits = regroup_uses_bits(t, tq.nq, tq.E);
+    DBuf<int32_t> own;
+    const int32_t *ncnt = group_records(t, tq, rg, nn, use_bits, counts, own, st);
+    const DBuf<int64_t> &noff = rg.noff;
+    DBuf<int64_t> nitems(nn + 1, st), ioff(nn + 1, st);
     const int32_t *lsize = t.nsize.get() + t.lvl_off[t.h - 1];
     DBuf<unsigned long long> pairs(1, st);
     GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
@@ -997,8 +1040,6 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
     GTS_CUDA(cudaStreamSynchronize(st));
     rg.n_pairs = (int64_t)total_pairs;
     rg.n_items = total_items;
-    rg.n_entries = total_entries;
-    rg.n_chunks = (total_entries + 127) / 128;
     if (total_items > 0) {
         rg.items.alloc(total_items, st);
         // window mode for nodes holding at least half of the batch
@@ -1006,6 +1047,34 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
         k_fill_items<<<nblk(nn), 256, 0, st>>>(ncnt, lsize, noff.get(), ioff.get(), nn, win_min, rg.items.get());
     }
     check_launch("tile regroup");
+    return total_items;
+}
+
+int64_t tc_regroup_children(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st) {
+    const int64_t nn = t.lvl_off[t.h - 1] - t.lvl_off[t.h - 2];      // the parents
+    const int64_t nc = t.lvl_off[t.h] - t.lvl_off[t.h - 1];          // their children
+    const int64_t words = nn * ((tq.nq + 31) / 32);
+    DBuf<int32_t> own;
+    const int32_t *ncnt =
+        group_records(t, tq, rg, nn, words * 8 <= ((int64_t)1 << 30) && words <= 4 * tq.E, nullptr, own, st);
+    const int32_t *csize = t.nsize.get() + t.lvl_off[t.h - 1];
+    DBuf<int64_t> nitems(nc + 1, st), ioff(nc + 1, st);
+    DBuf<unsigned long long> pairs(1, st);
+    GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
+    k_child_items<<<nblk(nc), 256, 0, st>>>(ncnt, csize, nc, t.F, nitems.get(), pairs.get());
+    exscan(nitems.get(), ioff.get(), nc + 1, st);
+    int64_t total_items = 0;
+    unsigned long long total_pairs = 0;
+    GTS_CUDA(cudaMemcpyAsync(&total_items, ioff.get() + nc, 8, cudaMemcpyDeviceToHost, st));
+    GTS_CUDA(cudaMemcpyAsync(&total_pairs, pairs.get(), 8, cudaMemcpyDeviceToHost, st));
+    GTS_CUDA(cudaStreamSynchronize(st));
+    rg.n_items = total_items;
+    rg.n_pairs = (int64_t)total_pairs;
+    if (total_items > 0) {
+        rg.items.alloc(total_items, st);
+        k_fill_child_items<<<nblk(nc), 256, 0, st>>>(ncnt, csize, rg.noff.get(), ioff.get(), nc, t.F, rg.items.get());
+    }
+    check_launch("child tile regroup");
     return total_items;
 }
 

@@ -70,3 +70,34 @@ def test_edit_bands_saved_and_cached_strings(gts, tmp_path):
         assert np.array_equal(r.dist, dist.astype(np.float32))
     ix.close()
     jx.close()
+
+
+def test_range_without_the_last_pivot_level(gts):
+    """Reads in many small families: the 3-gram filter lets almost nothing
+    through, so the rows of the last level are filtered without its pivots
+    (fewer pivot distances than entries); deleted rows stay out; radii on both
+    sides of the filter's whole-number limit."""
+    rng = np.random.default_rng(77)
+    base = random_strings(600, 100, 108, ACGT, rng)
+    items = [mutate(base.get(i % 600), int(rng.integers(0, 7)), ACGT, rng) for i in range(6007)]
+    S = strings_from_list(items)
+    Q = strings_from_list([mutate(base.get(int(rng.integers(0, 600))), int(rng.integers(0, 7)), ACGT, rng)
+                           for _ in range(201)])
+    ix = gts.Index.build(S, "edit", n_pivots=3, fanout=6, root_pivot=0)
+    radii = np.resize(np.array([0, 1, 8, 9], np.float32), 201)
+    s0 = ix.info()["seq"]
+    dele = rng.choice(6007, 300, replace=False)
+    for step in range(2):
+        r = ix.range(Q, radii, precision="bf16")
+        assert r.stats["pivot_dist"] < r.stats["frontier"]
+        ins = np.full(6007, -1, np.int64)
+        dl = np.full(6007, np.iinfo(np.int64).max, np.int64)
+        if step:
+            dl[dele] = s0 + np.arange(300)
+        off, ids, dist, _ = oracle.range_query("edit", S, Q, radii, ins, dl,
+                                               np.full(201, ix.info()["seq"], np.int64))
+        assert np.array_equal(r.offsets, off) and np.array_equal(r.ids, ids)
+        assert np.array_equal(r.dist, dist.astype(np.float32))
+        if not step:
+            ix.delete(dele)
+    ix.close()
