@@ -76,9 +76,26 @@ void ensure_device() {
 
 namespace {
 
+// (16 bytes a load from the first 16-byte boundary on: 0.092 ms for 10^6 x 128,
+// 5.5 TB/s; 4-byte loads took 0.225 ms)
 __global__ void k_nonfinite(const float *x, int64_t n, int *flag) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (!isfinite(x[i])) *flag = 1;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    int64_t head = (4 - (((uintptr_t)x >> 2) & 3)) & 3;
+    if (head > n) head = n;
+    const int64_t n4 = (n - head) / 4;
+    const float4 *x4 = reinterpret_cast<const float4 *>(x + head);
+    bool bad = false;
+    for (int64_t i = t; i < n4; i += 4 * step) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i + u * step < n4 ? __ldg(x4 + i + u * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            bad |= !(isfinite(v[u].x) && isfinite(v[u].y) && isfinite(v[u].z) && isfinite(v[u].w));
+    }
+    if (t < head) bad |= !isfinite(x[t]);
+    if (t < n - head - 4 * n4) bad |= !isfinite(x[head + 4 * n4 + t]);
+    if (bad) *flag = 1;
 }
 
 // Unit vectors for the angular distance: a warp per row sums the squares in

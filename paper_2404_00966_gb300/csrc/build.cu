@@ -133,6 +133,130 @@ __global__ void k_map_vec(const float *__restrict__ X, int dim, const int32_t *_
     }
 }
 
+// ---- mapping of vectors in double-single arithmetic
+//
+// The table holds RN32(d) of the FP64 distance summed in the reference order,
+// and GB300 has 2 FP64 lanes per SM and cycle: three FP64 operations per
+// coordinate of 10^6 x 128 take 0.61 ms per level (1.21 ms measured, a thread
+// per row; this form 0.34 ms), eight times the pass over the rows.  Here eight lanes take a row:
+// every difference (exact, Knuth's two-sum), square (Dekker's product by a
+// fused multiply-add) and partial sum is an unevaluated FP32 pair, and the
+// pair's proven error decides whether the FP32 rounding of the distance is
+// certain; if it is not (a few rows in ten thousand), the lane that holds the
+// row sums it in FP64 in the reference order.  The values are those of
+// k_map_vec bit for bit.
+//
+// Error of a lane's pair over n = ceil(dim / 8) + 3 terms, u = 2^-24, S the
+// sum: |lo| <= (n + 3) u S, two roundings of lo per term, the products'
+// dropped and rounded parts below 8 u^2 S, three merges: below (n^2 + 8 n +
+// 40) 2^-47 S; kMapErr doubles it, which also covers the FP64 reference's own
+// (dim + 4) 2^-53.  Results outside [1e-18, 1e30], where FP32 squares could
+// lose their low parts or overflow, take FP64.
+constexpr int kMapLanes = 8;
+constexpr int kMapSingleDim = 8;   // up to this dimension a thread sums a row in FP64 (a lane would hold one term)
+
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float bp = __fsub_rn(s, a), ap = __fsub_rn(s, bp);
+    e = __fadd_rn(__fsub_rn(a, ap), __fsub_rn(b, bp));
+}
+
+template <bool L2>
+__device__ __forceinline__ void ds_add_term(float a, float b, float &hi, float &lo, float &big) {
+    float s, e;
+    two_sum(a, -b, s, e);
+    big = fmaxf(big, fabsf(s));
+    float p, q;
+    if (L2) {
+        p = __fmul_rn(s, s);
+        q = __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p));
+    } else {
+        p = fabsf(s);
+        q = s < 0.f ? -e : e;
+    }
+    float t, r;
+    two_sum(hi, p, t, r);
+    hi = t;
+    lo = __fadd_rn(lo, __fadd_rn(r, q));
+}
+
+// RN32 of the distance whose (L2: squared) value lies within a relative del
+// of hi + lo, or -1 if two FP32 values are possible (or the first guess, one
+// Newton step from the root of hi, is not the nearest)
+template <bool L2>
+__device__ __forceinline__ float ds_round(float hi_s, float lo_s, double S, double del) {
+    float r;
+    if (L2) {
+        const float r0 = __fsqrt_rn(hi_s);
+        r = __fadd_rn(r0, __fdividef(__fadd_rn(__fmaf_rn(-r0, r0, hi_s), lo_s), r0 + r0));
+    } else {
+        r = __fadd_rn(hi_s, lo_s);
+    }
+    const double below = 0.5 * ((double)r + (double)__uint_as_float(__float_as_uint(r) - 1u));
+    const double above = 0.5 * ((double)r + (double)__uint_as_float(__float_as_uint(r) + 1u));
+    // (25-bit midpoints: their squares are exact in FP64)
+    const double lo = L2 ? below * below : below, hi = L2 ? above * above : above;
+    return lo < S * (1.0 - del) && S * (1.0 + del) < hi ? r : -1.f;
+}
+
+template <bool L2, bool V4>
+__global__ void __launch_bounds__(kThreads) k_map_vec_ds(const float *__restrict__ X, int dim,
+                                                         const int32_t *__restrict__ perm,
+                                                         const int32_t *__restrict__ pos_node,
+                                                         const int32_t *__restrict__ piv_obj, int64_t n, double del,
+                                                         float *__restrict__ Tl, int32_t *__restrict__ node_of) {
+    const int sub = threadIdx.x & (kMapLanes - 1);
+    const int64_t rows = (int64_t)gridDim.x * blockDim.x / kMapLanes;
+    // (p0 is the warp's first row: every lane runs the same iterations)
+    for (int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / kMapLanes; p0 < n; p0 += rows) {
+        const int64_t p = p0 + (threadIdx.x & 31) / kMapLanes;
+        const bool in = p < n;
+        const int32_t o = in ? perm[p] : 0;
+        const int32_t node = in ? pos_node[p] : 0;
+        const float *a = X + (int64_t)o * dim;
+        const float *b = X + (int64_t)(in ? piv_obj[node] : 0) * dim;
+        float hi = 0.f, lo = 0.f, big = 0.f;
+        if (in) {
+            if (V4) {
+                const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
+#pragma unroll 4
+                for (int i = sub; i < dim / 4; i += kMapLanes) {
+                    const float4 x = a4[i], y = b4[i];
+                    ds_add_term<L2>(x.x, y.x, hi, lo, big);
+                    ds_add_term<L2>(x.y, y.y, hi, lo, big);
+                    ds_add_term<L2>(x.z, y.z, hi, lo, big);
+                    ds_add_term<L2>(x.w, y.w, hi, lo, big);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = sub; i < dim; i += kMapLanes) ds_add_term<L2>(a[i], b[i], hi, lo, big);
+            }
+        }
+#pragma unroll
+        for (int off = 1; off < kMapLanes; off <<= 1) {
+            const float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
+            float t, r;
+            two_sum(hi, h2, t, r);
+            hi = t;
+            lo = __fadd_rn(__fadd_rn(lo, l2), r);
+            big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, off));
+        }
+        if (in && sub == 0) {
+            const double S = (double)hi + (double)lo;
+            float r = -1.f;
+            if (big == 0.f) r = 0.f;   // (a NaN cannot occur: builds reject non-finite coordinates)
+            else if (S >= 1e-18 && S <= 1e30) r = ds_round<L2>(hi, lo, S, del);
+            if (r < 0.f) {
+                double d = L2 ? l2sq_fp64_seq(a, b, dim) : l1_fp64_seq(a, b, dim);
+                if (L2) d = __dsqrt_rn(d);
+                r = __double2float_rn(d);
+            }
+            Tl[o] = r;
+            node_of[o] = node;
+        }
+    }
+}
+
 // Mapping for strings: a block takes a run of table positions; for every node
 // in the run it loads the node pivot's match masks into shared memory and each
 // thread computes one object's distance to the pivot (pattern = pivot).
@@ -209,13 +333,22 @@ __global__ void k_next_pos_node(int32_t *__restrict__ pos_node, int64_t n, const
     }
 }
 
-__global__ void k_gather_rows(const float *__restrict__ X, int dim, const int32_t *__restrict__ perm, int64_t n,
-                              float *__restrict__ Xl) {
-    const int64_t total = n * (int64_t)dim;
+// rows into leaf order: 16 bytes a thread where the rows allow it (10^6 x 128:
+// 0.20 ms; one float and a 64-bit division a thread took 0.70 ms)
+template <class V>
+__global__ void k_gather_rows(const V *__restrict__ X, int per_row, const int32_t *__restrict__ perm, int64_t n,
+                              V *__restrict__ Xl) {
+    const int64_t total = n * (int64_t)per_row;
+    if (total < ((int64_t)1 << 31)) {   // 32-bit division
+        const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, pr = (uint32_t)per_row;
+        if (t >= total) return;
+        const uint32_t p = t / pr;
+        Xl[t] = X[(int64_t)perm[p] * pr + (t - p * pr)];
+        return;
+    }
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = t / dim;
-        const int c = (int)(t - p * dim);
-        Xl[t] = X[(int64_t)perm[p] * dim + c];
+        const int64_t p = t / per_row;
+        Xl[t] = X[(int64_t)perm[p] * per_row + (t - p * per_row)];
     }
 }
 
@@ -264,6 +397,14 @@ void launch_map_str(const Objects &o, const int32_t *perm, const int32_t *pos_no
     const int chunk = 256;
     k_map_str<B><<<blocks_for(n, chunk), 128, 0, st>>>(o.S, o.Soff, perm, pos_node, piv, lpos, lsize, n, chunk, Tl,
                                                        node_of);
+}
+
+void gather_rows(const float *X, int dim, const int32_t *perm, int64_t n, float *out, cudaStream_t st) {
+    if (dim % 4 == 0 && (((uintptr_t)X | (uintptr_t)out) & 15) == 0)
+        k_gather_rows<float4><<<blocks_for(n * (dim / 4)), kThreads, 0, st>>>(
+            reinterpret_cast<const float4 *>(X), dim / 4, perm, n, reinterpret_cast<float4 *>(out));
+    else
+        k_gather_rows<float><<<blocks_for(n * (int64_t)dim), kThreads, 0, st>>>(X, dim, perm, n, out);
 }
 
 }  // namespace
@@ -338,12 +479,29 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
         if (l > 0) k_fft_pivot<<<(unsigned)nn, kThreads, 0, st>>>(perm.get(), T.get(), n, l, lpos, lsize, lpiv);
         check_launch("fft pivot");
         if (objs.dim > 0) {
-            if (metric == GTS_L2)
+            if (objs.dim > kMapSingleDim) {
+                const bool v4 = objs.dim % 4 == 0 && ((uintptr_t)objs.X & 15) == 0;
+                const double terms = (objs.dim + 7) / 8 + 3;
+                const double del = (terms * terms + 8 * terms + 40) / 70368744177664.0;   // 2^-46
+                const unsigned grid = blocks_for(n, kThreads / kMapLanes);
+#define GTS_MAP(L2V, V4V)                                                                                            \
+    k_map_vec_ds<L2V, V4V><<<grid, kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), pos_node.get(), lpiv, n, del, Tl, \
+                                                      node_of.get())
+                if (metric == GTS_L2) {
+                    if (v4) GTS_MAP(true, true);
+                    else GTS_MAP(true, false);
+                } else {
+                    if (v4) GTS_MAP(false, true);
+                    else GTS_MAP(false, false);
+                }
+#undef GTS_MAP
+            } else if (metric == GTS_L2) {
                 k_map_vec<true><<<blocks_for(n), kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), pos_node.get(), lpiv,
                                                                     n, Tl, node_of.get());
-            else
+            } else {
                 k_map_vec<false><<<blocks_for(n), kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), pos_node.get(), lpiv,
                                                                      n, Tl, node_of.get());
+            }
         } else {
             const int W = (t.max_len + 31) / 32;   // 32-bit words of the longest pattern
 #define GTS_MAP_STR(BB) \
@@ -377,12 +535,10 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
     k_fill_i64<<<blocks_for(n), kThreads, 0, st>>>(t.row_del.get(), n, kNever);
     if (objs.dim > 0) {
         t.X.alloc((size_t)n * objs.dim, st);
-        k_gather_rows<<<blocks_for(n * (int64_t)objs.dim), kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), n,
-                                                                             t.X.get());
+        gather_rows(objs.X, objs.dim, perm.get(), n, t.X.get(), st);
         if (raw_rows) {   // angular distance: the raw rows in the same (leaf) order
             t.Xr.alloc((size_t)(n > 0 ? n : 1) * objs.dim, st);
-            k_gather_rows<<<blocks_for(n * (int64_t)objs.dim), kThreads, 0, st>>>(raw_rows, objs.dim, perm.get(), n,
-                                                                                 t.Xr.get());
+            gather_rows(raw_rows, objs.dim, perm.get(), n, t.Xr.get(), st);
         }
     } else {
         DBuf<int64_t> len(n + 1, st);
