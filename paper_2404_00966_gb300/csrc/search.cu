@@ -3038,7 +3038,7 @@ struct Runner {
         tq.emask = mask.get();
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
-        tc_regroup(ix->tree, tq, rg, st, ncount ? ncount->get() : nullptr, ix->tree.tc.dim_p <= 128);
+        tc_regroup(ix->tree, tq, rg, st, ncount ? ncount->get() : nullptr, true);
         clk.end();
         tc_finish(tq, rg);
     }
