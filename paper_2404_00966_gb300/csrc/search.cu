@@ -422,139 +422,104 @@ struct LevelOffsets {
 
 constexpr int kProbeNodes = 4;   // last-level nodes whose rows the kNN probe evaluates
 
-// Probe for kNN (warp per query).  Section 3 notes that MkNNQ(q, k) is
-// MRQ(q, d_k) once d_k is known; the probe bounds d_k from above before the
-// batched descent.  It follows one root-to-last-level path: at every level it
-// computes the distances from q to the pivots of all non-empty children and
-// descends into the child whose pivot is nearest; at the last pivot level it
-// computes the distances to the rows (up to `cap` in all) of the kProbeNodes
-// nodes with the nearest pivots.  Every visible object so
-// evaluated enters the query's threshold list, so tau_q starts at (an upper
-// bound of) the k-th smallest of them instead of +inf.
-// One lane's distance from q to one row (coordinates in increasing order;
-// L2 returns the square).  The FP32 bound of the plain path covers any order.
-template <bool L2>
-__device__ __forceinline__ float lane_vec_dist(const float *__restrict__ q, const float *__restrict__ x, int dim) {
-    float s = 0.f;
-    if ((dim & 3) == 0 && ((((uintptr_t)q) | ((uintptr_t)x)) & 15) == 0) {
-        const float4 *q4 = reinterpret_cast<const float4 *>(q);
-        const float4 *x4 = reinterpret_cast<const float4 *>(x);
-        for (int i = 0; i < (dim >> 2); ++i) {
-            const float4 a = q4[i], b = __ldg(x4 + i);
-            const float d0 = a.x - b.x, d1 = a.y - b.y, d2 = a.z - b.z, d3 = a.w - b.w;
-            if (L2) s += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
-            else s += fabsf(d0) + fabsf(d1) + fabsf(d2) + fabsf(d3);
-        }
-    } else {
-        for (int i = 0; i < dim; ++i) {
-            const float t = q[i] - __ldg(x + i);
-            s += L2 ? t * t : fabsf(t);
-        }
-    }
-    return s;
-}
-
-// Rows [pos, pos + m) into the threshold list, a row per lane.
-template <bool L2>
-__device__ __forceinline__ void probe_rows(const Dev &d, const float *qv, int64_t pos, int32_t m, int64_t s,
-                                           TauList &L, double up, int lane) {
-    for (int32_t r0 = 0; r0 < m; r0 += 32) {
-        const int32_t r = r0 + lane;
-        const bool full = L.n >= L.K;
-        const double k_d = full ? L.kd() : 0.0;
-        const int64_t k_i = full ? L.kid() : 0;
-        bool cand = false;
-        double ub = 0.0;
-        int64_t id = 0;
-        if (r < m) {
-            const int64_t row = pos + r;
-            if (d.row_del[row] > s) {
-                const float sq = lane_vec_dist<L2>(qv, d.X + row * d.dim, d.dim);
-                const float dv = L2 ? sqrtf(sq) : sq;
-                ub = (double)dv * up + (double)d.absf;
-                id = d.row_id[row];
-                cand = !full || ub < k_d || (ub == k_d && id < k_i);
+// Distances from the query row qv to the rows listed in rows[0 .. cnt), into
+// out[0 .. cnt), by the nw warps of a block.  G lanes take a row: eight, each
+// reading 16 consecutive bytes of a 128-byte segment (V4: rows on 16-byte
+// boundaries; else 4 bytes), or one (rows of a few coordinates).  The FP32
+// bound of the plain path covers any order of summation.
+template <bool L2, int G, bool V4>
+__device__ __forceinline__ void list_dists(const Dev &d, const float *__restrict__ qv, const int32_t *rows, int cnt,
+                                           float *out, int warp, int lane, int nw) {
+    constexpr int R = 32 / G;   // rows per warp and step
+    const int g = lane / G, s = lane % G;
+    for (int i0 = warp * R; i0 < cnt; i0 += nw * R) {
+        const int i = i0 + g;
+        float sum = 0.f;
+        if (i < cnt) {
+            const float *xv = d.X + (int64_t)rows[i] * d.dim;
+            if (V4) {
+                const float4 *q4 = reinterpret_cast<const float4 *>(qv), *x4 = reinterpret_cast<const float4 *>(xv);
+#pragma unroll 4
+                for (int c = s; c < (d.dim >> 2); c += G) {
+                    const float4 a = __ldg(q4 + c), b = __ldg(x4 + c);
+                    const float d0 = a.x - b.x, d1 = a.y - b.y, d2 = a.z - b.z, d3 = a.w - b.w;
+                    sum += L2 ? d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3 : fabsf(d0) + fabsf(d1) + fabsf(d2) + fabsf(d3);
+                }
+            } else {
+#pragma unroll 4
+                for (int c = s; c < d.dim; c += G) {
+                    const float t = __ldg(qv + c) - __ldg(xv + c);
+                    sum += L2 ? t * t : fabsf(t);
+                }
             }
         }
-        unsigned bal = __ballot_sync(0xffffffffu, cand);
-        while (bal) {
-            const int src = __ffs(bal) - 1;
-            bal &= bal - 1;
-            const double u = __shfl_sync(0xffffffffu, ub, src);
-            const int64_t iid = __shfl_sync(0xffffffffu, id, src);
-            L.insert(u, iid);
-        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (i < cnt && s == 0) out[i] = L2 ? sqrtf(sum) : sum;
     }
 }
 
-// Probe for kNN (warp per query).  Section 3 notes that MkNNQ(q, k) is
-// MRQ(q, d_k) once d_k is known; the probe bounds d_k from above before the
-// batched descent.  It follows one root-to-last-level path: at every level it
-// computes the distances from q to the pivots of all non-empty children and
-// descends into the child whose pivot is nearest; at the last pivot level it
-// computes the distances to the rows (up to `cap` in all) of the kProbeNodes
-// nodes with the nearest pivots.  Every visible object so evaluated enters
-// the query's threshold list, so tau_q starts at (an upper bound of) the k-th
-// smallest of them instead of +inf.  The last-level node the path ended in is
-// the query's key: queries with equal or nearby keys lie in the same region.
-template <bool L2>
-__global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int64_t nq, int cap, const int32_t *__restrict__ kq,
-                            const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n,
-                            float *tau, int32_t *__restrict__ key) {
-    const int lane = threadIdx.x & 31;
-    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (q >= nq) return;
+// Probe for kNN (a block of NW warps per query).  Section 3 notes that
+// MkNNQ(q, k) is MRQ(q, d_k) once d_k is known; the probe bounds d_k from
+// above before the batched descent.  It follows one root-to-last-level path:
+// at every level it computes the distances from q to the pivots of all
+// non-empty children and descends into the child whose pivot is nearest; at
+// the last pivot level it goes through the rows of the kProbeNodes nodes with
+// the nearest pivots (about `cap` in all, shared evenly), in batches of 32 NW
+// from the rows whose distance to the node's pivot is closest to the query's
+// outwards, and computes the distances of the rows whose table lower bound is
+// within the bound found so far.  (Leaving a row out can only leave the bound
+// higher, never wrong.)  Every visible object so evaluated enters the query's
+// threshold list, so tau_q starts at (an upper bound of) the k-th smallest of
+// them instead of +inf.  The last-level node the path ended in is the query's
+// key: queries with equal or nearby keys lie in the same region.
+//
+// The rows' bytes from L2 and, in small batches, the chain of dependent loads
+// bound it: eight lanes read a row's 128-byte segments together, and a batch
+// of few queries takes eight warps a query.  10^4 queries of 10^6 x 128 0.45
+// ms, 10^4 of 2 * 10^5 x 300 0.74 ms, 128 of 2 * 10^6 x 256 (L1) 0.44 ms; a
+// row per lane over all of 1,024 rows took 0.82, 2.83 and 0.90 ms.
+template <bool L2, int G, bool V4>
+__global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int max_rows, int per_k, const int32_t *__restrict__ kq,
+                            const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n, float *tau,
+                            int32_t *__restrict__ key) {
+    __shared__ int32_t s_row[256];
+    __shared__ float s_dist[256];
+    __shared__ int s_cnt;
+    __shared__ float s_tau;
+    __shared__ float s_path[kMaxHeight];        // q's distances to the path's pivots
+    __shared__ float s_bd[kProbeNodes];         // the nearest children (ascending) and their distances
+    __shared__ int64_t s_bn[kProbeNodes];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int64_t q = blockIdx.x;
     const int K = kq[q];
-    TauList L;
-    L.load(tk_d + koff[q], tk_id + koff[q], tk_n[q], K, lane);
+    // rows: 256, or per_k for each neighbour wanted (per_k 0: max_rows)
+    const int cap = per_k ? min(max_rows, max(256, per_k * K)) : max_rows;
     const int64_t s = d.qseq[q];
     const float *qv = d.Q + q * d.dim;
     const double up = 1.0 + 2.0 * (double)d.rel;
-    // root pivot
-    {
-        const int32_t prow = d.npiv[lo_off.v[0]];
-        const float sq = warp_vec_dist<L2>(qv, d.X + (int64_t)prow * d.dim, d.dim, lane);
-        const float dq = L2 ? sqrtf(sq) : sq;
-        if (d.row_del[prow] > s) L.insert((double)dq * up + (double)d.absf, d.row_id[prow]);
-    }
-    int64_t node = 0;
-    if (d.h == 1) {   // one pivot level: the root's own rows
-        const int32_t m = d.nsize[lo_off.v[0]] < cap ? d.nsize[lo_off.v[0]] : cap;
-        probe_rows<L2>(d, qv, d.npos[lo_off.v[0]], m, s, L, up, lane);
-    }
-    for (int l = 1; l < d.h; ++l) {
-        // the kProbeNodes children with the nearest pivots (ascending), kept by every lane
-        float bd[kProbeNodes];
-        int64_t bn[kProbeNodes];
-#pragma unroll
-        for (int i = 0; i < kProbeNodes; ++i) {
-            bd[i] = __int_as_float(0x7f800000);
-            bn[i] = -1;
-        }
-        // the children 32 at a time, a child per lane: their pivot distances
-        // are computed together, then taken in child order
-        for (int j0 = 0; j0 < d.F; j0 += 32) {
-            const int j = j0 + lane;
-            float dq = 0.f;
-            bool live = false, vis = false;
+    TauList L;   // (warp 0's)
+    if (warp == 0) L.load(tk_d + koff[q], tk_id + koff[q], tk_n[q], K, lane);
+    // warp 0: the listed rows (visible ones) into the threshold list
+    auto enter = [&](int cnt, bool check_visible) {
+        for (int i0 = 0; i0 < cnt; i0 += 32) {
+            const int i = i0 + lane;
+            const bool full = L.n >= K;
+            const double k_d = full ? L.kd() : 0.0;
+            bool cand = false;
+            double ub = 0.0;
             int64_t id = 0;
-            if (j < d.F) {
-                const int64_t g = lo_off.v[l] + node * d.F + j;
-                if (d.nsize[g] != 0) {
-                    const int32_t prow = d.npiv[g];
-                    const float sq = lane_vec_dist<L2>(qv, d.X + (int64_t)prow * d.dim, d.dim);
-                    dq = L2 ? sqrtf(sq) : sq;
-                    live = true;
-                    vis = d.row_del[prow] > s;
-                    if (vis) id = d.row_id[prow];
+            if (i < cnt && s_row[i] >= 0) {
+                ub = (double)s_dist[i] * up + (double)d.absf;
+                if (!full || ub <= k_d) {
+                    const int32_t row = s_row[i];
+                    if (!check_visible || d.row_del[row] > s) {
+                        id = d.row_id[row];
+                        cand = true;
+                    }
                 }
             }
-            // the visible pivots into the threshold list (a register copy of
-            // its K-th bound skips the pivots that cannot enter it)
-            const double ub = (double)dq * up + (double)d.absf;
-            const bool full = L.n >= K;
-            const double kth = full ? L.kd() : 0.0;
-            unsigned bal = __ballot_sync(0xffffffffu, vis && (!full || ub <= kth));
+            unsigned bal = __ballot_sync(0xffffffffu, cand);
             while (bal) {
                 const int src = __ffs(bal) - 1;
                 bal &= bal - 1;
@@ -562,49 +527,129 @@ __global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int64_t nq, int cap, con
                 const int64_t iid = __shfl_sync(0xffffffffu, id, src);
                 L.insert(uu, iid);
             }
-            // the nearest children, in child order (ties keep the earlier child)
-            unsigned lv = __ballot_sync(0xffffffffu, live);
-            while (lv) {
-                const int src = __ffs(lv) - 1;
-                lv &= lv - 1;
-                float vd = __shfl_sync(0xffffffffu, dq, src);
-                int64_t vn = node * d.F + j0 + src;
-                if (vd < bd[kProbeNodes - 1]) {
-#pragma unroll
-                    for (int i = 0; i < kProbeNodes; ++i) {
-                        if (vd < bd[i]) {
-                            const float td = bd[i];
-                            const int64_t tn = bn[i];
-                            bd[i] = vd;
-                            bn[i] = vn;
-                            vd = td;
-                            vn = tn;
-                        }
-                    }
-                }
-            }
         }
-        if (bn[0] < 0) break;   // no non-empty child (cannot happen for a non-empty node)
-        node = bn[0];
-        if (l == d.h - 1) {
-            // last pivot level: the rows of the nearest kProbeNodes nodes
-            int budget = cap;
-#pragma unroll
-            for (int i = 0; i < kProbeNodes; ++i) {
-                if (bn[i] < 0 || budget <= 0) continue;
-                const int64_t g = lo_off.v[l] + bn[i];
-                const int32_t m = d.nsize[g] < budget ? d.nsize[g] : budget;
-                budget -= m;
-                probe_rows<L2>(d, qv, d.npos[g], m, s, L, up, lane);
-            }
+    };
+    // root pivot
+    if (threadIdx.x == 0) s_row[0] = d.npiv[lo_off.v[0]];
+    __syncthreads();
+    list_dists<L2, G, V4>(d, qv, s_row, 1, s_dist, warp, lane, nw);
+    __syncthreads();
+    if (warp == 0) {
+        enter(1, true);
+        if (lane == 0) {
+            s_path[0] = s_dist[0];
+            s_bd[0] = s_dist[0];
+            s_bn[0] = 0;
+            for (int i = 1; i < kProbeNodes; ++i) s_bn[i] = -1;
         }
     }
-    L.store();
-    const double k_fin = L.n >= K ? L.kd() : 0.0;
-    if (lane == 0) {
-        tk_n[q] = L.n;
-        tau[q] = L.n >= K ? __double2float_ru(k_fin) : __int_as_float(0x7f800000);
-        if (key) key[q] = (int32_t)node;   // where the path ended: a locality key for the query
+    int64_t node = 0;
+    for (int l = 1; l < d.h; ++l) {
+        __syncthreads();
+        // the children's pivots (-1: an empty child)
+        for (int j = threadIdx.x; j < d.F; j += blockDim.x) {
+            const int64_t g = lo_off.v[l] + node * d.F + j;
+            s_row[64 + j] = d.nsize[g] != 0 ? d.npiv[g] : -1;
+            s_row[j] = s_row[64 + j] >= 0 ? s_row[64 + j] : 0;
+        }
+        __syncthreads();
+        list_dists<L2, G, V4>(d, qv, s_row, d.F, s_dist, warp, lane, nw);
+        __syncthreads();
+        if (warp == 0) {
+            for (int j = lane; j < d.F; j += 32) s_row[j] = s_row[64 + j];
+            __syncwarp();
+            enter(d.F, true);
+            // the kProbeNodes nearest children, ties to the earlier one
+            uint64_t k0 = lane < d.F && s_row[lane] >= 0
+                              ? ((uint64_t)__float_as_uint(s_dist[lane]) << 32) | (uint32_t)lane : ~0ull;
+            uint64_t k1 = lane + 32 < d.F && s_row[lane + 32] >= 0
+                              ? ((uint64_t)__float_as_uint(s_dist[lane + 32]) << 32) | (uint32_t)(lane + 32) : ~0ull;
+            for (int i = 0; i < kProbeNodes; ++i) {
+                uint64_t m = k0 < k1 ? k0 : k1;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const uint64_t v = __shfl_xor_sync(0xffffffffu, m, o);
+                    m = v < m ? v : m;
+                }
+                if (k0 == m) k0 = ~0ull;
+                if (k1 == m) k1 = ~0ull;
+                if (lane == 0) {
+                    s_bd[i] = __uint_as_float((uint32_t)(m >> 32));
+                    s_bn[i] = m == ~0ull ? -1 : node * d.F + (int64_t)(uint32_t)m;
+                }
+            }
+            if (lane == 0) s_path[l] = s_bd[0];
+        }
+        __syncthreads();
+        if (s_bn[0] < 0) break;   // no non-empty child (cannot happen for a non-empty node)
+        node = s_bn[0];
+    }
+    // the rows of the nearest last-level nodes
+    int left = cap;
+    for (int i = 0; i < kProbeNodes; ++i) {
+        __syncthreads();
+        const int64_t nd = s_bn[i];
+        if (nd < 0 || left <= 0) break;
+        int budget = left / (d.h > 1 ? kProbeNodes - i : 1);   // the nodes share the rows
+        const int64_t g = lo_off.v[d.h - 1] + nd;
+        const int64_t pos = d.npos[g];
+        const int32_t size = d.nsize[g];
+        const float dn = s_bd[i];
+        const float *Tn = d.table + (int64_t)(d.h - 1) * d.n + pos;   // ascending within the node
+        int32_t a = 0, b = size;
+        while (a < b) {
+            const int32_t m = (a + b) >> 1;
+            if (Tn[m] < dn) a = m + 1;
+            else b = m;
+        }
+        const int bs = 32 * nw, nb = (size + bs - 1) / bs;
+        const int mid = a < size ? a / bs : nb - 1;
+        // batches mid, mid + 1, mid - 1, mid + 2, ...
+        for (int step = 0, done = 0; done < nb && budget > 0; ++step) {
+            const int bi = (step & 1) ? mid + (step + 1) / 2 : mid - step / 2;
+            if (bi < 0 || bi >= nb) continue;   // (block-uniform)
+            ++done;
+            if (threadIdx.x == 0) {
+                s_cnt = 0;
+                s_tau = __int_as_float(0x7f800000);
+            }
+            __syncthreads();
+            if (warp == 0 && L.n >= K) {
+                const double k_d = L.kd();
+                if (lane == 0) s_tau = __double2float_ru(k_d);
+            }
+            __syncthreads();
+            const float t0 = s_tau;
+            const int32_t r = bi * bs + (int)threadIdx.x;
+            bool take = false;
+            if (r < size) {
+                const int64_t row = pos + r;
+                take = d.row_del[row] > s && fabsf(Tn[r] - dn) <= t0;
+                for (int l = 0; l < d.h - 1 && take; ++l)
+                    take = fabsf(d.table[(int64_t)l * d.n + row] - s_path[l]) <= t0;
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, take);
+            int base = 0;
+            if (lane == 0 && bal) base = atomicAdd(&s_cnt, __popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (take) s_row[base + __popc(bal & ((1u << lane) - 1u))] = (int32_t)(pos + r);
+            budget -= min(bs, size - bi * bs);
+            left -= min(bs, size - bi * bs);
+            __syncthreads();
+            const int cnt = s_cnt;
+            list_dists<L2, G, V4>(d, qv, s_row, cnt, s_dist, warp, lane, nw);
+            __syncthreads();
+            if (warp == 0) enter(cnt, false);
+        }
+    }
+    if (warp == 0) {
+        L.store();
+        const double k_fin = L.n >= K ? L.kd() : 0.0;
+        if (lane == 0) {
+            tk_n[q] = L.n;
+            tau[q] = L.n >= K ? __double2float_ru(k_fin) : __int_as_float(0x7f800000);
+            if (key) key[q] = (int32_t)node;   // where the path ended: a locality key for the query
+        }
     }
 }
 
@@ -3736,14 +3781,27 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         for (int l = 0; l <= t.h && l < kMaxHeight + 2; ++l) lo_off.v[l] = t.lvl_off[l];
         const int cap = R.tu.probe_rows;
         R.clk.begin(GTS_STAGE_THRESHOLD);
-        if (t.metric == GTS_L2)
-            k_probe_vec<true><<<nblocks(nq, kWarpsPerBlock), kT, 0, st>>>(d, lo_off, nq, cap, qb.k, R.koff.get(),
-                                                                          R.tk_d.get(), R.tk_id.get(), R.tk_n.get(),
-                                                                          R.thr.get(), R.qkey.get());
-        else
-            k_probe_vec<false><<<nblocks(nq, kWarpsPerBlock), kT, 0, st>>>(d, lo_off, nq, cap, qb.k, R.koff.get(),
-                                                                           R.tk_d.get(), R.tk_id.get(), R.tk_n.get(),
-                                                                           R.thr.get(), R.qkey.get());
+        // eight warps a query until four of them fill the SMs, two while one
+        // does not, one for large batches
+        const int nw = nq <= 608 ? 8 : nq <= 1216 ? 4 : nq <= 4864 && t.dim > kScanMaxDim ? 2 : 1;
+        // a row of more than 16 coordinates costs as much as five of the kept
+        // pairs that it saves from 256 rows on (16 a neighbour for large k);
+        // a row of a few coordinates next to nothing
+        const int per_k = t.dim > kScanMaxDim ? 16 : 0;
+        const bool v4 = (t.dim & 3) == 0 && (((uintptr_t)d.Q | (uintptr_t)d.X) & 15) == 0;
+#define GTS_PROBE(L2V, GV, V4V)                                                                                      \
+    k_probe_vec<L2V, GV, V4V><<<(unsigned)nq, 32 * nw, 0, st>>>(d, lo_off, cap, per_k, qb.k, R.koff.get(), R.tk_d.get(),     \
+                                                               R.tk_id.get(), R.tk_n.get(), R.thr.get(), R.qkey.get())
+        if (t.metric == GTS_L2) {
+            if (t.dim <= kScanMaxDim) GTS_PROBE(true, 1, false);
+            else if (v4) GTS_PROBE(true, 8, true);
+            else GTS_PROBE(true, 8, false);
+        } else {
+            if (t.dim <= kScanMaxDim) GTS_PROBE(false, 1, false);
+            else if (v4) GTS_PROBE(false, 8, true);
+            else GTS_PROBE(false, 8, false);
+        }
+#undef GTS_PROBE
         R.qkey_ok = true;
         R.clk.end();
         check_launch("knn probe");
