@@ -128,7 +128,10 @@ struct DevObjects {
     std::vector<int64_t> h_off;   // host offsets (strings)
 };
 
-void load_objects(const gts_objects *o, int want_dim_or_neg, DevObjects &out, cudaStream_t st, const char *what) {
+// check_now = false: the coordinates' check is left to the caller, who
+// launches k_nonfinite over out.v
+void load_objects(const gts_objects *o, int want_dim_or_neg, DevObjects &out, cudaStream_t st, const char *what,
+                  bool check_now = true) {
     GTS_REQUIRE(o != nullptr, GTS_EINVAL, std::string(what) + " is NULL");
     GTS_REQUIRE(o->n >= 0, GTS_EINVAL, std::string(what) + ": negative n");
     GTS_REQUIRE(o->n < ((int64_t)1 << 31), GTS_EINVAL, std::string(what) + ": n >= 2^31");
@@ -150,7 +153,7 @@ void load_objects(const gts_objects *o, int want_dim_or_neg, DevObjects &out, cu
             if (cnt) GTS_CUDA(cudaMemcpyAsync(out.X.get(), o->data, cnt * 4, cudaMemcpyHostToDevice, st));
             out.v.X = out.X.get();
         }
-        if (cnt) {
+        if (cnt && check_now) {
             DBuf<int> flag(1, st);
             GTS_CUDA(cudaMemsetAsync(flag.get(), 0, 4, st));
             k_nonfinite<<<std::min<int64_t>(nb((int64_t)cnt), 4096), kT, 0, st>>>(out.v.X, (int64_t)cnt, flag.get());
@@ -221,6 +224,36 @@ void copy_small_to_device(const T *src, int64_t n, bool on_device, DBuf<T> &dst,
         std::memcpy(host.data(), src, n * sizeof(T));
         GTS_CUDA(cudaMemcpyAsync(dst.get(), src, n * sizeof(T), cudaMemcpyHostToDevice, st));
     }
+}
+
+// What a query call reads back about its device-resident inputs, in one copy.
+struct QueryCheck {
+    int nonfinite, bad;           // a coordinate / a radius or k is out of range
+    unsigned long long max_k, sum_k;
+};
+__global__ void k_check_k(const int32_t *__restrict__ k, int64_t n, QueryCheck *__restrict__ c) {
+    unsigned long long mx = 0, sum = 0;
+    bool bad = false;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t v = k[i];
+        bad |= v < 1 || v > 1024;
+        mx = v > 0 && (unsigned long long)v > mx ? (unsigned long long)v : mx;
+        sum += v > 0 ? (unsigned long long)v : 0ull;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = m2 > mx ? m2 : mx;
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    if (bad) c->bad = 1;
+    if ((threadIdx.x & 31) == 0 && sum) {
+        atomicMax(&c->max_k, mx);
+        atomicAdd(&c->sum_k, sum);
+    }
+}
+__global__ void k_check_radii(const float *__restrict__ r, int64_t n, QueryCheck *__restrict__ c) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        if (!(isfinite(r[i]) && r[i] >= 0.f)) c->bad = 1;
 }
 
 __global__ void k_scatter_marks(int64_t *dst, const int64_t *pos, const int64_t *val, int64_t n) {
@@ -600,11 +633,80 @@ gts_status query_common(gts_index *ix, const gts_objects *q, const float *radii,
         GTS_REQUIRE(q != nullptr, GTS_EINVAL, "queries are NULL");
         GTS_REQUIRE((ix->metric == GTS_EDIT) == (q->dim == 0), GTS_EINVAL, "query kind does not match the metric");
         DevObjects dq;
-        load_objects(q, ix->dim, dq, st, "queries");
+        load_objects(q, ix->dim, dq, st, "queries", /*check_now=*/false);
         const int64_t nq = dq.v.n;
+        const bool dev = q->on_device != 0;
         QueryBatch qb;
         qb.nq = nq;
         qb.dim = ix->dim;
+        DBuf<float> drad;
+        DBuf<int32_t> dk;
+        DBuf<int64_t> dseq;
+        std::vector<float> hrad;
+        std::vector<int64_t> hseq;
+        // the coordinates and, where they are on the device, k or the radii
+        // are checked there and the verdict read once
+        DBuf<QueryCheck> chk(1, st);
+        QueryCheck hc = {0, 0, 0, 0};
+        bool read = false;
+        GTS_CUDA(cudaMemsetAsync(chk.get(), 0, sizeof(QueryCheck), st));
+        const int64_t coords = ix->dim > 0 ? nq * ix->dim : 0;
+        if (coords > 0) {
+            k_nonfinite<<<std::min<int64_t>(nb((coords + 15) / 16), 4096), kT, 0, st>>>(dq.v.X, coords,
+                                                                                       &chk.get()->nonfinite);
+            read = true;
+        }
+        if (knn) {
+            GTS_REQUIRE(nq == 0 || k != nullptr, GTS_EINVAL, "k is NULL");
+            if (dev) {
+                dk.alloc(nq > 0 ? nq : 1, st);   // (a copy: what is checked is what is used)
+                if (nq > 0) {
+                    GTS_CUDA(cudaMemcpyAsync(dk.get(), k, nq * 4, cudaMemcpyDeviceToDevice, st));
+                    k_check_k<<<std::min<int64_t>(nb(nq), 256), kT, 0, st>>>(dk.get(), nq, chk.get());
+                    read = true;
+                }
+                qb.k = dk.get();
+            } else {
+                std::vector<int32_t> hk;
+                copy_small_to_device(k, nq, false, dk, hk, st);
+                for (int64_t i = 0; i < nq; ++i) {
+                    GTS_REQUIRE(hk[i] >= 1 && hk[i] <= 1024, GTS_EINVAL, "k must be in 1 .. 1024");
+                    hc.max_k = std::max<unsigned long long>(hc.max_k, (unsigned long long)hk[i]);
+                    hc.sum_k += (unsigned long long)hk[i];
+                }
+                qb.k = dk.get();
+                qb.max_k = (int64_t)hc.max_k;
+                qb.sum_k = (int64_t)hc.sum_k;
+            }
+        } else {
+            GTS_REQUIRE(nq == 0 || radii != nullptr, GTS_EINVAL, "radii is NULL");
+            if (dev && ix->metric != GTS_COS) {
+                drad.alloc(nq > 0 ? nq : 1, st);
+                if (nq > 0) {
+                    GTS_CUDA(cudaMemcpyAsync(drad.get(), radii, nq * 4, cudaMemcpyDeviceToDevice, st));
+                    k_check_radii<<<std::min<int64_t>(nb(nq), 256), kT, 0, st>>>(drad.get(), nq, chk.get());
+                    read = true;
+                }
+                qb.radii = drad.get();
+            } else {   // (the angular limits are formed on the host)
+                copy_small_to_device(radii, nq, dev, drad, hrad, st);
+                for (int64_t i = 0; i < nq; ++i)
+                    GTS_REQUIRE(std::isfinite(hrad[i]) && hrad[i] >= 0.f, GTS_EINVAL, "radius must be finite and >= 0");
+                qb.radii = drad.get();
+            }
+        }
+        if (read) {
+            QueryCheck got;
+            GTS_CUDA(cudaMemcpyAsync(&got, chk.get(), sizeof(got), cudaMemcpyDeviceToHost, st));
+            GTS_CUDA(cudaStreamSynchronize(st));
+            GTS_REQUIRE(got.nonfinite == 0, GTS_EINVAL, "queries: NaN or infinite coordinate");
+            GTS_REQUIRE(got.bad == 0, GTS_EINVAL,
+                        knn ? "k must be in 1 .. 1024" : "radius must be finite and >= 0");
+            if (knn && dev) {
+                qb.max_k = (int64_t)got.max_k;
+                qb.sum_k = (int64_t)got.sum_k;
+            }
+        }
         qb.Q = dq.v.X;
         DBuf<float> qunit;
         if (ix->metric == GTS_COS) {   // unit query vectors for the L2 kernels, the raw ones for the FP64 keys
@@ -616,27 +718,6 @@ gts_status query_common(gts_index *ix, const gts_objects *q, const float *radii,
         qb.Soff = dq.v.Soff;
         qb.max_len = dq.v.max_len;
         qb.seq_now = ix->seq;
-        DBuf<float> drad;
-        DBuf<int32_t> dk;
-        DBuf<int64_t> dseq;
-        std::vector<float> hrad;
-        std::vector<int32_t> hk;
-        std::vector<int64_t> hseq;
-        if (knn) {
-            GTS_REQUIRE(nq == 0 || k != nullptr, GTS_EINVAL, "k is NULL");
-            copy_small_to_device(k, nq, q->on_device != 0, dk, hk, st);
-            for (int64_t i = 0; i < nq; ++i) {
-                GTS_REQUIRE(hk[i] >= 1 && hk[i] <= 1024, GTS_EINVAL, "k must be in 1 .. 1024");
-                qb.max_k = std::max<int64_t>(qb.max_k, hk[i]);
-            }
-            qb.k = dk.get();
-        } else {
-            GTS_REQUIRE(nq == 0 || radii != nullptr, GTS_EINVAL, "radii is NULL");
-            copy_small_to_device(radii, nq, q->on_device != 0, drad, hrad, st);
-            for (int64_t i = 0; i < nq; ++i)
-                GTS_REQUIRE(std::isfinite(hrad[i]) && hrad[i] >= 0.f, GTS_EINVAL, "radius must be finite and >= 0");
-            qb.radii = drad.get();
-        }
         DBuf<double> dlim;
         if (!knn && ix->metric == GTS_COS && nq > 0) {
             // the FP64 limits 1 - cos(r) of the range test, on the host

@@ -33,6 +33,7 @@
 #include "tile_str.cuh"
 #include "tile_tc.cuh"
 #include "scan.cuh"
+#include "scan_block.cuh"
 
 namespace gts {
 namespace {
@@ -2305,8 +2306,9 @@ __global__ void k_knn_counts(const int32_t *bn, int64_t nq, int64_t *counts) {
 __global__ void k_knn_emit(const int64_t *__restrict__ offsets, const int64_t *__restrict__ koff,
                            const double *__restrict__ bd, const int64_t *__restrict__ bi, const int32_t *__restrict__ bn,
                            int64_t nq, bool l2, bool cosine, int64_t *__restrict__ ids, float *__restrict__ dist,
-                           double *__restrict__ keys) {
+                           double *__restrict__ keys, unsigned long long *__restrict__ total) {
     const int64_t q = blockIdx.x;
+    if (q == 0 && threadIdx.x == 0) *total = (unsigned long long)offsets[nq];
     if (q >= nq) return;
     for (int i = threadIdx.x; i < bn[q]; i += blockDim.x) {
         const double key = bd[koff[q] + i];
@@ -2463,7 +2465,7 @@ struct Runner {
     std::vector<DBuf<uint64_t>> rkeys;
     std::vector<DBuf<float>> rdists;
     std::vector<int64_t> rcounts;
-    DBuf<unsigned long long> counters;   // [0] rechecks, [1] scanned rows
+    DBuf<unsigned long long> counters;   // [0] rechecks, [1] scanned rows, [2] kNN: answers
     int64_t st_pivots = 0, st_frontier = 0, st_cands = 0, st_groups = 0, st_cache = 0;
     int64_t st_tiles = 0, st_tile_entries = 0, st_table_pass = 0;
     int64_t st_scan_rows = 0, st_scan_records = 0;   // node-major scan: table rows read, records tested
@@ -2500,8 +2502,14 @@ struct Runner {
     }
 
     void scan_i32(const DBuf<int32_t> &cnt, int64_t E, DBuf<int64_t> &off) {
-        DBuf<int64_t> c64(E + 1, st);
         off.alloc(E + 1, st);
+        if (E <= kScanBlockMax) {
+            clk.begin(GTS_STAGE_OTHER);
+            k_scan_block<int32_t><<<1, 1024, 0, st>>>(cnt.get(), E, off.get());
+            clk.end();
+            return;
+        }
+        DBuf<int64_t> c64(E + 1, st);
         clk.begin(GTS_STAGE_OTHER, 2);
         k_i32_to_i64<<<nblocks(E, kT), kT, 0, st>>>(cnt.get(), E, c64.get());
         exclusive_scan(c64.get(), off.get(), E + 1, st);
@@ -2643,8 +2651,15 @@ struct Runner {
         return out;
     }
 
-    void group_range(const DBuf<int64_t> &off, int64_t g0, int64_t g1, int64_t &o0, int64_t &o1,
-                     DBuf<int64_t> &offg) {
+    // the group [g0, g1) of E entries: its first and last offset, and its
+    // offsets from 0 on (the one group of a batch that fits: `off` itself)
+    const int64_t *group_range(const DBuf<int64_t> &off, int64_t E, int64_t total, int64_t g0, int64_t g1, int64_t &o0,
+                               int64_t &o1, DBuf<int64_t> &offg) {
+        if (g0 == 0 && g1 == E) {
+            o0 = 0;
+            o1 = total;
+            return off.get();
+        }
         GTS_CUDA(cudaMemcpyAsync(&o0, off.get() + g0, 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaMemcpyAsync(&o1, off.get() + g1, 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
@@ -2652,6 +2667,7 @@ struct Runner {
         clk.begin(GTS_STAGE_OTHER);
         k_shift<<<nblocks(g1 - g0 + 1, kT), kT, 0, st>>>(off.get() + g0, g1 - g0 + 1, o0, offg.get());
         clk.end();
+        return offg.get();
     }
 
     void process(Level &L, int64_t e0, int64_t e1, int l) {
@@ -2693,7 +2709,7 @@ struct Runner {
                 const int64_t g0 = gb[g], g1 = gb[g + 1];
                 int64_t o0 = 0, o1 = 0;
                 DBuf<int64_t> offg;
-                group_range(off, g0, g1, o0, o1, offg);
+                const int64_t *goff = group_range(off, E, total, g0, g1, o0, o1, offg);
                 Level N;
                 N.E = o1 - o0;
                 if (N.E == 0) continue;
@@ -2703,7 +2719,7 @@ struct Runner {
                 clk.begin(GTS_STAGE_EXPAND);
                 k_expand<1><<<cap(nblocks(g1 - g0, kWarpsPerBlock)), kT, 0, st>>>(
                     d, L.q.get(), L.node.get(), L.path.get(), l, lvl_next, e0 + g0, e0 + g1, thr.get(), nullptr,
-                    offg.get(), N.q.get(), N.node.get(), N.path.get(), cmask.get() + g0);
+                    goff, N.q.get(), N.node.get(), N.path.get(), cmask.get() + g0);
                 clk.end();
                 check_launch("expand write");
                 process(N, 0, N.E, l + 1);
@@ -2744,14 +2760,14 @@ struct Runner {
                 const int64_t g0 = gb[g], g1 = gb[g + 1];
                 int64_t o0 = 0, o1 = 0;
                 DBuf<int64_t> offg;
-                group_range(off, g0, g1, o0, o1, offg);
+                const int64_t *goff = group_range(off, E, total, g0, g1, o0, o1, offg);
                 const int64_t C = o1 - o0;
                 if (C == 0) continue;
                 DBuf<int32_t> cq(C, st), crow(C, st);
                 clk.begin(GTS_STAGE_LEAF_SCAN);
                 k_leafscan<true><<<nblocks(g1 - g0, kWarpsPerBlock), kT, 0, st>>>(
                     d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0, thr.get(),
-                    nullptr, offg.get(), cq.get(), crow.get(), nullptr);
+                    nullptr, goff, cq.get(), crow.get(), nullptr);
                 clk.end();
                 check_launch("leaf scan write");
                 verify_and_collect(cq, crow, C);
@@ -3636,6 +3652,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     Tree &t = ix->tree;
     Cache &c = ix->cache;
     const int64_t nq = qb.nq;
+    Arena arena(st);
     Runner R(ix, qb, knn, budget, st);
     {
         std::lock_guard<std::mutex> g(ix->tune_mu);
@@ -3662,6 +3679,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     if (precision == GTS_PREC_BF16 && !low_dim && tc_supported(t)) {
         {
             std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build it once
+            Arena::Pause index_owned;
             tc_prepare(t, t.tc, st);
             if (tc_dense_supported(t, t.tc)) tc_prepare_pivots(t, t.tc, st);
         }
@@ -3710,6 +3728,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         {
             std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build it once
             if (!t.qg_ready) {
+                Arena::Pause index_owned;
                 t.qg.alloc(t.n * kQgBuckets, st);
                 k_qgram_hist<<<nblocks(t.n, 256), 256, 0, st>>>(t.S.get(), t.Soff.get(), t.n, t.qg.get());
                 GTS_CUDA(cudaStreamSynchronize(st));
@@ -3743,8 +3762,8 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     R.clk.end();
     d.qseq = qseq.get();
     R.thr.alloc(nq, st);
-    R.counters.alloc(2, st);
-    GTS_CUDA(cudaMemsetAsync(R.counters.get(), 0, 16, st));
+    R.counters.alloc(3, st);
+    GTS_CUDA(cudaMemsetAsync(R.counters.get(), 0, 24, st));
     if (qb.count_table_pass) {
         R.tp_count.alloc(2, st);
         GTS_CUDA(cudaMemsetAsync(R.tp_count.get(), 0, 16, st));
@@ -3756,7 +3775,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         k_k_to_i64<<<nblocks(nq, kT), kT, 0, st>>>(qb.k, nq, k64.get());
         exclusive_scan(k64.get(), R.koff.get(), nq + 1, st);
         R.clk.end();
-        const int64_t ktot = d2h_i64(R.koff.get() + nq, st);
+        const int64_t ktot = qb.sum_k;
         R.tk_d.alloc(ktot, st);
         R.tk_id.alloc(ktot, st);
         R.bd.alloc(ktot, st);
@@ -3820,30 +3839,40 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     }
     if (nq > 0) R.cache_pass();
     // ---- assemble the CSR answer
-    out.offsets.alloc(nq + 1, st);
+    // (the answers' arrays may outlive the call; kNN: room for every k, the
+    // number of answers is read with the counters at the end)
+    {
+        Arena::Pause answers;
+        out.offsets.alloc(nq + 1, st);
+        if (knn) {
+            const int64_t room = std::max<int64_t>(qb.sum_k, 1);
+            out.ids.alloc(room, st);
+            out.dist.alloc(room, st);
+            if (qb.want_keys) out.key.alloc(room, st);
+        }
+    }
     if (knn) {
         DBuf<int64_t> counts(nq + 1, st);
         R.clk.begin(GTS_STAGE_OTHER, 2);
         k_knn_counts<<<nblocks(nq, kT), kT, 0, st>>>(R.bn.get(), nq, counts.get());
         exclusive_scan(counts.get(), out.offsets.get(), nq + 1, st);
         R.clk.end();
-        out.total = d2h_i64(out.offsets.get() + nq, st);
-        out.ids.alloc(out.total ? out.total : 1, st);
-        out.dist.alloc(out.total ? out.total : 1, st);
-        if (qb.want_keys) out.key.alloc(out.total ? out.total : 1, st);
         R.clk.begin(GTS_STAGE_OTHER);
         k_knn_emit<<<(unsigned)(nq > 0 ? nq : 1), 128, 0, st>>>(out.offsets.get(), R.koff.get(), R.bd.get(),
                                                                 R.bi.get(), R.bn.get(), nq, t.metric == GTS_L2,
                                                                 t.cosine, out.ids.get(), out.dist.get(),
-                                                                out.key.get());
+                                                                out.key.get(), R.counters.get() + 2);
         R.clk.end();
     } else {
         int64_t Rt = 0;
         for (auto v : R.rcounts) Rt += v;
         DBuf<uint64_t> keys(Rt ? Rt : 1, st), keys2(Rt ? Rt : 1, st);
         DBuf<float> dd(Rt ? Rt : 1, st);
-        out.dist.alloc(Rt ? Rt : 1, st);
-        out.ids.alloc(Rt ? Rt : 1, st);
+        {
+            Arena::Pause answers;
+            out.dist.alloc(Rt ? Rt : 1, st);
+            out.ids.alloc(Rt ? Rt : 1, st);
+        }
         // ids are below next_id (< 2^31): the keys keep idbits id bits
         int idbits = 1;
         while (idbits < 32 && ((int64_t)1 << idbits) < ix->next_id) ++idbits;
@@ -3878,10 +3907,11 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         out.total = Rt;
     }
     check_launch("assemble");
-    unsigned long long hc[2] = {0, 0}, htp[2] = {0, 0};
-    GTS_CUDA(cudaMemcpyAsync(hc, R.counters.get(), 16, cudaMemcpyDeviceToHost, st));
+    unsigned long long hc[3] = {0, 0, 0}, htp[2] = {0, 0};
+    GTS_CUDA(cudaMemcpyAsync(hc, R.counters.get(), 24, cudaMemcpyDeviceToHost, st));
     if (qb.count_table_pass) GTS_CUDA(cudaMemcpyAsync(htp, R.tp_count.get(), 16, cudaMemcpyDeviceToHost, st));
     GTS_CUDA(cudaStreamSynchronize(st));
+    if (knn) out.total = (int64_t)hc[2];
     if (stage_ms) R.clk.collect(stage_ms);
     if (stats) {
         stats[GTS_STAT_PIVOT_DIST] = R.st_pivots;

@@ -39,6 +39,7 @@
 
 #include "gts_impl.cuh"
 #include "metric.cuh"
+#include "scan_block.cuh"
 #include "tc.cuh"
 #include "tile_tc.cuh"
 
@@ -903,11 +904,31 @@ void exscan(const T *in, T *out, int64_t n, cudaStream_t st) {
     GTS_CUDA(cub::DeviceScan::ExclusiveSum(tmp.get(), tb, in, out, n, st));
 }
 
+// offsets [n + 1] of n counts
+template <class T>
+void count_offsets(const T *cnt, int64_t *off, int64_t n, cudaStream_t st);
+
 inline unsigned nblk(int64_t n, int per = 256) {
     int64_t b = (n + per - 1) / per;
     if (b < 1) b = 1;
     if (b > 0x7fffffffLL) b = 0x7fffffffLL;
     return (unsigned)b;
+}
+
+template <>
+void count_offsets<int32_t>(const int32_t *cnt, int64_t *off, int64_t n, cudaStream_t st) {
+    if (n <= kScanBlockMax) {
+        k_scan_block<int32_t><<<1, 1024, 0, st>>>(cnt, n, off);
+        return;
+    }
+    DBuf<int64_t> c64(n + 1, st);
+    k_i32_to_i64_tc<<<nblk(n), 256, 0, st>>>(cnt, n, c64.get());
+    exscan(c64.get(), off, n + 1, st);
+}
+template <>
+void count_offsets<int64_t>(const int64_t *cnt, int64_t *off, int64_t n, cudaStream_t st) {   // (cnt[n] = 0)
+    if (n <= kScanBlockMax) k_scan_block<int64_t><<<1, 1024, 0, st>>>(cnt, n, off);
+    else exscan(cnt, off, n + 1, st);
 }
 
 size_t tile_smem_bytes(int dim_p, int h, int kNQ, int SB, int SM) {
@@ -993,11 +1014,9 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
         }
     }
     const int32_t *ncnt = (counts && !use_bits) ? counts : own.get();
-    DBuf<int64_t> c64(nn + 1, st);
     DBuf<int64_t> &noff = rg.noff;
     noff.alloc(nn + 1, st);
-    k_i32_to_i64_tc<<<nblk(nn), 256, 0, st>>>(ncnt, nn, c64.get());
-    exscan(c64.get(), noff.get(), nn + 1, st);
+    count_offsets(ncnt, noff.get(), nn, st);
     int64_t total_entries = 0;
     GTS_CUDA(cudaMemcpyAsync(&total_entries, noff.get() + nn, 8, cudaMemcpyDeviceToHost, st));
     GTS_CUDA(cudaStreamSynchronize(st));
@@ -1032,7 +1051,7 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
     DBuf<unsigned long long> pairs(1, st);
     GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
     k_items_per_node<<<nblk(nn), 256, 0, st>>>(ncnt, lsize, nn, nitems.get(), pairs.get());
-    exscan(nitems.get(), ioff.get(), nn + 1, st);
+    count_offsets((const int64_t *)nitems.get(), ioff.get(), nn, st);
     int64_t total_items = 0;
     unsigned long long total_pairs = 0;
     GTS_CUDA(cudaMemcpyAsync(&total_items, ioff.get() + nn, 8, cudaMemcpyDeviceToHost, st));
@@ -1062,7 +1081,7 @@ int64_t tc_regroup_children(const Tree &t, const TcQuery &tq, TcRegroup &rg, cud
     DBuf<unsigned long long> pairs(1, st);
     GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
     k_child_items<<<nblk(nc), 256, 0, st>>>(ncnt, csize, nc, t.F, nitems.get(), pairs.get());
-    exscan(nitems.get(), ioff.get(), nc + 1, st);
+    count_offsets((const int64_t *)nitems.get(), ioff.get(), nc, st);
     int64_t total_items = 0;
     unsigned long long total_pairs = 0;
     GTS_CUDA(cudaMemcpyAsync(&total_items, ioff.get() + nc, 8, cudaMemcpyDeviceToHost, st));
@@ -1085,15 +1104,14 @@ int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegro
     rg.wpre.alloc(nn * nw, st);
     k_bits_rows<<<(unsigned)std::min<int64_t>(nn, 65535), 256, 0, st>>>(rg.bits.get(), nn, nw, rg.wpre.get(),
                                                                          ncnt.get());
-    DBuf<int64_t> c64(nn + 1, st), nitems(nn + 1, st), ioff(nn + 1, st);
+    DBuf<int64_t> nitems(nn + 1, st), ioff(nn + 1, st);
     rg.noff.alloc(nn + 1, st);
-    k_i32_to_i64_tc<<<nblk(nn), 256, 0, st>>>(ncnt.get(), nn, c64.get());
-    exscan(c64.get(), rg.noff.get(), nn + 1, st);
+    count_offsets((const int32_t *)ncnt.get(), rg.noff.get(), nn, st);
     const int32_t *lsize = t.nsize.get() + t.lvl_off[t.h - 1];
     DBuf<unsigned long long> pairs(1, st);
     GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
     k_items_per_node<<<nblk(nn), 256, 0, st>>>(ncnt.get(), lsize, nn, nitems.get(), pairs.get());
-    exscan(nitems.get(), ioff.get(), nn + 1, st);
+    count_offsets((const int64_t *)nitems.get(), ioff.get(), nn, st);
     int64_t total_items = 0, total_entries = 0;
     unsigned long long total_pairs = 0;
     GTS_CUDA(cudaMemcpyAsync(&total_items, ioff.get() + nn, 8, cudaMemcpyDeviceToHost, st));
