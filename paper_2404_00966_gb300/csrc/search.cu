@@ -959,6 +959,59 @@ __global__ void k_leafscan(Dev d, const int32_t *__restrict__ eq, const int32_t 
     }
 }
 
+// The same for nodes of a few rows, a thread per entry (a warp per entry leaves
+// most lanes idle: 0.36 + 0.26 ms for 6 * 10^5 entries of 2.4 rows, here 0.033 +
+// 0.033).
+constexpr int kLeafThreadRows = 8;   // average rows per node up to which a thread takes an entry
+template <bool WRITE>
+__global__ void k_leafscan_small(Dev d, const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
+                                 const float *__restrict__ path, int64_t lvl_last, int64_t e0, int64_t e1,
+                                 const uint64_t *__restrict__ mask, const float *__restrict__ thr_q,
+                                 int32_t *__restrict__ cnt, const int64_t *__restrict__ off, int32_t *__restrict__ cq,
+                                 int32_t *__restrict__ crow, unsigned long long *__restrict__ scanned) {
+    const int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    int32_t count = 0, tested = 0;
+    if (e < e1) {
+        const uint64_t m = mask[e - e0];
+        if (m != 0) {
+            const int32_t q = eq[e];
+            const int64_t node = lvl_last + enode[e];
+            const int32_t pos = d.npos[node], size = d.nsize[node];
+            const int32_t avg = size / d.F;
+            const int64_t s = d.qseq[q];
+            const float thr = thr_q[q];
+            const int64_t base = WRITE ? off[e - e0] : 0;
+            // (the bound keeps every write inside this entry's slot)
+            const int64_t lim = WRITE ? off[e - e0 + 1] : 0;
+            for (int32_t r = 0; r < size; ++r) {
+                int32_t j = avg > 0 ? r / avg : d.F - 1;
+                if (j > d.F - 1) j = d.F - 1;
+                if (!((m >> j) & 1ull)) continue;
+                ++tested;
+                const int64_t row = pos + r;
+                if (d.row_del[row] <= s) continue;
+                bool pass = true;
+                for (int t = 0; t < d.h && pass; ++t) {
+                    const float T = d.table[(int64_t)t * d.n + row], dq = path[e * d.h + t];
+                    const float eps = (d.epsc > 0.f ? d.epsc * (T + dq + thr) : 0.f) + d.lslack[t];
+                    if (fabsf(T - dq) > thr + eps) pass = false;
+                }
+                if (!pass) continue;
+                if (WRITE && base + count < lim) {
+                    cq[base + count] = q;
+                    crow[base + count] = pos + r;
+                }
+                ++count;
+            }
+        }
+        if (!WRITE) cnt[e - e0] = count;
+    }
+    if (!WRITE) {
+        tested = __reduce_add_sync(0xffffffffu, (unsigned)tested);
+        if ((threadIdx.x & 31) == 0 && tested) atomicAdd(scanned, (unsigned long long)tested);
+    }
+}
+
 // ---------------------------------------------------------------- diagnostics
 
 // Per-query distances to every pivot level, for the count below.
@@ -2474,6 +2527,7 @@ struct Runner {
     bool use_l1 = false;   // FP32 CUDA-core tiles at the last level (L1)
     bool use_f32 = false;  // GTS_PREC_FP32: FP32 CUDA-core tiles where the last level's nodes hold enough queries
     bool use_qg = false;   // 3-gram filtering tiles at the last level (edit distance)
+    bool use_qg_large = false;   // the same for large batches only (qgram_tiles_pay)
     bool use_scan = false; // low-dim vectors: node-major table scan + CUDA-core verification
     Tuning tu;             // launch parameters (a copy of the index's)
     // dense query-to-pivot matrices per level (tile paths): state 0 undecided, 1 ready, 2 not used
@@ -2599,7 +2653,10 @@ struct Runner {
             }
 #undef GTS_PV
         } else {
-            const int chunk = tu.str_chunk;
+            // at most str_chunk entries a block, fewer while that leaves SMs idle (a
+            // block goes through its queries' runs one after another: 256
+            // root entries are 256 runs, 0.3 ms in one block)
+            const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(tu.str_chunk, E / (2 * max_blocks)));
 #define GTS_PIV(WW)                                                                                                  \
     k_pivdist_str<WW><<<nblocks(E, chunk), 128, 0, st>>>(d, L.q.get(), L.node.get(), base, e0, e1, chunk, L.path.get(), \
                                                          l)
@@ -2688,7 +2745,7 @@ struct Runner {
                                                                    nullptr, nullptr, nullptr, cmask.get());
             clk.end();
             check_launch("expand count");
-            if (use_qg && !knn && l == h - 2 && filter_beats_last_pivots(L, e0, e1, cnt)) {
+            if (!knn && l == h - 2 && qgram_tiles_pay(E * F) && filter_beats_last_pivots(L, e0, e1, cnt)) {
                 str_leaf_children(L, e0, e1, cmask);
                 return;
             }
@@ -2735,7 +2792,7 @@ struct Runner {
                 tc_leaf(L, e0, e1, mask);
                 return;
             }
-            if (use_qg) {
+            if (qgram_tiles_pay(E)) {
                 count_table_pass(L, e0, e1, mask);
                 str_leaf(L, e0, e1, mask);
                 return;
@@ -2743,10 +2800,16 @@ struct Runner {
             DBuf<int32_t> cnt(E, st);
             const int64_t lvl_last = ix->tree.lvl_off[h - 1];
             clk.begin(GTS_STAGE_LEAF_SCAN);
-            k_leafscan<false><<<nblocks(E, kWarpsPerBlock), kT, 0, st>>>(d, L.q.get(), L.node.get(), L.path.get(),
-                                                                         lvl_last, e0, e1, mask.get(), thr.get(),
-                                                                         cnt.get(), nullptr, nullptr, nullptr,
-                                                                         counters.get() + 1);
+            const bool small_nodes =
+                ix->tree.n <= kLeafThreadRows * (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
+            if (small_nodes)
+                k_leafscan_small<false><<<nblocks(E, kT), kT, 0, st>>>(d, L.q.get(), L.node.get(), L.path.get(), lvl_last,
+                                                                       e0, e1, mask.get(), thr.get(), cnt.get(),
+                                                                       nullptr, nullptr, nullptr, counters.get() + 1);
+            else
+                k_leafscan<false><<<nblocks(E, kWarpsPerBlock), kT, 0, st>>>(
+                    d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0, e1, mask.get(), thr.get(), cnt.get(),
+                    nullptr, nullptr, nullptr, counters.get() + 1);
             clk.end();
             check_launch("leaf scan count");
             DBuf<int64_t> off;
@@ -2765,6 +2828,11 @@ struct Runner {
                 if (C == 0) continue;
                 DBuf<int32_t> cq(C, st), crow(C, st);
                 clk.begin(GTS_STAGE_LEAF_SCAN);
+                if (small_nodes)
+                    k_leafscan_small<true><<<nblocks(g1 - g0, kT), kT, 0, st>>>(
+                        d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0,
+                        thr.get(), nullptr, goff, cq.get(), crow.get(), nullptr);
+                else
                 k_leafscan<true><<<nblocks(g1 - g0, kWarpsPerBlock), kT, 0, st>>>(
                     d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0, thr.get(),
                     nullptr, goff, cq.get(), crow.get(), nullptr);
@@ -3165,6 +3233,15 @@ struct Runner {
         verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
     }
 
+    // Strings: whether E last-level entries go through the 3-gram tiles: always
+    // with GTS_PREC_BF16, with GTS_PREC_FP32 (the same exact distances) from
+    // the number of (entry, row) pairs on that pays for the regrouping.
+    bool qgram_tiles_pay(int64_t E) const {
+        if (use_qg) return true;
+        const int64_t nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
+        return use_qg_large && E * ((ix->tree.n + nn - 1) / nn) >= kF32TilePairs;
+    }
+
     // Range queries on the 3-gram tiles: whether to leave the last pivot level
     // out and filter every row of the children that survived the level above.
     // Per (query, last-level node) entry the pivot costs 0.6 ps per word-step
@@ -3250,6 +3327,27 @@ struct Runner {
         const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
         DBuf<int32_t> oq, orow;
         int nl = 0;
+        if (ix->tree.max_len <= kShortStr && qb.max_len <= kShortStr) {
+            ShortQuery hq;
+            hq.S = d.S;
+            hq.Soff = d.Soff;
+            hq.max_len = ix->tree.max_len;
+            hq.QS = d.QS;
+            hq.QSoff = d.QSoff;
+            DBuf<float> od;
+            clk.begin(GTS_STAGE_TILE);
+            const int64_t C = short_run(ix->tree, sq, hq, rg, oq, orow, od, hint, &nl, st);
+            clk.end();
+            if (rg.n_items > 0 && qb.nq > 0)
+                ix->tc_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+            ++st_groups;
+            if (C == 0) return;
+            st_cands += C;
+            DBuf<uint8_t> keep(C, st);
+            GTS_CUDA(cudaMemsetAsync(keep.get(), 1, C, st));
+            collect(oq, orow, od, keep, C, /*query_major=*/false);
+            return;
+        }
         clk.begin(GTS_STAGE_TILE);
         const int64_t C = qgram_run(ix->tree, sq, rg, oq, orow, hint, &nl, st);
         clk.end();
@@ -3676,6 +3774,9 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         R.use_f32 = true;
     if (precision == GTS_PREC_BF16 && t.dim == 0 && t.n > 0 && t.n < ((int64_t)1 << 31) && R.tu.str_qgram > 0)
         R.use_qg = true;
+    if (precision == GTS_PREC_FP32 && t.dim == 0 && t.n > 0 && t.n < ((int64_t)1 << 31) && R.tu.str_qgram > 0 &&
+        budget >= kF32TileBudget && !qb.count_table_pass)
+        R.use_qg_large = true;
     if (precision == GTS_PREC_BF16 && !low_dim && tc_supported(t)) {
         {
             std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build it once

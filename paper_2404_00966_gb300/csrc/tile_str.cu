@@ -17,6 +17,7 @@
 // at the query's sequence number and the bound does not exclude it.  The
 // kept pairs go on to the exact DP.
 #include "gts_impl.cuh"
+#include "metric.cuh"
 #include "tile_str.cuh"
 
 namespace gts {
@@ -38,6 +39,7 @@ struct StrArgs {
     const uint8_t *qg;          // rows' bucket counts [n, 64]
     const uint8_t *qgq;         // queries' bucket counts [nq, 64]
     const TileRec *grec;
+    const int32_t *gq;          // the records' queries
     const int4 *items;
     int64_t i1;
     int *work_counter;
@@ -46,24 +48,29 @@ struct StrArgs {
     unsigned long long *out_count;
 };
 
+__device__ __forceinline__ void cpa16s(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 // NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 4 per thread.
 // The ALU pipe bounds it: 16 four-byte sums of absolute differences per pair
-// (19 T a second on the device, 60 of 64 lanes per SM and cycle: 2 * 10^10
-// pairs cannot take less than 16.8 ms).  A lane therefore holds two rows, so
-// that a query's 64 bytes -- four 16-byte broadcast loads -- serve 64 rows of
-// its warp, and the leaf and visibility tests run on the few pairs that pass:
-// 33.1 ms for 1.9 * 10^10 pairs (one row a lane and 4-byte loads: 53.0 ms).
+// (19 T a second on the device, 60 of 64 lanes per SM and cycle: 1.9 * 10^10
+// pairs cannot take less than 16 ms).  So a lane holds two rows, and a query's
+// 64 bytes -- four 16-byte broadcast loads -- serve 64 rows of its warp; the
+// sums start at -(limit + 1), so that the test is their sign bit, shifted into
+// the pass masks; a chunk's records and vectors are copied while the one before
+// is computed (the query ids they need are read two chunks ahead); and the
+// leaf and visibility tests run on the few pairs that pass.
 template <int NQS>
 __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
     constexpr int kPer = NQS / kGroups;
-    __shared__ uint4 sQ[NQS][kWords / 4];
-    __shared__ uint64_t sMask[NQS];
-    __shared__ int64_t sSeq[NQS];
-    __shared__ uint32_t sLim[NQS];
-    __shared__ int32_t sQid[NQS];
+    __shared__ uint4 sQ[2][NQS][kWords / 4];
+    __shared__ __align__(16) TileRec sRec[2][NQS];
     __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int group = warp >> 1;
+    const int cj = tid / 4, cw = tid & 3;   // the vector piece this thread copies (tid < 4 NQS)
     for (;;) {
         if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
         __syncthreads();
@@ -72,10 +79,27 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
         const int4 it = a.items[item];
         const int64_t g = a.lvl_last + it.x;
         const int first = it.y, total = it.z;
+        const int nchunk = (total + NQS - 1) / NQS;
+        // chunk c into buffer c & 1; qid: the query of this thread's piece
+        auto query_of = [&](int c) -> int32_t {
+            const int j = c * NQS + cj;
+            return cj < NQS && j < total ? a.gq[first + j] : -1;
+        };
+        auto stage = [&](int c, int32_t qid) {
+            const int cnt = min(NQS, total - c * NQS);
+            if (qid >= 0)
+                cpa16s(&sQ[c & 1][cj][cw], reinterpret_cast<const uint4 *>(a.qgq + (int64_t)qid * 64) + cw);
+            if (tid < 2 * cnt)
+                cpa16s(reinterpret_cast<uint4 *>(&sRec[c & 1][0]) + tid,
+                       reinterpret_cast<const uint4 *>(a.grec + first + c * NQS) + tid);
+        };
+        const int32_t qid0 = query_of(0);
+        int32_t qnext = query_of(1);
         const int rb = it.w * kRowsS;
         const int32_t pos = a.npos[g], size = a.nsize[g];
         const int nrow = min(kRowsS, size - rb);
         const int32_t avg = size / a.F;
+        stage(0, qid0);
         // this lane's two rows: bucket counts, leaf bits, delete marks
         uint32_t rw[2][kWords];
         uint64_t rowbit[2];
@@ -105,69 +129,229 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
         const uint64_t both = rowbit[0] | rowbit[1];
         const uint64_t wmask = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)both) |
                                ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(both >> 32)) << 32);
-        for (int c0 = 0; c0 < total; c0 += NQS) {
-            const int cnt = min(NQS, total - c0);
-            __syncthreads();   // the previous chunk's shared data is no longer read
-            for (int j = tid; j < cnt; j += kThreadsS) {
-                const TileRec rc = a.grec[first + c0 + j];
-                sMask[j] = rc.mask;
-                sSeq[j] = rc.seq;
-                // keep iff L1 <= 6 t (whole numbers; an unbounded t keeps all)
-                sLim[j] = rc.thr < 1e8f ? (uint32_t)(6.f * rc.thr) : 0xffffffffu;
-                sQid[j] = rc.q;
+        for (int c = 0; c < nchunk; ++c) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();   // chunk c has landed; the other buffer is no longer read
+            if (c + 1 < nchunk) {
+                stage(c + 1, qnext);
+                qnext = query_of(c + 2);
             }
-            for (int t = tid; t < cnt * (kWords / 4); t += kThreadsS) {
-                const int j = t / (kWords / 4), w = t - j * (kWords / 4);
-                sQ[j][w] = reinterpret_cast<const uint4 *>(a.qgq + (int64_t)a.grec[first + c0 + j].q * 64)[w];
+            const int cnt = min(NQS, total - c * NQS);
+            const TileRec *rec = sRec[c & 1];
+            const int j0 = group * kPer;
+            const int nj = max(0, min(kPer, cnt - j0));
+            // lane i < nj: query j0 + i's limit (keep iff L1 <= 6 t, whole
+            // numbers; an unbounded t keeps all) and whether the warp's rows
+            // hold a leaf it kept
+            int start = 0;
+            bool live = false;
+            if (lane < nj) {
+                const float t = rec[j0 + lane].thr;
+                start = -1 - (t < 1e8f ? (int)(6.f * t) : 1 << 30);
+                live = (rec[j0 + lane].mask & wmask) != 0;
+            }
+            const unsigned lives = __ballot_sync(0xffffffffu, live);
+            uint32_t p0 = 0, p1 = 0;   // bit nj - 1 - i: rows r0, r0 + 32 pass query j0 + i
+#pragma unroll 2
+            for (int i = 0; i < nj; ++i) {
+                uint32_t l0 = 0, l1 = 0;
+                if ((lives >> i) & 1u) {   // warp-uniform
+                    l0 = l1 = (uint32_t)__shfl_sync(0xffffffffu, start, i);
+                    const uint4 *qv = sQ[c & 1][j0 + i];
+#pragma unroll
+                    for (int v = 0; v < kWords / 4; ++v) {
+                        const uint4 x = qv[v];
+                        l0 = __vsadu4(rw[0][4 * v], x.x) + l0;
+                        l1 = __vsadu4(rw[1][4 * v], x.x) + l1;
+                        l0 = __vsadu4(rw[0][4 * v + 1], x.y) + l0;
+                        l1 = __vsadu4(rw[1][4 * v + 1], x.y) + l1;
+                        l0 = __vsadu4(rw[0][4 * v + 2], x.z) + l0;
+                        l1 = __vsadu4(rw[1][4 * v + 2], x.z) + l1;
+                        l0 = __vsadu4(rw[0][4 * v + 3], x.w) + l0;
+                        l1 = __vsadu4(rw[1][4 * v + 3], x.w) + l1;
+                    }
+                }
+                p0 = __funnelshift_l(l0, p0, 1);
+                p1 = __funnelshift_l(l1, p1, 1);
+            }
+            if (__any_sync(0xffffffffu, (p0 | p1) != 0)) {
+                for (uint32_t left = p0; left; left &= left - 1) {   // leaf and visibility of the passing pairs
+                    const int b = __ffs(left) - 1;
+                    const TileRec &rc = rec[j0 + nj - 1 - b];
+                    if (!(rc.mask & rowbit[0]) || rdel[0] <= rc.seq) p0 &= ~(1u << b);
+                }
+                for (uint32_t left = p1; left; left &= left - 1) {
+                    const int b = __ffs(left) - 1;
+                    const TileRec &rc = rec[j0 + nj - 1 - b];
+                    if (!(rc.mask & rowbit[1]) || rdel[1] <= rc.seq) p1 &= ~(1u << b);
+                }
+                const int np = __popc(p0) + __popc(p1);
+                int incl = np;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                const int wtot = __shfl_sync(0xffffffffu, incl, 31);
+                if (wtot > 0) {
+                    unsigned long long base = 0;
+                    if (lane == 31) base = atomicAdd(a.out_count, (unsigned long long)wtot);
+                    base = __shfl_sync(0xffffffffu, base, 31);
+                    unsigned long long o = base + (unsigned long long)(incl - np);
+                    while (p0 | p1) {
+                        const bool h0 = p0 != 0;
+                        const int b = __ffs(h0 ? p0 : p1) - 1;
+                        if (h0) p0 &= p0 - 1;
+                        else p1 &= p1 - 1;
+                        if ((int64_t)o < a.cap) {
+                            a.out_q[o] = rec[j0 + nj - 1 - b].q;
+                            a.out_row[o] = pos + rb + r0 + (h0 ? 0 : 32);
+                        }
+                        ++o;
+                    }
+                }
+            }
+        }
+    }
+}
+
+// ---- short strings: filter and distance in one tile
+//
+// For words the 3-gram bound excludes little (two words of ten letters differ
+// in at most 16 3-grams, 6 t passes that at t = 3), and nearly every pair went
+// through a candidate list, a sort by query and a verification pass: 3.3 ms
+// for 50 M pairs (here 0.95), of which the distances themselves need 0.4.  Here a
+// thread holds one row of the block, its text (eight words) and its 3-gram
+// counts, the chunk's queries have their match masks in shared memory (one word
+// per character and query), and a pair costs 13 operations per character of
+// its row; only pairs within the threshold are written, with their distance.
+// The integer / logic pipe bounds it.
+constexpr int kNQD = 32;        // queries per chunk
+struct ShortArgs {
+    StrArgs s;
+    const uint8_t *S, *QS;
+    const int64_t *Soff, *QSoff;
+    int max_len;
+    float *out_d;
+};
+
+__global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
+    const StrArgs &a = A.s;
+    constexpr int kPer = kNQD / 2;
+    __shared__ __align__(16) uint32_t sPeq[kNQD][256];
+    __shared__ uint4 sQ[kNQD][kWords / 4];
+    __shared__ TileRec sRec[kNQD];
+    __shared__ int sLen[kNQD];
+    __shared__ int s_item;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int r = tid % kRowsS, half = tid / kRowsS;
+    for (;;) {
+        if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
+        __syncthreads();
+        const int64_t item = s_item;
+        if (item >= a.i1) break;
+        const int4 it = a.items[item];
+        const int64_t g = a.lvl_last + it.x;
+        const int first = it.y, total = it.z;
+        const int rb = it.w * kRowsS;
+        const int32_t pos = a.npos[g], size = a.nsize[g];
+        const bool valid = rb + r < size;
+        const int64_t row = (int64_t)pos + (valid ? rb + r : 0);
+        const int32_t avg = size / a.F;
+        int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
+        if (jl > a.F - 1) jl = a.F - 1;
+        if (a.children) jl = it.x % a.F;
+        const uint64_t rowbit = valid ? (1ull << jl) : 0ull;
+        const int64_t rdel = (valid && a.any_deleted) ? a.row_del[row] : kNever;
+        const int len = (int)(A.Soff[row + 1] - A.Soff[row]);
+        uint32_t tw[kShortStr / 4], rw[kWords];
+        {
+            TextWords tr(A.S + A.Soff[row], len);
+#pragma unroll
+            for (int i = 0; i < kShortStr / 4; ++i) tw[i] = 4 * i < len ? tr.next4() : 0u;
+            const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + row * 64);
+#pragma unroll
+            for (int v = 0; v < kWords / 4; ++v) {
+                const uint4 x = src[v];
+                rw[4 * v] = x.x;
+                rw[4 * v + 1] = x.y;
+                rw[4 * v + 2] = x.z;
+                rw[4 * v + 3] = x.w;
+            }
+        }
+        for (int c0 = 0; c0 < total; c0 += kNQD) {
+            const int cnt = min(kNQD, total - c0);
+            __syncthreads();   // the previous chunk's shared data is no longer read
+            for (int i = tid; i < kNQD * 64; i += kThreadsS)
+                reinterpret_cast<uint4 *>(&sPeq[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+            const int qj = tid >> 3;   // eight threads a query
+            int32_t q = -1;
+            int m = 0;
+            if (qj < cnt) {
+                q = a.gq[first + c0 + qj];
+                m = (int)(A.QSoff[q + 1] - A.QSoff[q]);
+                if ((tid & 7) == 0) {
+                    sRec[qj] = a.grec[first + c0 + qj];
+                    sLen[qj] = m;
+                }
+                if ((tid & 7) >= 4)
+                    sQ[qj][tid & 3] = reinterpret_cast<const uint4 *>(a.qgq + (int64_t)q * 64)[tid & 3];
             }
             __syncthreads();
-            uint32_t pass = 0;   // bit jj: row r0, bit 16 + jj: row r0 + 32
-            const int j0 = group * kPer, j1 = min(j0 + kPer, cnt);
-#pragma unroll 2
+            if (q >= 0) {
+                const uint8_t *p = A.QS + A.QSoff[q];
+                for (int i = tid & 7; i < m; i += 8) atomicOr(&sPeq[qj][p[i]], 1u << i);
+            }
+            __syncthreads();
+            const int j0 = half * kPer, j1 = min(j0 + kPer, cnt);
             for (int j = j0; j < j1; ++j) {
-                if (!(sMask[j] & wmask)) continue;   // warp-uniform
-                uint32_t l0 = 0, l1 = 0;
+                const TileRec &rc = sRec[j];
+                const int mq = sLen[j];
+                const int lim = rc.thr < 1e8f ? (int)rc.thr : 1 << 24;
+                bool on = (rc.mask & rowbit) && rdel > rc.seq && abs(mq - len) <= lim;
+                // the 3-gram bound, where it can exclude anything
+                if (6 * (int64_t)lim < mq + A.max_len - 4) {
+                    uint32_t l1 = 0;
 #pragma unroll
-                for (int v = 0; v < kWords / 4; ++v) {
-                    const uint4 x = sQ[j][v];
-                    l0 = __vsadu4(rw[0][4 * v], x.x) + l0;
-                    l1 = __vsadu4(rw[1][4 * v], x.x) + l1;
-                    l0 = __vsadu4(rw[0][4 * v + 1], x.y) + l0;
-                    l1 = __vsadu4(rw[1][4 * v + 1], x.y) + l1;
-                    l0 = __vsadu4(rw[0][4 * v + 2], x.z) + l0;
-                    l1 = __vsadu4(rw[1][4 * v + 2], x.z) + l1;
-                    l0 = __vsadu4(rw[0][4 * v + 3], x.w) + l0;
-                    l1 = __vsadu4(rw[1][4 * v + 3], x.w) + l1;
-                }
-                const uint32_t lim = sLim[j];
-                if (l0 <= lim) pass |= 1u << (j - j0);
-                if (l1 <= lim) pass |= 65536u << (j - j0);
-            }
-            for (uint32_t left = pass; left; left &= left - 1) {   // leaf and visibility of the passing pairs
-                const int b = __ffs(left) - 1, h = b >> 4, j = j0 + (b & 15);
-                if (!(sMask[j] & (h ? rowbit[1] : rowbit[0])) || (h ? rdel[1] : rdel[0]) <= sSeq[j]) pass &= ~(1u << b);
-            }
-            const int np = __popc(pass);
-            int incl = np;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int wtot = __shfl_sync(0xffffffffu, incl, 31);
-            if (wtot > 0) {
-                unsigned long long base = 0;
-                if (lane == 31) base = atomicAdd(a.out_count, (unsigned long long)wtot);
-                base = __shfl_sync(0xffffffffu, base, 31);
-                unsigned long long o = base + (unsigned long long)(incl - np);
-                while (pass) {
-                    const int b = __ffs(pass) - 1;
-                    pass &= pass - 1;
-                    if ((int64_t)o < a.cap) {
-                        a.out_q[o] = sQid[j0 + (b & 15)];
-                        a.out_row[o] = pos + rb + r0 + 32 * (b >> 4);
+                    for (int v = 0; v < kWords / 4; ++v) {
+                        const uint4 x = sQ[j][v];
+                        l1 = __vsadu4(rw[4 * v], x.x) + l1;
+                        l1 = __vsadu4(rw[4 * v + 1], x.y) + l1;
+                        l1 = __vsadu4(rw[4 * v + 2], x.z) + l1;
+                        l1 = __vsadu4(rw[4 * v + 3], x.w) + l1;
                     }
-                    ++o;
+                    on = on && l1 <= 6u * (uint32_t)lim;
+                }
+                int d = 1 << 25;
+                if (on) {
+                    uint32_t Pv = ~0u, Mv = 0u;
+                    const uint32_t *peq = sPeq[j];
+#pragma unroll
+                    for (int i = 0; i < kShortStr; ++i) {
+                        if (i < len) {
+                            const uint32_t Eq = peq[(tw[i / 4] >> (8 * (i % 4))) & 255u];
+                            const uint32_t Xh = (((Eq & Pv) + Pv) ^ Pv) | Eq;
+                            const uint32_t Ph = ((Mv | ~(Xh | Pv)) << 1) | 1u;
+                            const uint32_t Mh = (Pv & Xh) << 1;
+                            const uint32_t Xv = Eq | Mv;
+                            Pv = Mh | ~(Xv | Ph);
+                            Mv = Ph & Xv;
+                        }
+                    }
+                    const uint32_t rows = mq >= 32 ? ~0u : (1u << mq) - 1u;
+                    d = len + __popc(Pv & rows) - __popc(Mv & rows);
+                }
+                const unsigned b = __ballot_sync(0xffffffffu, d <= lim);
+                if (b) {
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(a.out_count, (unsigned long long)__popc(b));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    const unsigned long long o = base + __popc(b & ((1u << lane) - 1u));
+                    if (((b >> lane) & 1u) && (int64_t)o < a.cap) {
+                        a.out_q[o] = rc.q;
+                        a.out_row[o] = (int32_t)row;
+                        A.out_d[o] = (float)d;
+                    }
                 }
             }
         }
@@ -175,7 +359,70 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
     }
 }
 
+StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg) {
+    StrArgs a;
+    a.F = t.F;
+    a.npos = t.npos.get();
+    a.nsize = t.nsize.get();
+    a.lvl_last = t.lvl_off[t.h - 1];
+    a.row_del = t.row_del.get();
+    a.any_deleted = sq.any_deleted;
+    a.children = sq.children ? 1 : 0;
+    a.qg = sq.qg;
+    a.qgq = sq.qgq;
+    a.grec = rg.grec.get();
+    a.gq = rg.gq.get();
+    a.items = rg.items.get();
+    a.i1 = rg.n_items;
+    return a;
+}
+
 }  // namespace
+
+int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, DBuf<int32_t> &out_q,
+                  DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st) {
+    *launches = 0;
+    if (rg.n_items == 0) return 0;
+    int dev = 0, sms = 0, per_sm = 0;
+    GTS_CUDA(cudaGetDevice(&dev));
+    GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_short, kThreadsS, 0));
+    if (per_sm < 1) per_sm = 1;
+    const int64_t grid = std::min<int64_t>(rg.n_items, (int64_t)sms * per_sm);
+    DBuf<int> counter(1, st);
+    DBuf<unsigned long long> count(1, st);
+    int64_t cap = cap_hint > 0 ? cap_hint : 1 << 20;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        out_q.alloc(cap, st);
+        out_row.alloc(cap, st);
+        out_d.alloc(cap, st);
+        GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
+        GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
+        ShortArgs A;
+        A.s = str_args(t, sq, rg);
+        A.s.work_counter = counter.get();
+        A.s.out_q = out_q.get();
+        A.s.out_row = out_row.get();
+        A.s.cap = cap;
+        A.s.out_count = count.get();
+        A.S = hq.S;
+        A.Soff = hq.Soff;
+        A.max_len = hq.max_len;
+        A.QS = hq.QS;
+        A.QSoff = hq.QSoff;
+        A.out_d = out_d.get();
+        k_tile_short<<<(unsigned)grid, kThreadsS, 0, st>>>(A);
+        ++*launches;
+        check_launch("short-string tile");
+        unsigned long long hcount = 0;
+        GTS_CUDA(cudaMemcpyAsync(&hcount, count.get(), 8, cudaMemcpyDeviceToHost, st));
+        GTS_CUDA(cudaStreamSynchronize(st));
+        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        cap = (int64_t)hcount;   // rerun with room for every pair
+    }
+    GTS_REQUIRE(false, GTS_ECUDA, "short-string tile: output count changed between identical runs");
+    return 0;
+}
 
 int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<int32_t> &out_q,
                   DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st) {
@@ -199,19 +446,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<i
         out_row.alloc(cap, st);
         GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
-        StrArgs a;
-        a.F = t.F;
-        a.npos = t.npos.get();
-        a.nsize = t.nsize.get();
-        a.lvl_last = t.lvl_off[t.h - 1];
-        a.row_del = t.row_del.get();
-        a.any_deleted = sq.any_deleted;
-        a.children = sq.children ? 1 : 0;
-        a.qg = sq.qg;
-        a.qgq = sq.qgq;
-        a.grec = rg.grec.get();
-        a.items = rg.items.get();
-        a.i1 = rg.n_items;
+        StrArgs a = str_args(t, sq, rg);
         a.work_counter = counter.get();
         a.out_q = out_q.get();
         a.out_row = out_row.get();

@@ -15,6 +15,23 @@ struct StrQuery {
     bool children = false;          // records from tc_regroup_children: masks name the parent's children
 };
 
+// Both sides at most 32 characters: the tiles also run the edit distance itself
+// (one 32-bit word per column) on the pairs the bound keeps.
+constexpr int kShortStr = 32;
+
+struct ShortQuery {
+    const uint8_t *S = nullptr;     // the tree rows' bytes and offsets
+    const int64_t *Soff = nullptr;
+    int max_len = 0;                // the longest row
+    const uint8_t *QS = nullptr;    // the queries'
+    const int64_t *QSoff = nullptr;
+};
+
+// run the tiles over a regrouping of short strings: the (query, row, distance)
+// triples within the records' thresholds
+int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, DBuf<int32_t> &out_q,
+                  DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st);
+
 // run the tiles over a regrouping (its records carry each query's threshold);
 // returns the number of (query, row) pairs written, the pairs the bound keeps
 int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<int32_t> &out_q,

@@ -33,7 +33,7 @@ def family(lo, hi, n, nq, seed, edits):
 
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
-@pytest.mark.parametrize("lo,hi", [(1, 33), (31, 34), (60, 70), (100, 130), (126, 131), (250, 262), (508, 520),
+@pytest.mark.parametrize("lo,hi", [(1, 8), (1, 32), (29, 32), (1, 33), (31, 34), (60, 70), (100, 130), (126, 131), (250, 262), (508, 520),
                                    (1000, 1024)])
 def test_edit_bands_and_words(gts, prec, lo, hi):
     n, nq = (700, 48) if hi <= 140 else (260, 24)
@@ -100,4 +100,33 @@ def test_range_without_the_last_pivot_level(gts):
         assert np.array_equal(r.dist, dist.astype(np.float32))
         if not step:
             ix.delete(dele)
+    ix.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_short_string_tiles(gts, prec):
+    """Words: both precisions run the filter and the distance in one tile once
+    the batch holds 6 M (entry, row) pairs; deleted rows stay out."""
+    rng = np.random.default_rng(9)
+    alpha = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz", np.uint8)
+    S = random_strings(40_003, 0, 16, alpha, rng)
+    Q = strings_from_list([mutate(S.get(int(rng.integers(0, 40_003))), int(rng.integers(0, 4)), alpha, rng)
+                           for _ in range(401)])
+    ix = gts.Index.build(S, "edit", fanout=20, root_pivot=0)
+    s0 = ix.info()["seq"]
+    dele = rng.choice(40_003, 900, replace=False)
+    ix.delete(dele)
+    dl = np.full(40_003, np.iinfo(np.int64).max, np.int64)
+    dl[dele] = s0 + np.arange(900)
+    ins, qs = np.full(40_003, -1, np.int64), np.full(401, ix.info()["seq"], np.int64)
+    r = ix.knn(Q, 6, precision=prec)
+    assert r.stats["tiles"] > 0
+    off, ids, dist, _ = oracle.knn_query("edit", S, Q, 6, ins, dl, qs)
+    assert np.array_equal(r.offsets, off) and np.array_equal(r.ids, ids)
+    assert np.array_equal(r.dist, dist.astype(np.float32))
+    radii = np.resize(np.array([0, 1, 2, 5], np.float32), 401)
+    r = ix.range(Q, radii, precision=prec)
+    off, ids, dist, _ = oracle.range_query("edit", S, Q, radii, ins, dl, qs)
+    assert np.array_equal(r.offsets, off) and np.array_equal(r.ids, ids)
+    assert np.array_equal(r.dist, dist.astype(np.float32))
     ix.close()
