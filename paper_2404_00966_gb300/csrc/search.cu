@@ -40,8 +40,11 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kWarpsPerBlock = kT / 32;
+constexpr int64_t kCoarseRows = 64;              // tensor-core tiles: rows per last-level node below which range
+                                                 // queries may run over the level above (coarse_tiles_pay)
 constexpr int64_t kF32TileEntries = 4;           // FP32 tiles: least last-level entries per node
 constexpr int64_t kF32TilePairs = 6 << 20;       // and least (entry, row) pairs (f32_tiles_pay)
+constexpr int64_t kScanPairs = 16 << 20;         // table scan of low-dimensional vectors: least pairs
 constexpr int64_t kF32DenseQueries = 64;         // dense pivot matrices in FP32: one full tile of queries
 constexpr int64_t kF32TileBudget = (int64_t)1 << 30;   // and least memory budget: the regrouped records take about
                                                        // 60 bytes per entry beside the budgeted tables
@@ -477,9 +480,9 @@ __device__ __forceinline__ void list_dists(const Dev &d, const float *__restrict
 //
 // The rows' bytes from L2 and, in small batches, the chain of dependent loads
 // bound it: eight lanes read a row's 128-byte segments together, and a batch
-// of few queries takes eight warps a query.  10^4 queries of 10^6 x 128 0.45
-// ms, 10^4 of 2 * 10^5 x 300 0.74 ms, 128 of 2 * 10^6 x 256 (L1) 0.44 ms; a
-// row per lane over all of 1,024 rows took 0.82, 2.83 and 0.90 ms.
+// of few queries takes eight warps a query.  A row per lane over all 1,024
+// rows took 0.82 ms (10^4 queries, 10^6 x 128), 2.83 ms (10^4, 2 * 10^5 x 300)
+// and 0.90 ms (128 queries, 2 * 10^6 x 256, L1).
 template <bool L2, int G, bool V4>
 __global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int max_rows, int per_k, const int32_t *__restrict__ kq,
                             const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n, float *tau,
@@ -960,8 +963,7 @@ __global__ void k_leafscan(Dev d, const int32_t *__restrict__ eq, const int32_t 
 }
 
 // The same for nodes of a few rows, a thread per entry (a warp per entry leaves
-// most lanes idle: 0.36 + 0.26 ms for 6 * 10^5 entries of 2.4 rows, here 0.033 +
-// 0.033).
+// most lanes idle and takes 0.36 + 0.26 ms for 6 * 10^5 entries of 2.4 rows).
 constexpr int kLeafThreadRows = 8;   // average rows per node up to which a thread takes an entry
 template <bool WRITE>
 __global__ void k_leafscan_small(Dev d, const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
@@ -2752,6 +2754,10 @@ struct Runner {
             DBuf<int64_t> off;
             scan_i32(cnt, E, off);
             const int64_t total = d2h_i64(off.get() + E, st);
+            if (use_tc && !knn && l == h - 2 && coarse_tiles_pay(E, total)) {
+                tc_leaf_coarse(L, e0, e1, cmask);
+                return;
+            }
             if (use_tc && l == h - 2 && dense_last_ok(total)) {
                 dense_last_level(L, e0, e1, cmask);
                 return;
@@ -3172,6 +3178,37 @@ struct Runner {
         tc_finish(tq, rg);
     }
 
+    // Range queries on the tensor-core tiles: whether to run them over the
+    // nodes of the level above the last (E entries, masks over their children)
+    // instead of the last level's (`total` entries).  A tile spends a whole
+    // 128-row block on a node of few rows; nodes of fewer than kCoarseRows rows
+    // waste more than half of it, and the last level's pivot distances and leaf
+    // masks come on top.  The rows computed either way decide: E (parent blocks)
+    // against `total` (last-level blocks).  (3 * 10^5 x 100, 3,001 queries, nodes
+    // of 37 rows: COARSE_MS.)
+    bool coarse_tiles_pay(int64_t E, int64_t total) const {
+        const int64_t n = ix->tree.n, nl = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
+        const int64_t np = ix->tree.lvl_off[h - 1] - ix->tree.lvl_off[h - 2];
+        if (n >= kCoarseRows * nl || qb.count_table_pass) return false;
+        return E * ((n / np + 127) / 128) <= total;   // (a last-level node: one block)
+    }
+
+    void tc_leaf_coarse(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &cmask) {
+        TcQuery tq = tc_query_base();
+        tq.E = e1 - e0;
+        tq.eq = L.q.get() + e0;
+        tq.enode = L.node.get() + e0;
+        tq.path = L.path.get() + e0 * h;
+        tq.emask = cmask.get();
+        tq.h = h - 1;
+        tq.path_stride = h;
+        TcRegroup rg;
+        clk.begin(GTS_STAGE_OTHER, 6);
+        tc_regroup(ix->tree, tq, rg, st, nullptr, true);
+        clk.end();
+        tc_finish(tq, rg);
+    }
+
     // Last level of low-dimensional vectors: regroup the entries by node, scan
     // each node block's table rows once against all of its queries (leaf
     // mask, visibility, Lemma 1 / 2 lower bound), then verify the candidates
@@ -3375,9 +3412,12 @@ struct Runner {
     // us: 3 * 10^5 x 128, 32 queries (5 M pairs) 1501 / 1518, 100 (15 M) 2424 /
     // 1813, 1000 15877 / 5444; 3 * 10^5 x 17, 32: 1102 / 1161, 100: 1419 /
     // 1280; L1, 2 * 10^4 x 64, 100 (1 M): 895 / 1082, 3 * 10^5, 100: 2053 / 1743.
-    bool f32_tiles_pay(int64_t E) const {
+    // The node-major table scan of low-dimensional vectors needs more pairs
+    // (3-D kNN, 10^6 points, plain / scan: 200 queries 811 / 885, 5,000 3139 /
+    // 2345; 5 * 10^6, 200: 1091 / 1061, 5,000: 6751 / 4231).
+    bool f32_tiles_pay(int64_t E, int64_t least_pairs) const {
         const int64_t nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
-        return E >= kF32TileEntries * nn && E * ((ix->tree.n + nn - 1) / nn) >= kF32TilePairs;
+        return E >= kF32TileEntries * nn && E * ((ix->tree.n + nn - 1) / nn) >= least_pairs;
     }
 
     // Last level on the FP32 L2 tiles: regroup the entries by node, run the

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
 // For words the 3-gram bound excludes little (two words of ten letters differ
 // in at most 16 3-grams, 6 t passes that at t = 3), and nearly every pair went
 // through a candidate list, a sort by query and a verification pass: 3.3 ms
-// for 50 M pairs (here 0.95), of which the distances themselves need 0.4.  Here a
+// for 50 M pairs, of which the distances themselves need 0.4 ms.  Here a
 // thread holds one row of the block, its text (eight words) and its 3-gram
 // counts, the chunk's queries have their match masks in shared memory (one word
 // per character and query), and a pair costs 13 operations per character of

@@ -733,7 +733,7 @@ __global__ void k_query_consts(const float *__restrict__ thr, const float *__res
 
 __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
                                const uint64_t *__restrict__ emask, const float *__restrict__ path, int h, int hp,
-                               int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2, float cE1,
+                               int stride, int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2, float cE1,
                                float cE2, const int64_t *__restrict__ qseq, const int64_t *__restrict__ noff,
                                int32_t *__restrict__ cursor, TileRec *__restrict__ grec, int32_t *__restrict__ gq,
                                float *__restrict__ gpath) {
@@ -752,7 +752,7 @@ __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__
         grec[o] = r;
         gq[o] = q;
         if (path)
-            for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
+            for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * stride + l] : 0.f;
     }
 }
 
@@ -806,7 +806,7 @@ __global__ void k_bits_rows(const uint32_t *__restrict__ bits, int64_t nn, int64
 }
 
 __device__ __forceinline__ void write_rec(int64_t e, int64_t o, const int32_t *eq, const uint64_t *emask,
-                                          const float *path, int h, int hp, const float *thr, const float *qn2,
+                                          const float *path, int h, int hp, int stride, const float *thr, const float *qn2,
                                           float cE1, float cE2, const int64_t *qseq, TileRec *grec, int32_t *gq,
                                           float *gpath) {
     const int32_t q = eq[e];
@@ -819,12 +819,12 @@ __device__ __forceinline__ void write_rec(int64_t e, int64_t o, const int32_t *e
     grec[o] = r;
     gq[o] = q;
     if (path)
-        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
+        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * stride + l] : 0.f;
 }
 
 __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
                                     const uint64_t *__restrict__ emask, const float *__restrict__ path, int h, int hp,
-                                    int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2,
+                                    int stride, int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2,
                                     float cE1, float cE2, const int64_t *__restrict__ qseq,
                                     const int64_t *__restrict__ noff, const uint32_t *__restrict__ bits, const int32_t *__restrict__ wpre, int64_t nw,
                                     TileRec *__restrict__ grec, int32_t *__restrict__ gq, float *__restrict__ gpath) {
@@ -833,7 +833,7 @@ __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_
         const int32_t q = eq[e];
         const int64_t wi = (int64_t)enode[e] * nw + (q >> 5);
         const int64_t o = noff[enode[e]] + wpre[wi] + __popc(bits[wi] & ((1u << (q & 31)) - 1u));
-        write_rec(e, o, eq, emask, path, h, hp, thr, qn2, cE1, cE2, qseq, grec, gq, gpath);
+        write_rec(e, o, eq, emask, path, h, hp, stride, thr, qn2, cE1, cE2, qseq, grec, gq, gpath);
     }
 }
 
@@ -980,10 +980,11 @@ void tc_split_queries(const float *Q, int64_t nq, int dim, int dim_p, DBuf<uint8
     check_launch("split queries");
 }
 
-bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E) {
+bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E, int h) {
+    if (h == 0) h = t.h;
     // the bitmap costs a pass over nodes x query words; it pays when the
     // entries are dense in it (at least one per four words) and it stays small
-    const int64_t nn = t.lvl_off[t.h] - t.lvl_off[t.h - 1];
+    const int64_t nn = t.lvl_off[h] - t.lvl_off[h - 1];
     const int64_t words = nn * ((nq + 31) / 32);
     return words * 8 <= ((int64_t)1 << 30) && words <= 4 * E;
 }
@@ -1021,16 +1022,18 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
     GTS_CUDA(cudaMemcpyAsync(&total_entries, noff.get() + nn, 8, cudaMemcpyDeviceToHost, st));
     GTS_CUDA(cudaStreamSynchronize(st));
     const int64_t ne = total_entries > 0 ? total_entries : 1;
-    const int hp = (t.h + 3) & ~3;
+    const int h = tq.h ? tq.h : t.h, hp = (h + 3) & ~3;
+    const int stride = tq.path_stride ? tq.path_stride : t.h;
+    rg.h = h;
     rg.grec.alloc(ne, st);
     rg.gq.alloc(ne, st);
     rg.gpath.alloc(tq.path ? ne * hp : 1, st);
     if (use_bits)
-        k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, t.h, hp, E, tq.thr, tq.qn2,
+        k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
                                                      tq.cE1, tq.cE2, tq.qseq, noff.get(), bits.get(), wpre.get(), nw, rg.grec.get(),
                                                      rg.gq.get(), rg.gpath.get());
     else
-        k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, t.h, hp, E, tq.thr, tq.qn2,
+        k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
                                                 tq.cE1, tq.cE2, tq.qseq, noff.get(), cursor.get(), rg.grec.get(), rg.gq.get(),
                                                 rg.gpath.get());
     rg.n_entries = total_entries;
@@ -1040,14 +1043,15 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
 
 int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st, const int32_t *counts,
                    bool window_ok) {
-    const int64_t nn = t.lvl_off[t.h] - t.lvl_off[t.h - 1];
+    const int h = tq.h ? tq.h : t.h;
+    const int64_t nn = t.lvl_off[h] - t.lvl_off[h - 1];
     // the bitmap form when its two (node x query-word) arrays stay small
-    const bool use_bits = regroup_uses_bits(t, tq.nq, tq.E);
+    const bool use_bits = regroup_uses_bits(t, tq.nq, tq.E, h);
     DBuf<int32_t> own;
     const int32_t *ncnt = group_records(t, tq, rg, nn, use_bits, counts, own, st);
     const DBuf<int64_t> &noff = rg.noff;
     DBuf<int64_t> nitems(nn + 1, st), ioff(nn + 1, st);
-    const int32_t *lsize = t.nsize.get() + t.lvl_off[t.h - 1];
+    const int32_t *lsize = t.nsize.get() + t.lvl_off[h - 1];
     DBuf<unsigned long long> pairs(1, st);
     GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
     k_items_per_node<<<nblk(nn), 256, 0, st>>>(ncnt, lsize, nn, nitems.get(), pairs.get());
@@ -1135,6 +1139,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
                DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st, DBuf<float> *out_qx) {
     *launches = 0;
     if (rg.n_items == 0) return 0;
+    const int h = rg.h ? rg.h : t.h;
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1144,7 +1149,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     GTS_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     // TMEM: A (dim_p columns) and the slots' accumulators share 512 columns
     GTS_REQUIRE(c.dim_p + shp.sm * nq_chunk <= 512, GTS_ECUDA, "tensor-core tile: TMEM columns");
-    const size_t smem = tile_smem_bytes(c.dim_p, t.h, nq_chunk, shp.sb, shp.sm);
+    const size_t smem = tile_smem_bytes(c.dim_p, h, nq_chunk, shp.sb, shp.sm);
     GTS_REQUIRE(smem <= (size_t)smem_optin, GTS_ECUDA, "tensor-core tile: shared memory");
     void (*kern)(const CUtensorMap, const CUtensorMap, TileArgs) =
         nq_chunk == 96    ? k_tile_l2_tc<96, 4, 4>
@@ -1176,7 +1181,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     float cE1 = 0.f, cE2 = 0.f;
     tc_bound_coeffs(c.dim_p, cE1, cE2);
     // window mode: every node's non-empty windows
-    const int64_t nn = t.lvl_off[t.h] - t.lvl_off[t.h - 1];
+    const int64_t nn = t.lvl_off[h] - t.lvl_off[h - 1];
     const int64_t nwin = (tq.nq + nq_chunk - 1) / nq_chunk;
     const bool wl_on = rg.bits.get() != nullptr && rg.nw > 0;
     DBuf<int32_t> wl(wl_on ? nn * nwin : 1, st), wcnt(wl_on ? nn : 1, st);
@@ -1207,7 +1212,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.dim = t.dim;
         a.dim_p = c.dim_p;
         a.F = t.F;
-        a.h = t.h;
+        a.h = h;
         a.n = t.n;
         a.xn2 = c.xn2.get();
         a.Xh = reinterpret_cast<const __nv_bfloat16 *>(c.Xh.get());
@@ -1216,13 +1221,13 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.row_del = t.row_del.get();
         a.npos = t.npos.get();
         a.nsize = t.nsize.get();
-        a.lvl_last = t.lvl_off[t.h - 1];
+        a.lvl_last = t.lvl_off[h - 1];
         a.Qh = tq.Qh;
         a.Ql = tq.Ql;
         a.grec = rg.grec.get();
         a.gq = rg.gq.get();
         a.gpath = rg.gpath.get();
-        a.hp = (t.h + 3) & ~3;
+        a.hp = (h + 3) & ~3;
         a.items = rg.items.get();
         a.n_items = rg.n_items;
         a.work_counter = counter.get();

@@ -76,6 +76,9 @@ struct TcQuery {
     const int32_t *eq = nullptr, *enode = nullptr;
     const float *path = nullptr;
     const uint64_t *emask = nullptr;
+    // the entries' level is h - 1, their masks name the nodes' children at
+    // level h, and `path` holds path_stride floats per entry (0: the tree's h)
+    int h = 0, path_stride = 0;
     const float *Q = nullptr;
     const int64_t *qseq = nullptr;
     const float *thr = nullptr;
@@ -93,6 +96,7 @@ struct TcQuery {
 constexpr int kWindowItem = 1 << 30;
 
 struct TcRegroup {
+    int h = 0;             // the tiles' nodes are those of level h - 1 (0: the tree's h)
     const uint64_t *dmask = nullptr;   // dense last level: leaf masks [nodes, nq] (no records)
     DBuf<uint32_t> bits;   // node x query bitmap (when the regrouping used one)
     DBuf<int32_t> wpre;
@@ -118,7 +122,7 @@ void tc_split_queries(const float *Q, int64_t nq, int dim, int dim_p, DBuf<uint8
                       DBuf<float> &qn2, cudaStream_t st, const int32_t *sel = nullptr);
 // whether tc_regroup counts entries per node itself (a node x query bitmap),
 // so the caller need not
-bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E);
+bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E, int h = 0);
 // regroup the last-level entries by node into tiles; returns the tile count
 // counts: entries with a surviving leaf per last-level node, if already known
 // window_ok: mark dense nodes' items for window mode (tensor-core tiles of

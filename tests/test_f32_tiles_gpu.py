@@ -63,3 +63,18 @@ def test_f32_tiles_unaligned_queries_and_deletes(gts):
     assert r.stats["tiles"] > 0
     check(r, oracle.knn_query("l2", X, Q, 12, ins, dl, np.full(200, s1, np.int64)), "deletes")
     ix.close()
+
+
+@pytest.mark.parametrize("dim", [40, 128, 300])
+def test_range_tiles_over_the_parents_of_small_nodes(gts, dim):
+    """Range queries on nodes of a few rows run the tensor-core tiles over the
+    level above (masks over the nodes, path distances of fewer levels)."""
+    X, Q = small_vectors(9011, dim, 210, seed=600 + dim, dup_frac=0.1)
+    Q[:3] = X[[5, 9, 9010]]
+    ix = gts.Index.build(X, "l2", n_pivots=3, fanout=7, root_pivot=7)   # 49 nodes of 184 rows, 343 of 26
+    cal = oracle.knn_query("l2", X, Q[:10], 200)
+    radii = np.linspace(0.0, 1.5, 210).astype(np.float32) * np.float32(np.mean(cal[2][cal[0][1:] - 1]))
+    r = ix.range(Q, radii, precision="bf16")
+    assert r.stats["tiles"] <= 49 * 2 and r.stats["tiles"] > 0      # blocks of the parents, not of the 343 nodes
+    check(r, oracle.range_query("l2", X, Q, radii), f"coarse range {dim}")
+    ix.close()
