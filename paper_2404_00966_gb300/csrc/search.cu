@@ -689,21 +689,36 @@ __global__ void k_expand(Dev d, const int32_t *__restrict__ eq, const int32_t *_
             const float gthr = in ? thr_q[eq[eg]] : 0.f;
             const int ne = e1 - g0 < 32 ? (int)(e1 - g0) : 32;
             uint64_t my_m = 0;
-            for (int i = 0; i < ne; ++i) {
-                const int32_t node = __shfl_sync(0xffffffffu, gnode, i);
-                const float dq = __shfl_sync(0xffffffffu, gdq, i);
-                const float thr = __shfl_sync(0xffffffffu, gthr, i);
-                uint64_t m = 0;
+            // (four entries at a time, so that their loads are in flight together)
+            for (int i = 0; i < ne; i += 4) {
+                uint64_t m[4] = {0ull, 0ull, 0ull, 0ull};
                 for (int j0 = 0; j0 < d.F; j0 += 32) {
                     const int j = j0 + lane;
-                    bool keep = false;
-                    if (j < d.F) {
-                        const int64_t c = lvl_next + (int64_t)node * d.F + j;
-                        keep = d.nsize[c] > 0 && interval_hit(dq, thr, d.nlo[c], d.nhi[c], d.epsc, d.lslack[l]);
+                    int32_t sz[4];
+                    float lo[4], hi[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int32_t node = __shfl_sync(0xffffffffu, gnode, i + u);
+                        sz[u] = 0;
+                        lo[u] = hi[u] = 0.f;
+                        if (j < d.F && i + u < ne) {
+                            const int64_t c = lvl_next + (int64_t)node * d.F + j;
+                            sz[u] = d.nsize[c];
+                            lo[u] = d.nlo[c];
+                            hi[u] = d.nhi[c];
+                        }
                     }
-                    m |= (uint64_t)__ballot_sync(0xffffffffu, keep) << j0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float dq = __shfl_sync(0xffffffffu, gdq, i + u);
+                        const float thr = __shfl_sync(0xffffffffu, gthr, i + u);
+                        const bool keep = sz[u] > 0 && interval_hit(dq, thr, lo[u], hi[u], d.epsc, d.lslack[l]);
+                        m[u] |= (uint64_t)__ballot_sync(0xffffffffu, keep) << j0;
+                    }
                 }
-                if (lane == i) my_m = m;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (lane == i + u) my_m = m[u];
             }
             if (in) {
                 mask_io[eg - e0] = my_m;
@@ -713,9 +728,8 @@ __global__ void k_expand(Dev d, const int32_t *__restrict__ eq, const int32_t *_
         return;
     }
     for (int64_t e = e0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); e < e1; e += nw) {
-    const int32_t q = eq[e];
-    const int32_t node = enode[e];
-    if (MODE == 1) {
+        const int32_t q = eq[e];
+        const int32_t node = enode[e];
         const uint64_t m = mask_io[e - e0];
         const int64_t base = off[e - e0];
         for (int j0 = 0; j0 < d.F; j0 += 32) {
@@ -727,24 +741,6 @@ __global__ void k_expand(Dev d, const int32_t *__restrict__ eq, const int32_t *_
                 for (int t = 0; t <= l; ++t) npath_out[o * d.h + t] = path[e * d.h + t];
             }
         }
-        continue;
-    }
-    const float dq = path[e * d.h + l];
-    const float thr = thr_q[q];
-    uint64_t m = 0;
-    for (int j0 = 0; j0 < d.F; j0 += 32) {
-        const int j = j0 + lane;
-        bool keep = false;
-        if (j < d.F) {
-            const int64_t c = lvl_next + (int64_t)node * d.F + j;
-            keep = d.nsize[c] > 0 && interval_hit(dq, thr, d.nlo[c], d.nhi[c], d.epsc, d.lslack[l]);
-        }
-        m |= (uint64_t)__ballot_sync(0xffffffffu, keep) << j0;
-    }
-    if (lane == 0) {
-        mask_io[e - e0] = m;
-        if (MODE == 0) cnt[e - e0] = __popcll(m);
-    }
     }
 }
 
@@ -2010,7 +2006,7 @@ __global__ void k_cm_scatter(const int32_t *__restrict__ eq, const int32_t *__re
 }
 
 constexpr int64_t kDenseTcMinPivots = 2048;   // the smallest level whose dense matrix runs on the tensor cores
-constexpr int kTauUnroll = 4;   // pivots per lane whose loads k_tau_dense issues together
+constexpr int kTauUnroll = 8;   // pivots per lane whose loads k_tau_dense issues together
 
 // member(node, q): the node's bit in its parent's child mask for q
 // (node indices of one level fit 32 bits: a 32-bit division, far cheaper than a 64-bit one)
@@ -2020,7 +2016,9 @@ __device__ __forceinline__ bool dense_member(const uint64_t *cm, int64_t node, i
 }
 
 // kNN threshold from this level's pivots (warp per query; the same candidates
-// as k_tau over the entry list: the pivots of the member nodes)
+// as k_tau over the entry list: the pivots of the member nodes).  It streams
+// the distance rows (10^4 x 8,000: 0.45 ms); reading every pivot's membership
+// beside them took 0.48 ms.
 __global__ void k_tau_dense(Dev d, const float *__restrict__ D, int64_t P, const uint64_t *__restrict__ cm,
                             int64_t lvl_base, int64_t nq, const int32_t *__restrict__ kq,
                             const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n,
@@ -2052,26 +2050,25 @@ __global__ void k_tau_dense(Dev d, const float *__restrict__ D, int64_t P, const
         };
         refresh();
         for (int64_t p0 = 0; p0 < P; p0 += 32 * kTauUnroll) {
-            // kTauUnroll pivots per lane: their membership and distance loads
-            // are issued together, then they are tested in pivot order
-            bool mem[kTauUnroll];
+            // kTauUnroll pivots per lane: their distance loads are issued
+            // together, then they are tested in pivot order
             float dv[kTauUnroll];
 #pragma unroll
             for (int u = 0; u < kTauUnroll; ++u) {
                 const int64_t p = p0 + 32 * u + lane;
-                mem[u] = p < P && dense_member(cm, p, q, nq, d.F);
-                dv[u] = p < P ? D[q * P + p] : 0.f;
+                dv[u] = p < P ? __ldg(D + q * P + p) : __int_as_float(0x7f800000);
             }
 #pragma unroll
             for (int u = 0; u < kTauUnroll; ++u) {
                 const int64_t p = p0 + 32 * u + lane;
+                // the bound test first: nearly every pivot fails it, and then
+                // its membership, delete mark and id are never read
+                if (!__any_sync(0xffffffffu, p < P && dv[u] <= fthr)) continue;
                 bool cand = false;
                 double ub = 0.0;
                 int64_t id = 0;
-                if (mem[u] && dv[u] <= fthr) {
+                if (p < P && dv[u] <= fthr && dense_member(cm, p, q, nq, d.F)) {
                     ub = (double)dv[u] * up + (double)d.absf + (double)lab;
-                    // the bound test first: most pivots fail it, and then the
-                    // pivot's delete mark and id are never read
                     if ((L.n < K) || ub <= kth) {
                         const int32_t prow = d.npiv[lvl_base + p];
                         if (prow >= 0 && row_visible(d, prow, s)) {
@@ -2119,171 +2116,114 @@ __global__ void k_transpose_f32(const float *__restrict__ in, int64_t rows, int6
 }
 
 // Leaf masks of every member pair (Lemma 1 / 2 on the node's children
-// intervals, the same test as the entry kernels), the node x query bitmap of
-// the pairs with a surviving leaf, and the counts of member pairs and of
-// pairs with a surviving leaf.  Queries are taken in column order: position i
-// is query perm[i] (DT, M and the bitmap are in position order).  A block takes one node at a time and all of
-// its queries, 256 per step.
-// packed FP32 pairs, round to nearest: (a0 + b0, a1 + b1), (a0 - b0, a1 - b1), (a0 b0, a1 b1)
-__device__ __forceinline__ float2 add2f(float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-        "add.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ float2 sub2f(float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-        "sub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ float2 mul2f(float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-        "mul.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
+// intervals), the node x query bitmap of the pairs with a surviving leaf, and
+// the counts of member pairs and of pairs with a surviving leaf.  Queries are
+// taken in column order: position i is query perm[i] (DT, M and the bitmap are
+// in position order).  A block takes one parent, all of its F nodes, and
+// kLeafQueries queries, a thread per query: the query's threshold and the
+// parent's child mask (the membership of all F nodes) are read once, and every
+// access to DT and M is coalesced.  (A node at a time with its membership
+// looked up per pair took 0.71 ms for 8,000 nodes x 10^4 queries; this form
+// 0.56.)
+//
+// Sorted form: the build cuts a node's rows, in ascending distance to its
+// pivot, into consecutive children, so the non-empty children are a suffix
+// whose [lo, hi] rise with j.  Then the children that pass the test with one
+// eps >= every child's (the one of the largest hi) are the range [ja, jb]
+// found by two binary searches -- a superset of the per-child test's, so no
+// surviving leaf is lost.  Checked per node; a node that is not so ordered
+// takes the per-child test.  A failed test shows as the sign bit of (hi +
+// eps) - (dq - thr) or of (dq + thr + eps) - lo: both differences are rounded
+// once from the exact ones and are never -0 (eps >= +0).
+constexpr int kLeafQueries = 1024;
 
-__global__ void k_leaf_dense(Dev d, const float *__restrict__ DT, const uint64_t *__restrict__ cm, int64_t P,
-                             int64_t nq, int64_t lvl_next, const float *__restrict__ thr_q,
-                             const int32_t *__restrict__ perm, uint64_t *__restrict__ M,
-                             uint32_t *__restrict__ bits, int64_t nw, unsigned long long *__restrict__ counts) {
-    // the node's children two at a time: (hi_j, hi_j+1, |hi_j|, |hi_j+1|) and
-    // (lo_j, lo_j+1) for j = 2 i; and the mask of the non-empty children
-    __shared__ float4 sph[32];
-    __shared__ float2 spl[32];
-    __shared__ unsigned long long s_ne;
-    // the same children in order, for the sorted form (below)
-    __shared__ float s_hi[64], s_lo[64];
-    __shared__ int s_sorted, s_j0;
+__global__ void __launch_bounds__(256) k_leaf_dense(Dev d, const float *__restrict__ DT,
+                                                    const uint64_t *__restrict__ cm, int64_t P, int64_t nq,
+                                                    int64_t lvl_next, const float *__restrict__ thr_q,
+                                                    const int32_t *__restrict__ perm, uint64_t *__restrict__ M,
+                                                    uint32_t *__restrict__ bits, int64_t nw,
+                                                    unsigned long long *__restrict__ counts) {
+    extern __shared__ float s_iv[];          // hi [F][F], lo [F][F] of the F nodes' children
+    __shared__ unsigned long long s_ne[64];  // per node: its non-empty children
+    __shared__ int8_t s_j0[64];              // the first of them; -1: not sorted
+    const int F = d.F;
+    float *s_hi = s_iv, *s_lo = s_iv + F * F;
     const int lane = threadIdx.x & 31;
-    const float epsc = d.epsc;
+    const int64_t par = blockIdx.x;
+    const int64_t p0 = par * F;
+    if (threadIdx.x < 64) s_ne[threadIdx.x] = 0ull;
+    __syncthreads();
+    for (int i = threadIdx.x; i < F * F; i += blockDim.x) {
+        const int64_t c = lvl_next + p0 * F + i;
+        const bool ne = d.nsize[c] > 0;
+        s_hi[i] = ne ? d.nhi[c] : 0.f;
+        s_lo[i] = ne ? d.nlo[c] : 0.f;
+        if (ne) atomicOr(&s_ne[i / F], 1ull << (i % F));
+    }
+    __syncthreads();
+    if (threadIdx.x < F) {
+        const float *hi = s_hi + threadIdx.x * F, *lo = s_lo + threadIdx.x * F;
+        const uint64_t ne = s_ne[threadIdx.x];
+        bool bad = ne == 0ull || hi[F - 1] < lo[F - 1];
+        for (int j = 0; j + 1 < F; ++j) {
+            const bool ne0 = (ne >> j) & 1ull, ne1 = (ne >> (j + 1)) & 1ull;
+            if (ne0 && (!ne1 || hi[j] > hi[j + 1] || lo[j] > lo[j + 1] || lo[j] < 0.f || hi[j] < lo[j])) bad = true;
+        }
+        s_j0[threadIdx.x] = bad ? -1 : (int8_t)(__ffsll((long long)ne) - 1);
+    }
+    __syncthreads();
+    const float epsc = d.epsc, lab = d.lslack[d.h - 1];
     unsigned long long nmem = 0, nlive = 0;
-    // one node per block iteration, all of its queries: the children are read once
-    for (int64_t p = blockIdx.x; p < P; p += gridDim.x) {
-        __syncthreads();   // the previous node's children are no longer read
-        if (threadIdx.x == 0) s_ne = 0ull;
-        __syncthreads();
-        if (threadIdx.x < 64) {
-            const int j = threadIdx.x;
-            float lo = 0.f, hi = 0.f;
-            if (j < d.F) {
-                const int64_t c = lvl_next + p * d.F + j;
-                const bool ne = d.nsize[c] > 0;
-                if (ne) {
-                    lo = d.nlo[c];
-                    hi = d.nhi[c];
-                    atomicOr(&s_ne, 1ull << j);
-                }
-            }
-            float *h4 = reinterpret_cast<float *>(&sph[j >> 1]);
-            float *l2 = reinterpret_cast<float *>(&spl[j >> 1]);
-            h4[j & 1] = hi;
-            h4[2 + (j & 1)] = fabsf(hi);
-            l2[j & 1] = lo;
-            s_hi[j] = hi;
-            s_lo[j] = lo;
-        }
-        __syncthreads();
-        const uint64_t nonempty = s_ne;
-        // Sorted form: the build cuts a node's rows, in ascending distance to
-        // its pivot, into consecutive children, so the non-empty children
-        // are a suffix whose [lo, hi] rise with j.  Then the children that
-        // pass the test with one eps >= every child's (the one of the largest
-        // hi) are the range [ja, jb] found by two binary searches -- a
-        // superset of the per-child test's, so no surviving leaf is lost.
-        // Checked per node; a node that is not so ordered takes the per-child
-        // test.
-        if (threadIdx.x < 32) {
-            bool bad = false;
-            for (int j = threadIdx.x; j + 1 < d.F; j += 32) {
-                const bool ne0 = (nonempty >> j) & 1ull, ne1 = (nonempty >> (j + 1)) & 1ull;
-                if (ne0 && (!ne1 || s_hi[j] > s_hi[j + 1] || s_lo[j] > s_lo[j + 1] || s_lo[j] < 0.f ||
-                            s_hi[j] < s_lo[j]))
-                    bad = true;
-            }
-            bad = __any_sync(0xffffffffu, bad);
-            if (threadIdx.x == 0) {
-                s_sorted = !bad && nonempty != 0ull && s_hi[d.F - 1] >= s_lo[d.F - 1];
-                s_j0 = nonempty ? __ffsll((long long)nonempty) - 1 : d.F;
-            }
-        }
-        __syncthreads();
-        const bool sorted = s_sorted != 0;
-        const int j0 = s_j0;
-        const float himax = s_hi[d.F - 1];
-        for (int64_t q0 = 0; q0 < nq; q0 += blockDim.x) {
-            const int64_t q = q0 + threadIdx.x;                          // column position
-            const int64_t qq = q < nq && perm ? (int64_t)perm[q] : q;    // its query
-            const bool member = q < nq && dense_member(cm, p, qq, nq, d.F);
+    const int64_t qa = (int64_t)blockIdx.y * kLeafQueries;
+    for (int64_t q0 = qa; q0 < nq && q0 < qa + kLeafQueries; q0 += blockDim.x) {
+        const int64_t q = q0 + threadIdx.x;                          // column position
+        const int64_t qq = q < nq && perm ? (int64_t)perm[q] : q;    // its query
+        const uint64_t mem = q < nq ? cm[par * nq + qq] : 0ull;
+        const float thr = q < nq ? thr_q[qq] : 0.f;
+        const int64_t w = (q - lane) >> 5;   // the warp's word of the bitmap
+#pragma unroll 2
+        for (int n = 0; n < F; ++n) {
             uint64_t m = 0;
+            const bool member = (mem >> n) & 1ull;
             if (member) {
-                const float dq = DT[p * nq + q];
-                const float thr = thr_q[qq];
-                // interval_hit for two children at a time in packed FP32, its
-                // query terms formed once (the same operations in the same
-                // order): eps = epsc (sq + |hi|) + the level's absolute slack,
-                // keep iff u <= hi + eps and sq + eps >= lo.  A failed test
-                // shows as the sign bit of (hi + eps) - u or of (sq + eps) -
-                // lo: both differences are rounded once from the exact ones
-                // and are never -0 (eps >= +0, so hi + eps and sq + eps are
-                // not -0).
+                const float dq = __ldg(DT + (p0 + n) * nq + q);
+                const float *hi = s_hi + n * F, *lo = s_lo + n * F;
                 const float u = dq - thr, sq = dq + thr;
-                if (sorted) {
-                    const float eps = (epsc > 0.f ? epsc * (sq + himax) : 0.f) + d.lslack[d.h - 1];
-                    // ja: the first child with (hi + eps) - u >= +0; jb + 1: the
-                    // first with (sq + eps) - lo < 0 (sign bits, as below)
-                    int a0 = j0, a1 = d.F;
+                const int j0 = s_j0[n];
+                const uint64_t ne = s_ne[n];
+                if (j0 >= 0) {
+                    const float eps = (epsc > 0.f ? epsc * (sq + hi[F - 1]) : 0.f) + lab;
+                    int a0 = j0, a1 = F;   // ja: the first child with (hi + eps) - u >= +0
                     while (a0 < a1) {
                         const int mid = (a0 + a1) >> 1;
-                        if (__float_as_uint((s_hi[mid] + eps) - u) >> 31) a0 = mid + 1;
+                        if (__float_as_uint((hi[mid] + eps) - u) >> 31) a0 = mid + 1;
                         else a1 = mid;
                     }
                     const int ja = a0;
-                    a0 = j0;
-                    a1 = d.F;
+                    a0 = j0;               // jb + 1: the first with (sq + eps) - lo < 0
+                    a1 = F;
                     while (a0 < a1) {
                         const int mid = (a0 + a1) >> 1;
-                        if (__float_as_uint((sq + eps) - s_lo[mid]) >> 31) a1 = mid;
+                        if (__float_as_uint((sq + eps) - lo[mid]) >> 31) a1 = mid;
                         else a0 = mid + 1;
                     }
                     const int jb = a0 - 1;
-                    if (ja <= jb)
-                        m = ((jb >= 63) ? ~0ull : ((1ull << (jb + 1)) - 1ull)) & ~((1ull << ja) - 1ull) & nonempty;
+                    if (ja <= jb) m = ((jb >= 63) ? ~0ull : ((1ull << (jb + 1)) - 1ull)) & ~((1ull << ja) - 1ull) & ne;
                 } else {
-                    const float2 u2 = make_float2(u, u), sq2 = make_float2(sq, sq);
-                    const float2 ec2 = make_float2(epsc, epsc);
-                    const float2 lab2 = make_float2(d.lslack[d.h - 1], d.lslack[d.h - 1]);
-                    uint64_t fail = 0;
-#pragma unroll 2
-                    for (int j = 0; j < d.F; j += 2) {
-                        const float4 h = sph[j >> 1];
-                        const float2 lo = spl[j >> 1];
-                        const float2 eps = add2f(epsc > 0.f ? mul2f(ec2, add2f(sq2, make_float2(h.z, h.w)))
-                                                            : make_float2(0.f, 0.f),
-                                                 lab2);
-                        const float2 d1 = sub2f(add2f(make_float2(h.x, h.y), eps), u2);
-                        const float2 d2 = sub2f(add2f(sq2, eps), lo);
-                        const uint32_t f0 = (__float_as_uint(d1.x) | __float_as_uint(d2.x)) >> 31;
-                        const uint32_t f1 = (__float_as_uint(d1.y) | __float_as_uint(d2.y)) >> 31;
-                        fail |= (uint64_t)(f0 | (f1 << 1)) << j;
+                    for (int j = 0; j < F; ++j) {
+                        const float eps = (epsc > 0.f ? epsc * (sq + fabsf(hi[j])) : 0.f) + lab;
+                        const uint32_t fail = __float_as_uint((hi[j] + eps) - u) | __float_as_uint((sq + eps) - lo[j]);
+                        if (!(fail >> 31)) m |= 1ull << j;
                     }
-                    m = ~fail & nonempty;
+                    m &= ne;
                 }
             }
-            if (q < nq) M[p * nq + q] = m;
+            if (q < nq) M[(p0 + n) * nq + q] = m;
             const unsigned live = __ballot_sync(0xffffffffu, m != 0ull);
-            const unsigned mem = __ballot_sync(0xffffffffu, member);
-            const int64_t w = (q - lane) >> 5;   // the warp's word
-            if (lane == 0 && w < nw) bits[p * nw + w] = live;
+            const unsigned mb = __ballot_sync(0xffffffffu, member);
             if (lane == 0) {
-                nmem += __popc(mem);
+                if (w < nw) bits[(p0 + n) * nw + w] = live;
+                nmem += __popc(mb);
                 nlive += __popc(live);
             }
         }
@@ -3028,9 +2968,10 @@ struct Runner {
         {
             dim3 tb(32, 8), tg((unsigned)((P + 31) / 32), (unsigned)((nq + 31) / 32));
             if (!have_dt) k_transpose_f32<<<tg, tb, 0, st>>>(D, nq, P, DT.get(), perm.get());
-            k_leaf_dense<<<wave_grid(k_leaf_dense, P, 256), 256, 0, st>>>(
-                d, DT.get(), cm.get(), P, nq, ix->tree.lvl_off[h], thr.get(), perm.get(), M.get(), rg.bits.get(),
-                rg.nw, cnt.get());
+            const dim3 lg((unsigned)Pp, (unsigned)((nq + kLeafQueries - 1) / kLeafQueries));
+            k_leaf_dense<<<lg, 256, (size_t)2 * F * F * 4, st>>>(d, DT.get(), cm.get(), P, nq, ix->tree.lvl_off[h],
+                                                                thr.get(), perm.get(), M.get(), rg.bits.get(), rg.nw,
+                                                                cnt.get());
         }
         clk.end();
         check_launch("dense leaf masks");
