@@ -64,7 +64,8 @@ struct ScanArgs {
     const TileRec *grec;       // records grouped by node
     const float *gpath;        // their path distances [*, hp]
     const int4 *items;         // (node, first record, record count, row block)
-    int64_t n_items;
+    int64_t n_units;           // work units: item u / split, part u % split of its records
+    int split;
     int *work;
     float epsc;
     int any_deleted;
@@ -81,9 +82,9 @@ struct ScanArgs {
     int dim, l2;
     const float *X, *Q;
     const int64_t *row_id;
-    float rel;
+    float rel, absf;
     int warp_bytes;            // shared memory per warp
-    int claim;                 // items a warp takes per atomic on the work counter
+    int claim;                 // units a warp takes per atomic on the work counter
 };
 
 // Per-warp shared-memory layout (bytes), from h, hp and dim.
@@ -145,8 +146,11 @@ __device__ __forceinline__ void emit(const uint32_t *bits, int nstrips, int tota
     }
 }
 
-template <bool FUSED>
-__global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs a) {
+enum ScanMode { kScanPairs = 0, kScanRange = 1, kScanKnn = 2 };
+
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, MODE != kScanPairs ? 6 : 8) k_scan_warps(ScanArgs a) {
+    constexpr bool FUSED = MODE != kScanPairs;   // the pairs' FP32 distances decide here
     extern __shared__ __align__(16) uint8_t dyn[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const WarpLayout L = warp_layout(a.h, a.hp, a.dim, FUSED);
@@ -172,8 +176,8 @@ __global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs
     unsigned long long *cnt_acc = a.counts + kStripes + stripe;
     int32_t *oq = a.out_q + (int64_t)stripe * a.cap;
     int32_t *orow = a.out_row + (int64_t)stripe * a.cap;
-    uint64_t *okey = FUSED ? a.out_key + (int64_t)stripe * a.cap_acc : nullptr;
-    float *odist = FUSED ? a.out_dist + (int64_t)stripe * a.cap_acc : nullptr;
+    uint64_t *okey = MODE == kScanRange ? a.out_key + (int64_t)stripe * a.cap_acc : nullptr;
+    float *odist = FUSED ? a.out_dist + (int64_t)stripe * (MODE == kScanRange ? a.cap_acc : a.cap) : nullptr;
     unsigned long long staged = 0, tested = 0, passed = 0;
     const int64_t hn = (int64_t)a.h * a.n;
     bool ok = true;
@@ -187,14 +191,17 @@ __global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs
             if (lane == 0) it = atomicAdd(a.work, a.claim);
             it = __shfl_sync(kFull, it, 0);
             run_next = it;
-            run_end = (int)min((int64_t)it + a.claim, a.n_items);
+            run_end = (int)min((int64_t)it + a.claim, a.n_units);
         }
-        if (run_next >= a.n_items) break;
+        if (run_next >= a.n_units) break;
         const int it = run_next++;
-        const int4 w = a.items[it];
+        const int4 w = a.items[it / a.split];
         const int64_t node = a.lvl_last + w.x;
-        const int64_t first = w.y;
-        const int cnt = w.z, blk = w.w;
+        // this unit's share of the node's records
+        const int per = ((w.z + a.split - 1) / a.split + kRecW - 1) & ~(kRecW - 1);
+        const int64_t first = (int64_t)w.y + (int64_t)(it % a.split) * per;
+        const int cnt = min(per, w.z - (it % a.split) * per), blk = w.w;
+        if (cnt <= 0) continue;
         const int32_t pos = a.npos[node], size = a.nsize[node];
         const int32_t avg = size / a.F;
         const int r0 = blk * kRowsB;
@@ -288,6 +295,10 @@ __global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs
                                 for (int c2 = 0; c2 < a.dim; ++c2) sum += fabsf(qrow[c2] - xr[c2]);
                             }
                             const float d32 = a.l2 ? sqrtf(sum) : sum;
+                            dv[s] = d32;
+                            if (MODE == kScanKnn) {
+                                pass = d32 * (1.f - 2.f * a.rel) - a.absf <= thr;
+                            } else {
                             const float hi = d32 * (1.f + 2.f * a.rel) + kAbsFloor;
                             const float lo = d32 * (1.f - 2.f * a.rel) - kAbsFloor;
                             if (hi < thr * (1.f - 1e-9f)) {
@@ -296,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs
                             } else if (lo > thr * (1.f + 1e-9f)) {
                                 pass = false;
                             }
-                            dv[s] = d32;
+                            }
                         }
                     }
                     pb[s] = __ballot_sync(kFull, pass);
@@ -310,9 +321,10 @@ __global__ void __launch_bounds__(kThreads, FUSED ? 6 : 8) k_scan_warps(ScanArgs
                     if ((int64_t)o < a.cap) {
                         oq[o] = q;
                         orow[o] = (int32_t)(g0 + s * 32 + lane);
+                        if (MODE == kScanKnn) odist[o] = dv[s];
                     }
                 });
-                if (FUSED)
+                if (MODE == kScanRange)
                     emit(ab, nstrips, tot_acc, cnt_acc, lane, [&](int s, unsigned long long o) {
                         if ((int64_t)o < a.cap_acc) {
                             okey[o] = ((uint64_t)(uint32_t)q << 32) | (uint64_t)(uint32_t)a.row_id[g0 + s * 32 + lane];
@@ -370,31 +382,35 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
     if (rg.n_items == 0) return;
     GTS_REQUIRE(t.h >= 1 && t.h <= kMaxHeight && t.F <= kMaxFanout, GTS_EINVAL, "tree shape out of range for the scan");
     GTS_REQUIRE(!rg.dmask && rg.grec.get() && rg.gpath.get(), GTS_EINVAL, "the scan needs regrouped records");
-    GTS_REQUIRE(!sq.fused_range || (t.dim >= 1 && t.dim <= kScanMaxDim && sq.Q), GTS_EINVAL,
-                "fused range scan needs vectors of at most 16 dimensions");
-    const bool fused = sq.fused_range;
+    GTS_REQUIRE(!(sq.fused_range || sq.fused_knn) || (t.dim >= 1 && t.dim <= kScanMaxDim && sq.Q), GTS_EINVAL,
+                "a fused scan needs vectors of at most 16 dimensions");
+    const bool range = sq.fused_range, fused = range || sq.fused_knn;
     const int hp = (t.h + 3) & ~3;
     const WarpLayout L = warp_layout(t.h, hp, t.dim, fused);
     const int smem = L.bytes * kWarpsPerCta;
     int dev = 0, sms = 0, per_sm = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (fused) {
-        GTS_CUDA(cudaFuncSetAttribute(k_scan_warps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan_warps<true>, kThreads, smem));
-    } else {
-        GTS_CUDA(cudaFuncSetAttribute(k_scan_warps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scan_warps<false>, kThreads, smem));
-    }
-    const int64_t warps_needed = (rg.n_items + 0);
+    void (*kern)(ScanArgs) = range ? k_scan_warps<kScanRange> : fused ? k_scan_warps<kScanKnn> : k_scan_warps<kScanPairs>;
+    GTS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
     const int64_t resident = (int64_t)(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((warps_needed + kWarpsPerCta - 1) / kWarpsPerCta, resident));
+    // an item's records are split over several units while there are fewer
+    // than four units per resident warp and the parts still hold two chunks (a
+    // small tree: 400 items of 2,000 records kept 400 of 3,600 warps busy)
+    const int64_t avg_records = rg.n_entries / std::max<int64_t>(1, rg.n_nodes);
+    const int64_t split = std::max<int64_t>(
+        1, std::min<int64_t>(avg_records / (2 * kRecW), 4 * resident * kWarpsPerCta / rg.n_items));
+    const int64_t units = rg.n_items * split;
+    GTS_REQUIRE(units < ((int64_t)1 << 31) - 16 * resident * kWarpsPerCta, GTS_EINVAL, "too many scan units");
+    const unsigned grid =
+        (unsigned)std::max<int64_t>(1, std::min<int64_t>((units + kWarpsPerCta - 1) / kWarpsPerCta, resident));
     const int nc = 2 * kStripes + 3;
     DBuf<unsigned long long> counts(nc, st);
     DBuf<int> work(1, st), status(1, st);
     // per-stripe slices; fused: most passing pairs are accepted answers, few fall in the band
-    int64_t cap = std::max<int64_t>((fused ? cap_hint / 16 : cap_hint) / kStripes + 1, 1 << 12);
-    int64_t cap_acc = fused ? std::max<int64_t>(cap_hint / kStripes + 1, 1 << 12) : 0;
+    int64_t cap = std::max<int64_t>((range ? cap_hint / 16 : cap_hint) / kStripes + 1, 1 << 12);
+    int64_t cap_acc = range ? std::max<int64_t>(cap_hint / kStripes + 1, 1 << 12) : 0;
     std::vector<unsigned long long> hc(nc, 0);
     // Work stealing spreads the items over the warps (and so over the
     // stripes) differently on every launch: a relaunch sized by one launch's
@@ -404,8 +420,8 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
     for (int attempt = 0; attempt < 8 && !fits; ++attempt) {
         out.q.alloc(cap * kStripes, st);
         out.row.alloc(cap * kStripes, st);
-        out.key.alloc(fused ? cap_acc * kStripes : 1, st);
-        out.dist.alloc(fused ? cap_acc * kStripes : 1, st);
+        out.key.alloc(range ? cap_acc * kStripes : 1, st);
+        out.dist.alloc(range ? cap_acc * kStripes : fused ? cap * kStripes : 1, st);
         GTS_CUDA(cudaMemsetAsync(counts.get(), 0, nc * sizeof(unsigned long long), st));
         GTS_CUDA(cudaMemsetAsync(work.get(), 0, sizeof(int), st));
         GTS_CUDA(cudaMemsetAsync(status.get(), 0, sizeof(int), st));
@@ -422,7 +438,8 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
         a.grec = rg.grec.get();
         a.gpath = rg.gpath.get();
         a.items = rg.items.get();
-        a.n_items = rg.n_items;
+        a.n_units = units;
+        a.split = (int)split;
         a.work = work.get();
         a.epsc = sq.epsc;
         a.any_deleted = sq.any_deleted;
@@ -440,13 +457,11 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
         a.Q = sq.Q;
         a.row_id = t.row_id.get();
         a.rel = sq.rel;
+        a.absf = sq.absf;
         a.warp_bytes = L.bytes;
-        // runs of consecutive items: about 16 runs per warp, 1 .. 16 items each
-        a.claim = (int)std::max<int64_t>(1, std::min<int64_t>(16, rg.n_items / ((int64_t)grid * kWarpsPerCta * 16)));
-        if (fused)
-            k_scan_warps<true><<<grid, kThreads, smem, st>>>(a);
-        else
-            k_scan_warps<false><<<grid, kThreads, smem, st>>>(a);
+        // runs of consecutive units: about 16 runs per warp, 1 .. 16 units each
+        a.claim = (int)std::max<int64_t>(1, std::min<int64_t>(16, units / ((int64_t)grid * kWarpsPerCta * 16)));
+        kern<<<grid, kThreads, smem, st>>>(a);
         check_launch("table scan");
         stats.launches += 1;
         int hs = 0;
@@ -462,7 +477,7 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
         fits = mx <= cap && mxa <= cap_acc;
         if (!fits) {
             cap = std::max(cap, mx + mx / 4 + 1024);
-            cap_acc = fused ? std::max(cap_acc, mxa + mxa / 4 + 1024) : 0;
+            cap_acc = range ? std::max(cap_acc, mxa + mxa / 4 + 1024) : 0;
         }
     }
     GTS_REQUIRE(fits, GTS_ECUDA, "table scan: output slices kept overflowing");
@@ -473,7 +488,8 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
     }
     pack(out.q, counts.get(), cap, np, st);
     pack(out.row, counts.get(), cap, np, st);
-    if (fused) {
+    if (fused && !range) pack(out.dist, counts.get(), cap, np, st);
+    if (range) {
         pack(out.key, counts.get() + kStripes, cap_acc, na, st);
         pack(out.dist, counts.get() + kStripes, cap_acc, na, st);
     }

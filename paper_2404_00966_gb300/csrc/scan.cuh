@@ -27,14 +27,18 @@ struct ScanQuery {
     // decide it against the radius with the FP32 error band; accepted pairs
     // go straight to the answer, pairs inside the band to the FP64 recheck
     bool fused_range = false;
+    // kNN on such vectors: the same distance, and only the pairs whose lower
+    // bound is within tau_q are written, with their distance
+    bool fused_knn = false;
     const float *Q = nullptr; // queries [nq, dim]
     float rel = 0.f;          // FP32 relative error bound of one distance
+    float absf = 0.f;         // and its absolute slack
 };
 
 struct ScanOut {
     DBuf<int32_t> q, row;     // candidates (plain scan) or band pairs (fused range)
     DBuf<uint64_t> key;       // fused range: accepted answers, (query << 32) | object id
-    DBuf<float> dist;         // and their FP32 distances
+    DBuf<float> dist;         // and their FP32 distances (fused kNN: the pairs')
     int64_t n_pairs = 0;      // entries of q / row
     int64_t n_accepted = 0;   // entries of key / dist
 };

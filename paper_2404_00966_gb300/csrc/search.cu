@@ -2470,6 +2470,7 @@ struct Runner {
     bool use_f32 = false;  // GTS_PREC_FP32: FP32 CUDA-core tiles where the last level's nodes hold enough queries
     bool use_qg = false;   // 3-gram filtering tiles at the last level (edit distance)
     bool use_qg_large = false;   // the same for large batches only (qgram_tiles_pay)
+    bool use_scan_large = false;   // GTS_PREC_FP32: the same for large batches (f32_tiles_pay)
     bool use_scan = false; // low-dim vectors: node-major table scan + CUDA-core verification
     Tuning tu;             // launch parameters (a copy of the index's)
     // dense query-to-pivot matrices per level (tile paths): state 0 undecided, 1 ready, 2 not used
@@ -2671,7 +2672,8 @@ struct Runner {
 
     void process(Level &L, int64_t e0, int64_t e1, int l) {
         if (e1 <= e0) return;
-        if (l == h - 1 && (use_tc || use_l1 || use_scan || (use_f32 && f32_tiles_pay(e1 - e0)))) {
+        if (l == h - 1 && (use_tc || use_l1 || use_scan || (use_f32 && f32_tiles_pay(e1 - e0, kF32TilePairs)) ||
+                           (use_scan_large && f32_tiles_pay(e1 - e0, kScanPairs)))) {
             last_level_tc(L, e0, e1, l);
             return;
         }
@@ -3094,7 +3096,7 @@ struct Runner {
 
     void tc_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask, DBuf<int32_t> *ncount = nullptr) {
         count_table_pass(L, e0, e1, mask);
-        if (use_scan) {
+        if (use_scan || use_scan_large) {
             scan_leaf(L, e0, e1, mask, ncount);
             return;
         }
@@ -3181,8 +3183,10 @@ struct Runner {
         // range: decide the pairs in the scan (low dimension; the angular
         // distance takes its FP64 key for every pair, so not there)
         sq.fused_range = !knn && !d.cosine;
+        sq.fused_knn = knn;
         sq.Q = d.Q;
         sq.rel = d.rel;
+        sq.absf = d.absf;
         ScanOut so;
         ScanStats ss;
         clk.begin(GTS_STAGE_LEAF_SCAN);
@@ -3208,7 +3212,32 @@ struct Runner {
             return;
         }
         if (so.n_pairs == 0) return;
+        if (sq.fused_knn) {
+            st_cands += ss.candidates;
+            sort_and_merge(so.q, so.row, so.dist, so.n_pairs);
+            return;
+        }
         verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
+    }
+
+    // kNN pairs in any order into the answers: a stable radix sort by query
+    // with (row, distance) carried along, then the merge
+    void sort_and_merge(DBuf<int32_t> &q, DBuf<int32_t> &row, DBuf<float> &dist, int64_t C) {
+        DBuf<uint64_t> v1(C, st), v2(C, st);
+        DBuf<int32_t> q2(C, st), r2(C, st);
+        DBuf<float> d2(C, st);
+        int qbits = 1;
+        while (((int64_t)1 << qbits) < qb.nq) ++qbits;
+        size_t tb = 0;
+        cub::DeviceRadixSort::SortPairs(nullptr, tb, q.get(), q2.get(), v1.get(), v2.get(), C, 0, qbits, st);
+        DBuf<uint8_t> tmp(tb ? tb : 1, st);
+        clk.begin(GTS_STAGE_OTHER, 3);
+        k_pack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(row.get(), dist.get(), C, v1.get());
+        GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, q.get(), q2.get(), v1.get(), v2.get(), C, 0, qbits,
+                                                 st));
+        k_unpack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(v2.get(), C, r2.get(), d2.get());
+        clk.end();
+        merge_knn(q2, r2, d2, C);
     }
 
     // Strings: whether E last-level entries go through the 3-gram tiles: always
@@ -3321,6 +3350,10 @@ struct Runner {
             ++st_groups;
             if (C == 0) return;
             st_cands += C;
+            if (knn) {
+                sort_and_merge(oq, orow, od, C);
+                return;
+            }
             DBuf<uint8_t> keep(C, st);
             GTS_CUDA(cudaMemsetAsync(keep.get(), 1, C, st));
             collect(oq, orow, od, keep, C, /*query_major=*/false);
@@ -3465,21 +3498,7 @@ struct Runner {
             st_cands += C;
             DBuf<uint8_t> keep(C, st);
             if (knn) {   // the merge wants query-major order
-                DBuf<uint64_t> v1(C, st), v2(C, st);
-                DBuf<int32_t> q2(C, st), r2(C, st);
-                DBuf<float> d2(C, st);
-                int qbits = 1;
-                while (((int64_t)1 << qbits) < qb.nq) ++qbits;
-                size_t tb = 0;
-                cub::DeviceRadixSort::SortPairs(nullptr, tb, oq.get(), q2.get(), v1.get(), v2.get(), C, 0, qbits, st);
-                DBuf<uint8_t> tmp(tb ? tb : 1, st);
-                clk.begin(GTS_STAGE_OTHER, 3);
-                k_pack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(orow.get(), od.get(), C, v1.get());
-                GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, oq.get(), q2.get(), v1.get(), v2.get(), C, 0,
-                                                         qbits, st));
-                k_unpack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(v2.get(), C, r2.get(), d2.get());
-                clk.end();
-                merge_knn(q2, r2, d2, C);
+                sort_and_merge(oq, orow, od, C);
                 clk.begin(GTS_STAGE_THRESHOLD);
                 k_tau_from_answer<<<cap(nblocks(qb.nq, kT)), kT, 0, st>>>(qb.k, koff.get(), bd.get(), bn.get(), qb.nq,
                                                                          0, thr.get());
@@ -3584,22 +3603,8 @@ struct Runner {
             clk.end();
             if (query_major) {
                 merge_knn(kq2, krow2, kd2, R);
-            } else {   // stable radix sort by query, (row, distance) carried along
-                DBuf<uint64_t> v1(R, st), v2(R, st);
-                DBuf<int32_t> q3(R, st), r3(R, st);
-                DBuf<float> d3(R, st);
-                int qbits = 1;
-                while (((int64_t)1 << qbits) < qb.nq) ++qbits;
-                size_t tb = 0;
-                cub::DeviceRadixSort::SortPairs(nullptr, tb, kq2.get(), q3.get(), v1.get(), v2.get(), R, 0, qbits, st);
-                DBuf<uint8_t> tmp(tb ? tb : 1, st);
-                clk.begin(GTS_STAGE_OTHER, 3);
-                k_pack_row_dist<<<cap(nblocks(R, kT)), kT, 0, st>>>(krow2.get(), kd2.get(), R, v1.get());
-                GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, kq2.get(), q3.get(), v1.get(), v2.get(), R, 0,
-                                                         qbits, st));
-                k_unpack_row_dist<<<cap(nblocks(R, kT)), kT, 0, st>>>(v2.get(), R, r3.get(), d3.get());
-                clk.end();
-                merge_knn(q3, r3, d3, R);
+            } else {
+                sort_and_merge(kq2, krow2, kd2, R);
             }
         } else {
             DBuf<uint64_t> rk(R, st);
@@ -3747,6 +3752,8 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     const bool low_dim = t.dim > 0 && t.dim <= kScanMaxDim && (t.metric == GTS_L1 || t.metric == GTS_L2) &&
                          t.n > 0 && t.n < ((int64_t)1 << 31);
     if (precision == GTS_PREC_BF16 && low_dim) R.use_scan = true;
+    if (precision == GTS_PREC_FP32 && low_dim && budget >= kF32TileBudget && !qb.count_table_pass)
+        R.use_scan_large = true;
     if (precision == GTS_PREC_BF16 && !low_dim && l1_tiles_supported(t, qb.Q)) R.use_l1 = true;
     // GTS_PREC_FP32: node-major FP32 tiles for batches (the diagnostic count
     // needs the plain scan, whose candidates are the counted pairs)

@@ -1063,6 +1063,7 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
     GTS_CUDA(cudaStreamSynchronize(st));
     rg.n_pairs = (int64_t)total_pairs;
     rg.n_items = total_items;
+    rg.n_nodes = nn;
     if (total_items > 0) {
         rg.items.alloc(total_items, st);
         // window mode for nodes holding at least half of the batch

@@ -107,6 +107,7 @@ struct TcRegroup {
     DBuf<float> gpath;     // their path distances [*, hp]
     DBuf<int4> items;      // (node, first, count, 0)
     int64_t n_items = 0;
+    int64_t n_nodes = 0;   // nodes of the level
     int64_t n_entries = 0; // entries with a surviving leaf
     int64_t n_chunks = 0;  // query chunks over all blocks (tensor-core tiles)
     int64_t n_pairs = 0;   // (query, row) pairs of all blocks: sum over nodes of entries x rows
