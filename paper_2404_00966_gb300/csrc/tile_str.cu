@@ -25,9 +25,10 @@ namespace gts {
 namespace {
 
 constexpr int kRowsS = 128;     // rows of one node block (the regrouping's block size)
-constexpr int kThreadsS = 256;  // warp w: rows [64 (w % 2), + 64), two per lane; queries of group w / 2
+constexpr int kThreadsS = 256;
 constexpr int kWords = 16;      // 64 one-byte buckets as 16 words
-constexpr int kGroups = 4;      // query groups of a chunk
+constexpr int kGroups = kThreadsS / 32;   // query groups of a chunk, one per warp
+constexpr int kRPL = kRowsS / 32;         // rows per lane: lane + 32 h
 
 struct StrArgs {
     int F;
@@ -53,23 +54,25 @@ __device__ __forceinline__ void cpa16s(void *dst, const void *src) {
                  : "memory");
 }
 
-// NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 4 per thread.
+// NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 8 per warp.
 // The ALU pipe bounds it: 16 four-byte sums of absolute differences per pair
 // (19 T a second on the device, 60 of 64 lanes per SM and cycle: 1.9 * 10^10
-// pairs cannot take less than 16 ms).  So a lane holds two rows, and a query's
-// 64 bytes -- four 16-byte broadcast loads -- serve 64 rows of its warp; the
-// sums start at -(limit + 1), so that the test is their sign bit, shifted into
-// the pass masks; a chunk's records and vectors are copied while the one before
-// is computed (the query ids they need are read two chunks ahead); and the
-// leaf and visibility tests run on the few pairs that pass.
+// pairs cannot take less than 16 ms).  A warp therefore holds the whole block,
+// four rows a lane: a query's 64 bytes are four 16-byte broadcast loads, each
+// of which takes the shared-memory port four cycles to write back, and with
+// two rows a lane (31.9 ms; now 31.4) or one (53.0) they held the kernel back.
+// The sums
+// start at -(limit + 1), so that the test is their sign bit, shifted into the
+// pass masks; a chunk's records and vectors are copied while the one before is
+// computed (the query ids they need are read two chunks ahead); and the leaf
+// and visibility tests run on the few pairs that pass.
 template <int NQS>
-__global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
+__global__ void __launch_bounds__(kThreadsS, 2) k_tile_qgram(StrArgs a) {
     constexpr int kPer = NQS / kGroups;
     __shared__ uint4 sQ[2][NQS][kWords / 4];
     __shared__ __align__(16) TileRec sRec[2][NQS];
     __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int group = warp >> 1;
     const int cj = tid / 4, cw = tid & 3;   // the vector piece this thread copies (tid < 4 NQS)
     for (;;) {
         if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
@@ -100,22 +103,20 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
         const int nrow = min(kRowsS, size - rb);
         const int32_t avg = size / a.F;
         stage(0, qid0);
-        // this lane's two rows: bucket counts, leaf bits, delete marks
-        uint32_t rw[2][kWords];
-        uint64_t rowbit[2];
-        int64_t rdel[2];
-        const int r0 = (warp & 1) * 64 + lane;
+        // this lane's rows: bucket counts, leaf bits, delete marks
+        uint32_t rw[kRPL][kWords];
+        uint64_t rowbit[kRPL], any = 0;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int r = r0 + 32 * h;
+        for (int h = 0; h < kRPL; ++h) {
+            const int r = lane + 32 * h;
             const bool valid = r < nrow;
-            const int64_t row = (int64_t)pos + rb + r;
+            const int64_t row = (int64_t)pos + (valid ? rb + r : 0);
             int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
             if (jl > a.F - 1) jl = a.F - 1;
             if (a.children) jl = it.x % a.F;
             rowbit[h] = valid ? (1ull << jl) : 0ull;
-            rdel[h] = (valid && a.any_deleted) ? a.row_del[row] : kNever;
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + (valid ? row : (int64_t)pos) * 64);
+            any |= rowbit[h];
+            const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + row * 64);
 #pragma unroll
             for (int v = 0; v < kWords / 4; ++v) {
                 const uint4 x = src[v];
@@ -125,10 +126,9 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
                 rw[h][4 * v + 3] = x.w;
             }
         }
-        // the leaves of the warp's rows: a query that kept none of them is passed over
-        const uint64_t both = rowbit[0] | rowbit[1];
-        const uint64_t wmask = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)both) |
-                               ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(both >> 32)) << 32);
+        // the leaves of the block's rows: a query that kept none of them is passed over
+        const uint64_t wmask = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)any) |
+                               ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(any >> 32)) << 32);
         for (int c = 0; c < nchunk; ++c) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();   // chunk c has landed; the other buffer is no longer read
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
             }
             const int cnt = min(NQS, total - c * NQS);
             const TileRec *rec = sRec[c & 1];
-            const int j0 = group * kPer;
+            const int j0 = warp * kPer;
             const int nj = max(0, min(kPer, cnt - j0));
             // lane i < nj: query j0 + i's limit (keep iff L1 <= 6 t, whole
             // numbers; an unbounded t keeps all) and whether the warp's rows
@@ -151,41 +151,39 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
                 live = (rec[j0 + lane].mask & wmask) != 0;
             }
             const unsigned lives = __ballot_sync(0xffffffffu, live);
-            uint32_t p0 = 0, p1 = 0;   // bit nj - 1 - i: rows r0, r0 + 32 pass query j0 + i
-#pragma unroll 2
+            uint32_t pass = 0;   // bit 8 h + nj - 1 - i: row lane + 32 h passes query j0 + i
             for (int i = 0; i < nj; ++i) {
-                uint32_t l0 = 0, l1 = 0;
+                uint32_t l[kRPL] = {0u, 0u, 0u, 0u};
                 if ((lives >> i) & 1u) {   // warp-uniform
-                    l0 = l1 = (uint32_t)__shfl_sync(0xffffffffu, start, i);
+                    const uint32_t s0 = (uint32_t)__shfl_sync(0xffffffffu, start, i);
+#pragma unroll
+                    for (int h = 0; h < kRPL; ++h) l[h] = s0;
                     const uint4 *qv = sQ[c & 1][j0 + i];
 #pragma unroll
                     for (int v = 0; v < kWords / 4; ++v) {
                         const uint4 x = qv[v];
-                        l0 = __vsadu4(rw[0][4 * v], x.x) + l0;
-                        l1 = __vsadu4(rw[1][4 * v], x.x) + l1;
-                        l0 = __vsadu4(rw[0][4 * v + 1], x.y) + l0;
-                        l1 = __vsadu4(rw[1][4 * v + 1], x.y) + l1;
-                        l0 = __vsadu4(rw[0][4 * v + 2], x.z) + l0;
-                        l1 = __vsadu4(rw[1][4 * v + 2], x.z) + l1;
-                        l0 = __vsadu4(rw[0][4 * v + 3], x.w) + l0;
-                        l1 = __vsadu4(rw[1][4 * v + 3], x.w) + l1;
+#pragma unroll
+                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v], x.x) + l[h];
+#pragma unroll
+                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 1], x.y) + l[h];
+#pragma unroll
+                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 2], x.z) + l[h];
+#pragma unroll
+                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 3], x.w) + l[h];
                     }
                 }
-                p0 = __funnelshift_l(l0, p0, 1);
-                p1 = __funnelshift_l(l1, p1, 1);
+                // (nj <= 8: a row's bits stay inside its byte)
+                pass = (pass << 1) | (l[0] >> 31) | ((l[1] >> 31) << 8) | ((l[2] >> 31) << 16) | ((l[3] >> 31) << 24);
             }
-            if (__any_sync(0xffffffffu, (p0 | p1) != 0)) {
-                for (uint32_t left = p0; left; left &= left - 1) {   // leaf and visibility of the passing pairs
-                    const int b = __ffs(left) - 1;
-                    const TileRec &rc = rec[j0 + nj - 1 - b];
-                    if (!(rc.mask & rowbit[0]) || rdel[0] <= rc.seq) p0 &= ~(1u << b);
+            if (__any_sync(0xffffffffu, pass != 0)) {
+                for (uint32_t left = pass; left; left &= left - 1) {   // leaf and visibility of the passing pairs
+                    const int b = __ffs(left) - 1, h = b >> 3;
+                    const TileRec &rc = rec[j0 + nj - 1 - (b & 7)];
+                    const uint64_t rbit = h == 0 ? rowbit[0] : h == 1 ? rowbit[1] : h == 2 ? rowbit[2] : rowbit[3];
+                    if (!(rc.mask & rbit) || (a.any_deleted && a.row_del[(int64_t)pos + rb + lane + 32 * h] <= rc.seq))
+                        pass &= ~(1u << b);
                 }
-                for (uint32_t left = p1; left; left &= left - 1) {
-                    const int b = __ffs(left) - 1;
-                    const TileRec &rc = rec[j0 + nj - 1 - b];
-                    if (!(rc.mask & rowbit[1]) || rdel[1] <= rc.seq) p1 &= ~(1u << b);
-                }
-                const int np = __popc(p0) + __popc(p1);
+                const int np = __popc(pass);
                 int incl = np;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -198,14 +196,12 @@ __global__ void __launch_bounds__(kThreadsS) k_tile_qgram(StrArgs a) {
                     if (lane == 31) base = atomicAdd(a.out_count, (unsigned long long)wtot);
                     base = __shfl_sync(0xffffffffu, base, 31);
                     unsigned long long o = base + (unsigned long long)(incl - np);
-                    while (p0 | p1) {
-                        const bool h0 = p0 != 0;
-                        const int b = __ffs(h0 ? p0 : p1) - 1;
-                        if (h0) p0 &= p0 - 1;
-                        else p1 &= p1 - 1;
+                    while (pass) {
+                        const int b = __ffs(pass) - 1;
+                        pass &= pass - 1;
                         if ((int64_t)o < a.cap) {
-                            a.out_q[o] = rec[j0 + nj - 1 - b].q;
-                            a.out_row[o] = pos + rb + r0 + (h0 ? 0 : 32);
+                            a.out_q[o] = rec[j0 + nj - 1 - (b & 7)].q;
+                            a.out_row[o] = pos + rb + lane + 32 * (b >> 3);
                         }
                         ++o;
                     }
@@ -264,6 +260,7 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
         const uint64_t rowbit = valid ? (1ull << jl) : 0ull;
         const int64_t rdel = (valid && a.any_deleted) ? a.row_del[row] : kNever;
         const int len = (int)(A.Soff[row + 1] - A.Soff[row]);
+        const int wlen = __reduce_max_sync(0xffffffffu, len);   // the warp's longest row
         uint32_t tw[kShortStr / 4], rw[kWords];
         {
             TextWords tr(A.S + A.Soff[row], len);
@@ -327,15 +324,19 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
                     uint32_t Pv = ~0u, Mv = 0u;
                     const uint32_t *peq = sPeq[j];
 #pragma unroll
-                    for (int i = 0; i < kShortStr; ++i) {
-                        if (i < len) {
-                            const uint32_t Eq = peq[(tw[i / 4] >> (8 * (i % 4))) & 255u];
-                            const uint32_t Xh = (((Eq & Pv) + Pv) ^ Pv) | Eq;
-                            const uint32_t Ph = ((Mv | ~(Xh | Pv)) << 1) | 1u;
-                            const uint32_t Mh = (Pv & Xh) << 1;
-                            const uint32_t Xv = Eq | Mv;
-                            Pv = Mh | ~(Xv | Ph);
-                            Mv = Ph & Xv;
+                    for (int v = 0; v < kShortStr / 4; ++v) {
+                        if (4 * v >= wlen) break;
+#pragma unroll
+                        for (int i = 4 * v; i < 4 * v + 4; ++i) {
+                            if (i < len) {
+                                const uint32_t Eq = peq[(tw[v] >> (8 * (i % 4))) & 255u];
+                                const uint32_t Xh = (((Eq & Pv) + Pv) ^ Pv) | Eq;
+                                const uint32_t Ph = ((Mv | ~(Xh | Pv)) << 1) | 1u;
+                                const uint32_t Mh = (Pv & Xh) << 1;
+                                const uint32_t Xv = Eq | Mv;
+                                Pv = Mh | ~(Xv | Ph);
+                                Mv = Ph & Xv;
+                            }
                         }
                     }
                     const uint32_t rows = mq >= 32 ? ~0u : (1u << mq) - 1u;
