@@ -1426,7 +1426,7 @@ __global__ void k_verify_str(Dev d, const int32_t *__restrict__ cq, const int32_
 // distance from above again -- the k-th smallest of them, from a count per
 // (query, distance) -- and only those within it go on to the sort by query and
 // the merge (words, k = 5: 2,100 kept per query, a few dozen within the bound;
-// 10^3 queries of 10^5 words 2.00 -> 1.50 ms with the short rows' early end in
+// 999 queries, 5 10^4 words: 2.00 -> 1.50 ms with the short rows' early end in
 // k_tile_short).
 __global__ void k_edit_hist(const int32_t *__restrict__ cq, const float *__restrict__ cdist,
                             const uint8_t *__restrict__ keep, int64_t C, int D, uint32_t *__restrict__ hist) {
@@ -2281,6 +2281,11 @@ __global__ void k_range_pack(const int32_t *__restrict__ cq, const int32_t *__re
 __global__ void k_iota_i32(int32_t *a, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         a[i] = (int32_t)i;
+}
+
+__global__ void k_invert(const int32_t *__restrict__ perm, int64_t n, int32_t *__restrict__ inv) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        inv[perm[i]] = (int32_t)i;
 }
 
 __global__ void k_u8_to_i64(const uint8_t *a, int64_t n, int64_t *b) {
@@ -3420,6 +3425,25 @@ struct Runner {
         return E >= kF32TileEntries * nn && E * ((ix->tree.n + nn - 1) / nn) >= least_pairs;
     }
 
+    // pos_of[q]: the place of query q in the order of the probe keys
+    void region_order(DBuf<int32_t> &pos_of) {
+        const int64_t nq = qb.nq;
+        DBuf<int32_t> idx(nq, st), key2(nq, st), perm(nq, st);
+        pos_of.alloc(nq, st);
+        int kbits = 1;
+        while (kbits < 31 && ((int64_t)1 << kbits) < ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]) ++kbits;
+        size_t tb = 0;
+        cub::DeviceRadixSort::SortPairs(nullptr, tb, qkey.get(), key2.get(), idx.get(), perm.get(), nq, 0, kbits, st);
+        DBuf<uint8_t> tmp(tb > 0 ? tb : 1, st);
+        clk.begin(GTS_STAGE_OTHER, 3);
+        k_iota_i32<<<nblocks(nq, kT), kT, 0, st>>>(idx.get(), nq);
+        GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, qkey.get(), key2.get(), idx.get(), perm.get(), nq, 0,
+                                                 kbits, st));
+        k_invert<<<nblocks(nq, kT), kT, 0, st>>>(perm.get(), nq, pos_of.get());
+        clk.end();
+        check_launch("region order");
+    }
+
     // Last level on the FP32 L2 tiles: regroup the entries by node, run the
     // tiles (leaf mask, visibility and the FP32 distance bound), then verify
     // the kept pairs as the plain path does.
@@ -3436,6 +3460,13 @@ struct Runner {
         tq.thr = thr.get();
         tq.epsc = d.epsc;
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
+        // kNN: a node's queries in the order of the regions their probes ended
+        // in, so that a warp's queries keep much the same leaves of it
+        DBuf<int32_t> pos_of;
+        if (knn && qkey_ok && qb.nq > 32) {
+            region_order(pos_of);
+            tq.pos_of = pos_of.get();
+        }
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
         tc_regroup(ix->tree, tq, rg, st, ncount ? ncount->get() : nullptr);

@@ -762,10 +762,11 @@ __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__
 // so entries of a node land in ascending query order with no contended
 // atomics (each 32-bit word collects at most 32 entries).
 __global__ void k_bits_set(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
-                           const uint64_t *__restrict__ emask, int64_t E, int64_t nw, uint32_t *__restrict__ bits) {
+                           const uint64_t *__restrict__ emask, int64_t E, int64_t nw, uint32_t *__restrict__ bits,
+                           const int32_t *__restrict__ pos_of) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
         if (!emask[e]) continue;
-        const int32_t q = eq[e];
+        const int32_t q = pos_of ? pos_of[eq[e]] : eq[e];
         atomicOr(&bits[(int64_t)enode[e] * nw + (q >> 5)], 1u << (q & 31));
     }
 }
@@ -827,10 +828,11 @@ __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_
                                     int stride, int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2,
                                     float cE1, float cE2, const int64_t *__restrict__ qseq,
                                     const int64_t *__restrict__ noff, const uint32_t *__restrict__ bits, const int32_t *__restrict__ wpre, int64_t nw,
-                                    TileRec *__restrict__ grec, int32_t *__restrict__ gq, float *__restrict__ gpath) {
+                                    TileRec *__restrict__ grec, int32_t *__restrict__ gq, float *__restrict__ gpath,
+                                    const int32_t *__restrict__ pos_of) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
         if (!emask[e]) continue;
-        const int32_t q = eq[e];
+        const int32_t q = pos_of ? pos_of[eq[e]] : eq[e];
         const int64_t wi = (int64_t)enode[e] * nw + (q >> 5);
         const int64_t o = noff[enode[e]] + wpre[wi] + __popc(bits[wi] & ((1u << (q & 31)) - 1u));
         write_rec(e, o, eq, emask, path, h, hp, stride, thr, qn2, cE1, cE2, qseq, grec, gq, gpath);
@@ -1005,7 +1007,8 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
     DBuf<int32_t> cursor(use_bits ? 0 : nn, st);
     if (use_bits) {
         GTS_CUDA(cudaMemsetAsync(bits.get(), 0, nn * nw * 4, st));
-        k_bits_set<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, E, nw, bits.get());
+        k_bits_set<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, E, nw, bits.get(),
+                                            tq.pos_of);
         k_bits_rows<<<(unsigned)std::min<int64_t>(nn, 65535), 256, 0, st>>>(bits.get(), nn, nw, wpre.get(), own.get());
     } else {
         GTS_CUDA(cudaMemsetAsync(cursor.get(), 0, nn * 4, st));
@@ -1031,7 +1034,7 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
     if (use_bits)
         k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
                                                      tq.cE1, tq.cE2, tq.qseq, noff.get(), bits.get(), wpre.get(), nw, rg.grec.get(),
-                                                     rg.gq.get(), rg.gpath.get());
+                                                     rg.gq.get(), rg.gpath.get(), tq.pos_of);
     else
         k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
                                                 tq.cE1, tq.cE2, tq.qseq, noff.get(), cursor.get(), rg.grec.get(), rg.gq.get(),

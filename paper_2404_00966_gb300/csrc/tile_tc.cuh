@@ -79,6 +79,8 @@ struct TcQuery {
     // the entries' level is h - 1, their masks name the nodes' children at
     // level h, and `path` holds path_stride floats per entry (0: the tree's h)
     int h = 0, path_stride = 0;
+    // order of a node's records: by pos_of[query] (null: by query; the bitmap form only)
+    const int32_t *pos_of = nullptr;
     const float *Q = nullptr;
     const int64_t *qseq = nullptr;
     const float *thr = nullptr;
