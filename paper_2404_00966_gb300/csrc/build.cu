@@ -47,9 +47,43 @@ int tree_height(int64_t n, int F, int n_pivots) {
     return h < kMaxHeight ? h : kMaxHeight;
 }
 
+// thread per node of the pivot levels
+__global__ static void k_order_children(const int32_t *__restrict__ nsize, const float *__restrict__ nlo,
+                                        const float *__restrict__ nhi, int64_t nodes, int F, int8_t *__restrict__ nord) {
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (g >= nodes) return;
+    // (Eq. 1 over all levels in one array: the children of node g are nodes g F + 1 ..)
+    const int64_t c0 = g * F + 1;
+    int j0 = -1;
+    bool ok = true;
+    float lo = 0.f, hi = 0.f;
+    for (int j = 0; j < F; ++j) {
+        const bool ne = nsize[c0 + j] > 0;
+        if (!ne) {
+            if (j0 >= 0) ok = false;
+            continue;
+        }
+        const float l = nlo[c0 + j], h = nhi[c0 + j];
+        if (!(l >= lo && h >= hi && h >= l)) ok = false;   // (from 0 on: distances)
+        lo = l;
+        hi = h;
+        if (j0 < 0) j0 = j;
+    }
+    nord[g] = ok ? (int8_t)j0 : (int8_t)-1;
+}
+
+void order_children(Tree &t, cudaStream_t st) {
+    const int64_t nodes = t.lvl_off[t.h];
+    t.nord.alloc(nodes > 0 ? nodes : 1, st);
+    if (nodes > 0)
+        k_order_children<<<(unsigned)((nodes + 255) / 256), 256, 0, st>>>(t.nsize.get(), t.nlo.get(), t.nhi.get(), nodes,
+                                                                         t.F, t.nord.get());
+    check_launch("order of the children");
+}
+
 size_t Tree::device_bytes() const {
     return X.bytes() + S.bytes() + Soff.bytes() + row_id.bytes() + table.bytes() + row_del.bytes() + npos.bytes() +
-           nsize.bytes() + npiv.bytes() + nlo.bytes() + nhi.bytes() + tc.Xh.bytes() + tc.Xl.bytes() + tc.xn2.bytes() +
+           nsize.bytes() + npiv.bytes() + nlo.bytes() + nhi.bytes() + nord.bytes() + tc.Xh.bytes() + tc.Xl.bytes() + tc.xn2.bytes() +
            qg.bytes();
 }
 
@@ -528,6 +562,7 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
         k_next_pos_node<<<blocks_for(n), kThreads, 0, st>>>(pos_node.get(), n, lpos, lsize, F);
         check_launch("partitioning");
     }
+    order_children(t, st);
     // final gather into leaf order
     k_gather_meta<<<blocks_for(n), kThreads, 0, st>>>(perm.get(), n, h, T.get(), d_ids, t.table.get(),
                                                       t.row_id.get(), inv.get());

@@ -276,6 +276,10 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
         expect(r.dev(t.npiv, 1, st), nodes, "pivots");
         expect(r.dev(t.nlo, 1, st), nodes, "node bounds");
         expect(r.dev(t.nhi, 1, st), nodes, "node bounds");
+        if (t.n > 0) {
+            order_children(t, st);
+            GTS_CUDA(cudaStreamSynchronize(st));
+        }
         t.persist();
         Cache &c = ix->cache;
         c.count = r.pod<int64_t>();
