@@ -71,12 +71,40 @@ constexpr float kAbsFloor = 1e-17f;
 
 // The exact operation order of the CPU reference: increasing i, every
 // subtraction, product and sum rounded on its own (no fused multiply-add).
+// Rows on 16-byte boundaries are read 32 coordinates at a time (eight 16-byte
+// loads of each in flight; with a coordinate's loads at a time the sums waited
+// for memory: 130,000 keys of 128 coordinates 0.229 -> 0.193 ms), the sums keep
+// their order.
+template <class Term>
+__device__ __forceinline__ void fp64_terms(const float *q, const float *x, int dim, Term term) {
+    int i = 0;
+    if ((dim & 3) == 0 && ((((uintptr_t)q) | ((uintptr_t)x)) & 15) == 0) {
+        const float4 *q4 = reinterpret_cast<const float4 *>(q), *x4 = reinterpret_cast<const float4 *>(x);
+        for (; i + 32 <= dim; i += 32) {
+            float4 a[8], b[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                a[u] = __ldg(q4 + (i >> 2) + u);
+                b[u] = __ldg(x4 + (i >> 2) + u);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                term(a[u].x, b[u].x);
+                term(a[u].y, b[u].y);
+                term(a[u].z, b[u].z);
+                term(a[u].w, b[u].w);
+            }
+        }
+    }
+    for (; i < dim; ++i) term(q[i], x[i]);
+}
+
 __device__ __forceinline__ double l2sq_fp64_seq(const float *q, const float *x, int dim) {
     double s = 0.0;
-    for (int i = 0; i < dim; ++i) {
-        double t = __dsub_rn((double)q[i], (double)x[i]);
+    fp64_terms(q, x, dim, [&](float a, float b) {
+        const double t = __dsub_rn((double)a, (double)b);
         s = __dadd_rn(s, __dmul_rn(t, t));
-    }
+    });
     return s;
 }
 
@@ -86,12 +114,12 @@ __device__ __forceinline__ double l2sq_fp64_seq(const float *q, const float *x, 
 // order.
 __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *x, int dim) {
     double dot = 0.0, nq = 0.0, nx = 0.0;
-    for (int i = 0; i < dim; ++i) {
-        const double a = (double)q[i], b = (double)x[i];
+    fp64_terms(q, x, dim, [&](float fa, float fb) {
+        const double a = (double)fa, b = (double)fb;
         dot = __dadd_rn(dot, __dmul_rn(a, b));
         nq = __dadd_rn(nq, __dmul_rn(a, a));
         nx = __dadd_rn(nx, __dmul_rn(b, b));
-    }
+    });
     double c = __ddiv_rn(dot, __dmul_rn(__dsqrt_rn(nq), __dsqrt_rn(nx)));
     c = c > 1.0 ? 1.0 : (c < -1.0 ? -1.0 : c);
     return __dsub_rn(1.0, c);
@@ -99,7 +127,8 @@ __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *
 
 __device__ __forceinline__ double l1_fp64_seq(const float *q, const float *x, int dim) {
     double s = 0.0;
-    for (int i = 0; i < dim; ++i) s = __dadd_rn(s, fabs(__dsub_rn((double)q[i], (double)x[i])));
+    fp64_terms(q, x, dim,
+               [&](float a, float b) { s = __dadd_rn(s, fabs(__dsub_rn((double)a, (double)b))); });
     return s;
 }
 
