@@ -1330,6 +1330,145 @@ __global__ void k_compact_cands(const int32_t *__restrict__ cq, const int32_t *_
     }
 }
 
+// ---------------------------------------------------------------- small batches
+//
+// A few queries cannot fill the device on the way down the tree: the descent
+// is some thirty short launches with a host round trip per level (one query
+// of 10^5 x 128: 0.53 ms, of which the kernels take 0.24), while reading every
+// object once takes 8 us.  So for up to kSmallQueries FP32 queries whose
+// objects are read within a budget of bytes, every row's FP32 distance is
+// computed in one pass, four queries at a time, and only the rows that can be
+// answers go on -- range: within the radius by the error bound; kNN: within
+// the k-th smallest of the warps' nearest rows, an upper bound of the k-th
+// distance -- to the same verification, FP64 keys and selection as any
+// candidate.  G lanes take a row (eight, reading its 128-byte segments
+// together; one for rows of at most 16 coordinates); HBM bounds it.
+constexpr int64_t kSmallQueries = 8;
+// Objects read, over all passes of four queries, and distances; a quarter of
+// it for rows of up to 16 coordinates, whose 32 lanes have a row each and whose
+// trees prune better.  Descent / scan, us: 10^5 x 128, one query 477 / 270, 8:
+// 666 / 311; 10^6 x 128, one (0.5 GB) 698 / 475, 8 (1.06 GB) 1085 / 746; 10^7 x
+// 2, range, one (0.12 GB) 389 / 288, 8 (0.48 GB) 391 / 397, kNN, 8: 622 / 644.
+constexpr int64_t kSmallBytes = (int64_t)1 << 30;
+constexpr int kSmallQ = 4;                          // queries per pass
+
+template <bool L2, int G, bool V4, bool KNN>
+__global__ void __launch_bounds__(256) k_scan_small(Dev d, int64_t nq, const float *__restrict__ thr_q,
+                                                    float *__restrict__ d32, float *__restrict__ slots, int nslots,
+                                                    int32_t *__restrict__ oq, int32_t *__restrict__ orow, int64_t cap,
+                                                    unsigned long long *__restrict__ count) {
+    constexpr int R = 32 / G;
+    const int lane = threadIdx.x & 31, g = lane / G, s = lane % G;
+    const int64_t q0 = (int64_t)blockIdx.y * kSmallQ;
+    const int m = (int)(nq - q0 < kSmallQ ? nq - q0 : kSmallQ);
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    float best[kSmallQ], thr[kSmallQ];
+    int64_t seq[kSmallQ];
+#pragma unroll
+    for (int j = 0; j < kSmallQ; ++j) {
+        best[j] = __int_as_float(0x7f800000);
+        thr[j] = j < m ? thr_q[q0 + j] : 0.f;
+        seq[j] = j < m ? d.qseq[q0 + j] : 0;
+    }
+    for (int64_t r0 = w * R; r0 < d.n; r0 += nw * R) {   // (warp-uniform)
+        const int64_t row = r0 + g;
+        float sum[kSmallQ] = {0.f, 0.f, 0.f, 0.f};
+        if (row < d.n) {
+            const float *xv = d.X + row * d.dim;
+            if (V4) {
+                const float4 *x4 = reinterpret_cast<const float4 *>(xv);
+#pragma unroll 4
+                for (int c = s; c < (d.dim >> 2); c += G) {
+                    const float4 x = __ldg(x4 + c);
+#pragma unroll
+                    for (int j = 0; j < kSmallQ; ++j) {
+                        if (j < m) {
+                            const float4 a = __ldg(reinterpret_cast<const float4 *>(d.Q + (q0 + j) * d.dim) + c);
+                            const float e0 = a.x - x.x, e1 = a.y - x.y, e2 = a.z - x.z, e3 = a.w - x.w;
+                            sum[j] += L2 ? e0 * e0 + e1 * e1 + e2 * e2 + e3 * e3
+                                         : fabsf(e0) + fabsf(e1) + fabsf(e2) + fabsf(e3);
+                        }
+                    }
+                }
+            } else {
+#pragma unroll 4
+                for (int c = s; c < d.dim; c += G) {
+                    const float x = __ldg(xv + c);
+#pragma unroll
+                    for (int j = 0; j < kSmallQ; ++j) {
+                        if (j < m) {
+                            const float t = __ldg(d.Q + (q0 + j) * d.dim + c) - x;
+                            sum[j] += L2 ? t * t : fabsf(t);
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int j = 0; j < kSmallQ; ++j) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+        const int64_t del = row < d.n && s == 0 ? d.row_del[row] : 0;
+#pragma unroll
+        for (int j = 0; j < kSmallQ; ++j) {
+            if (j >= m) break;
+            const float dist = L2 ? sqrtf(sum[j]) : sum[j];
+            const bool vis = row < d.n && s == 0 && del > seq[j];
+            if (KNN) {
+                if (row < d.n && s == 0) d32[(q0 + j) * d.n + row] = vis ? dist : -1.f;
+                if (vis) best[j] = fminf(best[j], dist);
+            } else {
+                const bool keep = vis && !(dist * (1.f - 2.f * d.rel) - d.absf > thr[j]);
+                const unsigned b = __ballot_sync(0xffffffffu, keep);
+                if (b) {
+                    unsigned long long base = 0;
+                    if (lane == 0) base = atomicAdd(count, (unsigned long long)__popc(b));
+                    base = __shfl_sync(0xffffffffu, base, 0) + __popc(b & ((1u << lane) - 1u));
+                    if (keep && (int64_t)base < cap) {
+                        oq[base] = (int32_t)(q0 + j);
+                        orow[base] = (int32_t)row;
+                    }
+                }
+            }
+        }
+    }
+    if (KNN) {
+#pragma unroll
+        for (int j = 0; j < kSmallQ; ++j) {
+            if (j >= m) break;
+            float v = best[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (lane == 0) slots[(q0 + j) * nslots + w] = v;
+        }
+    }
+}
+
+// kNN rows that can be answers: lower bound within tau (-1: not visible)
+__global__ void k_small_emit(const float *__restrict__ d32, int64_t n, const float *__restrict__ thr_q, float rel,
+                             float absf, int32_t *__restrict__ oq, int32_t *__restrict__ orow, float *__restrict__ od,
+                             int64_t cap, unsigned long long *__restrict__ count) {
+    const int lane = threadIdx.x & 31;
+    const int64_t q = blockIdx.y, step = (int64_t)gridDim.x * blockDim.x;
+    const float thr = thr_q[q];
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += step) {
+        const int64_t i = i0 + lane;
+        const float v = i < n ? d32[q * n + i] : -1.f;
+        const bool keep = v != -1.f && !(v * (1.f - 2.f * rel) - absf > thr);
+        const unsigned b = __ballot_sync(0xffffffffu, keep);
+        if (!b) continue;
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(count, (unsigned long long)__popc(b));
+        base = __shfl_sync(0xffffffffu, base, 0) + __popc(b & ((1u << lane) - 1u));
+        if (keep && (int64_t)base < cap) {
+            oq[base] = (int32_t)q;
+            orow[base] = (int32_t)i;
+            od[base] = v;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- q-gram count filter
 //
 // A lower bound for edit distance from the counts of the strings' 3-grams
@@ -1587,6 +1726,25 @@ __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t *red) {
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
     __syncthreads();
     return t;
+}
+
+// tau_q from the warps' nearest rows (k_scan_small): the k-th smallest of them
+// belongs to k distinct visible rows.  A block per query.
+__global__ void __launch_bounds__(256) k_small_tau(const float *__restrict__ slots, int nslots,
+                                                   const int32_t *__restrict__ kq, float rel, float absf,
+                                                   float *__restrict__ thr) {
+    __shared__ unsigned hist[256];
+    __shared__ int64_t sh[4];
+    const int64_t q = blockIdx.x;
+    const int K = kq[q];
+    if (K > nslots) return;   // (tau stays as it was)
+    const float *v = slots + q * nslots;
+    const uint32_t u = (uint32_t)block_select8<32>(
+        nslots, K, [&](int64_t i, uint64_t &x) -> bool { x = __float_as_uint(v[i]); return true; }, hist, sh);
+    if (threadIdx.x == 0) {
+        const float t = __fadd_ru(__fmul_ru(__uint_as_float(u), 1.f + 2.f * rel), absf);
+        if (t < thr[q]) thr[q] = t;
+    }
 }
 
 // One block per query.  Merges this group's candidates into the query's
@@ -3775,6 +3933,90 @@ struct Runner {
         }
     }
 
+    // Small FP32 batches: every row in one pass per four queries (k_scan_small)
+    static bool small_batch(const Tree &t, int64_t nq) {
+        return t.dim > 0 && t.n > 0 && t.n < ((int64_t)1 << 31) && nq >= 1 && nq <= kSmallQueries &&
+               t.n <= kSmallBytes / (t.dim <= kScanMaxDim ? 16 : 4) /
+                          ((int64_t)t.dim * ((nq + kSmallQ - 1) / kSmallQ) + nq);
+    }
+
+    template <bool L2, bool KNN>
+    void launch_scan_small(dim3 grid, const float *d32, float *slots, int nslots, int32_t *oq, int32_t *orow,
+                           int64_t cap_, unsigned long long *count) {
+        const bool v4 = (d.dim & 3) == 0 && (((uintptr_t)d.Q | (uintptr_t)d.X) & 15) == 0;
+        float *dd = const_cast<float *>(d32);
+        if (d.dim <= kScanMaxDim)
+            k_scan_small<L2, 1, false, KNN><<<grid, kT, 0, st>>>(d, qb.nq, thr.get(), dd, slots, nslots, oq, orow, cap_,
+                                                                count);
+        else if (v4)
+            k_scan_small<L2, 8, true, KNN><<<grid, kT, 0, st>>>(d, qb.nq, thr.get(), dd, slots, nslots, oq, orow, cap_,
+                                                               count);
+        else
+            k_scan_small<L2, 8, false, KNN><<<grid, kT, 0, st>>>(d, qb.nq, thr.get(), dd, slots, nslots, oq, orow, cap_,
+                                                                count);
+    }
+
+    void scan_all() {
+        const int64_t n = ix->tree.n, nq = qb.nq;
+        const int rows_warp = d.dim <= kScanMaxDim ? 32 : 4;
+        const int64_t passes = (nq + kSmallQ - 1) / kSmallQ;
+        // at least four steps a warp, at most 48 warps an SM
+        const int64_t blocks = std::max<int64_t>(
+            1, std::min<int64_t>((n + 4 * 8 * rows_warp - 1) / (4 * 8 * rows_warp), (int64_t)(max_blocks / 8) * 6));
+        const dim3 grid((unsigned)blocks, (unsigned)passes);
+        const int nslots = (int)(blocks * (kT / 32));
+        DBuf<unsigned long long> count(1, st);
+        DBuf<float> d32(knn ? nq * n : 1, st), slots(knn ? nq * nslots : 1, st);
+        st_scan_rows += n * passes;
+        int64_t room = std::max<int64_t>(1 << 18, 2 * ix->small_pairs_hint[knn ? 1 : 0].load());
+        DBuf<int32_t> oq, orow;
+        DBuf<float> od;
+        int64_t C = 0;
+        for (int attempt = 0; attempt < 2; ++attempt) {
+            oq.alloc(room, st);
+            orow.alloc(room, st);
+            if (knn) od.alloc(room, st);
+            GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
+            clk.begin(GTS_STAGE_LEAF_SCAN, knn ? 3 : 1);
+            if (!knn) {
+                if (d.metric == GTS_L2)
+                    launch_scan_small<true, false>(grid, d32.get(), slots.get(), nslots, oq.get(), orow.get(), room,
+                                                   count.get());
+                else
+                    launch_scan_small<false, false>(grid, d32.get(), slots.get(), nslots, oq.get(), orow.get(), room,
+                                                    count.get());
+            } else {
+                if (attempt == 0) {
+                    if (d.metric == GTS_L2)
+                        launch_scan_small<true, true>(grid, d32.get(), slots.get(), nslots, nullptr, nullptr, 0, nullptr);
+                    else
+                        launch_scan_small<false, true>(grid, d32.get(), slots.get(), nslots, nullptr, nullptr, 0,
+                                                       nullptr);
+                    k_small_tau<<<(unsigned)nq, 256, 0, st>>>(slots.get(), nslots, qb.k, d.rel, d.absf, thr.get());
+                }
+                const dim3 eg((unsigned)std::min<int64_t>(nblocks(n, kT), max_blocks), (unsigned)nq);
+                k_small_emit<<<eg, kT, 0, st>>>(d32.get(), n, thr.get(), d.rel, d.absf, oq.get(), orow.get(), od.get(),
+                                                room, count.get());
+            }
+            clk.end();
+            check_launch("small-batch scan");
+            C = d2h_i64(reinterpret_cast<const int64_t *>(count.get()), st);
+            if (C <= room) break;
+            room = C;   // rerun with room for every pair
+        }
+        GTS_REQUIRE(C <= room, GTS_ECUDA, "small-batch scan: output count changed between identical runs");
+        ix->small_pairs_hint[knn ? 1 : 0].store(C);
+        ++st_groups;
+        if (C == 0) return;
+        if (!knn) {
+            verify_and_collect(oq, orow, C, /*query_major=*/false);
+            return;
+        }
+        st_cands += C;
+        if (nq == 1) merge_knn(oq, orow, od, C);
+        else sort_and_merge(oq, orow, od, C);
+    }
+
     // the first entry of each query's run among entries [e0, e1) of a
     // query-sorted level (relative to e0), for the per-query threshold kernel
     DBuf<int64_t> qrun_buf;
@@ -4040,7 +4282,11 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         R.clk.end();
     }
     check_launch("query setup");
-    if (knn && t.n > 0 && nq > 0 && t.dim > 0) {
+    // (the diagnostic count needs the plain scan's candidates)
+    const bool small = precision == GTS_PREC_FP32 && budget >= kF32TileBudget && !qb.count_table_pass &&
+                       Runner::small_batch(t, nq);
+    if (small) R.scan_all();
+    if (!small && knn && t.n > 0 && nq > 0 && t.dim > 0) {
         LevelOffsets lo_off;
         for (int l = 0; l <= t.h && l < kMaxHeight + 2; ++l) lo_off.v[l] = t.lvl_off[l];
         const int cap = R.tu.probe_rows;
@@ -4071,7 +4317,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         check_launch("knn probe");
         R.st_pivots += nq * (int64_t)t.h;
     }
-    if (t.n > 0 && nq > 0) {
+    if (!small && t.n > 0 && nq > 0) {
         Level L0;
         L0.E = nq;
         L0.q.alloc(nq, st);
