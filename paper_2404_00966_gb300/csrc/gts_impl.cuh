@@ -269,7 +269,8 @@ struct gts_index {
     std::mutex tune_mu;
     std::mutex prep_mu;   // lazily built per-index data (BF16 split rows, 3-gram counts)
     gts::Tuning tuning;
-    std::atomic<int64_t> tc_pairs_hint[2] = {{0}, {0}}; // last tensor-core output size per query (x1024)
+    std::atomic<int64_t> tc_pairs_hint[3] = {{0}, {0}, {0}};   // tensor-core / string tiles: output size per query
+                                                              // (x1024), range, kNN, kNN phase 1
     std::atomic<int64_t> l1_pairs_hint[4] = {{0}, {0}, {0}, {0}};  // L1 tiles: range, kNN phases 0..2 (same unit)
     std::atomic<int64_t> f32_pairs_hint[2] = {{0}, {0}};   // FP32 L2 tiles: pairs per query (x1024), range / kNN
     std::atomic<int64_t> small_pairs_hint[2] = {{0}, {0}}; // small-batch scan: pairs of the last call, range / kNN

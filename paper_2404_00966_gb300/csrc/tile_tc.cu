@@ -301,7 +301,9 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
             int4 it = make_int4(0, 0, 0, 0);
             int32_t pos = 0, size = 0;
             if (!stop) {
-                it = a.items[item];
+                // phase 0: items 0, stride, 2 stride ..; phase 1: the others
+                it = a.items[a.stride == 1 ? item : a.phase == 0 ? item * a.stride
+                                                                 : item + item / (a.stride - 1) + 1];
                 const int64_t gnode = a.lvl_last + it.x;
                 pos = a.npos[gnode];
                 size = a.nsize[gnode];
@@ -336,9 +338,9 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                 const int64_t wi = (int64_t)c * (kNQ / 32) + (ptid >> 5);
                 const int64_t q = (int64_t)c * kNQ + ptid;
                 if (window && ptid < kNQ && wi < a.nw) w.word = a.bits[(int64_t)it.x * a.nw + wi];
+                if (window && ptid < kNQ && q < a.nq) w.ab = a.ab_q[q];
                 if (window && a.dmask && ptid < kNQ && q < a.nq) {
                     w.dmask = a.dmask[(int64_t)it.x * a.nq + q];
-                    w.ab = a.ab_q[q];
                     w.seq = a.seq_q[q];
                     if (a.qperm) w.qid = a.qperm[q];
                 }
@@ -397,8 +399,8 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                                 a.noff[it.x] + a.wpre[wi] + __popc(cur.word & ((1u << (ptid & 31)) - 1u));
                             const TileRec r = a.grec[o];
                             *mr = r;
-                            ab[(ptid >> 1) * 4 + (ptid & 1)] = r.alpha;
-                            ab[(ptid >> 1) * 4 + 2 + (ptid & 1)] = r.beta;
+                            ab[(ptid >> 1) * 4 + (ptid & 1)] = cur.ab.x;
+                            ab[(ptid >> 1) * 4 + 2 + (ptid & 1)] = cur.ab.y;
                             float *mp = mpath(sl) + ptid * a.hp;
                             for (int l = 0; l < a.hp; ++l) mp[l] = a.gpath[o * a.hp + l];
                         } else {
@@ -1140,10 +1142,13 @@ int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegro
 }
 
 int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-               DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st, DBuf<float> *out_qx) {
+               DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st, DBuf<float> *out_qx, int phase, int stride) {
     *launches = 0;
     if (rg.n_items == 0) return 0;
     const int h = rg.h ? rg.h : t.h;
+    const int64_t first = (rg.n_items + stride - 1) / stride;   // items of phase 0
+    const int64_t n_items = stride == 1 || phase == 0 ? first : rg.n_items - first;
+    if (n_items == 0) return 0;
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1175,7 +1180,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     if (regs_cta > 0 && per_sm > regs_sm / regs_cta) per_sm = regs_sm / regs_cta;
     if (per_sm > 1) per_sm = 1;   // TMEM: every CTA takes all 512 columns
     if (per_sm < 1) per_sm = 1;
-    const int64_t grid = std::min<int64_t>(rg.n_items, (int64_t)sms * per_sm);
+    const int64_t grid = std::min<int64_t>(n_items, (int64_t)sms * per_sm);
     // the batch's split query rows, for window-mode chunks (TMA, 128 rows)
     const CUtensorMap map_qh = make_panel_map(tq.Qh, tq.nq, c.dim_p, nq_chunk);
     const CUtensorMap map_ql = make_panel_map(tq.Ql, tq.nq, c.dim_p, nq_chunk);
@@ -1195,11 +1200,11 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         check_launch("window lists");
         ++*launches;
     }
-    // dense last level: the queries' bound constants and sequence numbers in
-    // column order, once per batch
-    DBuf<float2> abq(rg.dmask ? tq.nq : 1, st);
-    DBuf<int64_t> seqp(rg.dmask ? tq.nq : 1, st);
-    if (rg.dmask) {
+    // windows: the queries' bound constants and sequence numbers in column
+    // order, with the thresholds of this launch
+    DBuf<float2> abq(wl_on ? tq.nq : 1, st);
+    DBuf<int64_t> seqp(wl_on ? tq.nq : 1, st);
+    if (wl_on) {
         k_query_consts<<<nblk(tq.nq), 256, 0, st>>>(tq.thr, tq.qn2, tq.qseq, tq.perm, tq.nq, cE1, cE2, abq.get(),
                                                     seqp.get());
         check_launch("query bound constants");
@@ -1233,7 +1238,9 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.gpath = rg.gpath.get();
         a.hp = (h + 3) & ~3;
         a.items = rg.items.get();
-        a.n_items = rg.n_items;
+        a.n_items = n_items;
+        a.phase = phase;
+        a.stride = stride;
         a.work_counter = counter.get();
         a.out_q = out_q.get();
         a.out_row = out_row.get();

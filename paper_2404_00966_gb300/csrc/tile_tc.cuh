@@ -34,7 +34,8 @@ struct TileArgs {
     const float *gpath;       // their path distances [*, hp], hp = h rounded up to 4
     int hp;
     const int4 *items;        // (node, first, count, row block | kWindowItem) over the records
-    int64_t n_items;
+    int64_t n_items;          // of this launch: number i is item pick(i), see tc_run
+    int phase, stride;
     int *work_counter;
     int32_t *out_q, *out_row;
     float *out_qx;            // null, or each kept pair's q.x~ (d~^2 = |q|^2 + |x|^2 - 2 q.x~ is within E of d^2)
@@ -57,7 +58,7 @@ struct TileArgs {
     // dense last level: no records; column q of node p takes its leaf mask
     // from dmask[p * nq + q] and its query data from the per-query arrays
     const uint64_t *dmask;    // null: records
-    const float2 *ab_q;       // per position: the query's bound constants (alpha, beta)
+    const float2 *ab_q;       // window mode, per position: the query's bound constants (alpha, beta)
     const int32_t *qperm;     // position -> query (null: the same)
     const int64_t *seq_q;
 };
@@ -143,10 +144,12 @@ int64_t tc_regroup_children(const Tree &t, const TcQuery &tq, TcRegroup &rg, cud
 int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegroup &rg, cudaStream_t st);
 // run the tiles; returns the number of (query, row) pairs written to out_q/out_row
 // (and, given out_qx, each pair's q.x~: d~^2 = |q|^2 + |x|^2 - 2 q.x~ is within
-// tc_bound_coeffs' E of d^2)
+// tc_bound_coeffs' E of d^2).  stride > 1: phase 0 runs every stride-th item,
+// phase 1 the others, with the thresholds as they are at the call (window
+// chunks; gathered chunks keep their records').
 int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegroup &rg, DBuf<int32_t> &out_q,
                DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st,
-               DBuf<float> *out_qx = nullptr);
+               DBuf<float> *out_qx = nullptr, int phase = 0, int stride = 1);
 // Dense query-to-pivot distances of one pivot level on the tensor cores
 // (dim_p <= 256, after tc_prepare and tc_prepare_pivots): out[q, p] for the
 // batch's split queries; returns the level's absolute slack, an upper bound of
