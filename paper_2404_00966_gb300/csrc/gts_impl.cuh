@@ -218,6 +218,8 @@ struct Tree {
     TcCache tc;
     DBuf<uint8_t> qg;               // strings: hashed 3-gram counts per row [n, 64] (built on first use)
     bool qg_ready = false;
+    DBuf<uint8_t> qcode;            // their codes for the tensor-core tiles [n, 256] (built on first use)
+    bool qcode_ready = false;
     size_t device_bytes() const;
     void persist() {   // every buffer the index keeps
         X.persist(); Xr.persist(); S.persist(); Soff.persist(); row_id.persist(); table.persist(); row_del.persist();

@@ -3785,8 +3785,30 @@ struct Runner {
             collect(oq, orow, od, keep, C, /*query_major=*/false);
             return;
         }
+        const bool tensor = qtc_pays(ix->tree, qb.nq, rg);
+        DBuf<uint8_t> qcode;
+        if (tensor) {
+            clk.begin(GTS_STAGE_OTHER, 1);
+            Tree &t = ix->tree;
+            {
+                std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build them once
+                if (!t.qcode_ready) {
+                    Arena::Pause index_owned;
+                    t.qcode.alloc(t.n * 256, st);
+                    qtc_codes(d.qg, t.n, nullptr, t.qcode.get(), st);
+                    GTS_CUDA(cudaStreamSynchronize(st));
+                    t.qcode.persist();
+                    t.qcode_ready = true;
+                }
+            }
+            qcode.alloc(qb.nq * 256, st);
+            qtc_codes(d.qgq, qb.nq, thr.get(), qcode.get(), st);
+            clk.end();
+        }
         clk.begin(GTS_STAGE_TILE);
-        const int64_t C = qgram_run(ix->tree, sq, rg, oq, orow, hint, &nl, st);
+        const int64_t C = tensor ? qtc_run(ix->tree, sq, rg, qb.nq, ix->tree.qcode.get(), qcode.get(), oq, orow, hint,
+                                           &nl, st)
+                                 : qgram_run(ix->tree, sq, rg, oq, orow, hint, &nl, st);
         clk.end();
         if (rg.n_items > 0 && qb.nq > 0)
             ix->tc_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
@@ -3802,7 +3824,7 @@ struct Runner {
         GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, oq.get(), q2.get(), orow.get(), r2.get(), C, 0, qbits,
                                                  st));
         clk.end();
-        verify_and_collect(q2, r2, C, true, /*qgram_done=*/true);
+        verify_and_collect(q2, r2, C, true, /*qgram_done=*/!tensor);
     }
 
     // GTS_PREC_FP32: whether the last level's E entries run as FP32 tiles or

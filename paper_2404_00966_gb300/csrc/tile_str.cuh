@@ -37,4 +37,15 @@ int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const
 int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<int32_t> &out_q,
                   DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st);
 
+// The same bound on the tensor cores (tile_qtc.cu), with the counts capped at
+// 4: keeps every pair that qgram_run keeps and a few more.  256-byte codes of the
+// rows and of the batch's queries (thr: their thresholds; rows: null).
+constexpr int64_t kQtcRows = 1 << 24;    // rows whose codes are kept with the index (4 GiB)
+constexpr int64_t kQtcPairs = 32 << 20;  // least (entry, row) pairs
+bool qtc_pays(const Tree &t, int64_t nq, const TcRegroup &rg);
+void qtc_codes(const uint8_t *qg, int64_t n, const float *thr, uint8_t *code, cudaStream_t st);
+int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t nq, const uint8_t *xcode,
+                const uint8_t *qcode, DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, int64_t cap_hint, int *launches,
+                cudaStream_t st);
+
 }  // namespace gts

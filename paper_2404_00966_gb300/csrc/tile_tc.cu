@@ -116,6 +116,24 @@ CUtensorMap make_panel_map(const void *base, int64_t rows, int dim_p, int box_ro
     return m;
 }
 
+}  // namespace
+
+// Rows of 256 bytes as two 128-byte panels, the same way
+CUtensorMap tc_byte_map(const void *base, int64_t rows, int box_rows) {
+    CUtensorMap m;
+    cuuint64_t dims[3] = {128, (cuuint64_t)(rows > 0 ? rows : 1), 2};
+    cuuint64_t strides[2] = {256, 128};
+    cuuint32_t box[3] = {128, (cuuint32_t)box_rows, 2};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void *>(base), dims, strides, box, estr,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    GTS_REQUIRE(r == CUDA_SUCCESS, GTS_ECUDA, "cuTensorMapEncodeTiled (bytes) failed (" + std::to_string((int)r) + ")");
+    return m;
+}
+
+namespace {
+
 // ---------------------------------------------------------------- preparation
 
 // Split every float32 row into bf16 hi / lo parts (padded with zeros to

@@ -116,6 +116,9 @@ struct TcRegroup {
     int64_t n_pairs = 0;   // (query, row) pairs of all blocks: sum over nodes of entries x rows
 };
 
+// a TMA map of `rows` rows of 256 bytes, boxes of box_rows rows: the rows' first
+// 128 bytes, then their second, each in the 128-byte swizzle
+CUtensorMap tc_byte_map(const void *base, int64_t rows, int box_rows);
 bool tc_supported(const Tree &t);
 // |d~^2 - d^2| <= cE1 |q||x| + cE2 (|q| + |x|)^2 for the split-bf16 products over dim_p columns
 void tc_bound_coeffs(int dim_p, float &cE1, float &cE2);
