@@ -216,6 +216,8 @@ struct Tree {
     int max_len = 0;                // longest string
     int64_t n_deleted = 0;          // rows carrying a delete mark
     TcCache tc;
+    DBuf<double> xrn2;              // angular distance: the raw rows' sums of squares (built on first use)
+    bool xrn2_ready = false;
     DBuf<uint8_t> qg;               // strings: hashed 3-gram counts per row [n, 64] (built on first use)
     bool qg_ready = false;
     DBuf<uint8_t> qcode;            // their codes for the tensor-core tiles [n, 256] (built on first use)

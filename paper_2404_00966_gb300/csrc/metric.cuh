@@ -112,6 +112,16 @@ __device__ __forceinline__ double l2sq_fp64_seq(const float *q, const float *x, 
 // increasing i, every product and sum rounded on its own, c = dot /
 // (sqrt(|q|^2) sqrt(|x|^2)) clamped to [-1, 1] -- the reference operation
 // order.
+__device__ __forceinline__ double cos_key_fp64(double dot, double nq, double nx) {
+    double c = __ddiv_rn(dot, __dmul_rn(__dsqrt_rn(nq), __dsqrt_rn(nx)));
+    c = c > 1.0 ? 1.0 : (c < -1.0 ? -1.0 : c);
+    return __dsub_rn(1.0, c);
+}
+__device__ __forceinline__ double dot_fp64_seq(const float *q, const float *x, int dim) {
+    double dot = 0.0;
+    fp64_terms(q, x, dim, [&](float a, float b) { dot = __dadd_rn(dot, __dmul_rn((double)a, (double)b)); });
+    return dot;
+}
 __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *x, int dim) {
     double dot = 0.0, nq = 0.0, nx = 0.0;
     fp64_terms(q, x, dim, [&](float fa, float fb) {
@@ -120,9 +130,7 @@ __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *
         nq = __dadd_rn(nq, __dmul_rn(a, a));
         nx = __dadd_rn(nx, __dmul_rn(b, b));
     });
-    double c = __ddiv_rn(dot, __dmul_rn(__dsqrt_rn(nq), __dsqrt_rn(nx)));
-    c = c > 1.0 ? 1.0 : (c < -1.0 ? -1.0 : c);
-    return __dsub_rn(1.0, c);
+    return cos_key_fp64(dot, nq, nx);
 }
 
 __device__ __forceinline__ double l1_fp64_seq(const float *q, const float *x, int dim) {

@@ -46,6 +46,7 @@ constexpr int64_t kF32TileEntries = 4;           // FP32 tiles: least last-level
 constexpr int64_t kF32TilePairs = 6 << 20;       // and least (entry, row) pairs (f32_tiles_pay)
 constexpr int64_t kScanPairs = 16 << 20;         // table scan of low-dimensional vectors: least pairs
 constexpr int64_t kTilePhaseItems = 1216;        // tensor-core tile kNN: items from which they run in two phases
+constexpr int64_t kCosNorms = 64;                 // angular batches: queries from which their sums are formed first
 constexpr int64_t kF32DenseQueries = 64;         // dense pivot matrices in FP32: one full tile of queries
 constexpr int64_t kF32TileBudget = (int64_t)1 << 30;   // and least memory budget: the regrouped records take about
                                                        // 60 bytes per entry beside the budgeted tables
@@ -91,6 +92,7 @@ struct Dev {
     // keys come from the raw rows and queries
     int cosine;
     const float *Xr, *cXr, *Qr;
+    const double *xrn2, *qrn2;   // null, or the raw tree rows' and queries' sums of squares, as the keys sum them
     const double *coslim;   // range: 1 - cos(r) per query
 };
 
@@ -109,7 +111,12 @@ __device__ __forceinline__ const float *vrow_raw(const Dev &d, int64_t row) {
 // squared sum, L1 the sum, angular distance 1 - cos on the raw vectors.
 template <bool L2>
 __device__ __forceinline__ double fp64_key(const Dev &d, int64_t q, int64_t row) {
-    if (d.cosine) return cos_key_fp64_seq(d.Qr + q * d.dim, vrow_raw(d, row), d.dim);
+    if (d.cosine) {
+        const float *qr = d.Qr + q * d.dim, *xr = vrow_raw(d, row);
+        // (rows of the cache list have no stored sum)
+        return d.qrn2 && row < d.n ? cos_key_fp64(dot_fp64_seq(qr, xr, d.dim), d.qrn2[q], d.xrn2[row])
+                                   : cos_key_fp64_seq(qr, xr, d.dim);
+    }
     const float *qv = d.Q + q * d.dim, *xv = vrow(d, row);
     return L2 ? l2sq_fp64_seq(qv, xv, d.dim) : l1_fp64_seq(qv, xv, d.dim);
 }
@@ -1777,7 +1784,8 @@ __global__ void __launch_bounds__(256) k_knn_bound_warp(Dev d, const int64_t *__
                                                         const int32_t *__restrict__ bn, double *__restrict__ ckey,
                                                         int64_t *__restrict__ rlist,
                                                         unsigned long long *__restrict__ rcount,
-                                                        const float *__restrict__ chi, int64_t nq) {
+                                                        const float *__restrict__ chi, int64_t nq,
+                                                        float *__restrict__ thr) {
     __shared__ uint32_t sx[8][kBoundStage];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1872,6 +1880,7 @@ __global__ void __launch_bounds__(256) k_knn_bound_warp(Dev d, const int64_t *__
         }
     }
     const float Uf = __uint_as_float(U);
+    if (thr && lane == 0 && Uf < thr[q]) thr[q] = Uf;
     // the candidates whose lower bound reaches U: counted first, then one
     // atomic per warp reserves their places in the list (a counter that every
     // warp hits once per candidate serialises)
@@ -1888,7 +1897,7 @@ __global__ void __launch_bounds__(256) k_knn_bound_warp(Dev d, const int64_t *__
     for (int64_t i0 = 0; i0 < M; i0 += 32) {
         const int64_t i = i0 + lane;
         const bool l = i < M && listed(i);
-        if (i < M) ckey[a + i] = __longlong_as_double(0x7ff0000000000000ll);   // +inf: not a candidate
+        if (ckey && i < M) ckey[a + i] = __longlong_as_double(0x7ff0000000000000ll);   // +inf: not a candidate
         const unsigned bal = __ballot_sync(0xffffffffu, l);
         if (l) rlist[base + __popc(bal & ((1u << lane) - 1u))] = a + i;
         base += __popc(bal);
@@ -2200,6 +2209,12 @@ __global__ void k_recheck_keys(Dev d, const int32_t *__restrict__ cq, const int3
     }
 }
 
+// sums of squares in the keys' order, a thread per row
+__global__ void k_raw_norms(const float *__restrict__ X, int64_t n, int dim, double *__restrict__ out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = dot_fp64_seq(X + i * dim, X + i * dim, dim);
+}
+
 // kNN: once a query's answer so far holds k objects, its k-th FP64 distance
 // (rounded up) bounds tau_q from above.
 __global__ void k_tau_from_answer(const int32_t *__restrict__ kq, const int64_t *__restrict__ koff,
@@ -2213,6 +2228,20 @@ __global__ void k_tau_from_answer(const int32_t *__restrict__ kq, const int64_t 
         const float t = cosine ? __fadd_ru(__double2float_ru(__dsqrt_ru(__dmul_ru(2.0, v))), absf)
                                : __double2float_ru(l2 ? __dsqrt_ru(v) : v);
         if (t < thr[q]) thr[q] = t;
+    }
+}
+
+// the listed pairs of a query-sorted set (packed: row, q.x~)
+__global__ void k_take_listed(const int64_t *__restrict__ list, const unsigned long long *__restrict__ count,
+                              const int32_t *__restrict__ q, const uint64_t *__restrict__ packed,
+                              int32_t *__restrict__ oq, int32_t *__restrict__ orow, float *__restrict__ od) {
+    const int64_t n = (int64_t)*count;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t c = list[i];
+        const uint64_t p = packed[c];
+        oq[i] = q[c];
+        orow[i] = (int32_t)(p >> 32);
+        od[i] = __uint_as_float((uint32_t)p);
     }
 }
 
@@ -3461,9 +3490,14 @@ struct Runner {
         // interval, the selection).  10^6 x 128, 10^4 queries: 9.6 M kept pairs
         // -> 2.0 M, 7.34 -> 7.11 ms; angular, 2 * 10^5 x 300: 20.2 M -> 4.2 M,
         // 8.85 -> 8.26 ms.
-        const int stride = knn && rg.n_items >= kTilePhaseItems ? 8 : 1;
-        for (int phase = 0; phase < (stride > 1 ? 2 : 1); ++phase) {
-            DBuf<int32_t> oq, orow;
+        // For k <= 32 the first phase gives only the thresholds, from its pairs'
+        // upper bounds, and the few pairs within them join the second's.
+        const int phases = knn && rg.n_items >= kTilePhaseItems ? 2 : 1;
+        const bool carry = phases == 2 && qb.max_k <= 32;
+        PairSet first;
+        DBuf<unsigned long long> ncarry(1, st);
+        for (int phase = 0; phase < phases; ++phase) {
+            PairSet p;
             int nl = 0;
             // output capacity: twice the last call's size (per query), at least 1 M
             // pairs; a larger output triggers one relaunch with the exact size
@@ -3473,23 +3507,29 @@ struct Runner {
             // kNN: the tiles also give each kept pair's q.x~, whose proven distance
             // interval stands in for the FP32 distance (the answers' distances
             // come from their FP64 keys), so the pairs skip the FP32 verification
-            DBuf<float> od2;
             clk.begin(GTS_STAGE_TILE);
-            const int64_t C = tc_run(ix->tree, ix->tree.tc, tq, rg, oq, orow, hint, &nl, st, knn ? &od2 : nullptr,
-                                     phase, stride);
+            p.n = tc_run(ix->tree, ix->tree.tc, tq, rg, p.q, p.row, hint, &nl, st, knn ? &p.qx : nullptr, phase,
+                         phases == 2 ? 8 : 1);
             clk.end();
-            if (rg.n_items > 0 && qb.nq > 0) known.store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+            if (rg.n_items > 0 && qb.nq > 0) known.store(std::max<int64_t>(per_q, p.n * 1024 / qb.nq));
             ++st_groups;
-            if (C == 0) continue;
             if (!knn) {
                 // verified in the tiles' node-major order (consecutive pairs share
                 // their object row); range pairs kept are then sorted by query and id
-                verify_and_collect(oq, orow, C, /*query_major=*/false);
+                if (p.n > 0) verify_and_collect(p.q, p.row, p.n, /*query_major=*/false);
                 continue;
             }
-            st_cands += C;
-            knn_from_intervals(oq, orow, od2, C, tq);
-            if (phase + 1 < (stride > 1 ? 2 : 1)) {
+            st_cands += p.n;
+            if (carry && phase == 0) {
+                if (p.n > 0) first = within_bound(p, tq, ncarry);
+                continue;
+            }
+            if (first.n > 0) first.n = d2h_i64(reinterpret_cast<const int64_t *>(ncarry.get()), st);
+            if (p.n + first.n == 0) continue;
+            SortedPairs sp;
+            sort_intervals(p, first, tq, sp);
+            merge_knn(sp.q, sp.row, sp.lo, p.n + first.n, sp.hi.get());
+            if (phase + 1 < phases) {
                 clk.begin(GTS_STAGE_THRESHOLD);
                 k_tau_from_answer<<<cap(nblocks(qb.nq, kT)), kT, 0, st>>>(qb.k, koff.get(), bd.get(), bn.get(), qb.nq, 1,
                                                                          d.cosine, d.absf, thr.get());
@@ -3503,25 +3543,71 @@ struct Runner {
     // in query order, turn each estimate into its distance interval, and
     // merge (FP64 keys for the candidates whose interval reaches the k-th
     // upper bound)
-    void knn_from_intervals(DBuf<int32_t> &cq, DBuf<int32_t> &crow, DBuf<float> &cd2, int64_t C, const TcQuery &tq) {
-        DBuf<uint64_t> v1(C, st), v2(C, st);
-        DBuf<int32_t> q3(C, st), r3(C, st);
-        DBuf<float> d3(C, st), hi(C, st);
+    struct PairSet {
+        DBuf<int32_t> q, row;
+        DBuf<float> qx;   // q.x~
+        int64_t n = 0;
+    };
+    struct SortedPairs {
+        DBuf<int32_t> q, row;
+        DBuf<float> lo, hi;
+        DBuf<uint64_t> packed;   // (row, q.x~)
+    };
+    void sort_intervals(const PairSet &a, const PairSet &b, const TcQuery &tq, SortedPairs &o) {
+        const int64_t C = a.n + b.n;
+        DBuf<uint64_t> v1(C, st);
+        DBuf<int32_t> both(b.n > 0 ? C : 0, st);
+        o.q.alloc(C, st);
+        o.row.alloc(C, st);
+        o.lo.alloc(C, st);
+        o.hi.alloc(C, st);
+        o.packed.alloc(C, st);
+        const int32_t *keys = a.q.get();
+        if (b.n > 0) {
+            if (a.n > 0) GTS_CUDA(cudaMemcpyAsync(both.get(), a.q.get(), a.n * 4, cudaMemcpyDeviceToDevice, st));
+            GTS_CUDA(cudaMemcpyAsync(both.get() + a.n, b.q.get(), b.n * 4, cudaMemcpyDeviceToDevice, st));
+            keys = both.get();
+        }
         int qbits = 1;
         while (((int64_t)1 << qbits) < qb.nq) ++qbits;
         size_t tb = 0;
-        cub::DeviceRadixSort::SortPairs(nullptr, tb, cq.get(), q3.get(), v1.get(), v2.get(), C, 0, qbits, st);
+        cub::DeviceRadixSort::SortPairs(nullptr, tb, keys, o.q.get(), v1.get(), o.packed.get(), C, 0, qbits, st);
         DBuf<uint8_t> tmp(tb ? tb : 1, st);
         clk.begin(GTS_STAGE_OTHER, 4);
-        k_pack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(crow.get(), cd2.get(), C, v1.get());
-        GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, cq.get(), q3.get(), v1.get(), v2.get(), C, 0, qbits,
+        if (a.n > 0) k_pack_row_dist<<<cap(nblocks(a.n, kT)), kT, 0, st>>>(a.row.get(), a.qx.get(), a.n, v1.get());
+        if (b.n > 0)
+            k_pack_row_dist<<<cap(nblocks(b.n, kT)), kT, 0, st>>>(b.row.get(), b.qx.get(), b.n, v1.get() + a.n);
+        GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, keys, o.q.get(), v1.get(), o.packed.get(), C, 0, qbits,
                                                  st));
-        k_unpack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(v2.get(), C, r3.get(), d3.get());
-        k_tile_intervals<<<cap(nblocks(C, kT)), kT, 0, st>>>(q3.get(), r3.get(), C, tq.qn2, ix->tree.tc.xn2.get(),
-                                                            tq.cE1, tq.cE2, d3.get(), hi.get());
+        k_unpack_row_dist<<<cap(nblocks(C, kT)), kT, 0, st>>>(o.packed.get(), C, o.row.get(), o.lo.get());
+        k_tile_intervals<<<cap(nblocks(C, kT)), kT, 0, st>>>(o.q.get(), o.row.get(), C, tq.qn2, ix->tree.tc.xn2.get(),
+                                                            tq.cE1, tq.cE2, o.lo.get(), o.hi.get());
         clk.end();
         check_launch("tile intervals");
-        merge_knn(q3, r3, d3, C, hi.get());
+    }
+
+    // The k-th upper bound of the pairs and the answer so far into tau_q; the
+    // pairs whose lower bound is within it (their number in *count; room for all)
+    PairSet within_bound(const PairSet &p, const TcQuery &tq, DBuf<unsigned long long> &count) {
+        SortedPairs sp;
+        sort_intervals(p, PairSet(), tq, sp);
+        PairSet o;
+        o.n = p.n;
+        o.q.alloc(p.n, st);
+        o.row.alloc(p.n, st);
+        o.qx.alloc(p.n, st);
+        DBuf<int64_t> qoff(qb.nq + 1, st), list(p.n, st);
+        GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
+        clk.begin(GTS_STAGE_THRESHOLD, 3);
+        k_query_runs<<<cap(nblocks(qb.nq + 1, kT)), kT, 0, st>>>(sp.q.get(), p.n, qb.nq, qoff.get());
+        k_knn_bound_warp<GTS_L2><<<(unsigned)((qb.nq + 7) / 8), 256, 0, st>>>(
+            d, qoff.get(), sp.lo.get(), p.n, qb.k, koff.get(), bd.get(), bn.get(), nullptr, list.get(), count.get(),
+            sp.hi.get(), qb.nq, thr.get());
+        k_take_listed<<<cap(nblocks(p.n, kT)), kT, 0, st>>>(list.get(), count.get(), sp.q.get(), sp.packed.get(),
+                                                            o.q.get(), o.row.get(), o.qx.get());
+        clk.end();
+        check_launch("tile tau update");
+        return o;
     }
 
     void tc_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask, DBuf<int32_t> *ncount = nullptr) {
@@ -4227,7 +4313,8 @@ struct Runner {
     do {                                                                                                         \
         if (warp_sel)                                                                                            \
             k_knn_bound_warp<MT><<<wgrid, 256, 0, st>>>(d, qoff.get(), kd2.get(), R, qb.k, koff.get(), bd.get(),  \
-                                                        bn.get(), ckey.get(), rlist.get(), rc.get(), chi, qb.nq); \
+                                                        bn.get(), ckey.get(), rlist.get(), rc.get(), chi, qb.nq,  \
+                                                        nullptr);                                             \
         else                                                                                                     \
             k_knn_merge<MT, 0><<<grid, kT, 0, st>>>(d, qoff.get(), krow2.get(), kd2.get(), R, qb.k, koff.get(), \
                                                     bd.get(), bi.get(), bn.get(), ckey.get(), rlist.get(),      \
@@ -4495,6 +4582,33 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     d.Xr = t.Xr.get();
     d.cXr = c.Xr.get();
     d.Qr = qb.Qr;
+    d.xrn2 = nullptr;
+    d.qrn2 = nullptr;
+    // angular batches: the FP64 keys' sums of squares, the rows' once per index
+    // (a key then takes one sum of products instead of three: 104,000 keys of
+    // 300 coordinates 0.71 -> 0.35 ms, bound by the FP64 units; the batch's sums
+    // 0.036 ms).
+    DBuf<double> qrn2(t.cosine && nq >= kCosNorms ? nq : 0, st);
+    if (t.cosine && nq >= kCosNorms && t.n > 0) {
+        {
+            std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build them once
+            if (!t.xrn2_ready) {
+                Arena::Pause index_owned;
+                t.xrn2.alloc(t.n, st);
+                k_raw_norms<<<nblocks(t.n, 256), 256, 0, st>>>(t.Xr.get(), t.n, t.dim, t.xrn2.get());
+                check_launch("raw norms");
+                GTS_CUDA(cudaStreamSynchronize(st));
+                t.xrn2.persist();
+                t.xrn2_ready = true;
+            }
+        }
+        R.clk.begin(GTS_STAGE_OTHER);
+        k_raw_norms<<<nblocks(nq, 64), 64, 0, st>>>(qb.Qr, nq, t.dim, qrn2.get());
+        R.clk.end();
+        check_launch("raw norms");
+        d.xrn2 = t.xrn2.get();
+        d.qrn2 = qrn2.get();
+    }
     d.coslim = qb.coslim;
     DBuf<int64_t> qseq(nq, st);
     R.clk.begin(GTS_STAGE_OTHER);
