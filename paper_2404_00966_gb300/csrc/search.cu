@@ -1518,26 +1518,54 @@ __global__ void k_qgram_hist(const uint8_t *__restrict__ S, const int64_t *__res
     }
 }
 
-// How selective the 3-gram bound is: of ns pairs spread over the entries [e0,
-// e0 + E) of a level (an entry's query, a row of its node), how many pass.
-__global__ void k_qgram_sample(Dev d, const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
-                               int64_t lvl_base, int64_t e0, int64_t E, const float *__restrict__ thr_q, int ns,
-                               unsigned long long *__restrict__ passed) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    bool pass = false;
-    if (i < ns) {
-        const int64_t e = e0 + (int64_t)i * E / ns;
-        const int32_t q = eq[e];
-        const int64_t g = lvl_base + enode[e];
-        const int64_t row = d.npos[g] + (uint32_t)(i * 2654435761u) % (uint32_t)d.nsize[g];
-        const uint32_t *qw = reinterpret_cast<const uint32_t *>(d.qgq + (int64_t)q * kQgBuckets);
-        const uint32_t *rw = reinterpret_cast<const uint32_t *>(d.qg + row * kQgBuckets);
-        uint32_t l1 = 0;
-        for (int w = 0; w < kQgBuckets / 4; ++w) l1 = __vsadu4(qw[w], rw[w]) + l1;
-        pass = (float)l1 <= 6.f * thr_q[q];
+// How far the pivots prune a batch of strings: for 32 random rows a block and one
+// of the batch's queries, the distances to the pivots of the row's path and
+// the levels whose interval tests let the row through; surv[l]: pairs alive
+// after level l's pivots, surv[h]: pairs that the 3-gram bound lets through.
+template <int B>
+__global__ void __launch_bounds__(128) k_path_sample(Dev d, LevelOffsets lo, int64_t nq,
+                                                     const float *__restrict__ thr_q, unsigned *__restrict__ surv) {
+    __shared__ __align__(16) uint32_t Peq[256 * B];
+    __shared__ float s_d[kMaxHeight][32];
+    const int64_t q = (int64_t)blockIdx.x * nq / gridDim.x;
+    const int m = (int)(d.QSoff[q + 1] - d.QSoff[q]);
+    if (m > 0) build_peq<B>(Peq, d.QS + d.QSoff[q], m);
+    auto row_of = [&](int i) { return (int64_t)((uint32_t)((blockIdx.x * 32 + i + 1) * 2654435761u) % (uint64_t)d.n); };
+    // the child, among a node's, that holds a row
+    auto child_of = [&](int64_t g, int64_t row) -> int {
+        const int32_t avg = d.nsize[g] / d.F;
+        return avg > 0 ? (int)min((row - d.npos[g]) / avg, (int64_t)(d.F - 1)) : d.F - 1;
+    };
+    for (int t = threadIdx.x; t < 32 * d.h; t += blockDim.x) {
+        const int i = t & 31, l = t >> 5;
+        const int64_t row = row_of(i);
+        int64_t nd = 0;
+        for (int u = 0; u < l; ++u) nd = nd * d.F + child_of(lo.v[u] + nd, row);
+        const uint8_t *tx;
+        int len;
+        srow(d, d.npiv[lo.v[l] + nd], tx, len);
+        s_d[l][i] = (float)(m > 0 ? edit_bits<B, TextWords>(Peq, m, tx, len) : len);
     }
-    const unsigned b = __ballot_sync(0xffffffffu, pass);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(passed, (unsigned long long)__popc(b));
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    const int64_t row = row_of(lane);
+    const float thr = thr_q[q];
+    int64_t nd = 0;
+    bool alive = true;
+    for (int l = 0; l < d.h; ++l) {
+        nd = nd * d.F + child_of(lo.v[l] + nd, row);
+        const int64_t c = lo.v[l + 1] + nd;
+        alive = alive && interval_hit(s_d[l][lane], thr, d.nlo[c], d.nhi[c], 0.f, 0.f);
+        const unsigned b = __ballot_sync(0xffffffffu, alive);
+        if (lane == 0 && b) atomicAdd(surv + l, (unsigned)__popc(b));
+    }
+    const uint32_t *qw = reinterpret_cast<const uint32_t *>(d.qgq + q * kQgBuckets);
+    const uint32_t *rw = reinterpret_cast<const uint32_t *>(d.qg + row * kQgBuckets);
+    uint32_t l1 = 0;
+    for (int w = 0; w < kQgBuckets / 4; ++w) l1 = __vsadu4(qw[w], rw[w]) + l1;
+    const unsigned b = __ballot_sync(0xffffffffu, (float)l1 <= 6.f * thr);
+    if (lane == 0 && b) atomicAdd(surv + d.h, (unsigned)__popc(b));
 }
 
 // Verification of (query, row) pairs under edit distance; consecutive pairs
@@ -3122,8 +3150,10 @@ struct Runner {
                                                                    nullptr, nullptr, nullptr, cmask.get());
             clk.end();
             check_launch("expand count");
-            if (!knn && l == h - 2 && qgram_tiles_pay(E * F) && filter_beats_last_pivots(L, e0, e1, cnt)) {
-                str_leaf_children(L, e0, e1, cmask);
+            if (!knn && l == 0) str_stop = plan_str_stop();
+            if (!knn && l == str_stop) {
+                st_frontier += sum_i32(cnt, E);
+                str_leaf(L, e0, e1, cmask, l + 1);
                 return;
             }
             DBuf<int64_t> off;
@@ -3175,7 +3205,7 @@ struct Runner {
             }
             if (qgram_tiles_pay(E)) {
                 count_table_pass(L, e0, e1, mask);
-                str_leaf(L, e0, e1, mask);
+                str_leaf(L, e0, e1, mask, h);
                 return;
             }
             DBuf<int32_t> cnt(E, st);
@@ -3765,50 +3795,69 @@ struct Runner {
         return use_qg_large && E * ((ix->tree.n + nn - 1) / nn) >= kF32TilePairs;
     }
 
-    // Range queries on the 3-gram tiles: whether to leave the last pivot level
-    // out and filter every row of the children that survived the level above.
-    // Per (query, last-level node) entry the pivot costs 0.6 ps per word-step
-    // of its DP and 150 ps for the entry (its expansion, leaf mask and
-    // regrouped record); filtering all R rows of the node costs 1 ps a row
-    // and 90 ps for each pair the bound lets through (sorting and verifying
-    // it).  The pass rate is measured on a sample.  (10^6 reads of 108, r = 8:
-    // R = 125, pass rate below 10^-3, and the pivots exclude 5 % of the
-    // entries: 100.5 -> 39.3 ms without them.  Dictionary words at r = 2: a
-    // third passes, so the pivots stay.)
-    bool filter_beats_last_pivots(Level &L, int64_t e0, int64_t e1, DBuf<int32_t> &cnt) {
-        if (qb.count_table_pass || h < 2) return false;
+    // Range queries on the 3-gram tiles: the pivot level after which every row
+    // of the children that survive goes through the tiles, without the pivots
+    // below (-1: after the last, as usual).  Stopping after level m costs, per
+    // query, the pivots that the levels above it let through (each 0.6 ps per
+    // word-step of its DP and 150 ps for the entry: its expansion, leaf mask
+    // and regrouped record) and the rows alive after it (0.25 ps on the tensor
+    // cores, per place of a 256-query window, 1.6 on the integer units, 16 for
+    // short strings with their distance) with 90 ps for each pair that the bound
+    // lets through (sorting and verifying it).  The fractions alive come from
+    // a sample of paths.  (10^6 reads of 108, r = 8: nothing is excluded above
+    // the last level, 5 % by its pivots: 9.3 -> 5.5 ms a call with the blocks
+    // below and the tile's epilogue; the sample takes 0.03 ms.  Dictionary words
+    // at r = 2: the pivots stay.)
+    int str_stop = -1;
+    int plan_str_stop() {
         const Tree &t = ix->tree;
-        const double nn = (double)(t.lvl_off[h] - t.lvl_off[h - 1]);
-        const double rows = (double)t.n / nn;
-        const double pivot_ps = 0.6 * W * ((double)t.S.bytes() / (double)t.n) + 150.0;
-        if (rows > pivot_ps) return false;
-        constexpr int kSample = 8192;
-        DBuf<unsigned long long> c(2, st);
-        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 16, st));
-        clk.begin(GTS_STAGE_OTHER, 2);
-        k_qgram_sample<<<kSample / kT, kT, 0, st>>>(d, L.q.get(), L.node.get(), t.lvl_off[h - 2], e0, e1 - e0,
-                                                    thr.get(), kSample, c.get());
-        k_sum_i32<<<cap(nblocks(e1 - e0, kT)), kT, 0, st>>>(cnt.get(), e1 - e0, c.get() + 1);
+        if (t.dim > 0 || qb.count_table_pass || h < 2 || !d.qg ||
+            !qgram_tiles_pay(qb.nq * (t.lvl_off[h] - t.lvl_off[h - 1])))
+            return -1;
+        constexpr int kBlocks = 32, kSample = 32 * kBlocks;
+        DBuf<unsigned> surv(h + 1, st);
+        GTS_CUDA(cudaMemsetAsync(surv.get(), 0, (h + 1) * 4, st));
+        LevelOffsets lo;
+        for (int l = 0; l <= h && l < kMaxHeight + 2; ++l) lo.v[l] = t.lvl_off[l];
+        clk.begin(GTS_STAGE_OTHER, 1);
+#define GTS_PS(WW) k_path_sample<WW><<<kBlocks, 128, 0, st>>>(d, lo, qb.nq, thr.get(), surv.get())
+        if (W <= 1) GTS_PS(1);
+        else if (W <= 2) GTS_PS(2);
+        else if (W <= 4) GTS_PS(4);
+        else if (W <= 8) GTS_PS(8);
+        else if (W <= 16) GTS_PS(16);
+        else GTS_PS(32);
+#undef GTS_PS
         clk.end();
-        check_launch("3-gram sample");
-        unsigned long long hc[2];
-        GTS_CUDA(cudaMemcpyAsync(hc, c.get(), 16, cudaMemcpyDeviceToHost, st));
+        check_launch("path sample");
+        unsigned hs[kMaxHeight + 1];
+        GTS_CUDA(cudaMemcpyAsync(hs, surv.get(), (h + 1) * 4, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        const double f = (double)hc[0] / kSample;
-        if (rows * (1.0 + 90.0 * f) > pivot_ps) return false;
-        st_frontier += (int64_t)hc[1];
-        return true;
+        const double pivot_ps = 0.6 * W * ((double)t.S.bytes() / (double)t.n) + 150.0;
+        const double pass_ps = 90.0 * hs[h] / kSample;
+        const double window = 256.0 * (double)((qb.nq + 255) / 256) / (double)qb.nq;
+        double row_ps = 1.6 + pass_ps;
+        if (t.max_len <= kShortStr && qb.max_len <= kShortStr) row_ps = 16.0;
+        else if (t.n <= kQtcRows && qb.nq * t.n >= kQtcPairs && window <= 6.0) row_ps = 0.25 * window + pass_ps;
+        double pivots = 0.0, alive = 1.0, best = 0.0;
+        int stop = -1;
+        for (int m = 0; m < h; ++m) {
+            pivots += (double)(t.lvl_off[m + 1] - t.lvl_off[m]) * alive * pivot_ps;
+            alive = (double)hs[m] / kSample;
+            const double cost = pivots + (double)t.n * alive * row_ps;
+            if (m == 0 || cost < best) {
+                best = cost;
+                stop = m;
+            }
+        }
+        return stop < h - 1 ? stop : -1;
     }
-
-    // The rows of every child of [e0, e1)'s nodes (level h - 2) that its
-    // query's mask kept, through the 3-gram tiles.
-    void str_leaf_children(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &cmask) {
-        TcQuery tq = str_query_base(L, e0, e1, cmask);
-        TcRegroup rg;
-        clk.begin(GTS_STAGE_OTHER, 6);
-        tc_regroup_children(ix->tree, tq, rg, st);
-        clk.end();
-        str_tiles(rg, tq.any_deleted, true);
+    int64_t sum_i32(const DBuf<int32_t> &a, int64_t n) {
+        DBuf<unsigned long long> c(1, st);
+        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 8, st));
+        k_sum_i32<<<cap(nblocks(n, kT)), kT, 0, st>>>(a.get(), n, c.get());
+        check_launch("sum");
+        return d2h_i64(reinterpret_cast<const int64_t *>(c.get()), st);
     }
 
     TcQuery str_query_base(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
@@ -3824,19 +3873,21 @@ struct Runner {
         return tq;
     }
 
-    // Last level for strings on the 3-gram tiles: regroup the entries by
-    // node, keep the pairs the 3-gram count bound does not exclude, then run
-    // the exact bit-parallel DP on those (query-major for its match masks).
-    void str_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+    // Strings on the 3-gram tiles: regroup the entries by node (level hl - 1;
+    // their masks name its children), keep the pairs the 3-gram count bound
+    // does not exclude, then run the exact bit-parallel DP on those
+    // (query-major for its match masks).
+    void str_leaf(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask, int hl) {
         TcQuery tq = str_query_base(L, e0, e1, mask);
+        tq.h = hl;
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
         tc_regroup(ix->tree, tq, rg, st, nullptr, false);
         clk.end();
-        str_tiles(rg, tq.any_deleted, false);
+        str_tiles(rg, tq.any_deleted);
     }
 
-    void str_tiles(TcRegroup &rg, int any_deleted, bool children) {
+    void str_tiles(TcRegroup &rg, int any_deleted) {
         st_tiles += rg.n_items;
         st_tile_entries += rg.n_entries;
         st_tile_pairs += rg.n_pairs;
@@ -3844,7 +3895,6 @@ struct Runner {
         sq.qg = d.qg;
         sq.qgq = d.qgq;
         sq.any_deleted = any_deleted;
-        sq.children = children;
         sq.queries = tu.str_qgram == 32 ? 32 : 64;
         const int64_t per_q = ix->tc_pairs_hint[knn ? 1 : 0].load();
         const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);

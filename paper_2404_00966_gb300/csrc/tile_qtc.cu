@@ -19,15 +19,16 @@
 // lies below 2^10, so the FP32 accumulation is exact in any order.
 //
 // What bounds it: 10^6 reads of 108 x 20,000 queries, 2 * 10^10 pairs of 256
-// places, 5.0 ms = 2.0 PFLOP/s (the byte-wise sums of tile_str.cu: 31.4 ms, at
-// the rate of the integer units); the epilogue warps hold the MMAs back.
+// places, 3.9 ms = 2.6 PFLOP/s (the byte-wise sums of tile_str.cu: 31.4 ms, at
+// the rate of the integer units).  With the two accumulators' epilogues on the
+// same eight warps, 32 columns at a time, they held the MMAs back: 5.0 ms.
 // Layout: a unit of work is two 128-row blocks of nodes (A, by TMA) against the
 // windows of 256 consecutive queries that either node has an entry in (B, by
 // TMA, two buffers; loaded once for both blocks, since reading B from L2 once
 // per block would take longer than the MMAs).  One thread issues per window and
 // block eight 128 x 256 x 32 MMAs from shared memory into the block's TMEM
-// accumulator; while the other block's run, eight epilogue warps read it and
-// look for a clear sign bit (one logic operation per two pairs).  The few pairs
+// accumulator; while the other block's run, the block's own eight epilogue warps
+// read it and look for a clear sign bit (one logic operation per two pairs).  The few pairs
 // found wait in a queue per warp until 32 of them look up their entry's record
 // (leaf mask, sequence number) together.
 #include <cuda_fp8.h>
@@ -44,8 +45,8 @@ constexpr int kRowsQ = 128;      // rows of a block (MMA M)
 constexpr int kWinQ = 256;       // queries of a window (MMA N)
 constexpr int kCode = 256;       // bytes of a string's code: two panels of 128
 constexpr int kPlaces = 249;     // of them levels; then |A|'s digits, the constants
-constexpr int kEpiQ = 8;         // epilogue warps
-constexpr int kThreadsQ = (4 + kEpiQ) * 32;   // warp 0 producer, 1 MMA, 2 TMEM, 4.. epilogue
+constexpr int kEpiQ = 8;         // epilogue warps of each block
+constexpr int kThreadsQ = (4 + 2 * kEpiQ) * 32;   // warp 0 producer, 1 MMA, 2 TMEM, 4.. epilogue
 constexpr int kABytes = kRowsQ * kCode, kBBytes = kWinQ * kCode;
 constexpr int kDescs = 4;        // window descriptors: the epilogue is at most two windows behind
 constexpr int kQueue = 64;
@@ -55,11 +56,11 @@ struct Window {
     int32_t stop, new_unit, last, w;
 };
 struct Block {
-    int32_t row0, nrow, rb, node, size, owner;   // owner: the node whose entries these are
+    int32_t row0, nrow, rb, node, size;
 };
 
 struct QtcArgs {
-    int F, children, any_deleted;
+    int F, any_deleted;
     const int32_t *npos, *nsize;
     int64_t lvl_last, nq, nw, nwin;
     const int64_t *row_del;
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
     __shared__ __align__(8) uint64_t b_full[2], b_empty[2], acc_full[2], acc_empty[2], d_full[kDescs], a_full, a_empty;
     __shared__ Window s_win[kDescs];
     __shared__ Block s_blk[kDescs][2];
-    __shared__ int4 s_queue[kEpiQ][kQueue];   // query, row, owner, leaf bit
+    __shared__ int4 s_queue[2 * kEpiQ][kQueue];   // query, row, node, leaf bit
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -214,7 +215,6 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
                     const bool has = i0 + b < a.n_items;   // (an odd last item: its block twice, the second without rows)
                     const int4 it = a.items[has ? i0 + b : i0];
                     blk[b].node = it.x;
-                    blk[b].owner = a.children ? it.x / a.F : it.x;
                     blk[b].size = a.nsize[a.lvl_last + it.x];
                     blk[b].rb = it.w * kRowsQ;
                     blk[b].row0 = a.npos[a.lvl_last + it.x] + blk[b].rb;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
                 };
                 int64_t pend = -1;   // a window found and not handed on yet
                 for (int64_t c = w0 / 32; ok && c * 32 < w1; ++c) {
-                    uint32_t m = a.wany[blk[0].owner * per + c] | a.wany[blk[1].owner * per + c];
+                    uint32_t m = a.wany[blk[0].node * per + c] | a.wany[blk[1].node * per + c];
                     while (ok && m) {
                         const int64_t w = c * 32 + __ffs(m) - 1;
                         m &= m - 1;
@@ -314,13 +314,13 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
         }
     } else if (warp >= 4) {
         // ================================================= epilogue
-        const int quad = warp & 3, half = (warp - 4) >> 2;
+        const int quad = warp & 3, half = ((warp - 4) >> 2) & 1, blk = (warp - 4) / kEpiQ;
         const int r = quad * 32 + lane;                     // row of the block
         int4 *queue = s_queue[warp - 4];
         int queued = 0;                                     // warp-uniform
         uint32_t unit = 0;
-        bool valid[2] = {false, false};
-        int32_t row[2] = {0, 0}, owner[2] = {0, 0}, leaf[2] = {0, 0};
+        bool valid = false;
+        int32_t row = 0, node = 0, leaf = 0;
         // the first n queued pairs: entry, leaf, visibility
         auto flush = [&](int n) {
             __syncwarp();
@@ -355,47 +355,45 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
             const Window win = s_win[k % kDescs];
             if (win.stop || s_abort) break;
             if (win.new_unit) {
-                for (int b = 0; b < 2; ++b) {
-                    const Block bl = s_blk[unit % kDescs][b];
-                    valid[b] = r < bl.nrow;
-                    row[b] = bl.row0 + r;
-                    owner[b] = bl.owner;
-                    const int32_t avg = bl.size / a.F;
-                    leaf[b] = a.children ? bl.node % a.F : min(avg > 0 ? (bl.rb + r) / avg : a.F - 1, a.F - 1);
-                }
+                const Block bl = s_blk[unit % kDescs][blk];
+                valid = r < bl.nrow;
+                row = bl.row0 + r;
+                node = bl.node;
+                const int32_t avg = bl.size / a.F;
+                leaf = min(avg > 0 ? (bl.rb + r) / avg : a.F - 1, a.F - 1);
                 ++unit;
             }
-            bool ok = true;
-            for (int b = 0; b < 2; ++b) {
-                if (!tc::mbar_wait(&acc_full[b], k & 1)) {
-                    fail(7);
-                    ok = false;
-                    break;
-                }
-                tc::tc_fence_after();
-                for (int g = 0; g < kWinQ / 64; ++g) {
-                    const int col = half * (kWinQ / 2) + 32 * g;
-                    const int64_t q0 = (int64_t)win.w * kWinQ + col;
-                    if (q0 >= a.nq) break;   // (warp-uniform)
-                    uint32_t v[32];
-                    tc::tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kWinQ + col), v);
-                    tc::tmem_ld_wait();
-                    uint32_t all = v[0];
+            if (!tc::mbar_wait(&acc_full[blk], k & 1)) {
+                fail(7);
+                break;
+            }
+            tc::tc_fence_after();
+            const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(blk * kWinQ + half * (kWinQ / 2));
+            // 64 columns at a time
+            for (int g = 0; g < kWinQ / 128; ++g) {
+                uint32_t v[2][32];
+                tc::tmem_ld32(acc + 64 * g, v[0]);
+                tc::tmem_ld32(acc + 64 * g + 32, v[1]);
+                tc::tmem_ld_wait();
 #pragma unroll
-                    for (int i = 1; i < 32; ++i) all &= v[i];
-                    if (!__any_sync(0xffffffffu, valid[b] && !(all >> 31))) continue;
+                for (int u = 0; u < 2; ++u) {
+                    const int64_t q0 = (int64_t)win.w * kWinQ + half * (kWinQ / 2) + 64 * g + 32 * u;
+                    uint32_t all = v[u][0];
+#pragma unroll
+                    for (int i = 1; i < 32; ++i) all &= v[u][i];
+                    if (!__any_sync(0xffffffffu, valid && !(all >> 31)) || q0 >= a.nq) continue;
                     uint32_t pass = 0;
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) pass |= (~v[i] >> 31) << i;
+                    for (int i = 0; i < 32; ++i) pass |= (~v[u][i] >> 31) << i;
                     if (q0 + 32 > a.nq) pass &= (1u << (a.nq - q0)) - 1u;   // (no queries past the batch)
-                    if (!valid[b]) pass = 0;
+                    if (!valid) pass = 0;
                     for (unsigned act = __ballot_sync(0xffffffffu, pass != 0); act;
                          act = __ballot_sync(0xffffffffu, pass != 0)) {
                         if (pass) {
                             const int i = __ffs(pass) - 1;
                             pass &= pass - 1;
                             queue[queued + __popc(act & ((1u << lane) - 1u))] =
-                                make_int4((int32_t)q0 + i, row[b], owner[b], leaf[b]);
+                                make_int4((int32_t)q0 + i, row, node, leaf);
                         }
                         queued += __popc(act);
                         if (queued >= 32) {
@@ -408,11 +406,10 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
                         }
                     }
                 }
-                tc::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&acc_empty[b]);
             }
-            if (!ok) break;
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&acc_empty[blk]);
         }
         if (queued > 0) flush(queued);
     }
@@ -427,7 +424,9 @@ __global__ void __launch_bounds__(kThreadsQ, 1)
 bool qtc_pays(const Tree &t, int64_t nq, const TcRegroup &rg) {
     if (rg.nw == 0 || rg.n_items == 0 || t.n > kQtcRows) return false;
     const int64_t win = (nq + kWinQ - 1) / kWinQ;
-    return rg.n_pairs >= kQtcPairs && rg.n_pairs / 128 * 4 >= rg.n_items * win * kWinQ;
+    // the integer units take 1.6 ps a pair, the tensor cores 0.25 ps a place of the
+    // windows
+    return rg.n_pairs >= kQtcPairs && rg.n_pairs * 6 >= std::min(t.n, rg.n_items * kRowsQ) * win * kWinQ;
 }
 
 void qtc_codes(const uint8_t *qg, int64_t n, const float *thr, uint8_t *code, cudaStream_t st) {
@@ -448,8 +447,7 @@ int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t 
     const int64_t nwin = (nq + kWinQ - 1) / kWinQ, pairs = (rg.n_items + 1) / 2;
     // at least four units per SM where the windows allow it
     const int split = (int)std::max<int64_t>(1, std::min<int64_t>(nwin, (4 * sms + pairs - 1) / pairs));
-    // the records' nodes: the items' or, with children, their parents
-    const int64_t nodes = sq.children ? t.lvl_off[t.h - 1] - t.lvl_off[t.h - 2] : t.lvl_off[t.h] - t.lvl_off[t.h - 1];
+    const int64_t nodes = t.lvl_off[rg.h] - t.lvl_off[rg.h - 1];
     const int64_t per = (nwin + 31) / 32;
     DBuf<uint32_t> wany(nodes * per, st);
     k_windows_any<<<(unsigned)std::min<int64_t>((nodes * per + 255) / 256, 1 << 16), 256, 0, st>>>(
@@ -466,11 +464,10 @@ int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t 
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
         QtcArgs a;
         a.F = t.F;
-        a.children = sq.children ? 1 : 0;
         a.any_deleted = sq.any_deleted;
         a.npos = t.npos.get();
         a.nsize = t.nsize.get();
-        a.lvl_last = t.lvl_off[t.h - 1];
+        a.lvl_last = t.lvl_off[rg.h - 1];
         a.nq = nq;
         a.nw = rg.nw;
         a.nwin = nwin;

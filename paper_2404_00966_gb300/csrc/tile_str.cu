@@ -36,7 +36,6 @@ struct StrArgs {
     int64_t lvl_last;
     const int64_t *row_del;
     int any_deleted;
-    int children;               // the masks' bits are the parent's children, not the node's leaves
     const uint8_t *qg;          // rows' bucket counts [n, 64]
     const uint8_t *qgq;         // queries' bucket counts [nq, 64]
     const TileRec *grec;
@@ -113,7 +112,6 @@ __global__ void __launch_bounds__(kThreadsS, 2) k_tile_qgram(StrArgs a) {
             const int64_t row = (int64_t)pos + (valid ? rb + r : 0);
             int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
             if (jl > a.F - 1) jl = a.F - 1;
-            if (a.children) jl = it.x % a.F;
             rowbit[h] = valid ? (1ull << jl) : 0ull;
             any |= rowbit[h];
             const uint4 *src = reinterpret_cast<const uint4 *>(a.qg + row * 64);
@@ -256,7 +254,6 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
         const int32_t avg = size / a.F;
         int32_t jl = avg > 0 ? (rb + r) / avg : a.F - 1;
         if (jl > a.F - 1) jl = a.F - 1;
-        if (a.children) jl = it.x % a.F;
         const uint64_t rowbit = valid ? (1ull << jl) : 0ull;
         const int64_t rdel = (valid && a.any_deleted) ? a.row_del[row] : kNever;
         const int len = (int)(A.Soff[row + 1] - A.Soff[row]);
@@ -365,10 +362,9 @@ StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg) {
     a.F = t.F;
     a.npos = t.npos.get();
     a.nsize = t.nsize.get();
-    a.lvl_last = t.lvl_off[t.h - 1];
+    a.lvl_last = t.lvl_off[rg.h - 1];
     a.row_del = t.row_del.get();
     a.any_deleted = sq.any_deleted;
-    a.children = sq.children ? 1 : 0;
     a.qg = sq.qg;
     a.qgq = sq.qgq;
     a.grec = rg.grec.get();

@@ -12,7 +12,6 @@ struct StrQuery {
     const uint8_t *qgq = nullptr;   // the batch's queries' [nq, 64]
     int any_deleted = 1;
     int queries = 64;               // queries per tile chunk: 32 or 64
-    bool children = false;          // records from tc_regroup_children: masks name the parent's children
 };
 
 // Both sides at most 32 characters: the tiles also run the edit distance itself

@@ -886,32 +886,6 @@ __global__ void k_fill_items(const int32_t *__restrict__ ncount, const int32_t *
     }
 }
 
-// The same for items over the children (level `cnode` sizes) of the counted
-// nodes: thread per child.
-__global__ void k_child_items(const int32_t *__restrict__ ncount, const int32_t *__restrict__ csize, int64_t nc, int F,
-                              int64_t *__restrict__ nitems, unsigned long long *__restrict__ pairs) {
-    unsigned long long p = 0;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = ncount[c / F];
-        nitems[c] = k > 0 ? (int64_t)((csize[c] + kRows - 1) / kRows) : 0;
-        p += (unsigned long long)k * (unsigned long long)csize[c];
-    }
-    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-    if ((threadIdx.x & 31) == 0 && p) atomicAdd(pairs, p);
-    if (blockIdx.x == 0 && threadIdx.x == 0) nitems[nc] = 0;
-}
-
-__global__ void k_fill_child_items(const int32_t *__restrict__ ncount, const int32_t *__restrict__ csize,
-                                   const int64_t *__restrict__ noff, const int64_t *__restrict__ ioff, int64_t nc,
-                                   int F, int4 *__restrict__ items) {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = ncount[c / F];
-        if (k == 0) continue;
-        const int32_t blocks = (csize[c] + kRows - 1) / kRows;
-        for (int32_t b = 0; b < blocks; ++b) items[ioff[c] + b] = make_int4((int)c, (int)noff[c / F], k, b);
-    }
-}
-
 __global__ void k_i32_to_i64_tc(const int32_t *a, int64_t n, int64_t *b) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         b[i] = a[i];
@@ -1094,34 +1068,6 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
         k_fill_items<<<nblk(nn), 256, 0, st>>>(ncnt, lsize, noff.get(), ioff.get(), nn, win_min, rg.items.get());
     }
     check_launch("tile regroup");
-    return total_items;
-}
-
-int64_t tc_regroup_children(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st) {
-    const int64_t nn = t.lvl_off[t.h - 1] - t.lvl_off[t.h - 2];      // the parents
-    const int64_t nc = t.lvl_off[t.h] - t.lvl_off[t.h - 1];          // their children
-    const int64_t words = nn * ((tq.nq + 31) / 32);
-    DBuf<int32_t> own;
-    const int32_t *ncnt =
-        group_records(t, tq, rg, nn, words * 8 <= ((int64_t)1 << 30) && words <= 4 * tq.E, nullptr, own, st);
-    const int32_t *csize = t.nsize.get() + t.lvl_off[t.h - 1];
-    DBuf<int64_t> nitems(nc + 1, st), ioff(nc + 1, st);
-    DBuf<unsigned long long> pairs(1, st);
-    GTS_CUDA(cudaMemsetAsync(pairs.get(), 0, 8, st));
-    k_child_items<<<nblk(nc), 256, 0, st>>>(ncnt, csize, nc, t.F, nitems.get(), pairs.get());
-    count_offsets((const int64_t *)nitems.get(), ioff.get(), nc, st);
-    int64_t total_items = 0;
-    unsigned long long total_pairs = 0;
-    GTS_CUDA(cudaMemcpyAsync(&total_items, ioff.get() + nc, 8, cudaMemcpyDeviceToHost, st));
-    GTS_CUDA(cudaMemcpyAsync(&total_pairs, pairs.get(), 8, cudaMemcpyDeviceToHost, st));
-    GTS_CUDA(cudaStreamSynchronize(st));
-    rg.n_items = total_items;
-    rg.n_pairs = (int64_t)total_pairs;
-    if (total_items > 0) {
-        rg.items.alloc(total_items, st);
-        k_fill_child_items<<<nblk(nc), 256, 0, st>>>(ncnt, csize, rg.noff.get(), ioff.get(), nc, t.F, rg.items.get());
-    }
-    check_launch("child tile regroup");
     return total_items;
 }
 

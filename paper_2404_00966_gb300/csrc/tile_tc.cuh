@@ -136,11 +136,6 @@ bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E, int h = 0);
 // every width: a window is one chunk of the tile's queries)
 int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st,
                    const int32_t *counts = nullptr, bool window_ok = false);
-// Regroup entries of the level above the last by node (tq.emask: their
-// surviving children) into tiles over the children: an item's node is a
-// last-level node, its records are its parent's, whose masks name the
-// children.  No path distances.  Needs t.h >= 2.
-int64_t tc_regroup_children(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t st);
 // dense last level: work items for every node with a set bit in the node x
 // query bitmap `bits` ([nodes, nw] words, nw = ceil(nq / 32)), all in window
 // mode; the leaf masks stay in dmask [nodes, nq]
