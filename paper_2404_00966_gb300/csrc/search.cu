@@ -3502,8 +3502,6 @@ struct Runner {
         tq.Q = d.Q;
         tq.qseq = d.qseq;
         tq.thr = thr.get();
-        tq.epsc = d.epsc;
-        for (int l = 0; l < kMaxHeight; ++l) tq.lslack[l] = d.lslack[l];
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
         return tq;
     }
@@ -3658,7 +3656,6 @@ struct Runner {
         tq.E = e1 - e0;
         tq.eq = L.q.get() + e0;
         tq.enode = L.node.get() + e0;
-        tq.path = L.path.get() + e0 * h;
         tq.emask = mask.get();
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
@@ -3687,10 +3684,8 @@ struct Runner {
         tq.E = e1 - e0;
         tq.eq = L.q.get() + e0;
         tq.enode = L.node.get() + e0;
-        tq.path = L.path.get() + e0 * h;
         tq.emask = cmask.get();
         tq.h = h - 1;
-        tq.path_stride = h;
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
         tc_regroup(ix->tree, tq, rg, st, nullptr, true);
@@ -3713,7 +3708,6 @@ struct Runner {
         tq.Q = d.Q;
         tq.qseq = d.qseq;
         tq.thr = thr.get();
-        tq.epsc = d.epsc;
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);
@@ -4006,12 +4000,10 @@ struct Runner {
         tq.nq = qb.nq;
         tq.eq = L.q.get() + e0;
         tq.enode = L.node.get() + e0;
-        tq.path = L.path.get() + e0 * h;
         tq.emask = mask.get();
         tq.Q = d.Q;
         tq.qseq = d.qseq;
         tq.thr = thr.get();
-        tq.epsc = d.epsc;
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
         // kNN: a node's queries in the order of the regions their probes ended
         // in, so that a warp's queries keep much the same leaves of it
@@ -4056,12 +4048,10 @@ struct Runner {
         tq.nq = qb.nq;
         tq.eq = L.q.get() + e0;
         tq.enode = L.node.get() + e0;
-        tq.path = L.path.get() + e0 * h;
         tq.emask = mask.get();
         tq.Q = d.Q;
         tq.qseq = d.qseq;
         tq.thr = thr.get();
-        tq.epsc = d.epsc;
         tq.any_deleted = ix->tree.n_deleted > 0 ? 1 : 0;
         TcRegroup rg;
         clk.begin(GTS_STAGE_OTHER, 6);

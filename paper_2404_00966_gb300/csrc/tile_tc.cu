@@ -14,9 +14,12 @@
 //     D += A_hi B_hi^T + A_hi B_lo^T + A_lo B_hi^T, FP32 accumulator in TMEM;
 //   * the epilogue reads q.x from TMEM, forms d~^2 = |q|^2 + |x|^2 - 2 q.x and
 //     keeps a (query, row) pair only if the row's leaf survived for the query,
-//     the row is visible at the query's sequence number, a proven lower bound
-//     of the distance is within the query's threshold (radius, or tau_q for
-//     kNN) and the table lower bound max_l |D_l - d_l| passes (Lemma 1 / 2).
+//     the row is visible at the query's sequence number and a proven lower
+//     bound of the distance is within the query's threshold (radius, or tau_q
+//     for kNN).  (The table's lower bound max_l |D_l - d_l| of Lemma 1 / 2 is at
+//     most the distance: it could only drop pairs within both error bands, and
+//     its path distances cost more than that: 10^4 queries, 2 * 10^5 x 300, 7.34
+//     -> 7.12 ms without.)
 // The pairs kept are a superset of the answers; they are finished by the FP32
 // distance with its FP64 boundary recheck, so results equal the plain path's.
 //
@@ -49,7 +52,7 @@ namespace {
 
 constexpr int kRows = 128;     // MMA M: rows of one node block
 // MMA N (queries per chunk) NQ, the number SB of query-row buffers (B, hi and
-// lo) and the number SM of chunk slots (records, path distances and one FP32
+// lo) and the number SM of chunk slots (records and one FP32
 // TMEM accumulator of 128 lanes x NQ columns each) are template parameters,
 // chosen so that the node block (dim_p TMEM columns, hi and lo) and the SM
 // accumulators fit TMEM's 512 columns and the SB buffers and the slots fit
@@ -208,17 +211,14 @@ constexpr int kMmaWarp = kEpiWarps + kProducers / 32;
 constexpr int kThreadsWS = (kMmaWarp + 1) * 32;
 
 // Stage chunk [start, start + cnt) of a block's queries with asynchronous
-// copies by the producer threads: the records and path distances (contiguous,
+// copies by the producer threads: the records (contiguous,
 // node-major), and the split bf16 query rows into the 128-byte swizzled
 // layout (each thread first reads the query ids of the rows it copies).
 template <int NQ>
-__device__ __forceinline__ void stage_chunk(const TileArgs &a, int start, int cnt, TileRec *mrec, float *mpath,
+__device__ __forceinline__ void stage_chunk(const TileArgs &a, int start, int cnt, TileRec *mrec,
                                             uint8_t *sBh, uint8_t *sBl, int chunks16, int ptid, int32_t *sqid) {
     const uint8_t *rsrc = reinterpret_cast<const uint8_t *>(a.grec + start);
     for (int t = ptid; t < cnt * 2; t += kProducers) cp_async16(reinterpret_cast<uint8_t *>(mrec) + t * 16, rsrc + t * 16);
-    const uint8_t *psrc = reinterpret_cast<const uint8_t *>(a.gpath + (int64_t)start * a.hp);
-    const int pch = cnt * a.hp / 4;
-    for (int t = ptid; t < pch; t += kProducers) cp_async16(reinterpret_cast<uint8_t *>(mpath) + t * 16, psrc + t * 16);
     // query ids first (one load per thread), then the rows: consecutive
     // threads copy consecutive 16-byte pieces of a row, so every warp
     // instruction reads whole 32-byte sectors
@@ -267,14 +267,13 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
     uint8_t *sB = smem;                                     // SB buffers x (hi, lo) x panels x kNQ x 128 B
     const int bbuf = 2 * panels * bpanel;                   // bytes of one buffer
     uint8_t *mbase = sB + SB * bbuf;
-    // slot: records [kNQ], path distances [kNQ][hp], bound constants [kNQ / 2][4], descriptor
-    const int mbytes = kNQ * (int)sizeof(TileRec) + kNQ * a.hp * 4 + kNQ * 8 + (int)sizeof(ChunkDesc);
+    // slot: records [kNQ], bound constants [kNQ / 2][4], descriptor
+    const int mbytes = kNQ * (int)sizeof(TileRec) + kNQ * 8 + (int)sizeof(ChunkDesc);
     auto mrec = [&](int sl) { return (TileRec *)(mbase + sl * mbytes); };
-    auto mpath = [&](int sl) { return (float *)(mbase + sl * mbytes + kNQ * sizeof(TileRec)); };
     // columns 2i, 2i + 1 as (alpha_2i, alpha_2i+1, beta_2i, beta_2i+1), for packed FP32 tests
-    auto mab = [&](int sl) { return (float *)(mbase + sl * mbytes + kNQ * sizeof(TileRec) + kNQ * a.hp * 4); };
+    auto mab = [&](int sl) { return (float *)(mbase + sl * mbytes + kNQ * sizeof(TileRec)); };
     auto mdesc = [&](int sl) {
-        return (ChunkDesc *)(mbase + sl * mbytes + kNQ * sizeof(TileRec) + kNQ * a.hp * 4 + kNQ * 8);
+        return (ChunkDesc *)(mbase + sl * mbytes + kNQ * sizeof(TileRec) + kNQ * 8);
     };
     uint64_t *bars = (uint64_t *)(mbase + SM * mbytes);    // full[SM], mma_done[SM], epi_done[SM], a_full
     uint64_t *full = bars, *mma_done = bars + SM, *epi_done = bars + 2 * SM, *a_full = bars + 3 * SM;
@@ -385,7 +384,7 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                     tc::tma_load_3d(sB + sb * bbuf, &map_qh, 0, c * kNQ, 0, &full[sl]);
                     tc::tma_load_3d(sB + sb * bbuf + panels * bpanel, &map_ql, 0, c * kNQ, 0, &full[sl]);
                 }
-                // slot sl (records, path distances, accumulator): chunk g - SM tested
+                // slot sl (records, accumulator): chunk g - SM tested
                 if (g >= SM && !tc::mbar_wait(&epi_done[sl], ((g - SM) / SM) & 1)) fail(7);
                 int cnt;
                 float *ab = mab(sl);
@@ -393,14 +392,12 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                     cnt = 0;
                 } else if (window) {
                     cnt = kNQ;
-                    // column ptid: its record, path distances and bound constants, or an empty record
+                    // column ptid: its record and bound constants, or an empty record
                     if (ptid < kNQ) {
                         TileRec *mr = mrec(sl) + ptid;
                         const bool has = (cur.word >> (ptid & 31)) & 1u;
                         if (a.dmask) {
                             // dense last level: the record from the per-query arrays
-                            // (no threshold: only the table test reads it, and
-                            // dense chunks skip that test)
                             TileRec r;
                             r.q = cur.qid;
                             r.thr = 0.f;
@@ -419,8 +416,6 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                             *mr = r;
                             ab[(ptid >> 1) * 4 + (ptid & 1)] = cur.ab.x;
                             ab[(ptid >> 1) * 4 + 2 + (ptid & 1)] = cur.ab.y;
-                            float *mp = mpath(sl) + ptid * a.hp;
-                            for (int l = 0; l < a.hp; ++l) mp[l] = a.gpath[o * a.hp + l];
                         } else {
                             mr->mask = 0;
                             mr->q = c * kNQ + ptid;
@@ -428,7 +423,7 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                     }
                 } else {
                     cnt = total - c * kNQ < kNQ ? total - c * kNQ : kNQ;
-                    stage_chunk<NQ>(a, it.y + c * kNQ, cnt, mrec(sl), mpath(sl), sB + sb * bbuf,
+                    stage_chunk<NQ>(a, it.y + c * kNQ, cnt, mrec(sl), sB + sb * bbuf,
                                     sB + sb * bbuf + panels * bpanel, chunks16, ptid, sqid);
                     // the bound constants, once every producer's record copies have landed
                     cp_async_wait_all();
@@ -598,7 +593,6 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
             tc::tc_fence_after();
             const int cnt = dsc.cnt;
             const TileRec *rec = mrec(sl);
-            const float *pth = mpath(sl);
             // columns (queries) with a surviving leaf among the warp's 32 rows
             const unsigned live = (cc < kNQ && cc < cnt)
                                       ? __ballot_sync(0xffffffffu, cc + lane < cnt && (rec[cc + lane].mask & wmask) != 0)
@@ -624,23 +618,14 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                     failbits |= ((__float_as_uint(t0) >> 31) << i) | ((__float_as_uint(t1) >> 31) << (i + 1));
                 }
                 uint32_t cand = ~failbits & live;
-                // the few survivors: the row's leaf, visibility and the table lower bound
+                // the few survivors: the row's leaf and visibility
                 uint32_t passbits = 0;
                 while (cand) {
                     const int i = __ffs(cand) - 1;
                     cand &= cand - 1;
                     const TileRec &rc = rec[cc + i];
                     if (!(rc.mask & rowbit) || rdel <= rc.seq) continue;
-                    bool ok = true;
-                    // (the table lower bound can only drop a pair that the
-                    // distance bound already dropped; dense chunks skip it)
-                    for (int l = 0; l < a.h && ok && !a.dmask; ++l) {
-                        const float T = a.table[(int64_t)l * a.n + row];
-                        const float pl = pth[(cc + i) * a.hp + l];
-                        const float eps = a.epsc * (T + pl + rc.thr) + a.lslack[l];
-                        if (fabsf(T - pl) > rc.thr + eps) ok = false;
-                    }
-                    if (ok) passbits |= 1u << i;
+                    passbits |= 1u << i;
                 }
                 const int np = __popc(passbits);
                 int incl = np;
@@ -753,7 +738,7 @@ __global__ void k_query_consts(const float *__restrict__ thr, const float *__res
 
 __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
                                const uint64_t *__restrict__ emask, const float *__restrict__ path, int h, int hp,
-                               int stride, int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2, float cE1,
+                               int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2, float cE1,
                                float cE2, const int64_t *__restrict__ qseq, const int64_t *__restrict__ noff,
                                int32_t *__restrict__ cursor, TileRec *__restrict__ grec, int32_t *__restrict__ gq,
                                float *__restrict__ gpath) {
@@ -772,7 +757,7 @@ __global__ void k_node_scatter(const int32_t *__restrict__ eq, const int32_t *__
         grec[o] = r;
         gq[o] = q;
         if (path)
-            for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * stride + l] : 0.f;
+            for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
     }
 }
 
@@ -827,7 +812,7 @@ __global__ void k_bits_rows(const uint32_t *__restrict__ bits, int64_t nn, int64
 }
 
 __device__ __forceinline__ void write_rec(int64_t e, int64_t o, const int32_t *eq, const uint64_t *emask,
-                                          const float *path, int h, int hp, int stride, const float *thr, const float *qn2,
+                                          const float *path, int h, int hp, const float *thr, const float *qn2,
                                           float cE1, float cE2, const int64_t *qseq, TileRec *grec, int32_t *gq,
                                           float *gpath) {
     const int32_t q = eq[e];
@@ -840,12 +825,12 @@ __device__ __forceinline__ void write_rec(int64_t e, int64_t o, const int32_t *e
     grec[o] = r;
     gq[o] = q;
     if (path)
-        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * stride + l] : 0.f;
+        for (int l = 0; l < hp; ++l) gpath[o * hp + l] = l < h ? path[e * h + l] : 0.f;
 }
 
 __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
                                     const uint64_t *__restrict__ emask, const float *__restrict__ path, int h, int hp,
-                                    int stride, int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2,
+                                    int64_t E, const float *__restrict__ thr, const float *__restrict__ qn2,
                                     float cE1, float cE2, const int64_t *__restrict__ qseq,
                                     const int64_t *__restrict__ noff, const uint32_t *__restrict__ bits, const int32_t *__restrict__ wpre, int64_t nw,
                                     TileRec *__restrict__ grec, int32_t *__restrict__ gq, float *__restrict__ gpath,
@@ -855,7 +840,7 @@ __global__ void k_node_scatter_bits(const int32_t *__restrict__ eq, const int32_
         const int32_t q = pos_of ? pos_of[eq[e]] : eq[e];
         const int64_t wi = (int64_t)enode[e] * nw + (q >> 5);
         const int64_t o = noff[enode[e]] + wpre[wi] + __popc(bits[wi] & ((1u << (q & 31)) - 1u));
-        write_rec(e, o, eq, emask, path, h, hp, stride, thr, qn2, cE1, cE2, qseq, grec, gq, gpath);
+        write_rec(e, o, eq, emask, path, h, hp, thr, qn2, cE1, cE2, qseq, grec, gq, gpath);
     }
 }
 
@@ -927,11 +912,11 @@ void count_offsets<int64_t>(const int64_t *cnt, int64_t *off, int64_t n, cudaStr
     else exscan(cnt, off, n + 1, st);
 }
 
-size_t tile_smem_bytes(int dim_p, int h, int kNQ, int SB, int SM) {
+size_t tile_smem_bytes(int dim_p, int kNQ, int SB, int SM) {
     const int panels = dim_p / 64;
     size_t b = 1024;                                              // alignment slack
     b += (size_t)SB * 2 * panels * kNQ * 128;
-    b += SM * ((size_t)kNQ * sizeof(TileRec) + (size_t)kNQ * ((h + 3) & ~3) * 4 + (size_t)kNQ * 8 + 32);
+    b += SM * ((size_t)kNQ * sizeof(TileRec) + (size_t)kNQ * 8 + 32);
     b += (3 * SM + 1) * 8 + 4 + 4 * 4 + 16 + (size_t)kNQ * 4;
     return b;
 }
@@ -1020,17 +1005,16 @@ static const int32_t *group_records(const Tree &t, const TcQuery &tq, TcRegroup 
     GTS_CUDA(cudaStreamSynchronize(st));
     const int64_t ne = total_entries > 0 ? total_entries : 1;
     const int h = tq.h ? tq.h : t.h, hp = (h + 3) & ~3;
-    const int stride = tq.path_stride ? tq.path_stride : t.h;
     rg.h = h;
     rg.grec.alloc(ne, st);
     rg.gq.alloc(ne, st);
     rg.gpath.alloc(tq.path ? ne * hp : 1, st);
     if (use_bits)
-        k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
+        k_node_scatter_bits<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, E, tq.thr, tq.qn2,
                                                      tq.cE1, tq.cE2, tq.qseq, noff.get(), bits.get(), wpre.get(), nw, rg.grec.get(),
                                                      rg.gq.get(), rg.gpath.get(), tq.pos_of);
     else
-        k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, stride, E, tq.thr, tq.qn2,
+        k_node_scatter<<<nblk(E), 256, 0, st>>>(tq.eq, tq.enode, tq.emask, tq.path, h, hp, E, tq.thr, tq.qn2,
                                                 tq.cE1, tq.cE2, tq.qseq, noff.get(), cursor.get(), rg.grec.get(), rg.gq.get(),
                                                 rg.gpath.get());
     rg.n_entries = total_entries;
@@ -1122,7 +1106,7 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     GTS_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     // TMEM: A (dim_p columns) and the slots' accumulators share 512 columns
     GTS_REQUIRE(c.dim_p + shp.sm * nq_chunk <= 512, GTS_ECUDA, "tensor-core tile: TMEM columns");
-    const size_t smem = tile_smem_bytes(c.dim_p, h, nq_chunk, shp.sb, shp.sm);
+    const size_t smem = tile_smem_bytes(c.dim_p, nq_chunk, shp.sb, shp.sm);
     GTS_REQUIRE(smem <= (size_t)smem_optin, GTS_ECUDA, "tensor-core tile: shared memory");
     void (*kern)(const CUtensorMap, const CUtensorMap, TileArgs) =
         nq_chunk == 96    ? k_tile_l2_tc<96, 4, 4>
@@ -1185,12 +1169,10 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.dim = t.dim;
         a.dim_p = c.dim_p;
         a.F = t.F;
-        a.h = h;
         a.n = t.n;
         a.xn2 = c.xn2.get();
         a.Xh = reinterpret_cast<const __nv_bfloat16 *>(c.Xh.get());
         a.Xl = reinterpret_cast<const __nv_bfloat16 *>(c.Xl.get());
-        a.table = t.table.get();
         a.row_del = t.row_del.get();
         a.npos = t.npos.get();
         a.nsize = t.nsize.get();
@@ -1199,8 +1181,6 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.Ql = tq.Ql;
         a.grec = rg.grec.get();
         a.gq = rg.gq.get();
-        a.gpath = rg.gpath.get();
-        a.hp = (h + 3) & ~3;
         a.items = rg.items.get();
         a.n_items = n_items;
         a.phase = phase;
@@ -1212,8 +1192,6 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.cap = cap;
         a.out_count = count.get();
         a.status = status.get();
-        a.epsc = tq.epsc;
-        for (int l = 0; l < kMaxHeight; ++l) a.lslack[l] = tq.lslack[l];
         a.cE1 = cE1;
         a.cE2 = cE2;
         a.any_deleted = tq.any_deleted;

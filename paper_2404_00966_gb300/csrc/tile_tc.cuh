@@ -20,19 +20,16 @@ struct __align__(16) TileRec {
 };
 
 struct TileArgs {
-    int dim, dim_p, F, h;
+    int dim, dim_p, F;
     int64_t n;
     const float *xn2;         // |x|^2 of every row (FP64 sum, rounded)
     const __nv_bfloat16 *Xh, *Xl;   // every row, split bf16 [n, dim_p]
-    const float *table;       // [h, n]
     const int64_t *row_del;
     const int32_t *npos, *nsize;
     int64_t lvl_last;         // first node of the last pivot level
     const __nv_bfloat16 *Qh, *Ql;   // the batch's queries, split bf16 [nq, dim_p]
     const TileRec *grec;      // entries of the last pivot level regrouped by node
     const int32_t *gq;        // their queries (for the row copies)
-    const float *gpath;       // their path distances [*, hp], hp = h rounded up to 4
-    int hp;
     const int4 *items;        // (node, first, count, row block | kWindowItem) over the records
     int64_t n_items;          // of this launch: number i is item pick(i), see tc_run
     int phase, stride;
@@ -42,8 +39,7 @@ struct TileArgs {
     int64_t cap;
     unsigned long long *out_count;
     int *status;
-    float epsc, cE1, cE2;     // pruning slack; error-bound coefficients
-    float lslack[kMaxHeight]; // absolute slack of each level's query-to-pivot distances
+    float cE1, cE2;           // error-bound coefficients
     int any_deleted;          // 0: no row has a delete mark, skip the visibility test
     // window mode (dense nodes): the node x query bitmap of the regrouping
     const uint32_t *bits;     // [nodes, nw]
@@ -78,15 +74,13 @@ struct TcQuery {
     const float *path = nullptr;
     const uint64_t *emask = nullptr;
     // the entries' level is h - 1, their masks name the nodes' children at
-    // level h, and `path` holds path_stride floats per entry (0: the tree's h)
-    int h = 0, path_stride = 0;
+    // level h (0: the tree's h)
+    int h = 0;
     // order of a node's records: by pos_of[query] (null: by query; the bitmap form only)
     const int32_t *pos_of = nullptr;
     const float *Q = nullptr;
     const int64_t *qseq = nullptr;
     const float *thr = nullptr;
-    float epsc = 0.f;
-    float lslack[kMaxHeight] = {};   // absolute slack of each level's path distances
     int any_deleted = 1;
 };
 
@@ -107,7 +101,7 @@ struct TcRegroup {
     int64_t nw = 0;
     DBuf<TileRec> grec;    // entry records grouped by node
     DBuf<int32_t> gq;      // their queries
-    DBuf<float> gpath;     // their path distances [*, hp]
+    DBuf<float> gpath;     // their path distances [*, hp], if asked for (tq.path): hp = h rounded up to 4
     DBuf<int4> items;      // (node, first, count, 0)
     int64_t n_items = 0;
     int64_t n_nodes = 0;   // nodes of the level
