@@ -187,7 +187,7 @@ struct TcCache {
     bool ready = false;
     int dim_p = 0;
     DBuf<uint8_t> Xh, Xl;
-    DBuf<float> xn2;
+    DBuf<float> xn2, xr;   // |x|^2; |x - x_hi|, rounded up
     // every pivot level's pivots as split rows (node order; empty nodes: zero rows)
     bool piv_ready = false;
     DBuf<uint8_t> Ph, Pl;

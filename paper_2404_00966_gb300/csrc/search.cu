@@ -2259,6 +2259,38 @@ __global__ void k_tau_from_answer(const int32_t *__restrict__ kq, const int64_t 
     }
 }
 
+// Of a first phase's pairs (a warp per query), those that one product's bound would
+// let through at the lowered threshold: count[0], over the queries whose first
+// threshold reached past it (their pairs are all here): count[1].
+__global__ void __launch_bounds__(256) k_single_count(const int64_t *__restrict__ qoff,
+                                                      const uint64_t *__restrict__ packed, int64_t nq,
+                                                      const float *__restrict__ qn2, const float *__restrict__ xn2,
+                                                      const float *__restrict__ xr, const float *__restrict__ rho,
+                                                      float gamma, const float *__restrict__ before,
+                                                      const float *__restrict__ thr, unsigned long long *count) {
+    const int lane = threadIdx.x & 31;
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (q >= nq) return;
+    const float t = thr[q], qn = sqrtf(qn2[q]), rg = *rho + gamma;
+    unsigned n = 0;
+    float widest = 0.f;
+    for (int64_t i = qoff[q] + lane; i < qoff[q + 1]; i += 32) {
+        const uint64_t p = packed[i];
+        const int64_t row = (int64_t)(p >> 32);
+        const float x2 = xn2[row], e = 2.02f * qn * (xr[row] + rg * sqrtf(x2));
+        const float d2 = qn2[q] + x2 - 2.f * __uint_as_float((uint32_t)p);
+        n += d2 <= t * t + e ? 1u : 0u;
+        widest = fmaxf(widest, e);
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) widest = fmaxf(widest, __shfl_xor_sync(0xffffffffu, widest, o));
+    if (lane == 0 && before[q] * before[q] >= t * t + widest) {
+        if (n) atomicAdd(count, (unsigned long long)n);
+        atomicAdd(count + 1, 1ull);
+    }
+}
+
 // the listed pairs of a query-sorted set (packed: row, q.x~)
 __global__ void k_take_listed(const int64_t *__restrict__ list, const unsigned long long *__restrict__ count,
                               const int32_t *__restrict__ q, const uint64_t *__restrict__ packed,
@@ -2934,7 +2966,7 @@ struct Runner {
     bool whole_batch = true;   // no level has been split into groups so far
     int64_t st_dense_last = 0;
     DBuf<uint8_t> tcQh, tcQl;   // the batch's queries as split bf16 rows (tensor-core path)
-    DBuf<float> tcqn2;
+    DBuf<float> tcqn2, tcrho;
     DBuf<int32_t> qkey;         // kNN: the probe's last-level node per query (qkey_ok once written)
     bool qkey_ok = false;
     DBuf<unsigned long long> tp_count;   // diagnostics: [0] pairs passing the table bound, [1] scratch
@@ -3497,6 +3529,7 @@ struct Runner {
         tq.Qh = (const __nv_bfloat16 *)tcQh.get();
         tq.Ql = (const __nv_bfloat16 *)tcQl.get();
         tq.qn2 = tcqn2.get();
+        tq.rho = tcrho.get();
         tq.chunk = tu.tc_queries;
         tc_bound_coeffs(ix->tree.tc.dim_p, tq.cE1, tq.cE2);
         tq.Q = d.Q;
@@ -3523,7 +3556,8 @@ struct Runner {
         const int phases = knn && rg.n_items >= kTilePhaseItems ? 2 : 1;
         const bool carry = phases == 2 && qb.max_k <= 32;
         PairSet first;
-        DBuf<unsigned long long> ncarry(1, st);
+        DBuf<unsigned long long> first_counts(3, st);   // pairs carried, within one product's bound, queries they tell
+        bool single = false;
         for (int phase = 0; phase < phases; ++phase) {
             PairSet p;
             int nl = 0;
@@ -3536,8 +3570,8 @@ struct Runner {
             // interval stands in for the FP32 distance (the answers' distances
             // come from their FP64 keys), so the pairs skip the FP32 verification
             clk.begin(GTS_STAGE_TILE);
-            p.n = tc_run(ix->tree, ix->tree.tc, tq, rg, p.q, p.row, hint, &nl, st, knn ? &p.qx : nullptr, phase,
-                         phases == 2 ? 8 : 1);
+            p.n = tc_run(ix->tree, ix->tree.tc, tq, rg, p.q, p.row, hint, &nl, st, knn && !single ? &p.qx : nullptr, phase,
+                         phases == 2 ? 8 : 1, single ? 1 : 3);
             clk.end();
             if (rg.n_items > 0 && qb.nq > 0) known.store(std::max<int64_t>(per_q, p.n * 1024 / qb.nq));
             ++st_groups;
@@ -3547,12 +3581,34 @@ struct Runner {
                 if (p.n > 0) verify_and_collect(p.q, p.row, p.n, /*query_major=*/false);
                 continue;
             }
-            st_cands += p.n;
+            if (!single) st_cands += p.n;
             if (carry && phase == 0) {
-                if (p.n > 0) first = within_bound(p, tq, ncarry);
+                if (p.n > 0) {
+                    first = within_bound(p, tq, first_counts);
+                    unsigned long long hc[3];
+                    GTS_CUDA(cudaMemcpyAsync(hc, first_counts.get(), 24, cudaMemcpyDeviceToHost, st));
+                    GTS_CUDA(cudaStreamSynchronize(st));
+                    first.n = (int64_t)hc[0];
+                    single = single_pays(rg.n_pairs, hc[1], hc[2]);
+                }
                 continue;
             }
-            if (first.n > 0) first.n = d2h_i64(reinterpret_cast<const int64_t *>(ncarry.get()), st);
+            if (single) {
+                // the carried pairs with them: all take their FP32 distance
+                const int64_t C = p.n + first.n;
+                if (C == 0) continue;
+                DBuf<int32_t> cq(C, st), crow(C, st);
+                const PairSet *sets[2] = {&p, &first};
+                int64_t o = 0;
+                for (const PairSet *x : sets) {
+                    if (x->n == 0) continue;
+                    GTS_CUDA(cudaMemcpyAsync(cq.get() + o, x->q.get(), x->n * 4, cudaMemcpyDeviceToDevice, st));
+                    GTS_CUDA(cudaMemcpyAsync(crow.get() + o, x->row.get(), x->n * 4, cudaMemcpyDeviceToDevice, st));
+                    o += x->n;
+                }
+                verify_and_collect(cq, crow, C, /*query_major=*/false);
+                continue;
+            }
             if (p.n + first.n == 0) continue;
             SortedPairs sp;
             sort_intervals(p, first, tq, sp);
@@ -3614,8 +3670,22 @@ struct Runner {
         check_launch("tile intervals");
     }
 
+    // Whether the second phase runs with one product: its three take 6 dim flops
+    // a pair at 1.0 PFLOP/s, one saves about half of that; each pair that the
+    // wider bound lets through costs 0.15 ns (its extraction, FP32 distance and
+    // sort).  Their number is seven times the first phase's, counted there in the
+    // queries whose first threshold reached past the wider bound (within: pairs,
+    // told: queries; for fewer than half of the queries it stays open).
+    bool single_pays(int64_t n_pairs, unsigned long long within, unsigned long long told) const {
+        if ((int64_t)told * 2 < qb.nq) return false;
+        const double pairs = 7.0 * (double)within * (double)qb.nq / (double)told;
+        const double saved_ns = 0.5 * 7.0 / 8.0 * (double)n_pairs * 6.0 * ix->tree.tc.dim_p / 1.0e6;
+        return pairs * 0.15 <= saved_ns;
+    }
+
     // The k-th upper bound of the pairs and the answer so far into tau_q; the
-    // pairs whose lower bound is within it (their number in *count; room for all)
+    // pairs whose lower bound is within it (their number in count[0]; room for
+    // all), and the counts for single_pays
     PairSet within_bound(const PairSet &p, const TcQuery &tq, DBuf<unsigned long long> &count) {
         SortedPairs sp;
         sort_intervals(p, PairSet(), tq, sp);
@@ -3625,14 +3695,19 @@ struct Runner {
         o.row.alloc(p.n, st);
         o.qx.alloc(p.n, st);
         DBuf<int64_t> qoff(qb.nq + 1, st), list(p.n, st);
-        GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
-        clk.begin(GTS_STAGE_THRESHOLD, 3);
+        DBuf<float> before(qb.nq, st);
+        GTS_CUDA(cudaMemcpyAsync(before.get(), thr.get(), qb.nq * 4, cudaMemcpyDeviceToDevice, st));
+        GTS_CUDA(cudaMemsetAsync(count.get(), 0, 24, st));
+        clk.begin(GTS_STAGE_THRESHOLD, 4);
         k_query_runs<<<cap(nblocks(qb.nq + 1, kT)), kT, 0, st>>>(sp.q.get(), p.n, qb.nq, qoff.get());
         k_knn_bound_warp<GTS_L2><<<(unsigned)((qb.nq + 7) / 8), 256, 0, st>>>(
             d, qoff.get(), sp.lo.get(), p.n, qb.k, koff.get(), bd.get(), bn.get(), nullptr, list.get(), count.get(),
             sp.hi.get(), qb.nq, thr.get());
         k_take_listed<<<cap(nblocks(p.n, kT)), kT, 0, st>>>(list.get(), count.get(), sp.q.get(), sp.packed.get(),
                                                             o.q.get(), o.row.get(), o.qx.get());
+        k_single_count<<<(unsigned)((qb.nq + 7) / 8), 256, 0, st>>>(
+            qoff.get(), sp.packed.get(), qb.nq, tq.qn2, ix->tree.tc.xn2.get(), ix->tree.tc.xr.get(), tq.rho,
+            tc_gamma(ix->tree.tc.dim_p), before.get(), thr.get(), count.get() + 1);
         clk.end();
         check_launch("tile tau update");
         return o;
@@ -4554,7 +4629,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         }
         R.use_tc = true;
         R.clk.begin(GTS_STAGE_OTHER);
-        tc_split_queries(qb.Q, nq, t.dim, t.tc.dim_p, R.tcQh, R.tcQl, R.tcqn2, st);
+        tc_split_queries(qb.Q, nq, t.dim, t.tc.dim_p, R.tcQh, R.tcQl, R.tcqn2, st, nullptr, &R.tcrho);
         R.clk.end();
     }
     R.h = t.h;

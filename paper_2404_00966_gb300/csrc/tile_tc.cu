@@ -32,6 +32,16 @@
 //   | d~^2 - d^2 | <= E = cE1 |q| |x| + cE2 (|q| + |x|)^2,
 //   cE1 = 2.02 (3.01 * 2^-16 + gamma_{3K+2}(2^-23)),  cE2 = 2^-21,
 // and d <= thr is possible only if d~^2 <= thr^2 + E.
+//
+// One product.  With A_hi B_hi^T alone, and r_x = |x - x_hi|, r_q = |q - q_hi| (as
+// computed, rounded up; about 0.0016 of the norms),
+//   | q.x - q_hi.x_hi | <= |q| r_x + r_q |x_hi|,   |x_hi| <= |x| + r_x,
+// and the K exact products are summed within gamma_{K+2}(2^-23) |q_hi| |x_hi|, so
+//   | d~^2 - d^2 | <= E' = |q| y_x + cE2 (|q| + |x|)^2,
+//   y_x = 2.02 (r_x + (rho + gamma_{K+2}) |x|),   rho = max over the batch r_q / |q|.
+// The second phase of a kNN batch runs so where the pairs that E' lets through
+// are few (single_pays): they take the FP32 distance.  10^4 queries, 2 * 10^5 x 300,
+// the angle: 20 pairs a query, the tile 3.7 -> 1.4 ms, the call 7.12 -> 5.13.
 #include <cstring>
 
 #include <cuda.h>
@@ -66,7 +76,14 @@ constexpr int kRows = 128;     // MMA M: rows of one node block
 struct TileShape {
     int nq, sb, sm;
 };
-inline TileShape shape_for(int dim_p, int pref) {
+// One product needs half of A's columns and of B: 128 queries up to 384 columns.
+inline TileShape shape_for(int dim_p, int pref, int products) {
+    if (products == 1) {
+        if (dim_p <= 192) return {128, 3, 3};
+        if (dim_p <= 256) return {128, 2, 3};
+        if (dim_p <= 384) return {128, 2, 2};
+        return {64, 3, 3};
+    }
     if (dim_p <= 128) return pref == 96 ? TileShape{96, 4, 4} : TileShape{128, 3, 3};
     if (dim_p <= 192) return {64, 4, 4};
     if (dim_p <= 256) return {32, 4, 4};
@@ -74,7 +91,6 @@ inline TileShape shape_for(int dim_p, int pref) {
     if (dim_p <= 384) return {32, 2, 4};
     return {32, 2, 2};
 }
-inline int nq_for(int dim_p, int pref) { return shape_for(dim_p, pref).nq; }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -141,26 +157,39 @@ namespace {
 
 // Split every float32 row into bf16 hi / lo parts (padded with zeros to
 // dim_p columns) and its squared norm, summed in FP64 and rounded once
-// (output row i from input row sel[i] when sel is given).
+// (output row i from input row sel[i] when sel is given).  res: the norms of x -
+// x_hi (the differences are exact), rounded up; rho: their largest ratio to |x|.
 __global__ void k_split_rows(const float *__restrict__ X, int dim, int dim_p, int64_t n,
                              __nv_bfloat16 *__restrict__ Xh, __nv_bfloat16 *__restrict__ Xl,
-                             float *__restrict__ n2, const int32_t *__restrict__ sel) {
+                             float *__restrict__ n2, const int32_t *__restrict__ sel,
+                             float *__restrict__ res, float *__restrict__ rho) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; row < n; row += nw) {
         // output row `row` takes input row `src` (a negative src: a zero row)
         const int64_t src = sel ? (int64_t)sel[row] : row;
-        double s = 0.0;
+        double s = 0.0, rs = 0.0;
         for (int k = lane; k < dim_p; k += 32) {
             const float v = k < dim && src >= 0 ? X[src * dim + k] : 0.f;
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
-            const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
+            const float e = v - __bfloat162float(h);
+            const __nv_bfloat16 l = __float2bfloat16_rn(e);
+            rs += (double)e * (double)e;
             Xh[row * dim_p + k] = h;
             Xl[row * dim_p + k] = l;
             s += (double)v * (double)v;
         }
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) n2[row] = __double2float_rn(s);
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            rs += __shfl_xor_sync(0xffffffffu, rs, o);
+        }
+        if (lane == 0) {
+            n2[row] = __double2float_rn(s);
+            const float re = __fmul_ru(__fsqrt_ru(__double2float_ru(rs)), 1.f + 1e-6f);
+            if (res) res[row] = re;
+            if (rho && re > 0.f)
+                atomicMax(reinterpret_cast<int *>(rho), __float_as_int(__fdiv_ru(re, __fsqrt_rd(__double2float_rd(s)))));
+        }
     }
 }
 
@@ -214,7 +243,7 @@ constexpr int kThreadsWS = (kMmaWarp + 1) * 32;
 // copies by the producer threads: the records (contiguous,
 // node-major), and the split bf16 query rows into the 128-byte swizzled
 // layout (each thread first reads the query ids of the rows it copies).
-template <int NQ>
+template <int NQ, int PROD>
 __device__ __forceinline__ void stage_chunk(const TileArgs &a, int start, int cnt, TileRec *mrec,
                                             uint8_t *sBh, uint8_t *sBl, int chunks16, int ptid, int32_t *sqid) {
     const uint8_t *rsrc = reinterpret_cast<const uint8_t *>(a.grec + start);
@@ -225,7 +254,7 @@ __device__ __forceinline__ void stage_chunk(const TileArgs &a, int start, int cn
     tc::named_sync(1, kProducers);   // every producer is done with the previous chunk's ids
     for (int j = ptid; j < cnt; j += kProducers) sqid[j] = a.gq[start + j];
     tc::named_sync(1, kProducers);
-    const int per_q = 2 * chunks16;                  // 16-byte copies per query (hi and lo)
+    const int per_q = (PROD == 3 ? 2 : 1) * chunks16;   // 16-byte copies per query (hi and lo)
 #pragma unroll 4
     for (int t = ptid; t < cnt * per_q; t += kProducers) {
         const int j = t / per_q, c = t - j * per_q;
@@ -254,7 +283,9 @@ __device__ __forceinline__ void stage_chunk(const TileArgs &a, int start, int cn
 // operands in shared memory a 128 x 128 x 16 MMA reads 8 KB, all that the port
 // delivers in the MMA's 64 cycles, and the MMAs ran at about 60 % of the
 // tensor rate.
-template <int NQ, int SB, int SM>
+// PROD: 3 products or 1 (then A_hi and B_hi alone are staged, and the
+// accumulators start at column dim_p / 2).
+template <int NQ, int SB, int SM, int PROD>
 __global__ void __launch_bounds__(kThreadsWS, 1)
     k_tile_l2_tc(const __grid_constant__ CUtensorMap map_qh, const __grid_constant__ CUtensorMap map_ql, TileArgs a) {
     static_assert(SB <= SM, "a B buffer is reused no later than its slot");
@@ -265,7 +296,7 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
     const int panels = a.dim_p / 64;
     const int bpanel = kNQ * 128;
     uint8_t *sB = smem;                                     // SB buffers x (hi, lo) x panels x kNQ x 128 B
-    const int bbuf = 2 * panels * bpanel;                   // bytes of one buffer
+    const int bbuf = (PROD == 3 ? 2 : 1) * panels * bpanel; // bytes of one buffer
     uint8_t *mbase = sB + SB * bbuf;
     // slot: records [kNQ], bound constants [kNQ / 2][4], descriptor
     const int mbytes = kNQ * (int)sizeof(TileRec) + kNQ * 8 + (int)sizeof(ChunkDesc);
@@ -298,7 +329,8 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tslot;
-    const uint32_t tacc = tmem + (uint32_t)a.dim_p;        // accumulator 0
+    const int acols = PROD == 3 ? a.dim_p : a.dim_p / 2;    // TMEM columns of A
+    const uint32_t tacc = tmem + (uint32_t)acols;           // accumulator 0
     const int chunks16 = a.dim_p / 8;                       // 16-byte chunks per bf16 row
     auto fail = [&](int code) {
         *sabort = 1;
@@ -380,9 +412,10 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                 if (g >= SB && !tc::mbar_wait(&mma_done[(g - SB) % SM], ((g - SB) / SM) & 1)) fail(4);
                 if (window && ptid == 0) {
                     // the window's query rows, every panel of hi and of lo
-                    tc::mbar_expect_tx_only(&full[sl], (uint32_t)(2 * panels * bpanel));
+                    tc::mbar_expect_tx_only(&full[sl], (uint32_t)bbuf);
                     tc::tma_load_3d(sB + sb * bbuf, &map_qh, 0, c * kNQ, 0, &full[sl]);
-                    tc::tma_load_3d(sB + sb * bbuf + panels * bpanel, &map_ql, 0, c * kNQ, 0, &full[sl]);
+                    if (PROD == 3)
+                        tc::tma_load_3d(sB + sb * bbuf + panels * bpanel, &map_ql, 0, c * kNQ, 0, &full[sl]);
                 }
                 // slot sl (records, accumulator): chunk g - SM tested
                 if (g >= SM && !tc::mbar_wait(&epi_done[sl], ((g - SM) / SM) & 1)) fail(7);
@@ -423,15 +456,16 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                     }
                 } else {
                     cnt = total - c * kNQ < kNQ ? total - c * kNQ : kNQ;
-                    stage_chunk<NQ>(a, it.y + c * kNQ, cnt, mrec(sl), sB + sb * bbuf,
+                    stage_chunk<NQ, PROD>(a, it.y + c * kNQ, cnt, mrec(sl), sB + sb * bbuf,
                                     sB + sb * bbuf + panels * bpanel, chunks16, ptid, sqid);
                     // the bound constants, once every producer's record copies have landed
                     cp_async_wait_all();
                     tc::named_sync(1, kProducers);
                     for (int j = ptid; j < cnt; j += kProducers) {
                         const TileRec &r = mrec(sl)[j];
-                        ab[(j >> 1) * 4 + (j & 1)] = r.alpha;
-                        ab[(j >> 1) * 4 + 2 + (j & 1)] = r.beta;
+                        const float2 c2 = PROD == 3 ? make_float2(r.alpha, r.beta) : a.ab_q[r.q];
+                        ab[(j >> 1) * 4 + (j & 1)] = c2.x;
+                        ab[(j >> 1) * 4 + 2 + (j & 1)] = c2.y;
                     }
                 }
                 if (ptid == 0) {
@@ -497,8 +531,10 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
                         tc::mma_bf16_ts(dt, tmem + ka + 8 * s, bh + po + 2 * s, idesc, (pnl | s) != 0);
-                        tc::mma_bf16_ts(dt, tmem + ka + 8 * s, bl + po + 2 * s, idesc, 1u);
-                        tc::mma_bf16_ts(dt, alo + ka + 8 * s, bh + po + 2 * s, idesc, 1u);
+                        if (PROD == 3) {
+                            tc::mma_bf16_ts(dt, tmem + ka + 8 * s, bl + po + 2 * s, idesc, 1u);
+                            tc::mma_bf16_ts(dt, alo + ka + 8 * s, bh + po + 2 * s, idesc, 1u);
+                        }
                     }
                 }
                 tc::mma_commit(&mma_done[sl]);
@@ -549,6 +585,10 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                 if (valid) {
                     xn2 = a.xn2[row];
                     xn = sqrtf(xn2) * (1.f + 1e-6f);
+                    if (PROD == 1)   // y_x, with the |q||x| term of cE2
+                        xn = __fmul_ru(__fadd_ru(__fmul_ru(2.02f, __fadd_ru(a.xr[row], __fmul_ru(__fadd_ru(*a.rho, a.cG), xn))),
+                                                 __fmul_ru(2.f * a.cE2, xn)),
+                                       1.f + 1e-6f);
                     if (a.any_deleted) rdel = a.row_del[row];
                 }
                 // rows outside the node block match no leaf bit
@@ -558,9 +598,7 @@ __global__ void __launch_bounds__(kThreadsWS, 1)
                 // the row's split coordinates into TMEM (rows outside the block:
                 // zeros).  Every MMA of the previous block is done: this warp
                 // has waited for the previous chunk's.
-                const int ncol = a.dim_p / 4;                  // this warp's share of A's dim_p columns
-                for (int p = 0; p < ncol; p += 16) {
-                    const int col = (warp >> 2) * ncol + p;
+                for (int col = (warp >> 2) * 16; col < acols; col += 64) {
                     const bool lo = col >= a.dim_p / 2;
                     const int k0 = 2 * (lo ? col - a.dim_p / 2 : col);   // first coordinate
                     uint32_t v[16];
@@ -726,11 +764,13 @@ __global__ void k_window_list(const uint32_t *__restrict__ bits, int64_t nn, int
 // each column position of the dense last level (query perm[i] at position i)
 __global__ void k_query_consts(const float *__restrict__ thr, const float *__restrict__ qn2,
                                const int64_t *__restrict__ qseq, const int32_t *__restrict__ perm, int64_t nq,
-                               float cE1, float cE2, float2 *__restrict__ ab, int64_t *__restrict__ seq) {
+                               float cE1, float cE2, int products, float2 *__restrict__ ab,
+                               int64_t *__restrict__ seq) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nq; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t q = perm ? (int64_t)perm[i] : i;
         float al, be;
         bound_consts(thr[q], qn2 ? qn2[q] : 0.f, cE1, cE2, al, be);
+        if (products == 1) al = sqrtf(qn2[q]) * (1.f + 2e-6f);   // |q|, against the rows' y_x
         ab[i] = make_float2(al, be);
         seq[i] = qseq[q];
     }
@@ -912,10 +952,10 @@ void count_offsets<int64_t>(const int64_t *cnt, int64_t *off, int64_t n, cudaStr
     else exscan(cnt, off, n + 1, st);
 }
 
-size_t tile_smem_bytes(int dim_p, int kNQ, int SB, int SM) {
+size_t tile_smem_bytes(int dim_p, int kNQ, int SB, int SM, int products) {
     const int panels = dim_p / 64;
     size_t b = 1024;                                              // alignment slack
-    b += (size_t)SB * 2 * panels * kNQ * 128;
+    b += (size_t)SB * (products == 3 ? 2 : 1) * panels * kNQ * 128;
     b += SM * ((size_t)kNQ * sizeof(TileRec) + (size_t)kNQ * 8 + 32);
     b += (3 * SM + 1) * 8 + 4 + 4 * 4 + 16 + (size_t)kNQ * 4;
     return b;
@@ -932,6 +972,8 @@ void tc_bound_coeffs(int dim_p, float &cE1, float &cE2) {
     cE2 = (float)(1.0 / 2097152.0);
 }
 
+float tc_gamma(int dim_p) { return (float)((dim_p + 2.0) / 8388608.0 * 1.02); }
+
 bool tc_supported(const Tree &t) { return t.metric == GTS_L2 && t.dim > 0 && t.dim <= 448 && t.n > 0; }
 
 void tc_prepare(Tree &t, TcCache &c, cudaStream_t st) {
@@ -940,24 +982,31 @@ void tc_prepare(Tree &t, TcCache &c, cudaStream_t st) {
     c.Xh.alloc((size_t)t.n * c.dim_p * 2, st);
     c.Xl.alloc((size_t)t.n * c.dim_p * 2, st);
     c.xn2.alloc(t.n, st);
+    c.xr.alloc(t.n, st);
     k_split_rows<<<nblk(t.n * 32), 256, 0, st>>>(t.X.get(), t.dim, c.dim_p, t.n, (__nv_bfloat16 *)c.Xh.get(),
-                                                (__nv_bfloat16 *)c.Xl.get(), c.xn2.get(), nullptr);
+                                                (__nv_bfloat16 *)c.Xl.get(), c.xn2.get(), nullptr, c.xr.get(), nullptr);
     check_launch("split rows");
     GTS_CUDA(cudaStreamSynchronize(st));
     c.Xh.persist();
     c.Xl.persist();
     c.xn2.persist();
+    c.xr.persist();
     c.ready = true;
 }
 
 void tc_split_queries(const float *Q, int64_t nq, int dim, int dim_p, DBuf<uint8_t> &Qh, DBuf<uint8_t> &Ql,
-                      DBuf<float> &qn2, cudaStream_t st, const int32_t *sel) {
+                      DBuf<float> &qn2, cudaStream_t st, const int32_t *sel, DBuf<float> *rho) {
     Qh.alloc((size_t)(nq > 0 ? nq : 1) * dim_p * 2, st);
     Ql.alloc((size_t)(nq > 0 ? nq : 1) * dim_p * 2, st);
     qn2.alloc(nq > 0 ? nq : 1, st);
+    if (rho) {
+        rho->alloc(1, st);
+        GTS_CUDA(cudaMemsetAsync(rho->get(), 0, 4, st));
+    }
     if (nq > 0)
         k_split_rows<<<nblk(nq * 32), 256, 0, st>>>(Q, dim, dim_p, nq, (__nv_bfloat16 *)Qh.get(),
-                                                   (__nv_bfloat16 *)Ql.get(), qn2.get(), sel);
+                                                   (__nv_bfloat16 *)Ql.get(), qn2.get(), sel, nullptr,
+                                                   rho ? rho->get() : nullptr);
     check_launch("split queries");
 }
 
@@ -1090,7 +1139,8 @@ int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegro
 }
 
 int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-               DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st, DBuf<float> *out_qx, int phase, int stride) {
+               DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st, DBuf<float> *out_qx,
+               int phase, int stride, int products) {
     *launches = 0;
     if (rg.n_items == 0) return 0;
     const int h = rg.h ? rg.h : t.h;
@@ -1100,21 +1150,25 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const TileShape shp = shape_for(c.dim_p, tq.chunk);
+    const TileShape shp = shape_for(c.dim_p, tq.chunk, products);
     const int nq_chunk = shp.nq;
     int smem_optin = 0;
     GTS_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     // TMEM: A (dim_p columns) and the slots' accumulators share 512 columns
-    GTS_REQUIRE(c.dim_p + shp.sm * nq_chunk <= 512, GTS_ECUDA, "tensor-core tile: TMEM columns");
-    const size_t smem = tile_smem_bytes(c.dim_p, nq_chunk, shp.sb, shp.sm);
+    GTS_REQUIRE((products == 3 ? c.dim_p : c.dim_p / 2) + shp.sm * nq_chunk <= 512, GTS_ECUDA, "tensor-core tile: TMEM columns");
+    const size_t smem = tile_smem_bytes(c.dim_p, nq_chunk, shp.sb, shp.sm, products);
     GTS_REQUIRE(smem <= (size_t)smem_optin, GTS_ECUDA, "tensor-core tile: shared memory");
     void (*kern)(const CUtensorMap, const CUtensorMap, TileArgs) =
-        nq_chunk == 96    ? k_tile_l2_tc<96, 4, 4>
-        : nq_chunk == 128 ? k_tile_l2_tc<128, 3, 3>
-        : shp.sb == 4     ? (nq_chunk == 64 ? k_tile_l2_tc<64, 4, 4> : k_tile_l2_tc<32, 4, 4>)
-        : nq_chunk == 64  ? k_tile_l2_tc<64, 2, 3>
-        : shp.sm == 4     ? k_tile_l2_tc<32, 2, 4>
-                          : k_tile_l2_tc<32, 2, 2>;
+        products == 1     ? (shp.nq == 64   ? k_tile_l2_tc<64, 3, 3, 1>
+                             : shp.sb == 3 ? k_tile_l2_tc<128, 3, 3, 1>
+                             : shp.sm == 3 ? k_tile_l2_tc<128, 2, 3, 1>
+                                           : k_tile_l2_tc<128, 2, 2, 1>)
+        : nq_chunk == 96  ? k_tile_l2_tc<96, 4, 4, 3>
+        : nq_chunk == 128 ? k_tile_l2_tc<128, 3, 3, 3>
+        : shp.sb == 4     ? (nq_chunk == 64 ? k_tile_l2_tc<64, 4, 4, 3> : k_tile_l2_tc<32, 4, 4, 3>)
+        : nq_chunk == 64  ? k_tile_l2_tc<64, 2, 3, 3>
+        : shp.sm == 4     ? k_tile_l2_tc<32, 2, 4, 3>
+                          : k_tile_l2_tc<32, 2, 2, 3>;
     GTS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // CTAs per SM: shared memory (each CTA also has 1 KB reserved), the 512
     // TMEM columns, and registers
@@ -1150,10 +1204,12 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
     }
     // windows: the queries' bound constants and sequence numbers in column
     // order, with the thresholds of this launch
-    DBuf<float2> abq(wl_on ? tq.nq : 1, st);
-    DBuf<int64_t> seqp(wl_on ? tq.nq : 1, st);
-    if (wl_on) {
-        k_query_consts<<<nblk(tq.nq), 256, 0, st>>>(tq.thr, tq.qn2, tq.qseq, tq.perm, tq.nq, cE1, cE2, abq.get(),
+    const bool consts = wl_on || products == 1;
+    DBuf<float2> abq(consts ? tq.nq : 1, st);
+    DBuf<int64_t> seqp(consts ? tq.nq : 1, st);
+    if (consts) {
+        k_query_consts<<<nblk(tq.nq), 256, 0, st>>>(tq.thr, tq.qn2, tq.qseq, tq.perm, tq.nq, cE1, cE2, products,
+                                                    abq.get(),
                                                     seqp.get());
         check_launch("query bound constants");
         ++*launches;
@@ -1194,6 +1250,9 @@ int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegro
         a.status = status.get();
         a.cE1 = cE1;
         a.cE2 = cE2;
+        a.cG = tc_gamma(c.dim_p);
+        a.xr = c.xr.get();
+        a.rho = tq.rho;
         a.any_deleted = tq.any_deleted;
         a.bits = rg.bits.get();
         a.wpre = rg.wpre.get();
@@ -1466,7 +1525,8 @@ void tc_prepare_pivots(const Tree &t, TcCache &c, cudaStream_t st) {
     c.pn2.alloc(nodes > 0 ? nodes : 1, st);
     if (nodes > 0)
         k_split_rows<<<nblk(nodes * 32), 256, 0, st>>>(t.X.get(), t.dim, c.dim_p, nodes, (__nv_bfloat16 *)c.Ph.get(),
-                                                       (__nv_bfloat16 *)c.Pl.get(), c.pn2.get(), t.npiv.get());
+                                                       (__nv_bfloat16 *)c.Pl.get(), c.pn2.get(), t.npiv.get(), nullptr,
+                                                       nullptr);
     check_launch("split pivots");
     GTS_CUDA(cudaStreamSynchronize(st));
     c.Ph.persist();

@@ -40,6 +40,8 @@ struct TileArgs {
     unsigned long long *out_count;
     int *status;
     float cE1, cE2;           // error-bound coefficients
+    float cG;                 // one product: its summation's (tc_gamma), the rows' |x - x_hi|, the batch's rho
+    const float *xr, *rho;
     int any_deleted;          // 0: no row has a delete mark, skip the visibility test
     // window mode (dense nodes): the node x query bitmap of the regrouping
     const uint32_t *bits;     // [nodes, nw]
@@ -63,6 +65,7 @@ struct TcQuery {
     int64_t E = 0;
     int64_t nq = 0;
     const __nv_bfloat16 *Qh = nullptr, *Ql = nullptr;   // split bf16 queries [nq, dim_p]
+    const float *rho = nullptr;                          // max |q - q_hi| / |q| (tc_split_queries)
     const float *qn2 = nullptr;                          // |q|^2 (null: not needed, records get 0)
     float cE1 = 0.f, cE2 = 0.f;                          // bf16 error-bound coefficients (tc_bound_coeffs)
     int chunk = 128;                                     // tensor-core tiles up to 128 columns: 128 or 96 queries
@@ -116,11 +119,13 @@ CUtensorMap tc_byte_map(const void *base, int64_t rows, int box_rows);
 bool tc_supported(const Tree &t);
 // |d~^2 - d^2| <= cE1 |q||x| + cE2 (|q| + |x|)^2 for the split-bf16 products over dim_p columns
 void tc_bound_coeffs(int dim_p, float &cE1, float &cE2);
+// one product: gamma_{K+2} of its FP32 summation
+float tc_gamma(int dim_p);
 void tc_prepare(Tree &t, TcCache &c, cudaStream_t st);
 // split a batch's queries into bf16 hi / lo rows [nq, dim_p] and squared norms
 // (sel: row i of the output is query sel[i]; null: query i)
 void tc_split_queries(const float *Q, int64_t nq, int dim, int dim_p, DBuf<uint8_t> &Qh, DBuf<uint8_t> &Ql,
-                      DBuf<float> &qn2, cudaStream_t st, const int32_t *sel = nullptr);
+                      DBuf<float> &qn2, cudaStream_t st, const int32_t *sel = nullptr, DBuf<float> *rho = nullptr);
 // whether tc_regroup counts entries per node itself (a node x query bitmap),
 // so the caller need not
 bool regroup_uses_bits(const Tree &t, int64_t nq, int64_t E, int h = 0);
@@ -138,10 +143,11 @@ int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegro
 // (and, given out_qx, each pair's q.x~: d~^2 = |q|^2 + |x|^2 - 2 q.x~ is within
 // tc_bound_coeffs' E of d^2).  stride > 1: phase 0 runs every stride-th item,
 // phase 1 the others, with the thresholds as they are at the call (window
-// chunks; gathered chunks keep their records').
+// chunks; gathered chunks keep their records').  products: 3, or 1 with its wider
+// bound (needs tq.rho).
 int64_t tc_run(const Tree &t, const TcCache &c, const TcQuery &tq, const TcRegroup &rg, DBuf<int32_t> &out_q,
                DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st,
-               DBuf<float> *out_qx = nullptr, int phase = 0, int stride = 1);
+               DBuf<float> *out_qx = nullptr, int phase = 0, int stride = 1, int products = 3);
 // Dense query-to-pivot distances of one pivot level on the tensor cores
 // (dim_p <= 256, after tc_prepare and tc_prepare_pivots): out[q, p] for the
 // batch's split queries; returns the level's absolute slack, an upper bound of
