@@ -282,17 +282,21 @@ __global__ void k_pivdist_str(Dev d, const int32_t *__restrict__ eq, const int32
 // Insert (u, id) into the ascending list D/I of n (<= K) distinct ids if it
 // belongs among the K smallest (u, id).  Warp-cooperative: every lane passes
 // the same arguments and gets the same n back; the duplicate test, the
-// insert position and the shift take n / 32 steps per lane.
+// insert position and the shift take n / 32 steps per lane.  Bounds are >= +0
+// and compare by their bits: the FP64 units would take sixteen cycles a
+// comparison (128 queries, k to 100: k_tau 0.54 -> 0.43 ms, the probe 0.45 -> 0.31).
 __device__ __forceinline__ void warp_tau_insert(double *D, int64_t *I, int &n, int K, double u, int64_t id,
                                                 int lane) {
-    if (n >= K && !(u < D[K - 1] || (u == D[K - 1] && id < I[K - 1]))) return;
+    const long long ub = __double_as_longlong(u);
+    const long long *B = reinterpret_cast<const long long *>(D);
+    if (n >= K && !(ub < B[K - 1] || (ub == B[K - 1] && id < I[K - 1]))) return;
     bool dup = false;
     int below = 0;
     for (int i = lane; i < n; i += 32) {
-        const double di = D[i];
+        const long long di = B[i];
         const int64_t ii = I[i];
         dup |= ii == id;
-        below += (di < u || (di == u && ii < id)) ? 1 : 0;
+        below += (di < ub || (di == ub && ii < id)) ? 1 : 0;
     }
     if (__any_sync(0xffffffffu, dup)) return;
 #pragma unroll
@@ -357,14 +361,16 @@ struct TauList {
             warp_tau_insert(D, I, n, K, u, id, lane);
             return;
         }
+        const long long ub = __double_as_longlong(u);
         if (n >= K) {
-            const double k_d = kd();
+            const long long k_d = __double_as_longlong(kd());
             const int64_t k_i = kid();
-            if (!(u < k_d || (u == k_d && id < k_i))) return;
+            if (!(ub < k_d || (ub == k_d && id < k_i))) return;
         }
         const bool live = lane < n;
         if (__any_sync(0xffffffffu, live && ri == id)) return;
-        const int below = __popc(__ballot_sync(0xffffffffu, live && (rd < u || (rd == u && ri < id))));
+        const long long rb = __double_as_longlong(rd);
+        const int below = __popc(__ballot_sync(0xffffffffu, live && (rb < ub || (rb == ub && ri < id))));
         const double pd = __shfl_up_sync(0xffffffffu, rd, 1);
         const int64_t pi = (int64_t)__shfl_up_sync(0xffffffffu, (long long)ri, 1);
         const int last = n < K ? n : K - 1;   // entries [below, last) move up one; a full list drops entry K-1
