@@ -518,8 +518,8 @@ __device__ __forceinline__ void list_dists(const Dev &d, const float *__restrict
 // rows took 0.82 ms (10^4 queries, 10^6 x 128), 2.83 ms (10^4, 2 * 10^5 x 300)
 // and 0.90 ms (128 queries, 2 * 10^6 x 256, L1).
 template <bool L2, int G, bool V4>
-__global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int max_rows, int per_k, const int32_t *__restrict__ kq,
-                            const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n, float *tau,
+__global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int max_rows, int least, int per_k,
+                            const int32_t *__restrict__ kq, const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id, int32_t *tk_n, float *tau,
                             int32_t *__restrict__ key) {
     __shared__ int32_t s_row[256];
     __shared__ float s_dist[256];
@@ -531,8 +531,8 @@ __global__ void k_probe_vec(Dev d, LevelOffsets lo_off, int max_rows, int per_k,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t q = blockIdx.x;
     const int K = kq[q];
-    // rows: 256, or per_k for each neighbour wanted (per_k 0: max_rows)
-    const int cap = per_k ? min(max_rows, max(256, per_k * K)) : max_rows;
+    // rows: `least`, or per_k for each neighbour wanted (per_k 0: max_rows)
+    const int cap = per_k ? min(max_rows, max(least, per_k * K)) : max_rows;
     const int64_t s = d.qseq[q];
     const float *qv = d.Q + q * d.dim;
     const double up = 1.0 + 2.0 * (double)d.rel;
@@ -4788,10 +4788,20 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         // a row of more than 16 coordinates costs as much as five of the kept
         // pairs that it saves from 256 rows on (16 a neighbour for large k);
         // a row of a few coordinates next to nothing
-        const int per_k = t.dim > kScanMaxDim ? 16 : 0;
+        int per_k = t.dim > kScanMaxDim ? 16 : 0, least = 256;
+        // The tiles' first phase lowers the thresholds better than the probe:
+        // 64 rows, or four a neighbour, then do (10^4 queries, rows 512 / 256 /
+        // 128 / 64: 10^6 x 128 6.65 / 6.64 / 6.54 / 6.48 ms, angular 2 * 10^5 x
+        // 300 5.27 / 5.28 / 5.04 / 4.92)
+        const int64_t blocks = std::max(t.lvl_off[t.h] - t.lvl_off[t.h - 1], t.n / 128);
+        if (R.use_tc && qb.max_k <= 32 && blocks >= kTilePhaseItems && per_k) {
+            per_k = 4;
+            least = 64;
+        }
         const bool v4 = (t.dim & 3) == 0 && (((uintptr_t)d.Q | (uintptr_t)d.X) & 15) == 0;
 #define GTS_PROBE(L2V, GV, V4V)                                                                                      \
-    k_probe_vec<L2V, GV, V4V><<<(unsigned)nq, 32 * nw, 0, st>>>(d, lo_off, cap, per_k, qb.k, R.koff.get(), R.tk_d.get(),     \
+    k_probe_vec<L2V, GV, V4V><<<(unsigned)nq, 32 * nw, 0, st>>>(d, lo_off, cap, least, per_k, qb.k, R.koff.get(),       \
+                                                               R.tk_d.get(),                                        \
                                                                R.tk_id.get(), R.tk_n.get(), R.thr.get(), R.qkey.get())
         if (t.metric == GTS_L2) {
             if (t.dim <= kScanMaxDim) GTS_PROBE(true, 1, false);
