@@ -898,16 +898,19 @@ __global__ void k_items_per_node(const int32_t *__restrict__ ncount, const int32
     if (blockIdx.x == 0 && threadIdx.x == 0) nitems[nn] = 0;
 }
 
-// win_min: nodes with at least this many entries get window-mode items
+// win_min: nodes with at least this many entries get window-mode items.  A warp
+// per node: one node may hold every block (7,800 took one thread 0.1 ms).
 __global__ void k_fill_items(const int32_t *__restrict__ ncount, const int32_t *__restrict__ nsize,
                              const int64_t *__restrict__ noff, const int64_t *__restrict__ ioff, int64_t nn,
                              int64_t win_min, int4 *__restrict__ items) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nn; i += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nn; i += nw) {
         const int32_t c = ncount[i];
         if (c == 0) continue;
         const int32_t blocks = (nsize[i] + kRows - 1) / kRows;
         const int flag = c >= win_min ? kWindowItem : 0;
-        for (int32_t b = 0; b < blocks; ++b) items[ioff[i] + b] = make_int4((int)i, (int)noff[i], c, b | flag);
+        for (int32_t b = lane; b < blocks; b += 32) items[ioff[i] + b] = make_int4((int)i, (int)noff[i], c, b | flag);
     }
 }
 
@@ -1098,7 +1101,7 @@ int64_t tc_regroup(const Tree &t, const TcQuery &tq, TcRegroup &rg, cudaStream_t
         rg.items.alloc(total_items, st);
         // window mode for nodes holding at least half of the batch
         const int64_t win_min = (use_bits && window_ok) ? std::max<int64_t>(1, (tq.nq + 1) / 2) : INT64_MAX;
-        k_fill_items<<<nblk(nn), 256, 0, st>>>(ncnt, lsize, noff.get(), ioff.get(), nn, win_min, rg.items.get());
+        k_fill_items<<<nblk(nn * 32), 256, 0, st>>>(ncnt, lsize, noff.get(), ioff.get(), nn, win_min, rg.items.get());
     }
     check_launch("tile regroup");
     return total_items;
@@ -1132,7 +1135,7 @@ int64_t tc_dense_items(const Tree &t, int64_t nq, const uint64_t *dmask, TcRegro
     rg.n_chunks = 0;
     if (total_items > 0) {
         rg.items.alloc(total_items, st);
-        k_fill_items<<<nblk(nn), 256, 0, st>>>(ncnt.get(), lsize, rg.noff.get(), ioff.get(), nn, 0, rg.items.get());
+        k_fill_items<<<nblk(nn * 32), 256, 0, st>>>(ncnt.get(), lsize, rg.noff.get(), ioff.get(), nn, 0, rg.items.get());
     }
     check_launch("dense tile items");
     return total_items;
