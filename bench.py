@@ -54,16 +54,11 @@ FP32_LANES_PER_SM = 128       # FP32 FMA lanes per SM
 ALU_LANES_PER_SM = 64         # integer / bit-logic ALU pipe: 2 warp instructions per SM cycle (ncu: the ALU
                               # instructions executed per active SM cycle are exactly 2 x its pipe utilization)
 
-# DRAM bytes per launch of the dominant kernel from one ncu capture (profiles/):
-# k_tile_l2_tc at half size, 0.467 GB read + write (node rows, the node x
-# query leaf-mask matrix and the kept pairs' q.x), all of which double at full
-# size.  None once the kernel has changed since the counters were taken.
-TRAFFIC = {"kernel": "tile", "bytes_per_launch": 0.934e9}
-# the zipf2d table scan (k_scan_warps, fused range form): DRAM read + write of
-# one launch over a 10,000-query batch from its ncu capture
-# (profiles/scan_warps_zipf2d_10M.md), 227.1 + 101.6 MB.  None once the kernel
-# changes.
-SCAN_TRAFFIC = 328.7e6
+# DRAM bytes per launch of the dominant kernel and of the zipf2d table scan
+# (k_scan_warps, fused range form).  None: the kernels have changed since their
+# counters were taken (profiles/).
+TRAFFIC = {"kernel": "tile", "bytes_per_launch": None}
+SCAN_TRAFFIC = None
 
 # ALU-pipe thread instructions per full-DP-equivalent cell (|q| x |o| per pair)
 # of the bit-parallel edit-distance kernels: sm__inst_executed_pipe_alu.sum x 32
@@ -312,8 +307,8 @@ def run_ours(args):
         # a contraction on the tensor cores: the algorithm's work is 2 D flops
         # per (query, row) pair that passes the table lower bound (C_q), against
         # the sustained bf16 peak (the kernel runs inside a long step).  The
-        # tiles compute every row of a surviving node block (covered pairs),
-        # and the split-bf16 form executes 3 products per pair.
+        # tiles compute every row of a surviving node block (covered pairs)
+        # with three split-bf16 products or, in a second phase, one.
         tf, tsrc = tensor_peak()
         sec = dom_ms / 1e3
         achieved = cq * 2 * dim / sec / 1e12 if dom_ms > 0 else 0.0
@@ -324,8 +319,7 @@ def run_ours(args):
                 "launches_per_step": stage_launch[dom], "ms_per_step": round(dom_ms, 4),
                 "algorithmic_pairs_per_step": int(cq),
                 "covered_pairs_per_step": int(stats0["tile_pairs"]),
-                "covered_tflops": round(covered, 1), "covered_frac": round(covered / tf, 4),
-                "executed_tflops": round(3 * covered, 1), "executed_frac": round(3 * covered / tf, 4)}
+                "covered_tflops": round(covered, 1), "covered_frac": round(covered / tf, 4)}
     else:
         roof = {"bound": "latency", "kernel": dom, "achieved": None, "peak": None, "unit": None, "frac": None,
                 "traffic": None, "launches_per_step": stage_launch[dom], "ms_per_step": round(dom_ms, 4)}
@@ -756,7 +750,7 @@ def bench_wordvec(args):
         out["roofline"] = {"bound": "tensor", "kernel": "k_tile_l2_tc (stage tile)", "achieved": round(ach, 2),
                            "peak": tf, "unit": "TFLOP/s", "frac": round(ach / tf, 5), "peak_source": tsrc,
                            "traffic": None, "ms_per_step": round(stage_ms[dom], 4),
-                           "covered_tflops": round(cov, 1), "executed_tflops": round(3 * cov, 1)}
+                           "covered_tflops": round(cov, 1)}
     else:
         out["roofline"] = {"bound": "latency", "kernel": dom, "achieved": None, "peak": None, "frac": None,
                            "traffic": None, "ms_per_step": round(stage_ms[dom], 4)}

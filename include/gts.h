@@ -65,7 +65,12 @@ typedef enum { GTS_EDIT = 0, GTS_L1 = 1, GTS_L2 = 2, GTS_COS = 3 } gts_metric;
 /* Verification precision for L2.  Both give the same result sets:
  *  GTS_PREC_FP32: FP32 CUDA-core distances, FP64 recheck of candidates whose
  *                 FP32 distance lies within a proven error bound of the radius
- *                 or of the running k-th distance.
+ *                 or of the running k-th distance.  Candidate by candidate, or
+ *                 for batches with enough (query, object) pairs in node-major
+ *                 FP32 tiles (the table scan up to 16 dimensions); up to eight
+ *                 queries over objects that are read in one pass (a GiB) take
+ *                 that pass instead of the descent.  With GTS_QUERY_COUNT_TABLE_PASS
+ *                 or a memory budget below 1 GiB always candidate by candidate.
  *  GTS_PREC_BF16: BF16 tensor-core distance tiles with FP32 accumulation and the
  *                 same FP64 recheck against a (wider) proven BF16 bound
  *                 (17 <= dim <= 448; vectors of at most 16 dimensions take the
@@ -74,7 +79,8 @@ typedef enum { GTS_EDIT = 0, GTS_L1 = 1, GTS_L2 = 2, GTS_COS = 3 } gts_metric;
  * same node-major tiles on the CUDA cores in FP32 (the arithmetic and the FP64
  * recheck of GTS_PREC_FP32, batched by node instead of by candidate); this
  * needs dim % 4 == 0 and 16-byte aligned query rows, else the plain path runs.
- * Edit distance ignores this field (exact int). */
+ * Edit distance is exact either way; GTS_PREC_BF16 sends batches of every size
+ * through the 3-gram tiles, GTS_PREC_FP32 large ones. */
 typedef enum { GTS_PREC_FP32 = 0, GTS_PREC_BF16 = 1 } gts_precision;
 
 /* A set of objects: vectors (dim > 0) or byte strings (dim == 0).
@@ -156,8 +162,9 @@ enum {
     GTS_STAT_GROUPS = 6,       /* query groups run by the two-stage scheduler */
     GTS_STAT_CACHE_ROWS = 7,   /* cache-list objects compared by brute force */
     GTS_STAT_LAUNCHES = 8,     /* kernels launched by the call */
-    GTS_STAT_TILES = 9,        /* tile work items: 128-row blocks of last-level nodes */
-    GTS_STAT_TILE_ENTRIES = 10,/* (query, last-level node) entries run against those blocks */
+    GTS_STAT_TILES = 9,        /* tile work items: 128-row blocks of nodes (last-level ones, or of a level
+                                  above where a range batch stops there) */
+    GTS_STAT_TILE_ENTRIES = 10,/* (query, node) entries run against those blocks */
     GTS_STAT_TILE_PAIRS = 11,  /* (query, row) pairs whose distance the tiles computed */
     GTS_STAT_DENSE_PAIRS = 12, /* (query, pivot) distances computed as dense per-level matrices */
     GTS_STAT_DENSE_LAST = 13,  /* 1 if the last level ran as dense matrices (no entry list) */
@@ -329,15 +336,17 @@ gts_status gts_multi_knn(gts_index *const *cols, int32_t m, const gts_objects *q
  *              node blocks with tau_q lowered from the answer so far in
  *              between (default 3).
  *  probe_rows: kNN probe, object rows evaluated before the descent to bound
- *              the k-th distance, 0 .. 4096 (default 1024).
+ *              the k-th distance, 0 .. 4096 (default 1024): at most that many,
+ *              taken from the rows nearest in the table; above 16 dimensions
+ *              256, or 16 per neighbour wanted if that is more.
  *  tc_queries: BF16 tensor-core tiles for dim <= 128, queries per chunk:
  *              128 (two staging slots, default) or 96 (three slots).
  *  str_chunk:  edit distance, (query, object) pairs per block of the
- *              bit-parallel DP kernels (pivot distances and verification):
- *              64, 128, 256 (default) or 512.
- *  str_qgram:  edit distance with GTS_PREC_BF16, the 3-gram count filter
- *              before the DP: 0 = off (the table scan alone), or its queries
- *              per tile chunk, 32 or 64 (default).
+ *              bit-parallel DP kernels (pivot distances, at most so many, and
+ *              verification): 64, 128, 256 (default) or 512.
+ *  str_qgram:  edit distance, the 3-gram count filter before the DP: 0 = off
+ *              (the table scan alone), or its queries per tile chunk on the
+ *              CUDA cores, 32 or 64 (default).
  *  tuned:      output only: 1 once gts_autotune has run on the index. */
 typedef struct {
     int32_t l1_queries;

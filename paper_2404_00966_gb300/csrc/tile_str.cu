@@ -9,12 +9,12 @@
 // (a substitution changes at most 3 of a string's 3-grams, an insertion or a
 // deletion at most 2 old and 3 new ones; summing counts into buckets and
 // capping them at 255 can only lower the L1 distance), so L1 > 6 t proves
-// d > t.  The surviving (query, last-level node) entries are regrouped by
-// node; one CTA takes a block of up to 128 node rows (each thread holds one
-// row's 64-byte bucket vector in registers) and the node's queries in chunks
-// of 32 or 64 (their vectors in shared memory); a pair is kept if the row's leaf
-// survived for the query, the row is visible
-// at the query's sequence number and the bound does not exclude it.  The
+// d > t.  The surviving (query, node) entries are regrouped by node; one CTA
+// takes a block of up to 128 node rows (a lane holds four rows' 64-byte bucket
+// vectors in registers) and the node's queries in chunks of 32 or 64 (their
+// vectors in shared memory); a pair is kept if the row's leaf survived for the
+// query, the row is visible at the query's sequence number and the bound does
+// not exclude it.  Well-filled batches take tile_qtc.cu instead.  The
 // kept pairs go on to the exact DP.
 #include "gts_impl.cuh"
 #include "metric.cuh"

@@ -723,8 +723,8 @@ __global__ void k_node_hist(const int32_t *__restrict__ enode, const uint64_t *_
 }
 
 // scatter each entry's record (query, threshold, norms, sequence number,
-// leaf mask) and path distances to its node's slot, so a tile reads its
-// queries' data contiguously
+// leaf mask) and, for the table scan, path distances to its node's slot, so a
+// tile reads its queries' data contiguously
 // the per-query constants of the squared-form bound test, all rounded up:
 // keep iff d~^2 <= thr^2 + cE1 |q||x| + cE2 (|q| + |x|)^2 with
 // d~^2 = |q|^2 + |x|^2 - 2 q.x, i.e. -2 q.x <= beta + alpha |x| + gamma_x,
