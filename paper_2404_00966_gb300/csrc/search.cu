@@ -403,54 +403,101 @@ __global__ void k_query_runs(const int32_t *__restrict__ cq, int64_t C, int64_t 
 // Warp per query.  The query's list of the k smallest (upper bound, id) of
 // distinct visible pivots seen so far is merged with this level's entries;
 // tau_q = the k-th bound, rounded up to float, or +inf while fewer than k.
+// An insertion is a chain of dependent steps, and a list that starts empty takes
+// k ln(n / k) of them: for k <= 128 and enough entries, a first pass finds the
+// k-th smallest of 128 minima (four a lane), which is at least the k-th smallest
+// of all, and only entries up to it are looked at.  Where too few of those were
+// visible or new, a second pass takes the others.  (128 queries, k to 100, 8,400
+// entries: 0.43 -> 0.31 ms; 2,000 queries, k = 10: 0.30 -> 0.14.)
 __global__ void k_tau(Dev d, const int64_t *__restrict__ qrun, const int32_t *__restrict__ enode, int64_t lvl_base,
                       int64_t e0, int64_t e1, const float *__restrict__ path, int l, int64_t nq,
                       const int32_t *__restrict__ kq, const int64_t *__restrict__ koff, double *tk_d, int64_t *tk_id,
                       int32_t *tk_n, float *tau) {
+    constexpr int kAhead = 4;   // loads in flight
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < nq; q += nw) {
-    const int64_t a = e0 + qrun[q], b = e0 + qrun[q + 1];
-    if (a == b) continue;
-    const int K = kq[q];
-    TauList L;
-    L.load(tk_d + koff[q], tk_id + koff[q], tk_n[q], K, lane);
-    const int64_t s = d.qseq[q];
+    const float inf = __int_as_float(0x7f800000);
     const double up = 1.0 + 2.0 * (double)d.rel;
-    for (int64_t base = a; base < b; base += 32) {
-        const int64_t e = base + lane;
-        const bool full = L.n >= K;
-        const double k_d = full ? L.kd() : 0.0;
-        const int64_t k_i = full ? L.kid() : 0;
-        bool cand = false;
-        double ub = 0.0;
-        int64_t id = 0;
-        if (e < b) {
-            const float dv = path[e * d.h + l];
-            ub = d.rel > 0.f ? (double)dv * up + (double)d.absf + (double)d.lslack[l] : (double)dv;
-            if (!full || ub <= k_d) {   // the bound test before the pivot's delete mark
-                const int32_t prow = d.npiv[lvl_base + enode[e]];
-                if (row_visible(d, prow, s)) {
-                    id = d.row_id[prow];
-                    cand = !full || ub < k_d || (ub == k_d && id < k_i);
+    auto bound = [&](float dv) -> double {
+        return d.rel > 0.f ? (double)dv * up + (double)d.absf + (double)d.lslack[l] : (double)dv;
+    };
+    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < nq; q += nw) {
+        const int64_t a = e0 + qrun[q], b = e0 + qrun[q + 1];
+        if (a == b) continue;
+        const int K = kq[q];
+        TauList L;
+        L.load(tk_d + koff[q], tk_id + koff[q], tk_n[q], K, lane);
+        const int64_t s = d.qseq[q];
+        float gate = inf;
+        if (K <= 128 && b - a >= 512) {
+            float m[kAhead] = {inf, inf, inf, inf};
+            for (int64_t base = a; base < b; base += 32 * kAhead) {
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const int64_t e = base + 32 * u + lane;
+                    if (e < b) m[u] = fminf(m[u], path[e * d.h + l]);
                 }
             }
+            // the largest x with fewer than K minima below it (distances are >= +0)
+            uint32_t x = 0;
+            for (int bit = 30; bit >= 0; --bit) {
+                const uint32_t y = x | (1u << bit);
+                int below = 0;
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u)
+                    below += __popc(__ballot_sync(0xffffffffu, __float_as_uint(m[u]) < y));
+                if (below < K) x = y;
+            }
+            if (x < 0x7f800000u) gate = __uint_as_float(x);
         }
-        unsigned bal = __ballot_sync(0xffffffffu, cand);
-        while (bal) {
-            const int src = __ffs(bal) - 1;
-            bal &= bal - 1;
-            const double u = __shfl_sync(0xffffffffu, ub, src);
-            const int64_t iid = __shfl_sync(0xffffffffu, id, src);
-            L.insert(u, iid);
+        for (int pass = 0; pass < 2; ++pass) {
+            for (int64_t base4 = a; base4 < b; base4 += 32 * kAhead) {
+                float dvs[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const int64_t e = base4 + 32 * u + lane;
+                    dvs[u] = e < b ? path[e * d.h + l] : inf;
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const int64_t e = base4 + 32 * u + lane;
+                    const float dv = dvs[u];
+                    if (!__any_sync(0xffffffffu, e < b && dv <= gate)) continue;
+                    const bool full = L.n >= K;
+                    const double k_d = full ? L.kd() : 0.0;
+                    const int64_t k_i = full ? L.kid() : 0;
+                    bool cand = false;
+                    double ub = 0.0;
+                    int64_t id = 0;
+                    if (e < b && dv <= gate) {
+                        ub = bound(dv);
+                        if (!full || ub <= k_d) {   // the bound test before the pivot's delete mark
+                            const int32_t prow = d.npiv[lvl_base + enode[e]];
+                            if (row_visible(d, prow, s)) {
+                                id = d.row_id[prow];
+                                cand = !full || ub < k_d || (ub == k_d && id < k_i);
+                            }
+                        }
+                    }
+                    unsigned bal = __ballot_sync(0xffffffffu, cand);
+                    while (bal) {
+                        const int src = __ffs(bal) - 1;
+                        bal &= bal - 1;
+                        const double uu = __shfl_sync(0xffffffffu, ub, src);
+                        const int64_t iid = __shfl_sync(0xffffffffu, id, src);
+                        L.insert(uu, iid);
+                    }
+                }
+            }
+            if (gate == inf || (L.n >= K && L.kd() <= bound(gate))) break;
+            gate = inf;
         }
-    }
-    L.store();
-    const double k_fin = L.n >= K ? L.kd() : 0.0;
-    if (lane == 0) {
-        tk_n[q] = L.n;
-        tau[q] = L.n >= K ? __double2float_ru(k_fin) : __int_as_float(0x7f800000);
-    }
+        L.store();
+        const double k_fin = L.n >= K ? L.kd() : 0.0;
+        if (lane == 0) {
+            tk_n[q] = L.n;
+            tau[q] = L.n >= K ? __double2float_ru(k_fin) : inf;
+        }
     }
 }
 
