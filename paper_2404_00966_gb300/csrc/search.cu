@@ -3315,6 +3315,13 @@ struct Runner {
             if (total == 0) return;
             const int64_t cand_bytes = 4 + 4 + 4 + 1 + 8 + 16;
             auto gb = groups(off, E, total, (budget / 2) / cand_bytes);
+            // every group writes with the thresholds it was counted with: collect()
+            // may lower tau_q between two groups (edit distance), and a pass that
+            // writes fewer candidates than were counted leaves the others unset
+            DBuf<float> thr_counted(knn && gb.size() > 2 ? qb.nq : 0, st);
+            if (thr_counted.get())
+                GTS_CUDA(cudaMemcpyAsync(thr_counted.get(), thr.get(), qb.nq * 4, cudaMemcpyDeviceToDevice, st));
+            const float *wthr = thr_counted.get() ? thr_counted.get() : thr.get();
             for (size_t g = 0; g + 1 < gb.size(); ++g) {
                 const int64_t g0 = gb[g], g1 = gb[g + 1];
                 int64_t o0 = 0, o1 = 0;
@@ -3327,11 +3334,11 @@ struct Runner {
                 if (small_nodes)
                     k_leafscan_small<true><<<nblocks(g1 - g0, kT), kT, 0, st>>>(
                         d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0,
-                        thr.get(), nullptr, goff, cq.get(), crow.get(), nullptr);
+                        wthr, nullptr, goff, cq.get(), crow.get(), nullptr);
                 else
-                k_leafscan<true><<<nblocks(g1 - g0, kWarpsPerBlock), kT, 0, st>>>(
-                    d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0, thr.get(),
-                    nullptr, goff, cq.get(), crow.get(), nullptr);
+                    k_leafscan<true><<<nblocks(g1 - g0, kWarpsPerBlock), kT, 0, st>>>(
+                        d, L.q.get(), L.node.get(), L.path.get(), lvl_last, e0 + g0, e0 + g1, mask.get() + g0, wthr,
+                        nullptr, goff, cq.get(), crow.get(), nullptr);
                 clk.end();
                 check_launch("leaf scan write");
                 verify_and_collect(cq, crow, C);
