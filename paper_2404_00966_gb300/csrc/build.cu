@@ -172,22 +172,35 @@ __global__ void k_map_vec(const float *__restrict__ X, int dim, const int32_t *_
 // The table holds RN32(d) of the FP64 distance summed in the reference order,
 // and GB300 has 2 FP64 lanes per SM and cycle: three FP64 operations per
 // coordinate of 10^6 x 128 take 0.61 ms per level (1.21 ms measured, a thread
-// per row; this form 0.34 ms), eight times the pass over the rows.  Here eight lanes take a row:
-// every difference (exact, Knuth's two-sum), square (Dekker's product by a
-// fused multiply-add) and partial sum is an unevaluated FP32 pair, and the
-// pair's proven error decides whether the FP32 rounding of the distance is
-// certain; if it is not (a few rows in ten thousand), the lane that holds the
-// row sums it in FP64 in the reference order.  The values are those of
-// k_map_vec bit for bit.
+// per row; this form 0.18 ms), eight times the pass over the rows.  Here eight
+// lanes sum a row: every difference (exact, Knuth's two-sum), square (Dekker's
+// product by a fused multiply-add) and partial sum is an unevaluated FP32 pair.
+// Then one warp of the block takes its 32 rows, a lane each: the pair's proven
+// error decides whether the FP32 rounding of the distance is certain; if it is
+// not (a few rows in ten thousand), the lane sums the row in FP64 in the
+// reference order.  The values are those of k_map_vec bit for bit.
+// (The test is some 19 FP64 instructions: by the lanes that had the sums, four
+// rows a warp, it took more FP64 time than the distances of up to 40 coordinates.)
 //
-// Error of a lane's pair over n = ceil(dim / 8) + 3 terms, u = 2^-24, S the
-// sum: |lo| <= (n + 3) u S, two roundings of lo per term, the products'
-// dropped and rounded parts below 8 u^2 S, three merges: below (n^2 + 8 n +
-// 40) 2^-47 S; kMapErr doubles it, which also covers the FP64 reference's own
-// (dim + 4) 2^-53.  Results outside [1e-18, 1e30], where FP32 squares could
-// lose their low parts or overflow, take FP64.
+// Error of a lane's pair over n <= dim / 8 + 4 terms, u = 2^-24, S the sum: lo is
+// folded into hi every four terms, so |lo| <= u S after that and at most 8 u S
+// before the next (each term's part of lo is below u S + 3 u p_i, p_i its square);
+// a term's two roundings of lo then add u^2 (10 S + 3 p_i), the products' dropped
+// and rounded parts 4 u^2 p_i, the three merges 60 u^2 S: below (10 n + 70) u^2 S
+// in all.  `del` is more than twice that, which also covers the FP64 reference's own
+// (dim + 4) 2^-53.  (Without the folding the error grows with the square of the
+// terms, and from 3,000 dimensions on many rows took FP64.)  Results outside [1e-18,
+// 1e30], where FP32 squares could lose their low parts or overflow, take FP64.
 constexpr int kMapLanes = 8;
-constexpr int kMapSingleDim = 8;   // up to this dimension a thread sums a row in FP64 (a lane would hold one term)
+// Up to these dimensions a thread sums a row in FP64, which is then as fast (L1
+// has one FP64 operation less per coordinate).  Builds of 10^6 rows, a thread a row / this form, us:
+// L2, 8 dimensions 2149 / 2084, 9: 2215 / 2048, 24: 2793 / 2200; L1, 9: 2083 / 2178,
+// 16: 2285 / 2272, 17: 2362 / 2224.  (Of 20,000 rows both take 0.52 ms up to 24.)
+constexpr int kMapSingleL2 = 8, kMapSingleL1 = 16;
+constexpr int kMapRows = kThreads / kMapLanes;   // rows of a block: one per lane of the warp that decides
+static_assert(kMapRows == 32, "one row per lane of the deciding warp");
+
+inline double map_error(int dim) { return (10.0 * (dim / 8 + 4) + 80.0) / 140737488355328.0; }   // 2^-47
 
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
@@ -213,6 +226,12 @@ __device__ __forceinline__ void ds_add_term(float a, float b, float &hi, float &
     hi = t;
     lo = __fadd_rn(lo, __fadd_rn(r, q));
 }
+// lo into hi (|lo| <= hi: the short form of the two-sum is exact)
+__device__ __forceinline__ void ds_fold(float &hi, float &lo) {
+    const float t = __fadd_rn(hi, lo);
+    lo = __fsub_rn(lo, __fsub_rn(t, hi));
+    hi = t;
+}
 
 // RN32 of the distance whose (L2: squared) value lies within a relative del
 // of hi + lo, or -1 if two FP32 values are possible (or the first guess, one
@@ -233,24 +252,21 @@ __device__ __forceinline__ float ds_round(float hi_s, float lo_s, double S, doub
     return lo < S * (1.0 - del) && S * (1.0 + del) < hi ? r : -1.f;
 }
 
+// block b: the rows at positions [32 b, 32 b + 32)
 template <bool L2, bool V4>
 __global__ void __launch_bounds__(kThreads) k_map_vec_ds(const float *__restrict__ X, int dim,
                                                          const int32_t *__restrict__ perm,
                                                          const int32_t *__restrict__ pos_node,
                                                          const int32_t *__restrict__ piv_obj, int64_t n, double del,
                                                          float *__restrict__ Tl, int32_t *__restrict__ node_of) {
+    __shared__ float s_hi[kMapRows], s_lo[kMapRows];   // hi < 0: every difference was 0
     const int sub = threadIdx.x & (kMapLanes - 1);
-    const int64_t rows = (int64_t)gridDim.x * blockDim.x / kMapLanes;
-    // (p0 is the warp's first row: every lane runs the same iterations)
-    for (int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / kMapLanes; p0 < n; p0 += rows) {
-        const int64_t p = p0 + (threadIdx.x & 31) / kMapLanes;
-        const bool in = p < n;
-        const int32_t o = in ? perm[p] : 0;
-        const int32_t node = in ? pos_node[p] : 0;
-        const float *a = X + (int64_t)o * dim;
-        const float *b = X + (int64_t)(in ? piv_obj[node] : 0) * dim;
+    const int64_t p0 = (int64_t)blockIdx.x * kMapRows;
+    {
+        const int64_t p = p0 + threadIdx.x / kMapLanes;
         float hi = 0.f, lo = 0.f, big = 0.f;
-        if (in) {
+        if (p < n) {
+            const float *a = X + (int64_t)perm[p] * dim, *b = X + (int64_t)piv_obj[pos_node[p]] * dim;
             if (V4) {
                 const float4 *a4 = reinterpret_cast<const float4 *>(a), *b4 = reinterpret_cast<const float4 *>(b);
 #pragma unroll 4
@@ -260,10 +276,14 @@ __global__ void __launch_bounds__(kThreads) k_map_vec_ds(const float *__restrict
                     ds_add_term<L2>(x.y, y.y, hi, lo, big);
                     ds_add_term<L2>(x.z, y.z, hi, lo, big);
                     ds_add_term<L2>(x.w, y.w, hi, lo, big);
+                    ds_fold(hi, lo);
                 }
             } else {
 #pragma unroll 4
-                for (int i = sub; i < dim; i += kMapLanes) ds_add_term<L2>(a[i], b[i], hi, lo, big);
+                for (int i = sub; i < dim; i += kMapLanes) {
+                    ds_add_term<L2>(a[i], b[i], hi, lo, big);
+                    if ((i & (3 * kMapLanes)) == 3 * kMapLanes) ds_fold(hi, lo);   // every fourth of the lane's terms
+                }
             }
         }
 #pragma unroll
@@ -275,20 +295,28 @@ __global__ void __launch_bounds__(kThreads) k_map_vec_ds(const float *__restrict
             lo = __fadd_rn(__fadd_rn(lo, l2), r);
             big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, off));
         }
-        if (in && sub == 0) {
-            const double S = (double)hi + (double)lo;
-            float r = -1.f;
-            if (big == 0.f) r = 0.f;   // (a NaN cannot occur: builds reject non-finite coordinates)
-            else if (S >= 1e-18 && S <= 1e30) r = ds_round<L2>(hi, lo, S, del);
-            if (r < 0.f) {
-                double d = L2 ? l2sq_fp64_seq(a, b, dim) : l1_fp64_seq(a, b, dim);
-                if (L2) d = __dsqrt_rn(d);
-                r = __double2float_rn(d);
-            }
-            Tl[o] = r;
-            node_of[o] = node;
+        if (sub == 0) {
+            s_hi[threadIdx.x / kMapLanes] = big == 0.f ? -1.f : fmaxf(hi, 0.f);
+            s_lo[threadIdx.x / kMapLanes] = lo;
         }
     }
+    __syncthreads();
+    const int64_t p = p0 + threadIdx.x;
+    if (threadIdx.x >= kMapRows || p >= n) return;
+    const float hi = s_hi[threadIdx.x], lo = s_lo[threadIdx.x];
+    const int32_t o = perm[p], node = pos_node[p];
+    const double S = (double)hi + (double)lo;
+    float r = -1.f;
+    if (hi < 0.f) r = 0.f;   // (a NaN cannot occur: builds reject non-finite coordinates)
+    else if (S >= 1e-18 && S <= 1e30) r = ds_round<L2>(hi, lo, S, del);
+    if (r < 0.f) {
+        const float *a = X + (int64_t)o * dim, *b = X + (int64_t)piv_obj[node] * dim;
+        double d = L2 ? l2sq_fp64_seq(a, b, dim) : l1_fp64_seq(a, b, dim);
+        if (L2) d = __dsqrt_rn(d);
+        r = __double2float_rn(d);
+    }
+    Tl[o] = r;
+    node_of[o] = node;
 }
 
 // Mapping for strings: a block takes a run of table positions; for every node
@@ -513,11 +541,10 @@ void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids, int metric, 
         if (l > 0) k_fft_pivot<<<(unsigned)nn, kThreads, 0, st>>>(perm.get(), T.get(), n, l, lpos, lsize, lpiv);
         check_launch("fft pivot");
         if (objs.dim > 0) {
-            if (objs.dim > kMapSingleDim) {
+            if (objs.dim > (metric == GTS_L2 ? kMapSingleL2 : kMapSingleL1)) {
                 const bool v4 = objs.dim % 4 == 0 && ((uintptr_t)objs.X & 15) == 0;
-                const double terms = (objs.dim + 7) / 8 + 3;
-                const double del = (terms * terms + 8 * terms + 40) / 70368744177664.0;   // 2^-46
-                const unsigned grid = blocks_for(n, kThreads / kMapLanes);
+                const double del = map_error(objs.dim);
+                const unsigned grid = blocks_for(n, kMapRows);
 #define GTS_MAP(L2V, V4V)                                                                                            \
     k_map_vec_ds<L2V, V4V><<<grid, kThreads, 0, st>>>(objs.X, objs.dim, perm.get(), pos_node.get(), lpiv, n, del, Tl, \
                                                       node_of.get())
