@@ -209,9 +209,9 @@ struct Tree {
     DBuf<float> table;
     DBuf<int64_t> row_del;
     std::vector<int64_t> lvl_off;   // h + 2 entries: first node of each level, last = total nodes
-    DBuf<int32_t> npos, nsize, npiv;
+    DBuf<int32_t> npos, nsize, npiv;   // (npiv holds the bytes of nord behind its own)
     DBuf<float> nlo, nhi;
-    DBuf<int8_t> nord;              // per pivot-level node: its first non-empty child if the children's intervals
+    int8_t *nord = nullptr;         // per pivot-level node: its first non-empty child if the children's intervals
                                     // rise from there on, else -1 (see order_children)
     int max_len = 0;                // longest string
     int64_t n_deleted = 0;          // rows carrying a delete mark
@@ -225,7 +225,7 @@ struct Tree {
     size_t device_bytes() const;
     void persist() {   // every buffer the index keeps
         X.persist(); Xr.persist(); S.persist(); Soff.persist(); row_id.persist(); table.persist(); row_del.persist();
-        npos.persist(); nsize.persist(); npiv.persist(); nlo.persist(); nhi.persist(); nord.persist();
+        npos.persist(); nsize.persist(); npiv.persist(); nlo.persist(); nhi.persist();
         tc.Xh.persist(); tc.Xl.persist(); tc.xn2.persist(); qg.persist();
     }
 };
@@ -298,8 +298,10 @@ void pair_keys(gts_index *ix, const gts_objects *queries, const std::vector<int3
 // the caller's rows in the same order (kept in leaf order as Tree::Xr)
 void build_tree(Tree &t, const Objects &objs, const int64_t *d_ids_or_null, int metric, int F, int h,
                 int64_t root_index, cudaStream_t st, const float *raw_rows = nullptr);
-// fills Tree::nord from the node list (after a build or a load)
+// fills Tree::nord from the node list (after a load; a build writes it with the children)
 void order_children(Tree &t, cudaStream_t st);
+// spare elements of Tree::npiv that hold nord
+inline int64_t nord_spare(const Tree &t) { return (t.lvl_off[t.h] + 3) / 4; }
 int tree_height(int64_t n, int F, int n_pivots);
 uint64_t splitmix64(uint64_t x);
 

@@ -273,7 +273,7 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
         expect(r.dev(t.row_del, 1, st), n, "delete marks");
         expect(r.dev(t.npos, 1, st), nodes, "node positions");
         expect(r.dev(t.nsize, 1, st), nodes, "node sizes");
-        expect(r.dev(t.npiv, 1, st), nodes, "pivots");
+        expect(r.dev(t.npiv, 1, st, nord_spare(t)), nodes, "pivots");
         expect(r.dev(t.nlo, 1, st), nodes, "node bounds");
         expect(r.dev(t.nhi, 1, st), nodes, "node bounds");
         if (t.n > 0) {

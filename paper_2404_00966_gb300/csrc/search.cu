@@ -4713,7 +4713,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     d.npiv = t.npiv.get();
     d.nlo = t.nlo.get();
     d.nhi = t.nhi.get();
-    d.nord = t.nord.get();
+    d.nord = t.nord;
     d.cn = c.count;
     d.cX = c.X.get();
     d.cS = c.S.get();
