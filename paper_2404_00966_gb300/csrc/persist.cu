@@ -254,6 +254,10 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
         t.n_deleted = n_deleted;
         t.lvl_off = r.host<int64_t>();
         GTS_REQUIRE((int)t.lvl_off.size() == h + 2, GTS_EINVAL, "index file is corrupt (levels)");
+        // level l holds F^l nodes (order_children below and every query index by it)
+        for (int64_t l = 0, first = 0, nn = 1; l < h + 2; ++l, first += nn, nn *= ix->F)
+            GTS_REQUIRE(t.lvl_off[l] == first && first <= (int64_t)1 << 28, GTS_EINVAL,
+                        "index file is corrupt (levels)");
         const int64_t nodes = t.lvl_off.back();
         auto expect = [&](int64_t got, int64_t want, const char *what) {
             GTS_REQUIRE(got == want, GTS_EINVAL, std::string("index file is corrupt (") + what + ")");
