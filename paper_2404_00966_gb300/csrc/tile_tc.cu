@@ -159,6 +159,9 @@ namespace {
 // dim_p columns) and its squared norm, summed in FP64 and rounded once
 // (output row i from input row sel[i] when sel is given).  res: the norms of x -
 // x_hi (the differences are exact), rounded up; rho: their largest ratio to |x|.
+// The FP64 conversions and sums bound it, so the residuals, of which any upper
+// bound will do, are summed in FP32 rounding up: in FP64 beside the norms they took
+// SPLITMS
 __global__ void k_split_rows(const float *__restrict__ X, int dim, int dim_p, int64_t n,
                              __nv_bfloat16 *__restrict__ Xh, __nv_bfloat16 *__restrict__ Xl,
                              float *__restrict__ n2, const int32_t *__restrict__ sel,
@@ -168,24 +171,25 @@ __global__ void k_split_rows(const float *__restrict__ X, int dim, int dim_p, in
     for (int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; row < n; row += nw) {
         // output row `row` takes input row `src` (a negative src: a zero row)
         const int64_t src = sel ? (int64_t)sel[row] : row;
-        double s = 0.0, rs = 0.0;
+        double s = 0.0;
+        float rs = 0.f;
         for (int k = lane; k < dim_p; k += 32) {
             const float v = k < dim && src >= 0 ? X[src * dim + k] : 0.f;
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
             const float e = v - __bfloat162float(h);
             const __nv_bfloat16 l = __float2bfloat16_rn(e);
-            rs += (double)e * (double)e;
+            rs = __fmaf_ru(e, e, rs);
             Xh[row * dim_p + k] = h;
             Xl[row * dim_p + k] = l;
             s += (double)v * (double)v;
         }
         for (int o = 16; o > 0; o >>= 1) {
             s += __shfl_xor_sync(0xffffffffu, s, o);
-            rs += __shfl_xor_sync(0xffffffffu, rs, o);
+            rs = __fadd_ru(rs, __shfl_xor_sync(0xffffffffu, rs, o));
         }
         if (lane == 0) {
             n2[row] = __double2float_rn(s);
-            const float re = __fmul_ru(__fsqrt_ru(__double2float_ru(rs)), 1.f + 1e-6f);
+            const float re = __fmul_ru(__fsqrt_ru(rs), 1.f + 1e-6f);
             if (res) res[row] = re;
             if (rho && re > 0.f)
                 atomicMax(reinterpret_cast<int *>(rho), __float_as_int(__fdiv_ru(re, __fsqrt_rd(__double2float_rd(s)))));
