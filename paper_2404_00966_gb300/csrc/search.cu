@@ -3033,6 +3033,23 @@ struct Runner {
     unsigned max_blocks = 152 * 8;   // grid cap for the grid-stride kernels (set from the SM count)
     unsigned cap(unsigned b) const { return b < max_blocks ? b : max_blocks; }
 
+    // Output room of a tile or scan launch, whose number of pairs is not known yet:
+    // twice the most pairs per query that this index has seen, at least 1 M and at
+    // most `most` (a larger output relaunches with the exact size).  Without the
+    // upper limit one batch that kept most rows would make every later, larger one
+    // ask for that many per query.
+    int64_t first_room(const std::atomic<int64_t> &known, int64_t most) const {
+        const double want = 2.0 * (double)known.load() * (double)qb.nq / 1024.0;
+        return std::max<int64_t>(1 << 20, want < (double)most ? (int64_t)want : most);
+    }
+    void seen_pairs(std::atomic<int64_t> &known, int64_t pairs) const {
+        if (qb.nq > 0) known.store(std::max<int64_t>(known.load(), pairs * 1024 / qb.nq));
+    }
+    // pairs that fit the budget at once, with what verifying them takes: the plain
+    // path's candidate groups
+    static constexpr int64_t kCandBytes = 4 + 4 + 4 + 1 + 8 + 16;
+    int64_t pair_room() const { return budget / 2 / kCandBytes; }
+
     int64_t limit_bytes(int l) const {   // Algorithm 4: size_GPU / ((h - layer + 1) * N_c), layer = l + 1
         return budget / ((int64_t)(h - l) * F);
     }
@@ -3313,8 +3330,7 @@ struct Runner {
             const int64_t total = d2h_i64(off.get() + E, st);
             st_table_pass += total;   // the plain scan's candidates are exactly the pairs passing the bound
             if (total == 0) return;
-            const int64_t cand_bytes = 4 + 4 + 4 + 1 + 8 + 16;
-            auto gb = groups(off, E, total, (budget / 2) / cand_bytes);
+            auto gb = groups(off, E, total, pair_room());
             // every group writes with the thresholds it was counted with: collect()
             // may lower tau_q between two groups (edit distance), and a pass that
             // writes fewer candidates than were counted leaves the others unset
@@ -3621,11 +3637,8 @@ struct Runner {
         for (int phase = 0; phase < phases; ++phase) {
             PairSet p;
             int nl = 0;
-            // output capacity: twice the last call's size (per query), at least 1 M
-            // pairs; a larger output triggers one relaunch with the exact size
             std::atomic<int64_t> &known = ix->tc_pairs_hint[knn ? 1 + phase : 0];
-            const int64_t per_q = known.load();
-            const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+            const int64_t hint = first_room(known, budget / 16);
             // kNN: the tiles also give each kept pair's q.x~, whose proven distance
             // interval stands in for the FP32 distance (the answers' distances
             // come from their FP64 keys), so the pairs skip the FP32 verification
@@ -3633,7 +3646,7 @@ struct Runner {
             p.n = tc_run(ix->tree, ix->tree.tc, tq, rg, p.q, p.row, hint, &nl, st, knn && !single ? &p.qx : nullptr, phase,
                          phases == 2 ? 8 : 1, single ? 1 : 3);
             clk.end();
-            if (rg.n_items > 0 && qb.nq > 0) known.store(std::max<int64_t>(per_q, p.n * 1024 / qb.nq));
+            seen_pairs(known, p.n);
             ++st_groups;
             if (!knn) {
                 // verified in the tiles' node-major order (consecutive pairs share
@@ -3850,8 +3863,7 @@ struct Runner {
         clk.end();
         st_tiles += rg.n_items;
         st_tile_entries += rg.n_entries;
-        const int64_t per_q = ix->scan_pairs_hint[knn ? 1 : 0].load();
-        const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+        std::atomic<int64_t> &known = ix->scan_pairs_hint[knn ? 1 : 0];
         ScanQuery sq;
         sq.epsc = d.epsc;
         sq.any_deleted = tq.any_deleted;
@@ -3865,13 +3877,12 @@ struct Runner {
         ScanOut so;
         ScanStats ss;
         clk.begin(GTS_STAGE_LEAF_SCAN);
-        scan_run(ix->tree, rg, sq, so, hint, ss, st);
+        scan_run(ix->tree, rg, sq, so, first_room(known, sq.fused_range ? budget / 16 : pair_room()), ss, st);
         clk.end();
         clk.launches[GTS_STAGE_LEAF_SCAN] += ss.launches > 1 ? ss.launches - 1 : 0;
         st_scan_rows += ss.staged_rows;
         st_scan_records += ss.records;
-        if (rg.n_items > 0 && qb.nq > 0)
-            ix->scan_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, ss.candidates * 1024 / qb.nq));
+        seen_pairs(known, ss.candidates);
         ++st_groups;
         if (sq.fused_range) {
             // the method's candidates are the pairs that passed the table
@@ -4025,8 +4036,8 @@ struct Runner {
         sq.qgq = d.qgq;
         sq.any_deleted = any_deleted;
         sq.queries = tu.str_qgram == 32 ? 32 : 64;
-        const int64_t per_q = ix->tc_pairs_hint[knn ? 1 : 0].load();
-        const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+        std::atomic<int64_t> &known = ix->tc_pairs_hint[knn ? 1 : 0];
+        const int64_t hint = first_room(known, pair_room());
         DBuf<int32_t> oq, orow;
         int nl = 0;
         if (ix->tree.max_len <= kShortStr && qb.max_len <= kShortStr) {
@@ -4040,8 +4051,7 @@ struct Runner {
             clk.begin(GTS_STAGE_TILE);
             const int64_t C = short_run(ix->tree, sq, hq, rg, oq, orow, od, hint, &nl, st);
             clk.end();
-            if (rg.n_items > 0 && qb.nq > 0)
-                ix->tc_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+            seen_pairs(known, C);
             ++st_groups;
             if (C == 0) return;
             st_cands += C;
@@ -4075,8 +4085,7 @@ struct Runner {
                                            &nl, st)
                                  : qgram_run(ix->tree, sq, rg, oq, orow, hint, &nl, st);
         clk.end();
-        if (rg.n_items > 0 && qb.nq > 0)
-            ix->tc_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+        seen_pairs(known, C);
         ++st_groups;
         if (C == 0) return;
         DBuf<int32_t> q2(C, st), r2(C, st);
@@ -4158,15 +4167,14 @@ struct Runner {
         lq.Q = d.Q;
         lq.absf = d.absf;
         lq.any_deleted = tq.any_deleted;
-        const int64_t per_q = ix->f32_pairs_hint[knn ? 1 : 0].load();
-        const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+        std::atomic<int64_t> &known = ix->f32_pairs_hint[knn ? 1 : 0];
+        const int64_t hint = first_room(known, pair_room());
         DBuf<int32_t> oq, orow;
         int nl = 0;
         clk.begin(GTS_STAGE_TILE);
         const int64_t C = l2f_run(ix->tree, lq, qb.nq, rg, oq, orow, hint, &nl, st);
         clk.end();
-        if (rg.n_items > 0 && qb.nq > 0)
-            ix->f32_pairs_hint[knn ? 1 : 0].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+        seen_pairs(known, C);
         ++st_groups;
         if (C > 0) verify_and_collect(oq, orow, C, /*query_major=*/false);
     }
@@ -4215,15 +4223,14 @@ struct Runner {
         if (rg.n_items > bounds.back()) bounds.push_back(rg.n_items);
         for (size_t p = 0; p + 1 < bounds.size(); ++p) {
             const int slot = knn ? 1 + (int)std::min<size_t>(p, 2) : 0;
-            const int64_t per_q = ix->l1_pairs_hint[slot].load();
-            const int64_t hint = std::max<int64_t>(1 << 20, 2 * per_q * (qb.nq > 0 ? qb.nq : 1) / 1024);
+            const int64_t hint = first_room(ix->l1_pairs_hint[slot], pair_room());
             DBuf<int32_t> oq, orow;
             DBuf<float> od;
             int nl = 0;
             clk.begin(GTS_STAGE_TILE);
             const int64_t C = l1_run(ix->tree, lq, rg, bounds[p], bounds[p + 1], oq, orow, od, hint, &nl, st);
             clk.end();
-            if (qb.nq > 0) ix->l1_pairs_hint[slot].store(std::max<int64_t>(per_q, C * 1024 / qb.nq));
+            seen_pairs(ix->l1_pairs_hint[slot], C);
             ++st_groups;
             if (C == 0) continue;
             if (!knn && use_f32) {   // GTS_PREC_FP32 reports the plain path's FP32 distances
