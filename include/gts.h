@@ -69,7 +69,8 @@ typedef enum { GTS_EDIT = 0, GTS_L1 = 1, GTS_L2 = 2, GTS_COS = 3 } gts_metric;
  *                 for batches with enough (query, object) pairs in node-major
  *                 FP32 tiles (the table scan up to 16 dimensions); up to eight
  *                 queries over objects that are read in one pass (a GiB) take
- *                 that pass instead of the descent.  With GTS_QUERY_COUNT_TABLE_PASS
+ *                 that pass instead of the descent, if a budget of 74 bytes holds each
+ *                 of their pairs.  With GTS_QUERY_COUNT_TABLE_PASS
  *                 or a memory budget below 1 GiB always candidate by candidate.
  *  GTS_PREC_BF16: BF16 tensor-core distance tiles with FP32 accumulation and the
  *                 same FP64 recheck against a (wider) proven BF16 bound

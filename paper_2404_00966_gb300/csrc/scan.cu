@@ -375,11 +375,12 @@ void pack(DBuf<T> &buf, const unsigned long long *dcounts, int64_t cap, int64_t 
 
 }  // namespace
 
-void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &out, int64_t cap_hint,
-              ScanStats &stats, cudaStream_t st) {
+int64_t scan_run(const Tree &t, const TcRegroup &rg, int64_t i0, int64_t i1, const ScanQuery &sq, ScanOut &out,
+                 int64_t cap_hint, int64_t most, ScanStats &stats, cudaStream_t st) {
     stats = ScanStats();
     out.n_pairs = out.n_accepted = 0;
-    if (rg.n_items == 0) return;
+    const int64_t n_items = i1 - i0;
+    if (n_items <= 0) return 0;
     GTS_REQUIRE(t.h >= 1 && t.h <= kMaxHeight && t.F <= kMaxFanout, GTS_EINVAL, "tree shape out of range for the scan");
     GTS_REQUIRE(!rg.dmask && rg.grec.get() && rg.gpath.get(), GTS_EINVAL, "the scan needs regrouped records");
     GTS_REQUIRE(!(sq.fused_range || sq.fused_knn) || (t.dim >= 1 && t.dim <= kScanMaxDim && sq.Q), GTS_EINVAL,
@@ -400,8 +401,8 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
     // small tree: 400 items of 2,000 records kept 400 of 3,600 warps busy)
     const int64_t avg_records = rg.n_entries / std::max<int64_t>(1, rg.n_nodes);
     const int64_t split = std::max<int64_t>(
-        1, std::min<int64_t>(avg_records / (2 * kRecW), 4 * resident * kWarpsPerCta / rg.n_items));
-    const int64_t units = rg.n_items * split;
+        1, std::min<int64_t>(avg_records / (2 * kRecW), 4 * resident * kWarpsPerCta / n_items));
+    const int64_t units = n_items * split;
     GTS_REQUIRE(units < ((int64_t)1 << 31) - 16 * resident * kWarpsPerCta, GTS_EINVAL, "too many scan units");
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((units + kWarpsPerCta - 1) / kWarpsPerCta, resident));
@@ -437,7 +438,7 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
         a.lvl_last = t.lvl_off[t.h - 1];
         a.grec = rg.grec.get();
         a.gpath = rg.gpath.get();
-        a.items = rg.items.get();
+        a.items = rg.items.get() + i0;
         a.n_units = units;
         a.split = (int)split;
         a.work = work.get();
@@ -469,13 +470,15 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
         GTS_CUDA(cudaMemcpyAsync(&hs, status.get(), sizeof(int), cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
         GTS_REQUIRE(hs == 0, GTS_ETIMEOUT, "table scan: a bounded wait for a staged record chunk ran out");
-        int64_t mx = 0, mxa = 0;
+        int64_t mx = 0, mxa = 0, total = 0;
         for (int s2 = 0; s2 < kStripes; ++s2) {
             mx = std::max<int64_t>(mx, (int64_t)hc[s2]);
             mxa = std::max<int64_t>(mxa, (int64_t)hc[kStripes + s2]);
+            total += (int64_t)hc[s2];
         }
         fits = mx <= cap && mxa <= cap_acc;
         if (!fits) {
+            if (total > most) return total;
             cap = std::max(cap, mx + mx / 4 + 1024);
             cap_acc = range ? std::max(cap_acc, mxa + mxa / 4 + 1024) : 0;
         }
@@ -498,6 +501,7 @@ void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &
     stats.candidates = fused ? (int64_t)hc[2 * kStripes + 2] : np;
     stats.staged_rows = (int64_t)hc[2 * kStripes];
     stats.records = (int64_t)hc[2 * kStripes + 1];
+    return 0;
 }
 
 }  // namespace gts

@@ -48,7 +48,9 @@ struct ScanOut {
 // the table list and tested against every record of its node; the pairs that
 // pass the leaf mask, visibility and the table lower bound are written to
 // out.q / out.row (node-major) -- or, with fused_range, decided on the spot.
-void scan_run(const Tree &t, const TcRegroup &rg, const ScanQuery &sq, ScanOut &out, int64_t cap_hint,
-              ScanStats &stats, cudaStream_t st);
+// Runs the items [i0, i1) and returns 0; where they give more than `most` pairs
+// (entries of out.q / out.row), their number, and nothing usable is written.
+int64_t scan_run(const Tree &t, const TcRegroup &rg, int64_t i0, int64_t i1, const ScanQuery &sq, ScanOut &out,
+                 int64_t cap_hint, int64_t most, ScanStats &stats, cudaStream_t st);
 
 }  // namespace gts

@@ -3049,10 +3049,35 @@ struct Runner {
     // path's candidate groups
     static constexpr int64_t kCandBytes = 4 + 4 + 4 + 1 + 8 + 16;
     int64_t pair_room() const { return budget / 2 / kCandBytes; }
+    // Runs the items [i0, i1) in as many launches as keep each one's pairs within
+    // the budget (at least 1 M; a single item is never split): run(a, b, most)
+    // launches the items [a, b) and verifies their pairs, or, where these are more
+    // than `most`, hands nothing on and returns their number.  A batch that fits takes
+    // one launch.
+    template <class Run>
+    void item_groups(int64_t i0, int64_t i1, Run run) {
+        const int64_t room = std::max<int64_t>(pair_room(), 1 << 20);
+        std::vector<std::pair<int64_t, int64_t>> todo;
+        if (i1 > i0) todo.push_back({i0, i1});
+        while (!todo.empty()) {
+            const int64_t a = todo.back().first, b = todo.back().second;
+            todo.pop_back();
+            const int64_t over = run(a, b, b - a > 1 ? room : INT64_MAX);
+            if (over == 0) {
+                ++st_groups;
+                continue;
+            }
+            const int64_t parts = std::min<int64_t>(b - a, over / room + 2);
+            for (int64_t p = parts; p > 0; --p)   // (the first part on top)
+                todo.push_back({a + (b - a) * (p - 1) / parts, a + (b - a) * p / parts});
+        }
+    }
 
     int64_t limit_bytes(int l) const {   // Algorithm 4: size_GPU / ((h - layer + 1) * N_c), layer = l + 1
         return budget / ((int64_t)(h - l) * F);
     }
+
+    int64_t entry_bytes() const { return 8 + 4 * (int64_t)h; }   // of a frontier table
 
     void scan_i32(const DBuf<int32_t> &cnt, int64_t E, DBuf<int64_t> &off) {
         off.alloc(E + 1, st);
@@ -3269,8 +3294,7 @@ struct Runner {
                 dense_last_level(L, e0, e1, cmask);
                 return;
             }
-            const int64_t entry_bytes = 8 + 4 * (int64_t)h;
-            auto gb = groups(off, E, total, limit_bytes(l) / entry_bytes);
+            auto gb = groups(off, E, total, limit_bytes(l) / entry_bytes());
             if (gb.size() > 2) {
                 st_groups += (int64_t)gb.size() - 1;
                 whole_batch = false;
@@ -3819,11 +3843,12 @@ struct Runner {
     // waste more than half of it, and the last level's pivot distances and leaf
     // masks come on top.  The rows computed either way decide: E (parent blocks)
     // against `total` (last-level blocks).  (3 * 10^5 x 100, 3,001 queries, nodes
-    // of 37 rows: COARSE_MS.)
+    // of 37 rows: COARSE_MS.)  Only where the last level's entries would be one
+    // group: the budget splits larger ones.
     bool coarse_tiles_pay(int64_t E, int64_t total) const {
         const int64_t n = ix->tree.n, nl = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
         const int64_t np = ix->tree.lvl_off[h - 1] - ix->tree.lvl_off[h - 2];
-        if (n >= kCoarseRows * nl || qb.count_table_pass) return false;
+        if (n >= kCoarseRows * nl || qb.count_table_pass || total > limit_bytes(h - 2) / entry_bytes()) return false;
         return E * ((n / np + 127) / 128) <= total;   // (a last-level node: one block)
     }
 
@@ -3874,36 +3899,40 @@ struct Runner {
         sq.Q = d.Q;
         sq.rel = d.rel;
         sq.absf = d.absf;
-        ScanOut so;
-        ScanStats ss;
-        clk.begin(GTS_STAGE_LEAF_SCAN);
-        scan_run(ix->tree, rg, sq, so, first_room(known, sq.fused_range ? budget / 16 : pair_room()), ss, st);
-        clk.end();
-        clk.launches[GTS_STAGE_LEAF_SCAN] += ss.launches > 1 ? ss.launches - 1 : 0;
-        st_scan_rows += ss.staged_rows;
-        st_scan_records += ss.records;
-        seen_pairs(known, ss.candidates);
-        ++st_groups;
-        if (sq.fused_range) {
-            // the method's candidates are the pairs that passed the table
-            // bound; the accepted ones are answers already, the band pairs get
-            // their FP64 recheck
-            st_cands += ss.candidates - so.n_pairs;
-            if (so.n_accepted > 0) {
-                rkeys.push_back(std::move(so.key));
-                rdists.push_back(std::move(so.dist));
-                rcounts.push_back(so.n_accepted);
+        int64_t seen = 0;
+        item_groups(0, rg.n_items, [&](int64_t i0, int64_t i1, int64_t most) -> int64_t {
+            ScanOut so;
+            ScanStats ss;
+            clk.begin(GTS_STAGE_LEAF_SCAN);
+            const int64_t over = scan_run(ix->tree, rg, i0, i1, sq, so,
+                                          first_room(known, sq.fused_range ? budget / 16 : pair_room()), most, ss, st);
+            clk.end();
+            clk.launches[GTS_STAGE_LEAF_SCAN] += ss.launches > 1 ? ss.launches - 1 : 0;
+            if (over) return over;
+            st_scan_rows += ss.staged_rows;
+            st_scan_records += ss.records;
+            seen += ss.candidates;
+            if (sq.fused_range) {
+                // the method's candidates are the pairs that passed the table
+                // bound; the accepted ones are answers already, the band pairs get
+                // their FP64 recheck
+                st_cands += ss.candidates - so.n_pairs;
+                if (so.n_accepted > 0) {
+                    rkeys.push_back(std::move(so.key));
+                    rdists.push_back(std::move(so.dist));
+                    rcounts.push_back(so.n_accepted);
+                }
             }
-            if (so.n_pairs > 0) verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
-            return;
-        }
-        if (so.n_pairs == 0) return;
-        if (sq.fused_knn) {
-            st_cands += ss.candidates;
-            sort_and_merge(so.q, so.row, so.dist, so.n_pairs);
-            return;
-        }
-        verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
+            if (so.n_pairs == 0) return 0;
+            if (sq.fused_knn) {
+                st_cands += ss.candidates;
+                sort_and_merge(so.q, so.row, so.dist, so.n_pairs);
+            } else {
+                verify_and_collect(so.q, so.row, so.n_pairs, /*query_major=*/false);
+            }
+            return 0;
+        });
+        seen_pairs(known, seen);
     }
 
     // kNN pairs in any order into the answers: a stable radix sort by query
@@ -4038,8 +4067,7 @@ struct Runner {
         sq.queries = tu.str_qgram == 32 ? 32 : 64;
         std::atomic<int64_t> &known = ix->tc_pairs_hint[knn ? 1 : 0];
         const int64_t hint = first_room(known, pair_room());
-        DBuf<int32_t> oq, orow;
-        int nl = 0;
+        int64_t seen = 0;
         if (ix->tree.max_len <= kShortStr && qb.max_len <= kShortStr) {
             ShortQuery hq;
             hq.S = d.S;
@@ -4047,17 +4075,23 @@ struct Runner {
             hq.max_len = ix->tree.max_len;
             hq.QS = d.QS;
             hq.QSoff = d.QSoff;
-            DBuf<float> od;
-            clk.begin(GTS_STAGE_TILE);
-            const int64_t C = short_run(ix->tree, sq, hq, rg, oq, orow, od, hint, &nl, st);
-            clk.end();
-            seen_pairs(known, C);
-            ++st_groups;
-            if (C == 0) return;
-            st_cands += C;
-            DBuf<uint8_t> keep(C, st);
-            GTS_CUDA(cudaMemsetAsync(keep.get(), 1, C, st));
-            collect(oq, orow, od, keep, C, /*query_major=*/false);
+            item_groups(0, rg.n_items, [&](int64_t i0, int64_t i1, int64_t most) -> int64_t {
+                DBuf<int32_t> oq, orow;
+                DBuf<float> od;
+                int nl = 0;
+                clk.begin(GTS_STAGE_TILE);
+                const int64_t C = short_run(ix->tree, sq, hq, rg, i0, i1, oq, orow, od, hint, most, &nl, st);
+                clk.end();
+                if (C > most) return C;
+                seen += C;
+                if (C == 0) return 0;
+                st_cands += C;
+                DBuf<uint8_t> keep(C, st);
+                GTS_CUDA(cudaMemsetAsync(keep.get(), 1, C, st));
+                collect(oq, orow, od, keep, C, /*query_major=*/false);
+                return 0;
+            });
+            seen_pairs(known, seen);
             return;
         }
         const bool tensor = qtc_pays(ix->tree, qb.nq, rg);
@@ -4080,25 +4114,31 @@ struct Runner {
             qtc_codes(d.qgq, qb.nq, thr.get(), qcode.get(), st);
             clk.end();
         }
-        clk.begin(GTS_STAGE_TILE);
-        const int64_t C = tensor ? qtc_run(ix->tree, sq, rg, qb.nq, ix->tree.qcode.get(), qcode.get(), oq, orow, hint,
-                                           &nl, st)
-                                 : qgram_run(ix->tree, sq, rg, oq, orow, hint, &nl, st);
-        clk.end();
-        seen_pairs(known, C);
-        ++st_groups;
-        if (C == 0) return;
-        DBuf<int32_t> q2(C, st), r2(C, st);
-        int qbits = 1;
-        while (((int64_t)1 << qbits) < qb.nq) ++qbits;
-        size_t tb = 0;
-        cub::DeviceRadixSort::SortPairs(nullptr, tb, oq.get(), q2.get(), orow.get(), r2.get(), C, 0, qbits, st);
-        DBuf<uint8_t> tmp(tb ? tb : 1, st);
-        clk.begin(GTS_STAGE_OTHER);
-        GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, oq.get(), q2.get(), orow.get(), r2.get(), C, 0, qbits,
-                                                 st));
-        clk.end();
-        verify_and_collect(q2, r2, C, true, /*qgram_done=*/!tensor);
+        item_groups(0, rg.n_items, [&](int64_t i0, int64_t i1, int64_t most) -> int64_t {
+            DBuf<int32_t> oq, orow;
+            int nl = 0;
+            clk.begin(GTS_STAGE_TILE);
+            const int64_t C = tensor ? qtc_run(ix->tree, sq, rg, i0, i1, qb.nq, ix->tree.qcode.get(), qcode.get(), oq,
+                                               orow, hint, most, &nl, st)
+                                     : qgram_run(ix->tree, sq, rg, i0, i1, oq, orow, hint, most, &nl, st);
+            clk.end();
+            if (C > most) return C;
+            seen += C;
+            if (C == 0) return 0;
+            DBuf<int32_t> q2(C, st), r2(C, st);
+            int qbits = 1;
+            while (((int64_t)1 << qbits) < qb.nq) ++qbits;
+            size_t tb = 0;
+            cub::DeviceRadixSort::SortPairs(nullptr, tb, oq.get(), q2.get(), orow.get(), r2.get(), C, 0, qbits, st);
+            DBuf<uint8_t> tmp(tb ? tb : 1, st);
+            clk.begin(GTS_STAGE_OTHER);
+            GTS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.get(), tb, oq.get(), q2.get(), orow.get(), r2.get(), C, 0,
+                                                     qbits, st));
+            clk.end();
+            verify_and_collect(q2, r2, C, true, /*qgram_done=*/!tensor);
+            return 0;
+        });
+        seen_pairs(known, seen);
     }
 
     // GTS_PREC_FP32: whether the last level's E entries run as FP32 tiles or
@@ -4169,14 +4209,19 @@ struct Runner {
         lq.any_deleted = tq.any_deleted;
         std::atomic<int64_t> &known = ix->f32_pairs_hint[knn ? 1 : 0];
         const int64_t hint = first_room(known, pair_room());
-        DBuf<int32_t> oq, orow;
-        int nl = 0;
-        clk.begin(GTS_STAGE_TILE);
-        const int64_t C = l2f_run(ix->tree, lq, qb.nq, rg, oq, orow, hint, &nl, st);
-        clk.end();
-        seen_pairs(known, C);
-        ++st_groups;
-        if (C > 0) verify_and_collect(oq, orow, C, /*query_major=*/false);
+        int64_t seen = 0;
+        item_groups(0, rg.n_items, [&](int64_t i0, int64_t i1, int64_t most) -> int64_t {
+            DBuf<int32_t> oq, orow;
+            int nl = 0;
+            clk.begin(GTS_STAGE_TILE);
+            const int64_t C = l2f_run(ix->tree, lq, qb.nq, rg, i0, i1, oq, orow, hint, most, &nl, st);
+            clk.end();
+            if (C > most) return C;
+            seen += C;
+            if (C > 0) verify_and_collect(oq, orow, C, /*query_major=*/false);
+            return 0;
+        });
+        seen_pairs(known, seen);
     }
 
     // Last level on the L1 tiles: regroup the entries by node, run the tiles
@@ -4224,36 +4269,41 @@ struct Runner {
         for (size_t p = 0; p + 1 < bounds.size(); ++p) {
             const int slot = knn ? 1 + (int)std::min<size_t>(p, 2) : 0;
             const int64_t hint = first_room(ix->l1_pairs_hint[slot], pair_room());
-            DBuf<int32_t> oq, orow;
-            DBuf<float> od;
-            int nl = 0;
-            clk.begin(GTS_STAGE_TILE);
-            const int64_t C = l1_run(ix->tree, lq, rg, bounds[p], bounds[p + 1], oq, orow, od, hint, &nl, st);
-            clk.end();
-            seen_pairs(ix->l1_pairs_hint[slot], C);
-            ++st_groups;
-            if (C == 0) continue;
-            if (!knn && use_f32) {   // GTS_PREC_FP32 reports the plain path's FP32 distances
-                verify_and_collect(oq, orow, C, /*query_major=*/false);
-                continue;
-            }
-            st_cands += C;
-            DBuf<uint8_t> keep(C, st);
-            if (knn) {   // the merge wants query-major order
-                sort_and_merge(oq, orow, od, C);
-                clk.begin(GTS_STAGE_THRESHOLD);
-                k_tau_from_answer<<<cap(nblocks(qb.nq, kT)), kT, 0, st>>>(qb.k, koff.get(), bd.get(), bn.get(), qb.nq,
-                                                                         0, 0, 0.f, thr.get());
+            int64_t seen = 0;
+            item_groups(bounds[p], bounds[p + 1], [&](int64_t i0, int64_t i1, int64_t most) -> int64_t {
+                DBuf<int32_t> oq, orow;
+                DBuf<float> od;
+                int nl = 0;
+                clk.begin(GTS_STAGE_TILE);
+                const int64_t C = l1_run(ix->tree, lq, rg, i0, i1, oq, orow, od, hint, most, &nl, st);
                 clk.end();
-                check_launch("L1 tau update");
-            } else {
-                clk.begin(GTS_STAGE_VERIFY);
-                k_decide_range_l1<<<cap(nblocks(C, kT)), kT, 0, st>>>(d, oq.get(), orow.get(), od.get(), C, thr.get(),
-                                                                      keep.get(), counters.get());
-                clk.end();
-                check_launch("L1 range decision");
-                collect(oq, orow, od, keep, C);
-            }
+                if (C > most) return C;
+                seen += C;
+                if (C == 0) return 0;
+                if (!knn && use_f32) {   // GTS_PREC_FP32 reports the plain path's FP32 distances
+                    verify_and_collect(oq, orow, C, /*query_major=*/false);
+                    return 0;
+                }
+                st_cands += C;
+                if (knn) {   // the merge wants query-major order
+                    sort_and_merge(oq, orow, od, C);
+                    clk.begin(GTS_STAGE_THRESHOLD);
+                    k_tau_from_answer<<<cap(nblocks(qb.nq, kT)), kT, 0, st>>>(qb.k, koff.get(), bd.get(), bn.get(),
+                                                                             qb.nq, 0, 0, 0.f, thr.get());
+                    clk.end();
+                    check_launch("L1 tau update");
+                } else {
+                    DBuf<uint8_t> keep(C, st);
+                    clk.begin(GTS_STAGE_VERIFY);
+                    k_decide_range_l1<<<cap(nblocks(C, kT)), kT, 0, st>>>(d, oq.get(), orow.get(), od.get(), C,
+                                                                          thr.get(), keep.get(), counters.get());
+                    clk.end();
+                    check_launch("L1 range decision");
+                    collect(oq, orow, od, keep, C);
+                }
+                return 0;
+            });
+            seen_pairs(ix->l1_pairs_hint[slot], seen);
         }
     }
 
@@ -4836,7 +4886,7 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
     check_launch("query setup");
     // (the diagnostic count needs the plain scan's candidates)
     const bool small = precision == GTS_PREC_FP32 && budget >= kF32TileBudget && !qb.count_table_pass &&
-                       Runner::small_batch(t, nq);
+                       Runner::small_batch(t, nq) && nq * t.n <= R.pair_room();
     if (small) R.scan_all();
     if (!small && knn && t.n > 0 && nq > 0 && t.dim > 0) {
         LevelOffsets lo_off;

@@ -276,7 +276,8 @@ bool l1_tiles_supported(const Tree &t, const float *Q) {
 }
 
 int64_t l1_run(const Tree &t, const L1Query &lq, const TcRegroup &rg, int64_t i0, int64_t i1, DBuf<int32_t> &out_q,
-               DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st) {
+               DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int64_t most, int *launches,
+               cudaStream_t st) {
     *launches = 0;
     if (i1 <= i0) return 0;
     int dev = 0, sms = 0;
@@ -329,7 +330,7 @@ int64_t l1_run(const Tree &t, const L1Query &lq, const TcRegroup &rg, int64_t i0
         unsigned long long hcount = 0;
         GTS_CUDA(cudaMemcpyAsync(&hcount, count.get(), 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        if ((int64_t)hcount <= cap || (int64_t)hcount > most) return (int64_t)hcount;
         cap = (int64_t)hcount;   // rerun with room for every pair
     }
     GTS_REQUIRE(false, GTS_ECUDA, "L1 tile: output count changed between identical runs");

@@ -21,6 +21,7 @@ bool l1_tiles_supported(const Tree &t, const float *Q);
 // run items [i0, i1) of a regrouping; returns the number of (query, row, FP32
 // distance) triples written
 int64_t l1_run(const Tree &t, const L1Query &lq, const TcRegroup &rg, int64_t i0, int64_t i1, DBuf<int32_t> &out_q,
-               DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st);
+               DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int64_t most, int *launches,
+               cudaStream_t st);
 
 }  // namespace gts

@@ -356,10 +356,12 @@ bool l2f_tiles_supported(const Tree &t) {
     return t.metric == GTS_L2 && t.dim > 0 && t.n > 0 && t.n < ((int64_t)1 << 31);
 }
 
-int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st) {
+int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &rg, int64_t i0, int64_t i1,
+                DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, int64_t cap_hint, int64_t most, int *launches,
+                cudaStream_t st) {
     *launches = 0;
-    if (rg.n_items == 0) return 0;
+    const int64_t n_items = i1 - i0;
+    if (n_items <= 0) return 0;
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -375,8 +377,8 @@ int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &
     const int64_t resident = (int64_t)(sms > 0 ? sms : 1) * per_sm;
     const int64_t max_chunks = (nq + kNQF - 1) / kNQF;
     const int64_t split =
-        std::max<int64_t>(1, std::min<int64_t>(max_chunks, (4 * resident + rg.n_items - 1) / rg.n_items));
-    const int64_t units = rg.n_items * split;
+        std::max<int64_t>(1, std::min<int64_t>(max_chunks, (4 * resident + n_items - 1) / n_items));
+    const int64_t units = n_items * split;
     GTS_REQUIRE(units < ((int64_t)1 << 31) - resident, GTS_EINVAL, "too many FP32 tiles");
     const int64_t grid = std::min<int64_t>(units, resident);
     DBuf<float> qn2(nq > 0 ? nq : 1, st);
@@ -401,7 +403,7 @@ int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &
         a.nsize = t.nsize.get();
         a.lvl_last = t.lvl_off[t.h - 1];
         a.grec = rg.grec.get();
-        a.items = rg.items.get();
+        a.items = rg.items.get() + i0;
         a.units = units;
         a.split = (int)split;
         a.work_counter = counter.get();
@@ -418,7 +420,7 @@ int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &
         unsigned long long hcount = 0;
         GTS_CUDA(cudaMemcpyAsync(&hcount, count.get(), 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        if ((int64_t)hcount <= cap || (int64_t)hcount > most) return (int64_t)hcount;
         cap = (int64_t)hcount;   // rerun with room for every pair
     }
     GTS_REQUIRE(false, GTS_ECUDA, "FP32 L2 tile: output count changed between identical runs");

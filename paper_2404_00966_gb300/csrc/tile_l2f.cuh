@@ -15,9 +15,11 @@ struct L2fQuery {
 
 // every FP32 vector set under L2 (dimension and alignment only choose the copy width)
 bool l2f_tiles_supported(const Tree &t);
-// run a regrouping's tiles; returns the number of (query, row) pairs written:
-// a superset of the pairs within the records' thresholds
-int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st);
+// run the tiles of a regrouping's items [i0, i1); returns the number of (query,
+// row) pairs written: a superset of the pairs within the records' thresholds.
+// More than `most`: their number, nothing usable is written.
+int64_t l2f_run(const Tree &t, const L2fQuery &lq, int64_t nq, const TcRegroup &rg, int64_t i0, int64_t i1,
+                DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, int64_t cap_hint, int64_t most, int *launches,
+                cudaStream_t st);
 
 }  // namespace gts

@@ -434,17 +434,18 @@ void qtc_codes(const uint8_t *qg, int64_t n, const float *thr, uint8_t *code, cu
     check_launch("3-gram codes");
 }
 
-int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t nq, const uint8_t *xcode,
-                const uint8_t *qcode, DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, int64_t cap_hint, int *launches,
-                cudaStream_t st) {
+int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1, int64_t nq,
+                const uint8_t *xcode, const uint8_t *qcode, DBuf<int32_t> &out_q, DBuf<int32_t> &out_row,
+                int64_t cap_hint, int64_t most, int *launches, cudaStream_t st) {
     *launches = 0;
-    if (rg.n_items == 0) return 0;
+    const int64_t n_items = i1 - i0;
+    if (n_items <= 0) return 0;
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     constexpr int smem = 2 * kABytes + 2 * kBBytes + 1024;
     GTS_CUDA(cudaFuncSetAttribute(k_tile_qgram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const int64_t nwin = (nq + kWinQ - 1) / kWinQ, pairs = (rg.n_items + 1) / 2;
+    const int64_t nwin = (nq + kWinQ - 1) / kWinQ, pairs = (n_items + 1) / 2;
     // at least four units per SM where the windows allow it
     const int split = (int)std::max<int64_t>(1, std::min<int64_t>(nwin, (4 * sms + pairs - 1) / pairs));
     const int64_t nodes = t.lvl_off[rg.h] - t.lvl_off[rg.h - 1];
@@ -477,8 +478,8 @@ int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t 
         a.wpre = rg.wpre.get();
         a.noff = rg.noff.get();
         a.grec = rg.grec.get();
-        a.items = rg.items.get();
-        a.n_items = rg.n_items;
+        a.items = rg.items.get() + i0;
+        a.n_items = n_items;
         a.split = split;
         a.work_counter = counter.get();
         a.out_q = out_q.get();
@@ -496,7 +497,7 @@ int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t 
         GTS_CUDA(cudaStreamSynchronize(st));
         GTS_REQUIRE(hstatus == 0, GTS_ETIMEOUT,
                     "3-gram tensor-core tile: a bounded mbarrier wait ran out (status " + std::to_string(hstatus) + ")");
-        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        if ((int64_t)hcount <= cap || (int64_t)hcount > most) return (int64_t)hcount;
         cap = (int64_t)hcount;   // rerun with room for every pair
     }
     GTS_REQUIRE(false, GTS_ECUDA, "3-gram tensor-core tile: output count changed between identical runs");

@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
     }
 }
 
-StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg) {
+StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1) {
     StrArgs a;
     a.F = t.F;
     a.npos = t.npos.get();
@@ -369,23 +369,24 @@ StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg) {
     a.qgq = sq.qgq;
     a.grec = rg.grec.get();
     a.gq = rg.gq.get();
-    a.items = rg.items.get();
-    a.i1 = rg.n_items;
+    a.items = rg.items.get() + i0;
+    a.i1 = i1 - i0;
     return a;
 }
 
 }  // namespace
 
-int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                  DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st) {
+int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, int64_t i0, int64_t i1,
+                  DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int64_t most,
+                  int *launches, cudaStream_t st) {
     *launches = 0;
-    if (rg.n_items == 0) return 0;
+    if (i1 <= i0) return 0;
     int dev = 0, sms = 0, per_sm = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_short, kThreadsS, 0));
     if (per_sm < 1) per_sm = 1;
-    const int64_t grid = std::min<int64_t>(rg.n_items, (int64_t)sms * per_sm);
+    const int64_t grid = std::min<int64_t>(i1 - i0, (int64_t)sms * per_sm);
     DBuf<int> counter(1, st);
     DBuf<unsigned long long> count(1, st);
     int64_t cap = cap_hint > 0 ? cap_hint : 1 << 20;
@@ -396,7 +397,7 @@ int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const
         GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
         ShortArgs A;
-        A.s = str_args(t, sq, rg);
+        A.s = str_args(t, sq, rg, i0, i1);
         A.s.work_counter = counter.get();
         A.s.out_q = out_q.get();
         A.s.out_row = out_row.get();
@@ -414,17 +415,17 @@ int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const
         unsigned long long hcount = 0;
         GTS_CUDA(cudaMemcpyAsync(&hcount, count.get(), 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        if ((int64_t)hcount <= cap || (int64_t)hcount > most) return (int64_t)hcount;
         cap = (int64_t)hcount;   // rerun with room for every pair
     }
     GTS_REQUIRE(false, GTS_ECUDA, "short-string tile: output count changed between identical runs");
     return 0;
 }
 
-int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                  DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st) {
+int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1, DBuf<int32_t> &out_q,
+                  DBuf<int32_t> &out_row, int64_t cap_hint, int64_t most, int *launches, cudaStream_t st) {
     *launches = 0;
-    if (rg.n_items == 0) return 0;
+    if (i1 <= i0) return 0;
     int dev = 0, sms = 0;
     GTS_CUDA(cudaGetDevice(&dev));
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -434,7 +435,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<i
     else
         GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_qgram<64>, kThreadsS, 0));
     if (per_sm < 1) per_sm = 1;
-    const int64_t grid = std::min<int64_t>(rg.n_items, (int64_t)sms * per_sm);
+    const int64_t grid = std::min<int64_t>(i1 - i0, (int64_t)sms * per_sm);
     DBuf<int> counter(1, st);
     DBuf<unsigned long long> count(1, st);
     int64_t cap = cap_hint > 0 ? cap_hint : 1 << 20;
@@ -443,7 +444,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<i
         out_row.alloc(cap, st);
         GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
-        StrArgs a = str_args(t, sq, rg);
+        StrArgs a = str_args(t, sq, rg, i0, i1);
         a.work_counter = counter.get();
         a.out_q = out_q.get();
         a.out_row = out_row.get();
@@ -458,7 +459,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<i
         unsigned long long hcount = 0;
         GTS_CUDA(cudaMemcpyAsync(&hcount, count.get(), 8, cudaMemcpyDeviceToHost, st));
         GTS_CUDA(cudaStreamSynchronize(st));
-        if ((int64_t)hcount <= cap) return (int64_t)hcount;
+        if ((int64_t)hcount <= cap || (int64_t)hcount > most) return (int64_t)hcount;
         cap = (int64_t)hcount;   // rerun with room for every pair
     }
     GTS_REQUIRE(false, GTS_ECUDA, "3-gram tile: output count changed between identical runs");

@@ -26,15 +26,19 @@ struct ShortQuery {
     const int64_t *QSoff = nullptr;
 };
 
-// run the tiles over a regrouping of short strings: the (query, row, distance)
-// triples within the records' thresholds
-int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                  DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int *launches, cudaStream_t st);
+// The tiles run the items [i0, i1) of a regrouping and return the number of pairs
+// written; more than `most`: their number, nothing usable is written.
 
-// run the tiles over a regrouping (its records carry each query's threshold);
-// returns the number of (query, row) pairs written, the pairs the bound keeps
-int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, DBuf<int32_t> &out_q,
-                  DBuf<int32_t> &out_row, int64_t cap_hint, int *launches, cudaStream_t st);
+// over a regrouping of short strings: the (query, row, distance) triples within
+// the records' thresholds
+int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const TcRegroup &rg, int64_t i0, int64_t i1,
+                  DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, DBuf<float> &out_d, int64_t cap_hint, int64_t most,
+                  int *launches, cudaStream_t st);
+
+// the (query, row) pairs that the bound keeps (the records carry each query's
+// threshold)
+int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1, DBuf<int32_t> &out_q,
+                  DBuf<int32_t> &out_row, int64_t cap_hint, int64_t most, int *launches, cudaStream_t st);
 
 // The same bound on the tensor cores (tile_qtc.cu), with the counts capped at
 // 4: keeps every pair that qgram_run keeps and a few more.  256-byte codes of the
@@ -43,8 +47,8 @@ constexpr int64_t kQtcRows = 1 << 24;    // rows whose codes are kept with the i
 constexpr int64_t kQtcPairs = 32 << 20;  // least (entry, row) pairs
 bool qtc_pays(const Tree &t, int64_t nq, const TcRegroup &rg);
 void qtc_codes(const uint8_t *qg, int64_t n, const float *thr, uint8_t *code, cudaStream_t st);
-int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t nq, const uint8_t *xcode,
-                const uint8_t *qcode, DBuf<int32_t> &out_q, DBuf<int32_t> &out_row, int64_t cap_hint, int *launches,
-                cudaStream_t st);
+int64_t qtc_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1, int64_t nq,
+                const uint8_t *xcode, const uint8_t *qcode, DBuf<int32_t> &out_q, DBuf<int32_t> &out_row,
+                int64_t cap_hint, int64_t most, int *launches, cudaStream_t st);
 
 }  // namespace gts
