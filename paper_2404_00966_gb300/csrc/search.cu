@@ -28,6 +28,7 @@
 #include "gts_impl.cuh"
 #include "metric.cuh"
 #include "pivot_dense.cuh"
+#include "qgram.cuh"
 #include "tile_l1.cuh"
 #include "tile_l2f.cuh"
 #include "tile_str.cuh"
@@ -1532,39 +1533,54 @@ __global__ void k_small_emit(const float *__restrict__ d32, int64_t n, const flo
 
 // ---------------------------------------------------------------- q-gram count filter
 //
-// A lower bound for edit distance from the counts of the strings' 3-grams
-// (Ukkonen 1992, q-gram distance): a substitution changes at most 3 of a
-// string's 3-grams and an insertion or deletion at most 2 old and 3 new ones,
-// so the L1 distance between the two 3-gram count vectors is at most 6 times
-// the edit distance.  Counting the 3-grams in 64 hashed buckets (sums of the
-// exact counts) and capping a count at 255 can only lower that L1 distance,
-// so L1(buckets) > 6 t proves d > t, and such a pair is not verified.
-constexpr int kQgBuckets = 64;
+// (the bound: qgram.cuh)
 
-// The bucket of a 3-gram: two bits of each character.  Bits 1 and 2 of ASCII
-// tell A, C, G and T apart, so the 64 3-grams of DNA get a bucket each (a
-// multiplicative hash of the three bytes left a third of the buckets empty and
-// let 164 M of 1.9 * 10^10 read pairs at t = 8 through; this one 2.3 M), and
-// they spread the letters of text over four even classes.
-__device__ __forceinline__ uint32_t qgram_bucket(uint32_t a, uint32_t b, uint32_t c) {
-    return ((a & 6u) << 3) | ((b & 6u) << 1) | ((c & 6u) >> 1);
+// The letter classes of an index, one block: the letters of up to 64 KB of its
+// strings, in 4,096 evenly spaced pieces of 16 bytes, are counted and ranked.
+__global__ void __launch_bounds__(1024) k_letter_classes(const uint8_t *__restrict__ S,
+                                                         const int64_t *__restrict__ Soff, int64_t n,
+                                                         uint8_t *__restrict__ cls) {
+    __shared__ uint32_t cnt[256];
+    __shared__ uint8_t order[256], out[256];
+    const int64_t bytes = Soff[n], pieces = bytes / 16;   // (S starts on a 16-byte boundary)
+    if (threadIdx.x < 256) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    if (pieces > 4096) {
+        for (int64_t p = threadIdx.x; p < 4096; p += blockDim.x) {
+            const uint4 v = reinterpret_cast<const uint4 *>(S)[pieces * p / 4096];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 16; ++i) atomicAdd(&cnt[(w[i >> 2] >> (8 * (i & 3))) & 255u], 1u);
+        }
+    } else {
+        for (int64_t i = threadIdx.x; i < bytes; i += blockDim.x) atomicAdd(&cnt[S[i]], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {   // its rank by (count falling, letter)
+        const uint32_t mine = cnt[threadIdx.x];
+        int rank = 0;
+        for (int c = 0; c < 256; ++c) rank += cnt[c] > mine || (cnt[c] == mine && c < (int)threadIdx.x);
+        order[rank] = (uint8_t)threadIdx.x;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) letter_classes(cnt, order, out);
+    __syncthreads();
+    if (threadIdx.x < 256) cls[threadIdx.x] = out[threadIdx.x];
 }
 
 // thread per string: its 64 bucket counts (saturating at 255)
 __global__ void k_qgram_hist(const uint8_t *__restrict__ S, const int64_t *__restrict__ Soff, int64_t n,
-                             uint8_t *__restrict__ out) {
-    __shared__ uint8_t hb[256][kQgBuckets];
+                             const uint8_t *__restrict__ cls, uint8_t *__restrict__ out) {
+    __shared__ __align__(16) uint8_t hb[256][kQgBuckets];
+    __shared__ uint8_t s_cls[256];
+    s_cls[threadIdx.x] = cls[threadIdx.x];   // (256 threads)
+    __syncthreads();
     uint8_t *h = hb[threadIdx.x];
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i - threadIdx.x < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (i >= n) continue;
         for (int b = 0; b < kQgBuckets; ++b) h[b] = 0;
-        const uint8_t *s = S + Soff[i];
-        const int64_t len = Soff[i + 1] - Soff[i];
-        for (int64_t j = 0; j + 2 < len; ++j) {
-            const uint32_t b = qgram_bucket(s[j], s[j + 1], s[j + 2]);
-            if (h[b] < 255) ++h[b];
-        }
+        qgram_counts(S + Soff[i], Soff[i + 1] - Soff[i], s_cls, h);
         uint32_t *o = reinterpret_cast<uint32_t *>(out + i * kQgBuckets);
         const uint32_t *hw = reinterpret_cast<const uint32_t *>(h);
         for (int w = 0; w < kQgBuckets / 4; ++w) o[w] = hw[w];
@@ -4791,15 +4807,18 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
             std::lock_guard<std::mutex> g(ix->prep_mu);   // concurrent queries build it once
             if (!t.qg_ready) {
                 Arena::Pause index_owned;
-                t.qg.alloc(t.n * kQgBuckets, st);
-                k_qgram_hist<<<nblocks(t.n, 256), 256, 0, st>>>(t.S.get(), t.Soff.get(), t.n, t.qg.get());
+                t.qg.alloc(t.n * kQgBuckets + 256, st);   // (and the letter classes behind the counts)
+                uint8_t *cls = t.qg.get() + t.n * kQgBuckets;
+                k_letter_classes<<<1, 1024, 0, st>>>(t.S.get(), t.Soff.get(), t.n, cls);
+                k_qgram_hist<<<nblocks(t.n, 256), 256, 0, st>>>(t.S.get(), t.Soff.get(), t.n, cls, t.qg.get());
+                check_launch("3-gram counts");
                 GTS_CUDA(cudaStreamSynchronize(st));
                 t.qg.persist();
                 t.qg_ready = true;
             }
         }
         qgq.alloc(nq * kQgBuckets, st);
-        k_qgram_hist<<<nblocks(nq, 256), 256, 0, st>>>(qb.S, qb.Soff, nq, qgq.get());
+        k_qgram_hist<<<nblocks(nq, 256), 256, 0, st>>>(qb.S, qb.Soff, nq, t.qg.get() + t.n * kQgBuckets, qgq.get());
         R.clk.end();
         check_launch("3-gram counts");
         d.qg = t.qg.get();

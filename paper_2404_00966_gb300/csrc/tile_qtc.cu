@@ -34,6 +34,7 @@
 #include <cuda_fp8.h>
 
 #include "gts_impl.cuh"
+#include "qgram.cuh"
 #include "tc.cuh"
 #include "tile_str.cuh"
 
@@ -44,7 +45,7 @@ namespace {
 constexpr int kRowsQ = 128;      // rows of a block (MMA M)
 constexpr int kWinQ = 256;       // queries of a window (MMA N)
 constexpr int kCode = 256;       // bytes of a string's code: two panels of 128
-constexpr int kPlaces = 249;     // of them levels; then |A|'s digits, the constants
+constexpr int kPlaces = kQgPlaces;   // of them levels; then |A|'s digits, the constants
 constexpr int kEpiQ = 8;         // epilogue warps of each block
 constexpr int kThreadsQ = (4 + 2 * kEpiQ) * 32;   // warp 0 producer, 1 MMA, 2 TMEM, 4.. epilogue
 constexpr int kABytes = kRowsQ * kCode, kBBytes = kWinQ * kCode;
@@ -90,7 +91,7 @@ __global__ void k_codes(const uint8_t *__restrict__ qg, int64_t n, const float *
     for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < n; i += nwarps) {
         const int c0 = qg[i * 64 + lane], c1 = qg[i * 64 + 32 + lane];
         uint8_t *o = code + i * kCode;
-        const bool fourth = 3 * 64 + 32 + lane < kPlaces;   // this lane's second bucket has its fourth level
+        const bool fourth = code_levels(32 + lane) == 4;   // this lane's second bucket has its fourth level
         const int ones = __reduce_add_sync(0xffffffffu, min(c0, 4) + min(c1, fourth ? 4 : 3));
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
