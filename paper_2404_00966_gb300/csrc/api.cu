@@ -987,7 +987,8 @@ gts_status gts_info(const gts_index *ix, gts_index_info *out) {
         out->metric = ix->metric;
         out->dim = ix->dim;
         const Cache &c = ix->cache;
-        out->device_bytes = (int64_t)(ix->tree.device_bytes() + c.X.bytes() + c.S.bytes() + c.Soff.bytes() +
+        std::lock_guard<std::mutex> g(ix->prep_mu);   // (queries on other threads may be building some of it)
+        out->device_bytes = (int64_t)(ix->tree.device_bytes() + c.X.bytes() + c.Xr.bytes() + c.S.bytes() + c.Soff.bytes() +
                                       c.id.bytes() + c.ins.bytes() + c.del.bytes());
     });
 }

@@ -82,9 +82,11 @@ void order_children(Tree &t, cudaStream_t st) {
 }
 
 size_t Tree::device_bytes() const {
-    return X.bytes() + S.bytes() + Soff.bytes() + row_id.bytes() + table.bytes() + row_del.bytes() + npos.bytes() +
-           nsize.bytes() + npiv.bytes() + nlo.bytes() + nhi.bytes() + tc.Xh.bytes() + tc.Xl.bytes() + tc.xn2.bytes() +
-           qg.bytes();
+    return X.bytes() + Xr.bytes() + S.bytes() + Soff.bytes() + row_id.bytes() + table.bytes() + row_del.bytes() +
+           npos.bytes() + nsize.bytes() + npiv.bytes() + nlo.bytes() + nhi.bytes() +
+           // built on first use
+           tc.Xh.bytes() + tc.Xl.bytes() + tc.xn2.bytes() + tc.xr.bytes() + tc.Ph.bytes() + tc.Pl.bytes() +
+           tc.pn2.bytes() + xrn2.bytes() + qg.bytes() + qcode.bytes();
 }
 
 namespace {

@@ -271,7 +271,7 @@ struct gts_index {
     int64_t rebuilds = 0;
     std::vector<cudaEvent_t> events;   // reused by per-stage timing
     std::mutex tune_mu;
-    std::mutex prep_mu;   // lazily built per-index data (BF16 split rows, 3-gram counts and codes, sums of squares)
+    mutable std::mutex prep_mu;   // lazily built per-index data (BF16 split rows, 3-gram counts and codes, sums of squares)
     gts::Tuning tuning;
     std::atomic<int64_t> tc_pairs_hint[3] = {{0}, {0}, {0}};   // tensor-core / string tiles: output size per query
                                                               // (x1024), range, kNN, kNN phase 1
