@@ -262,12 +262,25 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
         auto expect = [&](int64_t got, int64_t want, const char *what) {
             GTS_REQUIRE(got == want, GTS_EINVAL, std::string("index file is corrupt (") + what + ")");
         };
+        // the longest string, from the offsets: kernels size tables by it, so the
+        // file's own word for it is not taken
+        auto longest = [&](const std::vector<int64_t> &off, const char *what) {
+            int64_t most = 0;
+            for (size_t i = 0; i < off.size(); ++i) {
+                const int64_t len = off[i] - (i ? off[i - 1] : 0);
+                GTS_REQUIRE(len >= 0 && len <= (i ? kMaxStrLen : 0), GTS_EINVAL,
+                            std::string("index file is corrupt (") + what + ")");
+                most = std::max(most, len);
+            }
+            return (int)most;
+        };
         if (ix->dim > 0) {
             expect(r.dev(t.X, 1, st), n * ix->dim, "objects");
             if (t.cosine) expect(r.dev(t.Xr, 1, st), n * ix->dim, "raw objects");
         } else {
             std::vector<int64_t> soff = r.host<int64_t>();
             expect((int64_t)soff.size(), n + 1, "string offsets");
+            t.max_len = std::max(t.max_len, longest(soff, "string offsets"));
             t.Soff.alloc(n + 1, st);
             GTS_CUDA(cudaMemcpyAsync(t.Soff.get(), soff.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
             expect(r.dev(t.S, 1, st, kTextPad), soff[n], "strings");
@@ -288,7 +301,8 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
         Cache &c = ix->cache;
         c.count = r.pod<int64_t>();
         c.max_len = r.pod<int32_t>();
-        GTS_REQUIRE(c.count >= 0 && c.count <= ix->next_id, GTS_EINVAL, "index file is corrupt (cache)");
+        GTS_REQUIRE(c.count >= 0 && c.count <= ix->next_id && c.max_len >= 0 && c.max_len <= kMaxStrLen, GTS_EINVAL,
+                    "index file is corrupt (cache)");
         if (ix->dim > 0) {
             expect(r.dev(c.X, 1, st), c.count * ix->dim, "cache objects");
             if (t.cosine) expect(r.dev(c.Xr, 1, st), c.count * ix->dim, "raw cache objects");
@@ -296,6 +310,7 @@ extern "C" gts_status gts_load(const char *path, const gts_build_opts *opts, gts
             c.h_Soff = r.host<int64_t>();
             GTS_REQUIRE((int64_t)c.h_Soff.size() == (c.count > 0 ? c.count + 1 : (int64_t)c.h_Soff.size()),
                         GTS_EINVAL, "index file is corrupt (cache offsets)");
+            c.max_len = std::max(c.max_len, longest(c.h_Soff, "cache offsets"));
             c.s_bytes = c.h_Soff.empty() ? 0 : c.h_Soff.back();
             expect(r.dev(c.S, 1, st, kTextPad), c.s_bytes, "cache strings");
             c.Soff.alloc(c.h_Soff.size() + 1, st);
