@@ -162,7 +162,7 @@ __global__ void k_map_vec(const float *__restrict__ X, int dim, const int32_t *_
         const int32_t pv = piv_obj[node];
         const float *a = X + (int64_t)o * dim;
         const float *b = X + (int64_t)pv * dim;
-        double d = L2 ? l2sq_fp64_seq(a, b, dim) : l1_fp64_seq(a, b, dim);
+        double d = L2 ? l2sq_fp64_seq<false>(a, b, dim) : l1_fp64_seq<false>(a, b, dim);
         if (L2) d = __dsqrt_rn(d);
         Tl[o] = __double2float_rn(d);
         node_of[o] = node;

@@ -74,11 +74,14 @@ constexpr float kAbsFloor = 1e-17f;
 // Rows on 16-byte boundaries are read 32 coordinates at a time (eight 16-byte
 // loads of each in flight; with a coordinate's loads at a time the sums waited
 // for memory: 130,000 keys of 128 coordinates 0.229 -> 0.193 ms), the sums keep
-// their order.
-template <class Term>
+// their order.  WIDE = false: a coordinate at a time, for kernels that form few
+// keys beside other work or rows of up to 16 coordinates -- the wide form takes
+// 12 to 20 registers more (k_verify_vec 48 -> 64, and the range batches that it
+// decides 5 to 9 % longer).
+template <bool WIDE, class Term>
 __device__ __forceinline__ void fp64_terms(const float *q, const float *x, int dim, Term term) {
     int i = 0;
-    if ((dim & 3) == 0 && ((((uintptr_t)q) | ((uintptr_t)x)) & 15) == 0) {
+    if (WIDE && (dim & 3) == 0 && ((((uintptr_t)q) | ((uintptr_t)x)) & 15) == 0) {
         const float4 *q4 = reinterpret_cast<const float4 *>(q), *x4 = reinterpret_cast<const float4 *>(x);
         for (; i + 32 <= dim; i += 32) {
             float4 a[8], b[8];
@@ -96,12 +99,14 @@ __device__ __forceinline__ void fp64_terms(const float *q, const float *x, int d
             }
         }
     }
+#pragma unroll 4
     for (; i < dim; ++i) term(q[i], x[i]);
 }
 
+template <bool WIDE = true>
 __device__ __forceinline__ double l2sq_fp64_seq(const float *q, const float *x, int dim) {
     double s = 0.0;
-    fp64_terms(q, x, dim, [&](float a, float b) {
+    fp64_terms<WIDE>(q, x, dim, [&](float a, float b) {
         const double t = __dsub_rn((double)a, (double)b);
         s = __dadd_rn(s, __dmul_rn(t, t));
     });
@@ -117,14 +122,16 @@ __device__ __forceinline__ double cos_key_fp64(double dot, double nq, double nx)
     c = c > 1.0 ? 1.0 : (c < -1.0 ? -1.0 : c);
     return __dsub_rn(1.0, c);
 }
+template <bool WIDE = true>
 __device__ __forceinline__ double dot_fp64_seq(const float *q, const float *x, int dim) {
     double dot = 0.0;
-    fp64_terms(q, x, dim, [&](float a, float b) { dot = __dadd_rn(dot, __dmul_rn((double)a, (double)b)); });
+    fp64_terms<WIDE>(q, x, dim, [&](float a, float b) { dot = __dadd_rn(dot, __dmul_rn((double)a, (double)b)); });
     return dot;
 }
+template <bool WIDE = true>
 __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *x, int dim) {
     double dot = 0.0, nq = 0.0, nx = 0.0;
-    fp64_terms(q, x, dim, [&](float fa, float fb) {
+    fp64_terms<WIDE>(q, x, dim, [&](float fa, float fb) {
         const double a = (double)fa, b = (double)fb;
         dot = __dadd_rn(dot, __dmul_rn(a, b));
         nq = __dadd_rn(nq, __dmul_rn(a, a));
@@ -133,9 +140,10 @@ __device__ __forceinline__ double cos_key_fp64_seq(const float *q, const float *
     return cos_key_fp64(dot, nq, nx);
 }
 
+template <bool WIDE = true>
 __device__ __forceinline__ double l1_fp64_seq(const float *q, const float *x, int dim) {
     double s = 0.0;
-    fp64_terms(q, x, dim,
+    fp64_terms<WIDE>(q, x, dim,
                [&](float a, float b) { s = __dadd_rn(s, fabs(__dsub_rn((double)a, (double)b))); });
     return s;
 }

@@ -110,16 +110,16 @@ __device__ __forceinline__ const float *vrow_raw(const Dev &d, int64_t row) {
 }
 // The FP64 key of (query, row) in the reference operation order: L2 the
 // squared sum, L1 the sum, angular distance 1 - cos on the raw vectors.
-template <bool L2>
+template <bool L2, bool WIDE>
 __device__ __forceinline__ double fp64_key(const Dev &d, int64_t q, int64_t row) {
     if (d.cosine) {
         const float *qr = d.Qr + q * d.dim, *xr = vrow_raw(d, row);
         // (rows of the cache list have no stored sum)
-        return d.qrn2 && row < d.n ? cos_key_fp64(dot_fp64_seq(qr, xr, d.dim), d.qrn2[q], d.xrn2[row])
-                                   : cos_key_fp64_seq(qr, xr, d.dim);
+        return d.qrn2 && row < d.n ? cos_key_fp64(dot_fp64_seq<WIDE>(qr, xr, d.dim), d.qrn2[q], d.xrn2[row])
+                                   : cos_key_fp64_seq<WIDE>(qr, xr, d.dim);
     }
     const float *qv = d.Q + q * d.dim, *xv = vrow(d, row);
-    return L2 ? l2sq_fp64_seq(qv, xv, d.dim) : l1_fp64_seq(qv, xv, d.dim);
+    return L2 ? l2sq_fp64_seq<WIDE>(qv, xv, d.dim) : l1_fp64_seq<WIDE>(qv, xv, d.dim);
 }
 // the range limit on the FP64 key and the reported distance of a key
 template <bool L2>
@@ -1202,9 +1202,11 @@ __global__ void k_cache_cands(int64_t qa, int64_t qb, int64_t n, int64_t cn, int
 // candidate if its lower bound is within the query's threshold tau_q (an
 // upper bound of the k-th distance; a farther candidate cannot be in the top
 // k) and store its FP32 distance.
+// WIDE: FP64 keys with wide loads, for ranges under the angle, where they decide
+// every kept pair (from stored sums of squares on: one sum a key).
 constexpr int kVerifyGroup = 32;   // pairs per warp in k_verify_vec (at most 32: one per lane)
 
-template <bool L2, bool KNN, int NV>
+template <bool L2, bool KNN, int NV, bool WIDE>
 __global__ void k_verify_vec(Dev d, const int32_t *__restrict__ cq, const int32_t *__restrict__ crow, int64_t C,
                              const float *__restrict__ thr_q, float *__restrict__ cdist, uint8_t *__restrict__ keep,
                              unsigned long long *__restrict__ rechecks) {
@@ -1264,7 +1266,7 @@ __global__ void k_verify_vec(Dev d, const int32_t *__restrict__ cq, const int32_
         } else if (lo > r * (1.f + 1e-9f)) {
             keep[c] = 0;
         } else {
-            const double key = fp64_key<L2>(d, q, (int64_t)grow);
+            const double key = fp64_key<L2, WIDE>(d, q, (int64_t)grow);
             keep[c] = key <= fp64_limit<L2>(d, q, r) ? 1 : 0;
             cdist[c] = key_distance(d, L2, key);
             atomicAdd(rechecks, 1ull);
@@ -1310,7 +1312,7 @@ __global__ void k_verify_lowdim(Dev d, const int32_t *__restrict__ cq, const int
         } else if (lo > r * (1.f + 1e-9f)) {
             keep[c] = 0;
         } else {
-            const double key = fp64_key<L2>(d, q, row);
+            const double key = fp64_key<L2, false>(d, q, row);
             keep[c] = key <= fp64_limit<L2>(d, q, r) ? 1 : 0;
             cdist[c] = key_distance(d, L2, key);
             atomicAdd(rechecks, 1ull);
@@ -1358,7 +1360,7 @@ __global__ void k_cache_range_lowdim(Dev d, int64_t qa, int64_t qb, int64_t cn, 
                     kept = true;
                     dist = d32;
                 } else if (!(lo > r * (1.f + 1e-9f))) {
-                    const double key = fp64_key<L2>(d, q, row);
+                    const double key = fp64_key<L2, false>(d, q, row);
                     kept = key <= fp64_limit<L2>(d, q, r);
                     dist = key_distance(d, L2, key);
                     atomicAdd(rechecks, 1ull);
@@ -2281,7 +2283,7 @@ __global__ void k_decide_range_l1(Dev d, const int32_t *__restrict__ cq, const i
         } else if (lo > r * (1.f + 1e-9f)) {
             keep[c] = 0;
         } else {
-            const double key = l1_fp64_seq(d.Q + (int64_t)q * d.dim, vrow(d, crow[c]), d.dim);
+            const double key = l1_fp64_seq<false>(d.Q + (int64_t)q * d.dim, vrow(d, crow[c]), d.dim);
             keep[c] = key <= (double)r ? 1 : 0;
             cdist[c] = __double2float_rn(key);
             atomicAdd(rechecks, 1ull);
@@ -2302,7 +2304,7 @@ __global__ void k_recheck_keys(Dev d, const int32_t *__restrict__ cq, const int3
     const int64_t n = (int64_t)*rcount;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t c = rlist[i];
-        ckey[c] = fp64_key<METRIC == GTS_L2>(d, cq[c], crow[c]);
+        ckey[c] = fp64_key<METRIC == GTS_L2, true>(d, cq[c], crow[c]);
     }
 }
 
@@ -4335,9 +4337,16 @@ struct Runner {
         const unsigned grid = cap(nblocks(warps, kWarpsPerBlock));
         const bool aligned = ((uintptr_t)d.Q & 15) == 0;
         const int nv = (aligned && d.dim % 128 == 0 && d.dim <= 512) ? d.dim / 128 : 0;
-#define GTS_VV(NVV)                                                                                          \
-    k_verify_vec<L2, KNN, NVV><<<wave_grid(k_verify_vec<L2, KNN, NVV>, grid, kT), kT, 0, st>>>(                     \
+#define GTS_VW(NVV, WW)                                                                                     \
+    k_verify_vec<L2, KNN, NVV, WW><<<wave_grid(k_verify_vec<L2, KNN, NVV, WW>, grid, kT), kT, 0, st>>>(      \
         d, cq.get(), crow.get(), C, thr.get(), cdist.get(), keep.get(), counters.get())
+#define GTS_VV(NVV)                             \
+    do {                                        \
+        if (L2 && !KNN && d.qrn2)               \
+            GTS_VW(NVV, (L2 && !KNN));          \
+        else                                    \
+            GTS_VW(NVV, false);                 \
+    } while (0)
         switch (nv) {
             case 1: GTS_VV(1); break;
             case 2: GTS_VV(2); break;
@@ -4346,6 +4355,7 @@ struct Runner {
             default: GTS_VV(0); break;
         }
 #undef GTS_VV
+#undef GTS_VW
     }
 
     // query_major: the pairs come sorted by query (the kNN merge needs that
