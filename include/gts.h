@@ -338,8 +338,10 @@ gts_status gts_multi_knn(gts_index *const *cols, int32_t m, const gts_objects *q
  *              between (default 3).
  *  probe_rows: kNN probe, object rows evaluated before the descent to bound
  *              the k-th distance, 0 .. 4096 (default 1024): at most that many,
- *              taken from the rows nearest in the table; above 16 dimensions
- *              256, or 16 per neighbour wanted if that is more.
+ *              taken from the rows nearest in the table.  Batches above 16
+ *              dimensions that run distance tiles evaluate 256, or 16 per
+ *              neighbour wanted if that is more; 64, or 4 per neighbour, where
+ *              the tensor-core tiles run in two phases.
  *  tc_queries: BF16 tensor-core tiles for dim <= 128, queries per chunk:
  *              128 (two staging slots, default) or 96 (three slots).
  *  str_chunk:  edit distance, (query, object) pairs per block of the

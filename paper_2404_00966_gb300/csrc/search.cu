@@ -4927,8 +4927,12 @@ void run_query(gts_index *ix, const QueryBatch &qb, bool knn, int precision, int
         const int nw = nq <= 608 ? 8 : nq <= 1216 ? 4 : nq <= 4864 && t.dim > kScanMaxDim ? 2 : 1;
         // a row of more than 16 coordinates costs as much as five of the kept
         // pairs that it saves from 256 rows on (16 a neighbour for large k);
-        // a row of a few coordinates next to nothing
-        int per_k = t.dim > kScanMaxDim ? 16 : 0, least = 256;
+        // a row of a few coordinates next to nothing.  Where no tiles run,
+        // a pair saved is a candidate saved in every later pass, and all of
+        // probe_rows pay (256 / 1,024 rows: 10^5 x 33, L1, 2,000 queries 13.47 /
+        // 13.10 ms; x 17, 150 queries, 1 MiB budget 62.9 / 60.2)
+        const bool tiles = R.use_tc || R.use_l1 || R.use_f32;
+        int per_k = t.dim > kScanMaxDim && tiles ? 16 : 0, least = 256;
         // The tiles' first phase lowers the thresholds better than the probe:
         // 64 rows, or four a neighbour, then do (10^4 queries, rows 512 / 256 /
         // 128 / 64: 10^6 x 128 6.65 / 6.64 / 6.54 / 6.48 ms, angular 2 * 10^5 x
