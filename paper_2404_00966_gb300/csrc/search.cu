@@ -45,6 +45,8 @@ constexpr int64_t kCoarseRows = 64;              // tensor-core tiles: rows per 
                                                  // queries may run over the level above (coarse_tiles_pay)
 constexpr int64_t kF32TileEntries = 4;           // FP32 tiles: least last-level entries per node
 constexpr int64_t kF32TilePairs = 6 << 20;       // and least (entry, row) pairs (f32_tiles_pay)
+constexpr int64_t kF32LeastRows = 10;            // and least rows per node (f32_route)
+constexpr int64_t kF32SureL1 = 200, kF32SureL2 = 40;   // rows per node from which the tiles run without a sample
 constexpr int64_t kScanPairs = 16 << 20;         // table scan of low-dimensional vectors: least pairs
 constexpr int64_t kTilePhaseItems = 1216;        // tensor-core tile kNN: items from which they run in two phases
 constexpr int64_t kCosNorms = 64;                 // angular batches: queries from which their sums are formed first
@@ -1119,6 +1121,39 @@ __global__ void k_leafscan_small(Dev d, const int32_t *__restrict__ eq, const in
         tested = __reduce_add_sync(0xffffffffu, (unsigned)tested);
         if ((threadIdx.x & 31) == 0 && tested) atomicAdd(scanned, (unsigned long long)tested);
     }
+}
+
+// The leaf scan's candidates of `samples` evenly spaced entries, a warp each.
+__global__ void k_leaf_sample(Dev d, const int32_t *__restrict__ eq, const int32_t *__restrict__ enode,
+                              const float *__restrict__ path, int64_t lvl_last, int64_t e0, int64_t E, int64_t samples,
+                              const uint64_t *__restrict__ mask, const float *__restrict__ thr_q,
+                              unsigned long long *__restrict__ candidates) {
+    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (w >= samples) return;
+    const int64_t e = e0 + E * w / samples;
+    const uint64_t m = mask[e - e0];
+    if (m == 0) return;
+    const int32_t q = eq[e];
+    const int64_t node = lvl_last + enode[e];
+    const int32_t pos = d.npos[node], size = d.nsize[node];
+    const int32_t avg = size / d.F;
+    const int64_t s = d.qseq[q];
+    const float thr = thr_q[q];
+    unsigned count = 0;
+    for (int32_t r = lane; r < size; r += 32) {
+        const int32_t j = avg > 0 ? min(r / avg, d.F - 1) : d.F - 1;
+        if (!((m >> j) & 1ull) || d.row_del[pos + r] <= s) continue;
+        bool pass = true;
+        for (int t = 0; t < d.h && pass; ++t) {
+            const float T = d.table[(int64_t)t * d.n + pos + r], dq = path[e * d.h + t];
+            const float eps = (d.epsc > 0.f ? d.epsc * (T + dq + thr) : 0.f) + d.lslack[t];
+            pass = !(fabsf(T - dq) > thr + eps);
+        }
+        count += pass ? 1u : 0u;
+    }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0 && count) atomicAdd(candidates, (unsigned long long)count);
 }
 
 // ---------------------------------------------------------------- diagnostics
@@ -3278,7 +3313,8 @@ struct Runner {
 
     void process(Level &L, int64_t e0, int64_t e1, int l) {
         if (e1 <= e0) return;
-        if (l == h - 1 && (use_tc || use_l1 || use_scan || (use_f32 && f32_tiles_pay(e1 - e0, kF32TilePairs)) ||
+        const F32Route f32 = use_f32 && l == h - 1 ? f32_route(e1 - e0) : kF32Plain;
+        if (l == h - 1 && (use_tc || use_l1 || use_scan || f32 == kF32Tiles ||
                            (use_scan_large && f32_tiles_pay(e1 - e0, kScanPairs)))) {
             last_level_tc(L, e0, e1, l);
             return;
@@ -3343,7 +3379,7 @@ struct Runner {
                                                                    lvl_next, e0, e1, thr.get(), nullptr, nullptr,
                                                                    nullptr, nullptr, nullptr, mask.get());
             clk.end();
-            if (use_tc) {
+            if (use_tc || (f32 == kF32Ask && f32_sample_pays(L, e0, e1, mask))) {
                 tc_leaf(L, e0, e1, mask);
                 return;
             }
@@ -4169,9 +4205,61 @@ struct Runner {
     // The node-major table scan of low-dimensional vectors needs more pairs
     // (3-D kNN, 10^6 points, plain / scan: 200 queries 811 / 885, 5,000 3139 /
     // 2345; 5 * 10^6, 200: 1091 / 1061, 5,000: 6751 / 4231).
+    // Nodes of few rows leave most of a 128-row block empty (L1 tiles compute it
+    // whole, L2 tiles in groups of 32 rows): see f32_route.
     bool f32_tiles_pay(int64_t E, int64_t least_pairs) const {
         const int64_t nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
         return E >= kF32TileEntries * nn && E * ((ix->tree.n + nn - 1) / nn) >= least_pairs;
+    }
+
+    // FP32 tiles, by the rows of a node: always from kF32SureL1 / kF32SureL2 rows on,
+    // never below kF32LeastRows, and in between by the share of the pairs that the
+    // table bound leaves, which a sample of the entries tells (f32_sample_pays).
+    // Batches of 20 to 1,500 queries on 60,000 to 600,000 rows of 24 to 256 dimensions,
+    // trees of 3 to 10,000 rows a node, plain / tiles, least and median: L1, 200 rows
+    // and more 1.16 / 1.7 to 6.2, 40 to 200 rows 0.66 / 1.1 to 2.5, 8 to 20 rows 0.58 /
+    // 0.7 to 1.2, fewer 0.30 / 0.5; L2, from 40 rows on 0.90 / 1.2 to 7.8, 8 to 20 0.79 /
+    // 0.9 to 2.2, fewer 0.48 / 0.7 to 1.2.  (600,000 x 200, L1, 18 rows a node, 60 queries,
+    // range: tiles 2.23 ms, plain 1.21.)
+    enum F32Route { kF32Plain, kF32Ask, kF32Tiles };
+    F32Route f32_route(int64_t E) const {
+        if (!f32_tiles_pay(E, kF32TilePairs)) return kF32Plain;
+        const int64_t rows = ix->tree.n / (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
+        if (rows >= (d.metric == GTS_L1 ? kF32SureL1 : kF32SureL2)) return kF32Tiles;
+        return rows >= kF32LeastRows ? kF32Ask : kF32Plain;
+    }
+
+    // Whether the tiles beat the plain path on these entries.  Costs in ns, fitted to
+    // the batches above for nodes of 10 rows and more (errors of 5 to 10 %): plain, per
+    // entry and 32-row strip of its node (two table scans) and per candidate (wide
+    // rows: per 256 coordinates); tiles, per block, per 64 (L1) or 128 (L2) queries on
+    // its rows' coordinates, and per entry (regrouped); 150 us for the regrouping's launches
+    // and host round trips.  Of 553 such batches 16 took the slower route, the worst by
+    // 1.20.
+    bool f32_sample_pays(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+        const int64_t E = e1 - e0, nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
+        const int64_t samples = std::min<int64_t>(E, 2048);
+        DBuf<unsigned long long> c(1, st);
+        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 8, st));
+        clk.begin(GTS_STAGE_LEAF_SCAN);
+        k_leaf_sample<<<nblocks(samples, kWarpsPerBlock), kT, 0, st>>>(d, L.q.get(), L.node.get(), L.path.get(),
+                                                                       ix->tree.lvl_off[h - 1], e0, E, samples,
+                                                                       mask.get(), thr.get(), c.get());
+        clk.end();
+        check_launch("leaf sample");
+        const double per = (double)d2h_i64(reinterpret_cast<const int64_t *>(c.get()), st) / (double)samples;
+        const double rows = (double)ix->tree.n / (double)nn, blocks = (double)nn * std::ceil(rows / 128.0);
+        const double strips = std::ceil(rows / 32.0), ent = (double)E, wide = std::max(1.0, d.dim / 256.0);
+        double plain, tiles;
+        if (d.metric == GTS_L1) {
+            plain = (0.55 + 0.25 * strips) * ent + 0.12 * per * ent * wide;
+            tiles = 1.5e5 + blocks * (20.0 + 0.08 * d.dim) + 0.29 / 64.0 * ent * std::ceil(rows / 128.0) * d.dim +
+                    0.2 * ent + 0.017 * per * ent;
+        } else {
+            plain = 0.74 * strips * ent + 0.16 * per * ent * wide;
+            tiles = 1.5e5 + blocks * (17.0 + 0.07 * d.dim) + 0.64 / 128.0 * ent * strips / 4.0 * d.dim + 0.2 * ent;
+        }
+        return tiles < plain;
     }
 
     // pos_of[q]: the place of query q in the order of the probe keys
