@@ -2576,12 +2576,14 @@ __global__ void k_transpose_f32(const float *__restrict__ in, int64_t rows, int6
 // intervals), the node x query bitmap of the pairs with a surviving leaf, and
 // the counts of member pairs and of pairs with a surviving leaf.  Queries are
 // taken in column order: position i is query perm[i] (DT, M and the bitmap are
-// in position order).  A block takes one parent, all of its F nodes, and
-// kLeafQueries queries, a thread per query: the query's threshold and the
+// in position order).  A block takes nodes [z nodes, (z + 1) nodes) of one parent
+// and `queries` queries, a thread per query: the query's threshold and the
 // parent's child mask (the membership of all F nodes) are read once, and every
 // access to DT and M is coalesced.  (A node at a time with its membership
-// looked up per pair took 0.71 ms for 8,000 nodes x 10^4 queries; this form
-// 0.56.)
+// looked up per pair took 0.71 ms for 8,000 nodes x 10^4 queries; all F of them
+// 0.56.)  Few parents or queries take fewer nodes and queries a block, so that
+// the blocks fill the device (a parent of 64 nodes, 1,200 queries: two blocks; the
+// call 0.80 -> 0.48 ms).
 //
 // Sorted form: the build cuts a node's rows, in ascending distance to its
 // pivot, into consecutive children, so the non-empty children are a suffix
@@ -2597,20 +2599,21 @@ constexpr int kLeafQueries = 1024;
 __global__ void __launch_bounds__(256) k_leaf_dense(Dev d, const float *__restrict__ DT,
                                                     const uint64_t *__restrict__ cm, int64_t P, int64_t nq,
                                                     int64_t lvl_next, const float *__restrict__ thr_q,
-                                                    const int32_t *__restrict__ perm, uint64_t *__restrict__ M,
-                                                    uint32_t *__restrict__ bits, int64_t nw,
+                                                    const int32_t *__restrict__ perm, int queries, int nodes,
+                                                    uint64_t *__restrict__ M, uint32_t *__restrict__ bits, int64_t nw,
                                                     unsigned long long *__restrict__ counts) {
-    extern __shared__ float s_iv[];          // hi [F][F], lo [F][F] of the F nodes' children
+    extern __shared__ float s_iv[];          // hi [nodes][F], lo [nodes][F] of the nodes' children
     __shared__ unsigned long long s_ne[64];  // per node: its non-empty children
     __shared__ int8_t s_j0[64];              // the first of them; -1: not sorted
     const int F = d.F;
-    float *s_hi = s_iv, *s_lo = s_iv + F * F;
+    float *s_hi = s_iv, *s_lo = s_iv + nodes * F;
     const int lane = threadIdx.x & 31;
     const int64_t par = blockIdx.x;
-    const int64_t p0 = par * F;
+    const int n0 = (int)blockIdx.z * nodes, nn = min(nodes, F - n0);   // this block's nodes: p0 .. p0 + nn - 1
+    const int64_t p0 = par * F + n0;
     if (threadIdx.x < 64) s_ne[threadIdx.x] = 0ull;
     __syncthreads();
-    for (int i = threadIdx.x; i < F * F; i += blockDim.x) {
+    for (int i = threadIdx.x; i < nn * F; i += blockDim.x) {
         const int64_t c = lvl_next + p0 * F + i;
         const bool ne = d.nsize[c] > 0;
         s_hi[i] = ne ? d.nhi[c] : 0.f;
@@ -2618,7 +2621,7 @@ __global__ void __launch_bounds__(256) k_leaf_dense(Dev d, const float *__restri
         if (ne) atomicOr(&s_ne[i / F], 1ull << (i % F));
     }
     __syncthreads();
-    if (threadIdx.x < F) {
+    if (threadIdx.x < nn) {
         const float *hi = s_hi + threadIdx.x * F, *lo = s_lo + threadIdx.x * F;
         const uint64_t ne = s_ne[threadIdx.x];
         bool bad = ne == 0ull || hi[F - 1] < lo[F - 1];
@@ -2631,17 +2634,17 @@ __global__ void __launch_bounds__(256) k_leaf_dense(Dev d, const float *__restri
     __syncthreads();
     const float epsc = d.epsc, lab = d.lslack[d.h - 1];
     unsigned long long nmem = 0, nlive = 0;
-    const int64_t qa = (int64_t)blockIdx.y * kLeafQueries;
-    for (int64_t q0 = qa; q0 < nq && q0 < qa + kLeafQueries; q0 += blockDim.x) {
+    const int64_t qa = (int64_t)blockIdx.y * queries;
+    for (int64_t q0 = qa; q0 < nq && q0 < qa + queries; q0 += blockDim.x) {
         const int64_t q = q0 + threadIdx.x;                          // column position
         const int64_t qq = q < nq && perm ? (int64_t)perm[q] : q;    // its query
         const uint64_t mem = q < nq ? cm[par * nq + qq] : 0ull;
         const float thr = q < nq ? thr_q[qq] : 0.f;
         const int64_t w = (q - lane) >> 5;   // the warp's word of the bitmap
 #pragma unroll 2
-        for (int n = 0; n < F; ++n) {
+        for (int n = 0; n < nn; ++n) {
             uint64_t m = 0;
-            const bool member = (mem >> n) & 1ull;
+            const bool member = (mem >> (n0 + n)) & 1ull;
             if (member) {
                 const float dq = __ldg(DT + (p0 + n) * nq + q);
                 const float *hi = s_hi + n * F, *lo = s_lo + n * F;
@@ -3628,10 +3631,18 @@ struct Runner {
         {
             dim3 tb(32, 8), tg((unsigned)((P + 31) / 32), (unsigned)((nq + 31) / 32));
             if (!have_dt) k_transpose_f32<<<tg, tb, 0, st>>>(D, nq, P, DT.get(), perm.get());
-            const dim3 lg((unsigned)Pp, (unsigned)((nq + kLeafQueries - 1) / kLeafQueries));
-            k_leaf_dense<<<lg, 256, (size_t)2 * F * F * 4, st>>>(d, DT.get(), cm.get(), P, nq, ix->tree.lvl_off[h],
-                                                                thr.get(), perm.get(), M.get(), rg.bits.get(), rg.nw,
-                                                                cnt.get());
+            // 1,024 queries and all F nodes a block, fewer while that leaves less than
+            // four blocks an SM
+            int lq = kLeafQueries, ln = F;
+            auto grid = [&] {
+                return dim3((unsigned)Pp, (unsigned)((nq + lq - 1) / lq), (unsigned)((F + ln - 1) / ln));
+            };
+            auto few = [&] { return (int64_t)grid().x * grid().y * grid().z < max_blocks / 2; };
+            while (lq > 256 && few()) lq /= 2;
+            while (ln > 1 && few()) ln = (ln + 1) / 2;
+            k_leaf_dense<<<grid(), 256, (size_t)2 * ln * F * 4, st>>>(d, DT.get(), cm.get(), P, nq, ix->tree.lvl_off[h],
+                                                                     thr.get(), perm.get(), lq, ln, M.get(),
+                                                                     rg.bits.get(), rg.nw, cnt.get());
         }
         clk.end();
         check_launch("dense leaf masks");
