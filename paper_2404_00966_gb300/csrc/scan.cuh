@@ -27,7 +27,7 @@ struct ScanQuery {
     // decide it against the radius with the FP32 error band; accepted pairs
     // go straight to the answer, pairs inside the band to the FP64 recheck
     bool fused_range = false;
-    // kNN on such vectors: the same distance, and only the pairs whose lower
+    // kNN on such vectors (scan_decides_knn): the same distance, and only the pairs whose lower
     // bound is within tau_q are written, with their distance
     bool fused_knn = false;
     const float *Q = nullptr; // queries [nq, dim]

@@ -3931,6 +3931,19 @@ struct Runner {
         tc_finish(tq, rg);
     }
 
+    // Whether the table scan also forms the distances of kNN pairs.  It does so strip
+    // by strip, the lanes whose rows pass the table bound; with few of them the
+    // verification's full warps are faster.  10^5 and 10^6 points of 4 to 16 dimensions, 3 to 2,000
+    // rows a node, 400 and 3,000 queries, k = 1 to 100, candidates first / decided in
+    // the scan: fewer than 1 candidate a strip 0.7 to 1.0 (the more dimensions the less), 1
+    // to 2 0.8 to 1.0, 2 to 3 0.9 to 1.1, 5 and more 1.1 to 4.  Up to 4 dimensions and
+    // from 256 rows a node on it always decides.
+    bool scan_decides_knn(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+        const int64_t rows = ix->tree.n / (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
+        if (d.dim <= 4 || rows >= 256) return true;
+        return candidates_per_entry(L, e0, e1, mask) >= 2.0 * (double)((rows + 31) / 32);
+    }
+
     // Last level of low-dimensional vectors: regroup the entries by node, scan
     // each node block's table rows once against all of its queries (leaf
     // mask, visibility, Lemma 1 / 2 lower bound), then verify the candidates
@@ -3960,7 +3973,7 @@ struct Runner {
         // range: decide the pairs in the scan (low dimension; the angular
         // distance takes its FP64 key for every pair, so not there)
         sq.fused_range = !knn && !d.cosine;
-        sq.fused_knn = knn;
+        sq.fused_knn = knn && scan_decides_knn(L, e0, e1, mask);
         sq.Q = d.Q;
         sq.rel = d.rel;
         sq.absf = d.absf;
@@ -4240,6 +4253,20 @@ struct Runner {
         return rows >= kF32LeastRows ? kF32Ask : kF32Plain;
     }
 
+    // candidates of the table scan per last-level entry, from a sample of up to 2,048
+    double candidates_per_entry(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
+        const int64_t samples = std::min<int64_t>(e1 - e0, 2048);
+        DBuf<unsigned long long> c(1, st);
+        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 8, st));
+        clk.begin(GTS_STAGE_LEAF_SCAN);
+        k_leaf_sample<<<nblocks(samples, kWarpsPerBlock), kT, 0, st>>>(d, L.q.get(), L.node.get(), L.path.get(),
+                                                                       ix->tree.lvl_off[h - 1], e0, e1 - e0, samples,
+                                                                       mask.get(), thr.get(), c.get());
+        clk.end();
+        check_launch("leaf sample");
+        return (double)d2h_i64(reinterpret_cast<const int64_t *>(c.get()), st) / (double)samples;
+    }
+
     // Whether the tiles beat the plain path on these entries.  Costs in ns, fitted to
     // the batches above for nodes of 10 rows and more (errors of 5 to 10 %): plain, per
     // entry and 32-row strip of its node (two table scans) and per candidate (wide
@@ -4249,16 +4276,7 @@ struct Runner {
     // 1.20.
     bool f32_sample_pays(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
         const int64_t E = e1 - e0, nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
-        const int64_t samples = std::min<int64_t>(E, 2048);
-        DBuf<unsigned long long> c(1, st);
-        GTS_CUDA(cudaMemsetAsync(c.get(), 0, 8, st));
-        clk.begin(GTS_STAGE_LEAF_SCAN);
-        k_leaf_sample<<<nblocks(samples, kWarpsPerBlock), kT, 0, st>>>(d, L.q.get(), L.node.get(), L.path.get(),
-                                                                       ix->tree.lvl_off[h - 1], e0, E, samples,
-                                                                       mask.get(), thr.get(), c.get());
-        clk.end();
-        check_launch("leaf sample");
-        const double per = (double)d2h_i64(reinterpret_cast<const int64_t *>(c.get()), st) / (double)samples;
+        const double per = candidates_per_entry(L, e0, e1, mask);
         const double rows = (double)ix->tree.n / (double)nn, blocks = (double)nn * std::ceil(rows / 128.0);
         const double strips = std::ceil(rows / 32.0), ent = (double)E, wide = std::max(1.0, d.dim / 256.0);
         double plain, tiles;
