@@ -4141,6 +4141,7 @@ struct Runner {
         StrQuery sq;
         sq.qg = d.qg;
         sq.qgq = d.qgq;
+        sq.nq = qb.nq;
         sq.any_deleted = any_deleted;
         sq.queries = tu.str_qgram == 32 ? 32 : 64;
         std::atomic<int64_t> &known = ix->tc_pairs_hint[knn ? 1 : 0];

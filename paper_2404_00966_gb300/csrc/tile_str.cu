@@ -41,7 +41,8 @@ struct StrArgs {
     const TileRec *grec;
     const int32_t *gq;          // the records' queries
     const int4 *items;
-    int64_t i1;
+    int64_t units;              // work units: item u / split, its query chunks u % split, + split, ...
+    int split;
     int *work_counter;
     int32_t *out_q, *out_row;
     int64_t cap;
@@ -76,24 +77,31 @@ __global__ void __launch_bounds__(kThreadsS, 2) k_tile_qgram(StrArgs a) {
     for (;;) {
         if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
         __syncthreads();
-        const int64_t item = s_item;
-        if (item >= a.i1) break;
-        const int4 it = a.items[item];
+        const int64_t unit = s_item;
+        if (unit >= a.units) break;
+        const int4 it = a.items[unit / a.split];
+        const int part = (int)(unit % a.split);
         const int64_t g = a.lvl_last + it.x;
         const int first = it.y, total = it.z;
-        const int nchunk = (total + NQS - 1) / NQS;
+        // the unit's chunks: c = 0, 1, ..  is the node's chunk part + c split
+        const int nchunk = ((total + NQS - 1) / NQS - part + a.split - 1) / a.split;
+        if (nchunk <= 0) {
+            __syncthreads();   // s_item is read by everyone
+            continue;
+        }
+        auto begin = [&](int c) { return (part + c * a.split) * NQS; };
         // chunk c into buffer c & 1; qid: the query of this thread's piece
         auto query_of = [&](int c) -> int32_t {
-            const int j = c * NQS + cj;
-            return cj < NQS && j < total ? a.gq[first + j] : -1;
+            const int j = begin(c) + cj;
+            return c < nchunk && cj < NQS && j < total ? a.gq[first + j] : -1;
         };
         auto stage = [&](int c, int32_t qid) {
-            const int cnt = min(NQS, total - c * NQS);
+            const int cnt = min(NQS, total - begin(c));
             if (qid >= 0)
                 cpa16s(&sQ[c & 1][cj][cw], reinterpret_cast<const uint4 *>(a.qgq + (int64_t)qid * 64) + cw);
             if (tid < 2 * cnt)
                 cpa16s(reinterpret_cast<uint4 *>(&sRec[c & 1][0]) + tid,
-                       reinterpret_cast<const uint4 *>(a.grec + first + c * NQS) + tid);
+                       reinterpret_cast<const uint4 *>(a.grec + first + begin(c)) + tid);
         };
         const int32_t qid0 = query_of(0);
         int32_t qnext = query_of(1);
@@ -134,7 +142,7 @@ __global__ void __launch_bounds__(kThreadsS, 2) k_tile_qgram(StrArgs a) {
                 stage(c + 1, qnext);
                 qnext = query_of(c + 2);
             }
-            const int cnt = min(NQS, total - c * NQS);
+            const int cnt = min(NQS, total - begin(c));
             const TileRec *rec = sRec[c & 1];
             const int j0 = warp * kPer;
             const int nj = max(0, min(kPer, cnt - j0));
@@ -242,9 +250,10 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
     for (;;) {
         if (tid == 0) s_item = atomicAdd(a.work_counter, 1);
         __syncthreads();
-        const int64_t item = s_item;
-        if (item >= a.i1) break;
-        const int4 it = a.items[item];
+        const int64_t unit = s_item;
+        if (unit >= a.units) break;
+        const int4 it = a.items[unit / a.split];
+        const int part = (int)(unit % a.split);
         const int64_t g = a.lvl_last + it.x;
         const int first = it.y, total = it.z;
         const int rb = it.w * kRowsS;
@@ -273,7 +282,7 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
                 rw[4 * v + 3] = x.w;
             }
         }
-        for (int c0 = 0; c0 < total; c0 += kNQD) {
+        for (int c0 = part * kNQD; c0 < total; c0 += a.split * kNQD) {
             const int cnt = min(kNQD, total - c0);
             __syncthreads();   // the previous chunk's shared data is no longer read
             for (int i = tid; i < kNQD * 64; i += kThreadsS)
@@ -357,7 +366,13 @@ __global__ void __launch_bounds__(kThreadsS, 3) k_tile_short(ShortArgs A) {
     }
 }
 
-StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1) {
+// parts of an item's query chunks: more than one while there are fewer than four
+// units per resident CTA (5,000 words in 20 nodes, 2,000 queries: 40 blocks of rows)
+int chunk_parts(int64_t items, int64_t resident, int64_t nq, int chunk) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>((nq + chunk - 1) / chunk, (4 * resident + items - 1) / items));
+}
+
+StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t i0, int64_t i1, int split) {
     StrArgs a;
     a.F = t.F;
     a.npos = t.npos.get();
@@ -370,7 +385,8 @@ StrArgs str_args(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_t
     a.grec = rg.grec.get();
     a.gq = rg.gq.get();
     a.items = rg.items.get() + i0;
-    a.i1 = i1 - i0;
+    a.units = (i1 - i0) * split;
+    a.split = split;
     return a;
 }
 
@@ -386,7 +402,9 @@ int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const
     GTS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_short, kThreadsS, 0));
     if (per_sm < 1) per_sm = 1;
-    const int64_t grid = std::min<int64_t>(i1 - i0, (int64_t)sms * per_sm);
+    const int64_t resident = (int64_t)sms * per_sm;
+    const int split = chunk_parts(i1 - i0, resident, sq.nq, kNQD);
+    const int64_t grid = std::min<int64_t>((i1 - i0) * split, resident);
     DBuf<int> counter(1, st);
     DBuf<unsigned long long> count(1, st);
     int64_t cap = cap_hint > 0 ? cap_hint : 1 << 20;
@@ -397,7 +415,7 @@ int64_t short_run(const Tree &t, const StrQuery &sq, const ShortQuery &hq, const
         GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
         ShortArgs A;
-        A.s = str_args(t, sq, rg, i0, i1);
+        A.s = str_args(t, sq, rg, i0, i1, split);
         A.s.work_counter = counter.get();
         A.s.out_q = out_q.get();
         A.s.out_row = out_row.get();
@@ -435,7 +453,9 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_
     else
         GTS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_qgram<64>, kThreadsS, 0));
     if (per_sm < 1) per_sm = 1;
-    const int64_t grid = std::min<int64_t>(i1 - i0, (int64_t)sms * per_sm);
+    const int64_t resident = (int64_t)sms * per_sm;
+    const int split = chunk_parts(i1 - i0, resident, sq.nq, sq.queries == 32 ? 32 : 64);
+    const int64_t grid = std::min<int64_t>((i1 - i0) * split, resident);
     DBuf<int> counter(1, st);
     DBuf<unsigned long long> count(1, st);
     int64_t cap = cap_hint > 0 ? cap_hint : 1 << 20;
@@ -444,7 +464,7 @@ int64_t qgram_run(const Tree &t, const StrQuery &sq, const TcRegroup &rg, int64_
         out_row.alloc(cap, st);
         GTS_CUDA(cudaMemsetAsync(counter.get(), 0, 4, st));
         GTS_CUDA(cudaMemsetAsync(count.get(), 0, 8, st));
-        StrArgs a = str_args(t, sq, rg, i0, i1);
+        StrArgs a = str_args(t, sq, rg, i0, i1, split);
         a.work_counter = counter.get();
         a.out_q = out_q.get();
         a.out_row = out_row.get();

@@ -10,6 +10,7 @@ namespace gts {
 struct StrQuery {
     const uint8_t *qg = nullptr;    // the tree rows' 3-gram bucket counts [n, 64]
     const uint8_t *qgq = nullptr;   // the batch's queries' [nq, 64]
+    int64_t nq = 0;                 // queries of the batch
     int any_deleted = 1;
     int queries = 64;               // queries per tile chunk: 32 or 64
 };
