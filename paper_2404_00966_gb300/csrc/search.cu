@@ -4033,11 +4033,28 @@ struct Runner {
         merge_knn(q2, r2, d2, C);
     }
 
+    bool short_strings() const { return ix->tree.max_len <= kShortStr && qb.max_len <= kShortStr; }
+    // Short strings: filter and distance in one tile, or the 3-gram tile and the DP of
+    // its pairs.  A thread of the one tile holds a row, and kNN, whose thresholds
+    // let most pairs through to the distance, needs its warps filled (5,000 to 300,000 strings
+    // of 4 to 32 letters, 100 to 2,000 queries, two tiles / one, least and median: nodes of 8 to
+    // 12 rows 0.51 / 0.7, 12 to 20 0.58 / 0.9, 20 to 40 0.94 / 1.0, more 0.83 / 1.2 to 2.5;
+    // range 1.07 / 1.4 at any size).
+    bool short_tile_pays() const {
+        const int64_t rows = ix->tree.n / (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
+        return short_strings() && (!knn || rows >= 20);
+    }
+
     // Strings: whether E last-level entries go through the 3-gram tiles: always
     // with GTS_PREC_BF16, with GTS_PREC_FP32 (the same exact distances) from
-    // the number of (entry, row) pairs on that pays for the regrouping.
+    // the number of (entry, row) pairs on that pays for the regrouping.  Not kNN over
+    // long strings: its first thresholds, from the pivots, exclude next to nothing,
+    // and the pairs only take the longer way (40 to 200 letters, 60,000 to 300,000 strings: 0.87
+    // to 1.01 times the speed of the plain path; reads of 100 to 108 0.91 to 1.04, nodes of 9
+    // rows 1.1 to 1.2).
     bool qgram_tiles_pay(int64_t E) const {
         if (use_qg) return true;
+        if (knn && !short_strings()) return false;
         const int64_t nn = ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1];
         return use_qg_large && E * ((ix->tree.n + nn - 1) / nn) >= kF32TilePairs;
     }
@@ -4084,7 +4101,7 @@ struct Runner {
         const double pass_ps = 90.0 * hs[h] / kSample;
         const double window = 256.0 * (double)((qb.nq + 255) / 256) / (double)qb.nq;
         double row_ps = 1.6 + pass_ps;
-        if (t.max_len <= kShortStr && qb.max_len <= kShortStr) row_ps = 16.0;
+        if (short_strings()) row_ps = 16.0;
         else if (t.n <= kQtcRows && qb.nq * t.n >= kQtcPairs && window <= 6.0) row_ps = 0.25 * window + pass_ps;
         double pivots = 0.0, alive = 1.0, best = 0.0;
         int stop = -1;
@@ -4147,7 +4164,7 @@ struct Runner {
         std::atomic<int64_t> &known = ix->tc_pairs_hint[knn ? 1 : 0];
         const int64_t hint = first_room(known, pair_room());
         int64_t seen = 0;
-        if (ix->tree.max_len <= kShortStr && qb.max_len <= kShortStr) {
+        if (short_tile_pays()) {
             ShortQuery hq;
             hq.S = d.S;
             hq.Soff = d.Soff;
@@ -4173,7 +4190,10 @@ struct Runner {
             seen_pairs(known, seen);
             return;
         }
-        const bool tensor = qtc_pays(ix->tree, qb.nq, rg);
+        // (kNN: its first thresholds let most pairs through, and the tensor-core
+        // tile looks up every pair it keeps: 60,000 words in nodes of 15, 2,000 queries, 7.7 ms
+        // against 1.5 on the integer units)
+        const bool tensor = !knn && qtc_pays(ix->tree, qb.nq, rg);
         DBuf<uint8_t> qcode;
         if (tensor) {
             clk.begin(GTS_STAGE_OTHER, 1);

@@ -54,6 +54,23 @@ __device__ __forceinline__ void cpa16s(void *dst, const void *src) {
                  : "memory");
 }
 
+// l[h] += the L1 distances of the lane's first NH rows' counts and the query's
+template <int NH>
+__device__ __forceinline__ void add_l1(uint32_t (&l)[kRPL], const uint32_t (&rw)[kRPL][kWords], const uint4 *qv) {
+#pragma unroll
+    for (int v = 0; v < kWords / 4; ++v) {
+        const uint4 x = qv[v];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) l[h] = __vsadu4(rw[h][4 * v], x.x) + l[h];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) l[h] = __vsadu4(rw[h][4 * v + 1], x.y) + l[h];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) l[h] = __vsadu4(rw[h][4 * v + 2], x.z) + l[h];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) l[h] = __vsadu4(rw[h][4 * v + 3], x.w) + l[h];
+    }
+}
+
 // NQS: queries per chunk (32 or 64; a tuning parameter), NQS / 8 per warp.
 // The ALU pipe bounds it: 16 four-byte sums of absolute differences per pair
 // (19 T a second on the device, 60 of 64 lanes per SM and cycle: 1.9 * 10^10
@@ -63,7 +80,9 @@ __device__ __forceinline__ void cpa16s(void *dst, const void *src) {
 // two rows a lane (31.9 ms; now 31.4) or one (53.0) they held the kernel back.
 // The sums
 // start at -(limit + 1), so that the test is their sign bit, shifted into the
-// pass masks; a chunk's records and vectors are copied while the one before is
+// pass masks; a block of at most 32 or 64 rows (small nodes) skips the lanes' empty
+// rows (110 M pairs in nodes of 15 rows: 1.5 ms; a row a thread took 2.3); a
+// chunk's records and vectors are copied while the one before is
 // computed (the query ids they need are read two chunks ahead); and the leaf
 // and visibility tests run on the few pairs that pass.
 template <int NQS>
@@ -162,20 +181,16 @@ __global__ void __launch_bounds__(kThreadsS, 2) k_tile_qgram(StrArgs a) {
                 uint32_t l[kRPL] = {0u, 0u, 0u, 0u};
                 if ((lives >> i) & 1u) {   // warp-uniform
                     const uint32_t s0 = (uint32_t)__shfl_sync(0xffffffffu, start, i);
-#pragma unroll
-                    for (int h = 0; h < kRPL; ++h) l[h] = s0;
                     const uint4 *qv = sQ[c & 1][j0 + i];
-#pragma unroll
-                    for (int v = 0; v < kWords / 4; ++v) {
-                        const uint4 x = qv[v];
-#pragma unroll
-                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v], x.x) + l[h];
-#pragma unroll
-                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 1], x.y) + l[h];
-#pragma unroll
-                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 2], x.z) + l[h];
-#pragma unroll
-                        for (int h = 0; h < kRPL; ++h) l[h] = __vsadu4(rw[h][4 * v + 3], x.w) + l[h];
+                    l[0] = s0;
+                    if (nrow > 64) {
+                        l[1] = l[2] = l[3] = s0;
+                        add_l1<4>(l, rw, qv);
+                    } else if (nrow > 32) {
+                        l[1] = s0;
+                        add_l1<2>(l, rw, qv);
+                    } else {
+                        add_l1<1>(l, rw, qv);
                     }
                 }
                 // (nj <= 8: a row's bits stay inside its byte)
