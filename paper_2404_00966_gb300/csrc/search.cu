@@ -3318,7 +3318,7 @@ struct Runner {
         if (e1 <= e0) return;
         const F32Route f32 = use_f32 && l == h - 1 ? f32_route(e1 - e0) : kF32Plain;
         if (l == h - 1 && (use_tc || use_l1 || use_scan || f32 == kF32Tiles ||
-                           (use_scan_large && f32_tiles_pay(e1 - e0, kScanPairs)))) {
+                           (use_scan_large && !scan_asks() && f32_tiles_pay(e1 - e0, kScanPairs)))) {
             last_level_tc(L, e0, e1, l);
             return;
         }
@@ -3383,6 +3383,11 @@ struct Runner {
                                                                    nullptr, nullptr, nullptr, mask.get());
             clk.end();
             if (use_tc || (f32 == kF32Ask && f32_sample_pays(L, e0, e1, mask))) {
+                tc_leaf(L, e0, e1, mask);
+                return;
+            }
+            if (use_scan_large && scan_asks() && f32_tiles_pay(E, kScanPairs) &&
+                strips_filled(candidates_per_entry(L, e0, e1, mask))) {
                 tc_leaf(L, e0, e1, mask);
                 return;
             }
@@ -3938,10 +3943,19 @@ struct Runner {
     // the scan: fewer than 1 candidate a strip 0.7 to 1.0 (the more dimensions the less), 1
     // to 2 0.8 to 1.0, 2 to 3 0.9 to 1.1, 5 and more 1.1 to 4.  Up to 4 dimensions and
     // from 256 rows a node on it always decides.
+    bool strips_filled(double per) const {
+        const int64_t rows = ix->tree.n / (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
+        return per >= 2.0 * (double)((rows + 31) / 32);
+    }
+    // GTS_PREC_FP32, up to two dimensions: kNN asks first whether to scan at all, since
+    // a candidate costs the plain path next to nothing there (10^6 points, 3,000 and 10,000
+    // queries, k = 1, 0.8 candidates a strip: 777 and 1435 us against 965 and 1810; with 3
+    // dimensions 0.92 and more of the scan's speed, with more of them less than it).
+    bool scan_asks() const { return knn && d.dim <= 2; }
     bool scan_decides_knn(Level &L, int64_t e0, int64_t e1, DBuf<uint64_t> &mask) {
         const int64_t rows = ix->tree.n / (ix->tree.lvl_off[h] - ix->tree.lvl_off[h - 1]);
         if (d.dim <= 4 || rows >= 256) return true;
-        return candidates_per_entry(L, e0, e1, mask) >= 2.0 * (double)((rows + 31) / 32);
+        return strips_filled(candidates_per_entry(L, e0, e1, mask));
     }
 
     // Last level of low-dimensional vectors: regroup the entries by node, scan
