@@ -162,7 +162,13 @@ __global__ void k_map_vec(const float *__restrict__ X, int dim, const int32_t *_
         const int32_t pv = piv_obj[node];
         const float *a = X + (int64_t)o * dim;
         const float *b = X + (int64_t)pv * dim;
-        double d = L2 ? l2sq_fp64_seq<false>(a, b, dim) : l1_fp64_seq<false>(a, b, dim);
+        // (l2sq_fp64_seq / l1_fp64_seq without their unrolling, which long rows need: a
+        // level of 10^6 rows of 2 coordinates, us: L2 54.9 with, 44.6 without; L1 32.4, 26.3)
+        double d = 0.0;
+        for (int i = 0; i < dim; ++i) {
+            const double t = __dsub_rn((double)a[i], (double)b[i]);
+            d = __dadd_rn(d, L2 ? __dmul_rn(t, t) : fabs(t));
+        }
         if (L2) d = __dsqrt_rn(d);
         Tl[o] = __double2float_rn(d);
         node_of[o] = node;
