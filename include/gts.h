@@ -66,7 +66,8 @@ typedef enum { GTS_EDIT = 0, GTS_L1 = 1, GTS_L2 = 2, GTS_COS = 3 } gts_metric;
  *  GTS_PREC_FP32: FP32 CUDA-core distances, FP64 recheck of candidates whose
  *                 FP32 distance lies within a proven error bound of the radius
  *                 or of the running k-th distance.  Candidate by candidate, or
- *                 for batches with enough (query, object) pairs in node-major
+ *                 for batches with enough (query, object) pairs and rows per
+ *                 last-level node in node-major
  *                 FP32 tiles (the table scan up to 16 dimensions); up to eight
  *                 queries over objects that are read in one pass (a GiB) take
  *                 that pass instead of the descent, if a budget of 74 bytes holds each
@@ -81,7 +82,8 @@ typedef enum { GTS_EDIT = 0, GTS_L1 = 1, GTS_L2 = 2, GTS_COS = 3 } gts_metric;
  * recheck of GTS_PREC_FP32, batched by node instead of by candidate); this
  * needs dim % 4 == 0 and 16-byte aligned query rows, else the plain path runs.
  * Edit distance is exact either way; GTS_PREC_BF16 sends batches of every size
- * through the 3-gram tiles, GTS_PREC_FP32 large ones. */
+ * through the string tiles, GTS_PREC_FP32 large ones (kNN only over strings of up to
+ * 32 letters). */
 typedef enum { GTS_PREC_FP32 = 0, GTS_PREC_BF16 = 1 } gts_precision;
 
 /* A set of objects: vectors (dim > 0) or byte strings (dim == 0).

@@ -218,7 +218,7 @@ struct Tree {
     TcCache tc;
     DBuf<double> xrn2;              // angular distance: the raw rows' sums of squares (built on first use)
     bool xrn2_ready = false;
-    DBuf<uint8_t> qg;               // strings: hashed 3-gram counts per row [n, 64] (built on first use)
+    DBuf<uint8_t> qg;               // strings: 3-gram bucket counts per row [n, 64] (built on first use)
     bool qg_ready = false;
     DBuf<uint8_t> qcode;            // their codes for the tensor-core tiles [n, 256] (built on first use)
     bool qcode_ready = false;

@@ -1,5 +1,6 @@
 // Edit-distance filtering tiles on the tensor cores: the 3-gram count bound of
-// tile_str.cu for batches whose (node rows x queries) blocks are well filled.
+// tile_str.cu for ranges whose (node rows x queries) blocks are well filled (kNN's
+// first thresholds exclude little, and every pair kept is looked up).
 //
 // The L1 distance of two strings' bucket counts, each capped at 4, is the
 // Hamming distance of their thermometer codes (bucket b, level l: one if the

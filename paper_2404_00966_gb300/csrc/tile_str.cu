@@ -5,7 +5,7 @@
 // concentrate (random-like sequences), and most (query, row) pairs of the
 // surviving leaves reach verification.  Before the bit-parallel DP, each pair
 // is tested against the 3-gram count bound: the L1 distance between the
-// strings' hashed 3-gram bucket counts is at most 6 times the edit distance
+// strings' 3-gram bucket counts (qgram.cuh) is at most 6 times the edit distance
 // (a substitution changes at most 3 of a string's 3-grams, an insertion or a
 // deletion at most 2 old and 3 new ones; summing counts into buckets and
 // capping them at 255 can only lower the L1 distance), so L1 > 6 t proves
@@ -14,7 +14,7 @@
 // vectors in registers) and the node's queries in chunks of 32 or 64 (their
 // vectors in shared memory); a pair is kept if the row's leaf survived for the
 // query, the row is visible at the query's sequence number and the bound does
-// not exclude it.  Well-filled batches take tile_qtc.cu instead.  The
+// not exclude it.  Ranges that fill the blocks take tile_qtc.cu instead.  The
 // kept pairs go on to the exact DP.
 #include "gts_impl.cuh"
 #include "metric.cuh"

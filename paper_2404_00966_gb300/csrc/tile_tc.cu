@@ -161,7 +161,7 @@ namespace {
 // x_hi (the differences are exact), rounded up; rho: their largest ratio to |x|.
 // The FP64 conversions and sums bound it, so the residuals, of which any upper
 // bound will do, are summed in FP32 rounding up: in FP64 beside the norms they took
-// SPLITMS
+// as long again (10^6 x 128: 1.65 against 0.84 ms).
 __global__ void k_split_rows(const float *__restrict__ X, int dim, int dim_p, int64_t n,
                              __nv_bfloat16 *__restrict__ Xh, __nv_bfloat16 *__restrict__ Xl,
                              float *__restrict__ n2, const int32_t *__restrict__ sel,
